@@ -10,7 +10,7 @@
 //
 //   warp 0     producer   TMA loads of this CTA's A and B halves into a kStages-deep ring; the
 //                         transaction bytes of both CTAs land on the first CTA's "full" barrier
-//   warp 1     MMA        (first CTA only) one thread issues four M256 N256 K16 MMAs per K-block
+//   warp 1     MMA        (first CTA only) an elected lane issues four M256 N256 K16 MMAs per K-block
 //                         into one of two 256-column accumulators; tcgen05.commit, delivered to
 //                         both CTAs, frees the ring slot / publishes the accumulator
 //   warps 2-9  epilogue   warp w drains lanes 32 (w mod 4) .. +31, columns 128 ((w-2)/4) .. +127
@@ -147,6 +147,19 @@ __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, volatil
       return false;
     }
   }
+}
+
+// The same wait made by a whole converged warp; the answer is the same in all of its lanes.
+__device__ __forceinline__ bool mbar_wait_warp(unsigned bar, unsigned parity, volatile int* abort_flag) {
+  if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag)) != 0;
+}
+
+// One lane of a converged warp, the same one every time.
+__device__ __forceinline__ bool elect_one() {
+  unsigned p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
 }
 
 __device__ __forceinline__ void mbar_expect_tx(unsigned bar, unsigned bytes) {
@@ -396,21 +409,29 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
 
   if (warp == 0) {
     // ------------------------------------------------ producer (both CTAs)
-    if (lane == 0) {
-      // ring position kept as (slot, round parity) and stepped, not divided out of a running count:
-      // with a slot count that is not a power of two the division is a long instruction sequence,
-      // once per K-block
-      long long kb_iter = 0;
-      int slot = 0;
-      unsigned round = 0;
-      for (int tile = first; tile < p.total_tiles && !*abort_flag; tile += stride) {
-        const TileCoord tc = tile_coord(p, tile);
-        const int s_lo = p.chain ? 0 : tc.g, s_hi = p.chain ? p.nseg : tc.g + 1;
-        for (int s = s_lo; s < s_hi; ++s) {
-          const int nkb = p.kblocks[s];
-          for (int kb = 0; kb < nkb; ++kb, ++kb_iter, slot = slot + 1 == kSt ? 0 : slot + 1, round ^= (slot == 0)) {
-            const unsigned parity = round ^ 1;
-            if (!mbar_wait(smem_addr(&bar_empty[slot]), parity, abort_flag)) goto producer_done;
+    //
+    // Both single-issue roles run as whole warps: every lane walks the loop and waits on the barriers, one
+    // elected lane issues.  Ring position, addresses and descriptors are then the same in all lanes of a
+    // converged warp and can live in uniform registers, which the copy and MMA instructions take their
+    // operands from; with one lane alone inside the loop each operand was moved there per instruction.
+    // [8192,4096] x [4096,16384] + GeLU 755 -> 709 us back to back, fused classifier forward (512 x 512 x
+    // 2^20) 489 -> 456 us, its backward 577 -> 527 us (same GPU, MMA warp and producer about half each).
+    const bool leader = elect_one();
+    // ring position kept as (slot, round parity) and stepped, not divided out of a running count:
+    // with a slot count that is not a power of two the division is a long instruction sequence,
+    // once per K-block
+    long long kb_iter = 0;
+    int slot = 0;
+    unsigned round = 0;
+    for (int tile = first; tile < p.total_tiles; tile += stride) {
+      const TileCoord tc = tile_coord(p, tile);
+      const int s_lo = p.chain ? 0 : tc.g, s_hi = p.chain ? p.nseg : tc.g + 1;
+      for (int s = s_lo; s < s_hi; ++s) {
+        const int nkb = p.kblocks[s];
+        for (int kb = 0; kb < nkb; ++kb, ++kb_iter, slot = slot + 1 == kSt ? 0 : slot + 1, round ^= (slot == 0)) {
+          const unsigned parity = round ^ 1;
+          if (!mbar_wait_warp(smem_addr(&bar_empty[slot]), parity, abort_flag)) goto producer_done;
+          if (leader) {
             const unsigned full0 = map_to_cta(smem_addr(&bar_full[slot]), 0);
             if (rank == 0) mbar_expect_tx(smem_addr(&bar_full[slot]), 2 * kStBytes);
             unsigned char* sa0 = smem + slot * kStBytes;
@@ -436,34 +457,36 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
               tma_load_2d(smem_addr(sb), &p.map_b[s], kb * BK, bcol, full0);
             }
           }
+          __syncwarp();
         }
       }
-    producer_done:
-      if (*abort_flag && rank == 0) {
-        // give the loads still in flight a bounded chance to land before the CTA goes away
-        const long long issued = kb_iter;
-        for (long long i = issued > kSt ? issued - kSt : 0; i < issued; ++i) {
-          const unsigned long long t0 = now_ns();
-          while (!mbar_try(smem_addr(&bar_full[i % kSt]), (unsigned)((i / kSt) & 1)) && now_ns() - t0 < 100000000ull) {
-          }
+    }
+  producer_done:
+    if (*abort_flag && rank == 0 && leader) {
+      // give the loads still in flight a bounded chance to land before the CTA goes away
+      const long long issued = kb_iter;
+      for (long long i = issued > kSt ? issued - kSt : 0; i < issued; ++i) {
+        const unsigned long long t0 = now_ns();
+        while (!mbar_try(smem_addr(&bar_full[i % kSt]), (unsigned)((i / kSt) & 1)) && now_ns() - t0 < 100000000ull) {
         }
       }
     }
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer (first CTA of the pair only)
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
+      const bool leader = elect_one();
       int slot = 0;
       unsigned round = 0;
       int tile_iter = 0;
       constexpr unsigned idesc = make_idesc(AT, BT);
-      for (int tile = first; tile < p.total_tiles && !*abort_flag; tile += stride, ++tile_iter) {
+      for (int tile = first; tile < p.total_tiles; tile += stride, ++tile_iter) {
         const TileCoord tc = tile_coord(p, tile);
         // Square form: the two accumulators take turns, so a tile's MMAs run while the tile before
         // it is drained.  Tall form: accumulator h belongs to m-half h of every tile; the first
         // m-half may start as soon as ITS accumulator has been drained, the second waits for its own.
         const int acc = MH == 2 ? 0 : (tile_iter & 1);
         const unsigned empty_parity = MH == 2 ? (unsigned)((tile_iter & 1) ^ 1) : (unsigned)(((tile_iter >> 1) & 1) ^ 1);
-        if (!mbar_wait(smem_addr(&bar_acc_empty[acc]), empty_parity, abort_flag)) break;
+        if (!mbar_wait_warp(smem_addr(&bar_acc_empty[acc]), empty_parity, abort_flag)) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const int s_lo = p.chain ? 0 : tc.g, s_hi = p.chain ? p.nseg : tc.g + 1;
         unsigned accumulate = 0;
@@ -471,7 +494,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
         for (int s = s_lo; s < s_hi && ok; ++s) {
           const int nkb = p.kblocks[s];
           for (int kb = 0; kb < nkb; ++kb, slot = slot + 1 == kSt ? 0 : slot + 1, round ^= (slot == 0)) {
-            if (!mbar_wait(smem_addr(&bar_full[slot]), round, abort_flag)) {
+            if (!mbar_wait_warp(smem_addr(&bar_full[slot]), round, abort_flag)) {
               ok = false;
               break;
             }
@@ -480,38 +503,43 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
             const unsigned sb = sa0 + kStA;
 #pragma unroll
             for (int h = 0; h < MH; ++h) {
-            if (MH == 2 && h == 1 && accumulate == 0) {      // first K-block of the tile: the second accumulator must be free too
-              if (!mbar_wait(smem_addr(&bar_acc_empty[1]), empty_parity, abort_flag)) {
-                ok = false;
-                break;
+              if (MH == 2 && h == 1 && accumulate == 0) {      // first K-block of the tile: the second accumulator must be free too
+                if (!mbar_wait_warp(smem_addr(&bar_acc_empty[1]), empty_parity, abort_flag)) {
+                  ok = false;
+                  break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
               }
-              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            }
-            const unsigned sa = sa0 + h * kStageA;
-            const unsigned d_tmem = tmem_base + (MH == 2 ? h : acc) * BN;
+              const unsigned sa = sa0 + h * kStageA;
+              const unsigned d_tmem = tmem_base + (MH == 2 ? h : acc) * BN;
+              if (leader) {
 #pragma unroll
-            for (int kk = 0; kk < BK / 16; ++kk) {
-              // K-major tile (A as given, B transposed): rows of 128 bytes = 64 K-elements, 8-row
-              //    groups 1024 bytes apart; 16 K-elements = 32 bytes.
-              // MN-major tile (B as given, A transposed): 64-element chunks of the M / N index
-              //    BK*128 bytes apart, 8-row K groups 1024 bytes apart; 16 K-rows = 2048 bytes.
-              // Each CTA holds its 128 of the pair's 256 rows (A) or columns (B).
-              // (shared-memory addresses are below 256 KiB and the tiles 1024-byte aligned, so the
-              //  start-address field is address >> 4 and stepping it cannot carry out of the field)
-              constexpr unsigned a_lo = desc_lo_fixed(AT ? BK * 128 : 16), b_lo = desc_lo_fixed(BT ? 16 : BK * 128);
-              constexpr unsigned hi = desc_hi_fixed(1024);
-              const unsigned long long da = desc_pack(a_lo + (sa >> 4) + kk * (AT ? 128 : 2), hi);
-              const unsigned long long db = desc_pack(b_lo + (sb >> 4) + kk * (BT ? 2 : 128), hi);
-              umma_bf16(d_tmem, da, db, idesc, kk == 0 ? accumulate : 1u);
-            }
+                for (int kk = 0; kk < BK / 16; ++kk) {
+                  // K-major tile (A as given, B transposed): rows of 128 bytes = 64 K-elements, 8-row
+                  //    groups 1024 bytes apart; 16 K-elements = 32 bytes.
+                  // MN-major tile (B as given, A transposed): 64-element chunks of the M / N index
+                  //    BK*128 bytes apart, 8-row K groups 1024 bytes apart; 16 K-rows = 2048 bytes.
+                  // Each CTA holds its 128 of the pair's 256 rows (A) or columns (B).
+                  // (shared-memory addresses are below 256 KiB and the tiles 1024-byte aligned, so the
+                  //  start-address field is address >> 4 and stepping it cannot carry out of the field)
+                  constexpr unsigned a_lo = desc_lo_fixed(AT ? BK * 128 : 16), b_lo = desc_lo_fixed(BT ? 16 : BK * 128);
+                  constexpr unsigned hi = desc_hi_fixed(1024);
+                  const unsigned long long da = desc_pack(a_lo + (sa >> 4) + kk * (AT ? 128 : 2), hi);
+                  const unsigned long long db = desc_pack(b_lo + (sb >> 4) + kk * (BT ? 2 : 128), hi);
+                  umma_bf16(d_tmem, da, db, idesc, kk == 0 ? accumulate : 1u);
+                }
+              }
+              __syncwarp();
             }
             if (!ok) break;
             accumulate = 1;
-            umma_commit_pair(smem_addr(&bar_empty[slot]));   // slot reusable in both CTAs
+            if (leader) umma_commit_pair(smem_addr(&bar_empty[slot]));   // slot reusable in both CTAs
+            __syncwarp();
           }
         }
         if (!ok) break;
-        umma_commit_pair(smem_addr(&bar_acc_full[acc]));      // accumulator(s) complete in both CTAs
+        if (leader) umma_commit_pair(smem_addr(&bar_acc_full[acc]));      // accumulator(s) complete in both CTAs
+        __syncwarp();
       }
     }
   } else {
