@@ -1,10 +1,11 @@
 // MatMul under the SBP signatures of Table 1: signature rule -> grouped-GEMM plan -> kernel.
 //
-// Two kernels execute a plan:
+// Three kernels execute a plan:
 //   * the tensor-core kernel (matmul_tc.cu): bf16 operands, fp32 accumulation in tensor
 //     memory, TMA-fed tiles; taken whenever the shapes meet its alignment rules;
-//   * the FMA kernel in this file: fp32 operands (and bf16 operands whose shapes the tensor
-//     core kernel cannot take), fp32 accumulation with fused multiply-adds, k ascending.
+//   * the fp32 kernel (matmul_f32.cu): fp32 operands, fp32 fused multiply-adds, k ascending;
+//   * the FMA kernel in this file: bf16 operands that the tensor-core kernel cannot take and that no
+//     workspace was given for, same arithmetic.
 #include <cuda_bf16.h>
 
 #include "bounds_check.h"
@@ -17,6 +18,8 @@ namespace sbp {
 // when the plan does not meet the tensor-core kernel's rules; the caller then falls back
 // to the FMA kernel.
 sbp_status launch_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, cudaStream_t st, bool* taken);
+// Defined in matmul_f32.cu: fp32 operands and result.
+sbp_status launch_matmul_f32(const MatmulPlan& plan, cudaStream_t st);
 // Defined in softmax_xent.cu: reduces the per-chunk partials left by the fused classifier kernel.
 sbp_status launch_xent_finish(float* part_m, float* part_s, float* part_t, int parts, long long rows, float* stage,
                               sbp_tensor* loss, sbp_tensor* row_max, sbp_tensor* row_sum, int k, cudaStream_t st);
@@ -33,13 +36,6 @@ int tc_route(long long tiles_sq, long long tiles_tall, long long kb, int pairs, 
 __device__ __forceinline__ float gelu_erf(float v) { return 0.5f * v * (1.0f + erff(v * 0.70710678118654752440f)); }
 
 template <typename T>
-__device__ __forceinline__ float ld_f32(const T* p);
-template <>
-__device__ __forceinline__ float ld_f32<float>(const float* p) { return *p; }
-template <>
-__device__ __forceinline__ float ld_f32<__nv_bfloat16>(const __nv_bfloat16* p) { return __bfloat162float(*p); }
-
-template <typename T>
 __device__ __forceinline__ void st_out(T* p, float v);
 template <>
 __device__ __forceinline__ void st_out<float>(float* p, float v) { *p = v; }
@@ -48,8 +44,9 @@ __device__ __forceinline__ void st_out<__nv_bfloat16>(__nv_bfloat16* p, float v)
 
 constexpr int BM = 64, BN = 64, BK = 16;
 
-template <typename TI, typename TO>
+template <typename TO>
 __global__ void __launch_bounds__(256) matmul_fma_kernel(const __grid_constant__ MatmulPlan p) {
+  using TI = __nv_bfloat16;
   const int g = blockIdx.z;
   const long long M = p.m[g], N = p.n[g];
   const long long m0 = (long long)blockIdx.y * BM, n0 = (long long)blockIdx.x * BN;
@@ -75,23 +72,23 @@ __global__ void __launch_bounds__(256) matmul_fma_kernel(const __grid_constant__
       if (p.a_trans) {
         for (int e = threadIdx.x; e < BM * BK; e += 256) {
           const int c = e / BM, r = e % BM;   // consecutive threads walk the stored rows
-          As[c][r] = (m0 + r < M && k0 + c < K && SBP_GUARD(A + r * a_rs + (k0 + c) * a_ks, sizeof(TI))) ? ld_f32<TI>(A + r * a_rs + (k0 + c) * a_ks) : 0.f;
+          As[c][r] = (m0 + r < M && k0 + c < K && SBP_GUARD(A + r * a_rs + (k0 + c) * a_ks, sizeof(TI))) ? __bfloat162float(*(A + r * a_rs + (k0 + c) * a_ks)) : 0.f;
         }
       } else {
         for (int e = threadIdx.x; e < BM * BK; e += 256) {
           const int r = e / BK, c = e % BK;
-          As[c][r] = (m0 + r < M && k0 + c < K && SBP_GUARD(A + r * a_rs + (k0 + c) * a_ks, sizeof(TI))) ? ld_f32<TI>(A + r * a_rs + (k0 + c) * a_ks) : 0.f;
+          As[c][r] = (m0 + r < M && k0 + c < K && SBP_GUARD(A + r * a_rs + (k0 + c) * a_ks, sizeof(TI))) ? __bfloat162float(*(A + r * a_rs + (k0 + c) * a_ks)) : 0.f;
         }
       }
       if (p.b_trans) {
         for (int e = threadIdx.x; e < BK * BN; e += 256) {
           const int c = e / BK, r = e % BK;
-          Bs[r][c] = (k0 + r < K && n0 + c < N && SBP_GUARD(Bm + (k0 + r) * b_ks + c * b_cs, sizeof(TI))) ? ld_f32<TI>(Bm + (k0 + r) * b_ks + c * b_cs) : 0.f;
+          Bs[r][c] = (k0 + r < K && n0 + c < N && SBP_GUARD(Bm + (k0 + r) * b_ks + c * b_cs, sizeof(TI))) ? __bfloat162float(*(Bm + (k0 + r) * b_ks + c * b_cs)) : 0.f;
         }
       } else {
         for (int e = threadIdx.x; e < BK * BN; e += 256) {
           const int r = e / BN, c = e % BN;
-          Bs[r][c] = (k0 + r < K && n0 + c < N && SBP_GUARD(Bm + (k0 + r) * b_ks + c * b_cs, sizeof(TI))) ? ld_f32<TI>(Bm + (k0 + r) * b_ks + c * b_cs) : 0.f;
+          Bs[r][c] = (k0 + r < K && n0 + c < N && SBP_GUARD(Bm + (k0 + r) * b_ks + c * b_cs, sizeof(TI))) ? __bfloat162float(*(Bm + (k0 + r) * b_ks + c * b_cs)) : 0.f;
         }
       }
       __syncthreads();
@@ -139,14 +136,8 @@ static sbp_status launch_fma(const MatmulPlan& p, cudaStream_t st) {
   if (gx > 0x7fffffffLL || gy > 65535) return fail(SBP_ERR_UNSUPPORTED, "matrix too large for the FMA kernel");
   dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)p.ngroups);
   SBP_BOUNDS_UPLOAD(st);
-  if (p.in_dtype == SBP_F32 && p.out_dtype == SBP_F32)
-    matmul_fma_kernel<float, float><<<grid, 256, 0, st>>>(p);
-  else if (p.in_dtype == SBP_BF16 && p.out_dtype == SBP_BF16)
-    matmul_fma_kernel<__nv_bfloat16, __nv_bfloat16><<<grid, 256, 0, st>>>(p);
-  else if (p.in_dtype == SBP_BF16 && p.out_dtype == SBP_F32)
-    matmul_fma_kernel<__nv_bfloat16, float><<<grid, 256, 0, st>>>(p);
-  else
-    return fail(SBP_ERR_DTYPE, "F32 operands need an F32 result");
+  if (p.out_dtype == SBP_BF16) matmul_fma_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(p);
+  else matmul_fma_kernel<float><<<grid, 256, 0, st>>>(p);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "matmul launch");
   count_launch();
@@ -581,6 +572,7 @@ sbp_status sbp_matmul(const sbp_tensor* x, const sbp_tensor* w, sbp_tensor* y, u
   SBP_BOUNDS_TENSOR(w);
   SBP_BOUNDS_TENSOR(y);
   SBP_BOUNDS_ADD(ws, ws_bytes);
+  if (plan.in_dtype == SBP_F32) return launch_matmul_f32(plan, stream);
   bool taken = false;
   st = launch_matmul_tc(plan, nullptr, stream, &taken);
   if (taken) return st;

@@ -1,0 +1,400 @@
+// fp32 MatMul: executes a grouped-GEMM plan (matmul_plan.h) on the FMA pipes.
+//
+// Every element of the result is one chain of fused multiply-adds in fp32, k ascending, segments in rank
+// order; there is no reduced-precision product.  Bound: the FMA pipe (128 lanes per SM and clock, 74
+// TFLOP/s at 1.965 GHz) once a product fills the device, the latency of load -> shared memory -> first
+// FMA and the launch for the small ones.
+//
+//   * A CTA of 256 threads owns a (16 TM) x (16 TN) tile, TM x TN elements per thread.  Multiply-adds are
+//     issued as packed pairs (fma.rn.f32x2, each half an IEEE fma), which leaves half of the issue slots to
+//     the shared-memory reads.
+//   * Operands arrive through a kStages-deep ring of 16-deep K-slices filled with asynchronous copies: 16
+//     bytes each where base, leading dimension and offsets allow, else 4 bytes each; positions past an
+//     edge are zero-filled by the copy.  A slice keeps the order it has in memory -- K contiguous or M / N
+//     contiguous -- so nothing is transposed on the way and both stored forms of either operand cost the
+//     same.
+//   * A tile whose K is long and whose device is otherwise idle is split along K over the CTAs of a
+//     cluster (S = 2, 4, 8): each CTA runs its range of slices, then reads the others' partial sums of its
+//     own rows from their shared memory and adds them in slice order.  No workspace, no atomics, the same
+//     bits every time.
+#include <cuda_runtime.h>
+
+#include <atomic>
+
+#include "bounds_check.h"
+#include "matmul_plan.h"
+#include "sbp_internal.h"
+
+namespace sbp {
+
+namespace {
+
+constexpr int kBK = 16;          // K-slice
+constexpr int kStages = 4;
+constexpr int kThreads = 256;
+constexpr int kKPitch = kBK + 4; // floats per row of a K-contiguous slice: 16-byte aligned, and 4 (8) neighbouring
+                                 // rows read at once fall into different banks
+
+struct F32Params {
+  MatmulPlan plan;
+  int splits;                    // CTAs per tile (cluster size)
+  int a_vec, b_vec, y_vec;       // 16-byte copies / stores are possible everywhere
+};
+
+__device__ __forceinline__ void cp_async16(unsigned dst, const void* src, unsigned bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async4(unsigned dst, const void* src, unsigned bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(unsigned long long v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ void fma2(unsigned long long& acc, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ float gelu_erf(float v) { return 0.5f * v * (1.0f + erff(v * 0.70710678118654752440f)); }
+
+template <int EXT, bool KC>
+constexpr int slice_floats() {
+  return KC ? EXT * kKPitch : kBK * EXT;
+}
+
+// One slice of an operand: EXT positions of its M / N index x kBK of K.  g points at position (0, 0) of
+// the slice; ext / kk are how many positions / K-steps of it lie inside the operand (any may be <= 0).
+// KC: K is contiguous in memory (and in shared memory: rows of kKPitch floats), else the M / N index is.
+template <int EXT, bool KC>
+__device__ __forceinline__ void load_slice(float* s, const float* g, long long ld, long long ext, long long kk, bool vec, int tid) {
+  const unsigned base = (unsigned)__cvta_generic_to_shared(s);
+  constexpr int kRows = KC ? EXT : kBK, kCols = KC ? kBK : EXT, kPitch = KC ? kKPitch : EXT;
+  const long long rows = KC ? ext : kk, cols = KC ? kk : ext;
+  if (vec) {
+#pragma unroll
+    for (int j = 0; j < kRows * kCols / 4 / kThreads; ++j) {
+      const int idx = tid + j * kThreads, r = idx / (kCols / 4), c = idx % (kCols / 4) * 4;
+      const long long left = r < rows ? cols - c : 0;
+      int n = left >= 4 ? 4 : (left > 0 ? (int)left : 0);
+      const float* src = g + (long long)r * ld + c;
+      if (n > 0 && !SBP_GUARD(src, (size_t)n * 4)) n = 0;
+      cp_async16(base + (unsigned)(r * kPitch + c) * 4, n > 0 ? src : g, (unsigned)n * 4);
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < kRows * kCols / kThreads; ++j) {
+      const int idx = tid + j * kThreads, r = idx / kCols, c = idx % kCols;
+      const float* src = g + (long long)r * ld + c;
+      const bool in = r < rows && c < cols && SBP_GUARD(src, 4);
+      cp_async4(base + (unsigned)(r * kPitch + c) * 4, in ? src : g, in ? 4u : 0u);
+    }
+  }
+}
+
+// AT / BT: the operand is stored transposed.  A as given and B transposed are K-contiguous.
+template <int TM, int TN, int AT, int BT>
+__global__ void __launch_bounds__(kThreads, TM == 8 ? 2 : 3) matmul_f32_kernel(const __grid_constant__ F32Params P) {
+  constexpr int BM = 16 * TM, BN = 16 * TN;
+  constexpr bool AKC = !AT, BKC = BT;
+  constexpr int kA = slice_floats<BM, AKC>(), kB = slice_floats<BN, BKC>();
+  constexpr int KS = TM == 8 ? 2 : 4;              // K-steps whose A values a thread holds at once
+  extern __shared__ __align__(16) float smem[];
+  const MatmulPlan& p = P.plan;
+  const int g = blockIdx.z;
+  const int splits = P.splits, slice = (int)(blockIdx.x % (unsigned)splits);
+  const long long M = p.m[g], N = p.n[g];
+  const long long m0 = (long long)blockIdx.y * BM, n0 = (long long)(blockIdx.x / (unsigned)splits) * BN;
+  SBP_PDL_WAIT();
+  if (m0 >= M || n0 >= N) return;                  // the whole cluster
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ty = (warp >> 1) * 4 + (lane >> 3), tx = (warp & 1) * 8 + (lane & 7);
+  // element (i, j) of a thread: strided over a K-contiguous slice's rows, in runs of four otherwise
+  auto row_of = [&](int i) { return AKC ? i * 16 + ty : (i / 4) * 64 + ty * 4 + (i & 3); };
+  auto col_of = [&](int j) { return BKC ? j * 16 + tx : (j / 4) * 64 + tx * 4 + (j & 3); };
+
+  // this CTA's range of K-slices over all segments
+  const int s_lo = p.chain ? 0 : g, s_hi = p.chain ? p.nseg : g + 1;
+  long long total = 0;
+  for (int s = s_lo; s < s_hi; ++s) total += (p.kseg[s] + kBK - 1) / kBK;
+  const long long it0 = total * slice / splits, it1 = total * (slice + 1) / splits;
+  const int iters = (int)(it1 - it0);
+  int ls = s_lo;                                   // the loader's position: segment and K inside it
+  long long lk = it0 * kBK;
+  {
+    long long skip = it0;
+    while (ls < s_hi) {
+      const long long n = (p.kseg[ls] + kBK - 1) / kBK;
+      if (skip < n) break;
+      skip -= n;
+      ++ls;
+    }
+    lk = skip * kBK;
+  }
+  auto load_next = [&](int stage) {
+    while (ls < s_hi && lk >= p.kseg[ls]) { ++ls; lk = 0; }      // also steps over empty segments
+    const long long lda = p.lda[ls], ldb = p.ldb[ls], left = p.kseg[ls] - lk;
+    const float* A = static_cast<const float*>(p.a[ls]) + (AT ? lk * lda + p.row_off[g] + m0 : (p.row_off[g] + m0) * lda + lk);
+    const float* B = static_cast<const float*>(p.b[ls]) + (BT ? (p.col_off[g] + n0) * ldb + lk : lk * ldb + p.col_off[g] + n0);
+    float* sa = smem + stage * (kA + kB);
+    load_slice<BM, AKC>(sa, A, lda, M - m0, left, P.a_vec != 0, tid);
+    load_slice<BN, BKC>(sa + kA, B, ldb, N - n0, left, P.b_vec != 0, tid);
+    lk += kBK;
+  };
+
+  unsigned long long acc[TM][TN / 2];
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TN / 2; ++j) acc[i][j] = 0ull;
+
+#pragma unroll
+  for (int st = 0; st < kStages - 1; ++st) {
+    if (st < iters) load_next(st);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  int stage = 0, fill = kStages - 1;
+  for (int it = 0; it < iters; ++it) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
+    __syncthreads();                               // slice `it` is there, and everyone is done with the one before it
+    if (it + kStages - 1 < iters) load_next(fill);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const float* sa = smem + stage * (kA + kB);
+    const float* sb = sa + kA;
+#pragma unroll
+    for (int k0 = 0; k0 < kBK; k0 += KS) {
+      float a[TM][KS], b[TN][KS];
+      if constexpr (AKC) {
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+          if constexpr (KS == 4) *reinterpret_cast<float4*>(a[i]) = *reinterpret_cast<const float4*>(sa + row_of(i) * kKPitch + k0);
+          else *reinterpret_cast<float2*>(a[i]) = *reinterpret_cast<const float2*>(sa + row_of(i) * kKPitch + k0);
+        }
+      }
+      if constexpr (BKC) {
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+          if constexpr (KS == 4) *reinterpret_cast<float4*>(b[j]) = *reinterpret_cast<const float4*>(sb + col_of(j) * kKPitch + k0);
+          else *reinterpret_cast<float2*>(b[j]) = *reinterpret_cast<const float2*>(sb + col_of(j) * kKPitch + k0);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < KS; ++k) {
+        float ak[TM], bk[TN];
+#pragma unroll
+        for (int i = 0; i < TM; i += 4) {
+          if constexpr (AKC) { ak[i] = a[i][k]; ak[i + 1] = a[i + 1][k]; ak[i + 2] = a[i + 2][k]; ak[i + 3] = a[i + 3][k]; }
+          else *reinterpret_cast<float4*>(ak + i) = *reinterpret_cast<const float4*>(sa + (k0 + k) * BM + row_of(i));
+        }
+#pragma unroll
+        for (int j = 0; j < TN; j += 4) {
+          if constexpr (BKC) { bk[j] = b[j][k]; bk[j + 1] = b[j + 1][k]; bk[j + 2] = b[j + 2][k]; bk[j + 3] = b[j + 3][k]; }
+          else *reinterpret_cast<float4*>(bk + j) = *reinterpret_cast<const float4*>(sb + (k0 + k) * BN + col_of(j));
+        }
+        unsigned long long bp[TN / 2];
+#pragma unroll
+        for (int j = 0; j < TN / 2; ++j) bp[j] = pack2(bk[2 * j], bk[2 * j + 1]);
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+          const unsigned long long ap = pack2(ak[i], ak[i]);
+#pragma unroll
+          for (int j = 0; j < TN / 2; ++j) fma2(acc[i][j], ap, bp[j]);
+        }
+      }
+    }
+    stage = stage + 1 == kStages ? 0 : stage + 1;
+    fill = fill + 1 == kStages ? 0 : fill + 1;
+  }
+
+  // The next kernel's CTAs are let in only now: set up earlier, they take the free slots of the SMs that
+  // finish first and the next product runs unevenly (1000 x 1500 x 777 over four shards, back to back:
+  // 171 us released at the start, 99 us here).
+  SBP_PDL_RELEASE();
+
+  // four neighbouring results of one row: GeLU, then the result and its replicas
+  float* const y = static_cast<float*>(p.y[g]);
+  const long long ldy = p.ldy[g];
+  const int n_out = (g == 0 ? p.n_rep : 0) + 1;
+  auto store4 = [&](long long r, long long c, const float (&v)[4], int step) {
+    if (r >= M) return;
+    float o[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) o[e] = p.gelu ? gelu_erf(v[e]) : v[e];
+    for (int q = 0; q < n_out; ++q) {
+      float* at = (q == 0 ? y : static_cast<float*>(p.y_rep[q - 1])) + r * ldy + c;
+      if (step == 1 && P.y_vec && c + 3 < N) {
+        if (SBP_GUARD(at, 16)) *reinterpret_cast<float4*>(at) = make_float4(o[0], o[1], o[2], o[3]);
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (c + e * step < N && SBP_GUARD(at + e * step, 4)) at[e * step] = o[e];
+      }
+    }
+  };
+
+  if (splits == 1) {
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < TN; j += 4) {
+        float v[4];
+        unpack2(acc[i][j / 2], v[0], v[1]);
+        unpack2(acc[i][j / 2 + 1], v[2], v[3]);
+        store4(m0 + row_of(i), n0 + col_of(j), v, BKC ? 16 : 1);
+      }
+    return;
+  }
+
+  // K was split: park the partial tile, then add up the rows this CTA answers for, slice by slice.
+  // (The ring holds the tile: kStages slices of (BM + BN) x 16 are at least BM x BN floats.)
+  static_assert(kStages * (kA + kB) >= BM * BN, "the ring has to hold the partial tile");
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; j += 4) {
+      float v[4];
+      unpack2(acc[i][j / 2], v[0], v[1]);
+      unpack2(acc[i][j / 2 + 1], v[2], v[3]);
+      float* at = smem + row_of(i) * BN + col_of(j);
+      if constexpr (BKC) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) at[e * 16] = v[e];
+      } else {
+        *reinterpret_cast<float4*>(at) = make_float4(v[0], v[1], v[2], v[3]);
+      }
+    }
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  const int rows_each = BM / splits;
+  const unsigned mine = (unsigned)__cvta_generic_to_shared(smem);
+  for (int idx = tid; idx < rows_each * (BN / 4); idx += kThreads) {
+    const int r = slice * rows_each + idx / (BN / 4), c = idx % (BN / 4) * 4;
+    if (m0 + r >= M || n0 + c >= N) continue;
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int q = 0; q < splits; ++q) {
+      unsigned remote;
+      float x0, x1, x2, x3;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(mine + (unsigned)(r * BN + c) * 4), "r"(q));
+      asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x0), "=f"(x1), "=f"(x2), "=f"(x3) : "r"(remote) : "memory");
+      if (q == 0) { v[0] = x0; v[1] = x1; v[2] = x2; v[3] = x3; }
+      else { v[0] += x0; v[1] += x1; v[2] += x2; v[3] += x3; }
+    }
+    store4(m0 + r, n0 + c, v, 1);
+  }
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");      // nobody leaves while its tile may still be read
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+template <int TM, int TN, int AT, int BT>
+cudaError_t launch_form(const F32Params& P, dim3 grid, cudaStream_t st) {
+  constexpr int kSmem = kStages * (slice_floats<16 * TM, !AT>() + slice_floats<16 * TN, (bool)BT>()) * 4;
+  if (kSmem > 48 * 1024) {
+    static std::atomic<unsigned long long> opted{0};      // one bit per device
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (dev >= 64 || !(opted.load(std::memory_order_relaxed) & bit)) {
+      e = cudaFuncSetAttribute(matmul_f32_kernel<TM, TN, AT, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+      if (e != cudaSuccess) return e;
+      if (dev < 64) opted.fetch_or(bit, std::memory_order_relaxed);
+    }
+  }
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = kSmem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)P.splits;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = P.splits > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, matmul_f32_kernel<TM, TN, AT, BT>, P);
+}
+
+template <int TM, int TN>
+cudaError_t launch_stored(const F32Params& P, dim3 grid, cudaStream_t st) {
+  switch ((P.plan.a_trans ? 2 : 0) | (P.plan.b_trans ? 1 : 0)) {
+    case 0: return launch_form<TM, TN, 0, 0>(P, grid, st);
+    case 1: return launch_form<TM, TN, 0, 1>(P, grid, st);
+    case 2: return launch_form<TM, TN, 1, 0>(P, grid, st);
+    default: return launch_form<TM, TN, 1, 1>(P, grid, st);
+  }
+}
+
+bool aligned16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
+
+}  // namespace
+
+sbp_status launch_matmul_f32(const MatmulPlan& plan, cudaStream_t st) {
+  F32Params P;
+  P.plan = plan;
+  P.a_vec = P.b_vec = P.y_vec = 1;
+  long long iters = 0, mmax = 0, nmax = 0;
+  for (int s = 0; s < plan.nseg; ++s) {
+    if (!plan.chain && s >= plan.ngroups) continue;
+    if (!aligned16(plan.a[s]) || plan.lda[s] % 4 != 0) P.a_vec = 0;
+    if (!aligned16(plan.b[s]) || plan.ldb[s] % 4 != 0) P.b_vec = 0;
+    const long long n = (plan.kseg[s] + kBK - 1) / kBK;
+    iters = plan.chain ? iters + n : (n > iters ? n : iters);
+  }
+  for (int g = 0; g < plan.ngroups; ++g) {
+    mmax = plan.m[g] > mmax ? plan.m[g] : mmax;
+    nmax = plan.n[g] > nmax ? plan.n[g] : nmax;
+    if (plan.a_trans && plan.row_off[g] % 4 != 0) P.a_vec = 0;
+    if (!plan.b_trans && plan.col_off[g] % 4 != 0) P.b_vec = 0;
+    if (!aligned16(plan.y[g]) || plan.ldy[g] % 4 != 0) P.y_vec = 0;
+  }
+  for (int q = 0; q < plan.n_rep; ++q)
+    if (!aligned16(plan.y_rep[q])) P.y_vec = 0;
+  if (mmax == 0 || nmax == 0) return SBP_OK;
+  if (iters > 0x7fffffffLL) return fail(SBP_ERR_UNSUPPORTED, "contraction too long for one launch");
+
+  // Which tile and how many CTAs per tile: the smallest estimated time, in clocks.  Measured per K-slice
+  // of 16 (2048 clocks of the FMA pipe for a 128 x 128 tile, 512 for 64 x 64): the large tile takes 3590
+  // clocks alone on its SM and 3170 each once two share one; the small one 1500 alone, 1230 each for two,
+  // 1075 each from three.  A round of CTAs costs about 4000 clocks of launch and pipeline fill, a split
+  // its exchange through distributed shared memory.  (us, this rule / the other choices: 1000 x 1500 x 777
+  // on four shards 92 / 98-189, 700 x 2000 x 700 81 / 88-232, 100 x 2000 x 100 16 / 28-226.)
+  const int sms = 148;
+  int best_t = 0, best_s = 1;
+  double best = 1e300;
+  for (int t = 0; t < 2; ++t) {
+    const int b = t == 0 ? 128 : 64;
+    long long tiles = 0;
+    for (int g = 0; g < plan.ngroups; ++g) tiles += ((plan.m[g] + b - 1) / b) * ((plan.n[g] + b - 1) / b);
+    if ((mmax + b - 1) / b > 65535) continue;
+    for (int s = 1; s <= 8; s *= 2) {
+      if (s > 1 && iters < s) break;
+      const double per_sm = (double)((tiles * s + sms - 1) / sms), resident = t == 0 ? 2 : 3;
+      const double it = (double)((iters + s - 1) / s);
+      const double each = t == 0 ? (per_sm > 1 ? 3170 : 3590) : (per_sm > 2 ? 1075 : (per_sm > 1 ? 1230 : 1500));
+      const double exchange = s == 1 ? 0 : (t == 0 ? 4000 : 1000 + 450 * s);
+      const double rounds = (double)(long long)((per_sm + resident - 1) / resident);
+      const double cost = it * per_sm * each + rounds * (4000 + exchange);
+      if (cost < best) { best = cost; best_t = t; best_s = s; }
+    }
+  }
+  if (best == 1e300) return fail(SBP_ERR_UNSUPPORTED, "matrix too large for the FMA kernel");
+  const int b = best_t == 0 ? 128 : 64;
+  P.splits = best_s;
+  const long long gx = (nmax + b - 1) / b * best_s;
+  if (gx > 0x7fffffffLL) return fail(SBP_ERR_UNSUPPORTED, "matrix too large for the FMA kernel");
+  const dim3 grid((unsigned)gx, (unsigned)((mmax + b - 1) / b), (unsigned)plan.ngroups);
+  SBP_BOUNDS_UPLOAD(st);
+  const cudaError_t e = best_t == 0 ? launch_stored<8, 8>(P, grid, st) : launch_stored<4, 4>(P, grid, st);
+  if (e != cudaSuccess) return cuda_fail(e, "matmul launch");
+  count_launch();
+  return SBP_OK;
+}
+
+}  // namespace sbp
