@@ -1,4 +1,5 @@
-"""ctypes binding of include/sbp.h.  Argument marshalling only."""
+"""Binding of include/sbp.h.  Argument marshalling only: ctypes for queries and rarely made calls, the
+native module built from csrc/binding_native.cpp for the entry points a program makes at every step."""
 from __future__ import annotations
 
 import ctypes as C
@@ -137,6 +138,28 @@ def load_library():
     lib.sbp_embedding_backward.argtypes = [T, T, T, C.c_void_p, C.c_void_p]
     _LIB = lib
     return lib
+
+
+# Entry points called through the native module, in the order its bind() takes them.
+_NATIVE_ENTRIES = ("sbp_boxing", "sbp_boxing_shard", "sbp_matmul", "sbp_softmax_xent", "sbp_softmax_xent_static",
+                   "sbp_softmax_xent_backward", "sbp_matmul_softmax_xent", "sbp_matmul_softmax_xent_backward",
+                   "sbp_embedding", "sbp_embedding_backward")
+_NATIVE = None
+
+
+def _native():
+    """The native module, bound to the library this process loaded.  Raises if it has not been built."""
+    global _NATIVE
+    if _NATIVE is None:
+        lib = load_library()
+        try:
+            from . import _native as mod
+        except ImportError as e:
+            raise RuntimeError("the native part of the binding is missing or does not load "
+                               f"({e}): build it with `python -m paper_2110_15032_b200.build`") from e
+        mod.bind(*(C.cast(getattr(lib, n), C.c_void_p).value for n in _NATIVE_ENTRIES))
+        _NATIVE = mod
+    return _NATIVE
 
 
 def _check(status: int):
@@ -342,15 +365,17 @@ def sbp_boxing_set_copy_engine(engine: int) -> None:
 
 
 def sbp_boxing(src: SbpTensor, dst: SbpTensor, stream=None) -> None:
-    a, b = src._c(), dst._c()
-    _check(load_library().sbp_boxing(C.byref(a), C.byref(b), _stream_ptr(stream)))
+    st = (_NATIVE or _native()).boxing(src, dst, stream)
+    if st:
+        _check(st)
 
 
 def sbp_boxing_shard(src: SbpTensor, dst: SbpTensor, dst_shard: int, stream=None) -> None:
     """Only destination local tensor `dst_shard` of the boxing op (what one device of the
     destination placement executes); the other entries of dst.locals may be None."""
-    a, b = src._c(), dst._c()
-    _check(load_library().sbp_boxing_shard(C.byref(a), C.byref(b), int(dst_shard), _stream_ptr(stream)))
+    st = (_NATIVE or _native()).boxing_shard(src, dst, int(dst_shard), stream)
+    if st:
+        _check(st)
 
 
 def sbp_boxing_host_workspace_bytes(src_host: SbpTensor, dst_host: SbpTensor) -> int:
@@ -406,10 +431,9 @@ def sbp_matmul_workspace_bytes(x: SbpTensor, w: SbpTensor, y: SbpTensor, flags: 
 
 def sbp_matmul(x: SbpTensor, w: SbpTensor, y: SbpTensor, flags: int = 0,
                ws: Optional[torch.Tensor] = None, stream=None) -> None:
-    a, b, c = x._c(), w._c(), y._c()
-    wp = C.c_void_p(ws.data_ptr()) if ws is not None else C.c_void_p(0)
-    wb = ws.numel() * ws.element_size() if ws is not None else 0
-    _check(load_library().sbp_matmul(C.byref(a), C.byref(b), C.byref(c), flags, wp, wb, _stream_ptr(stream)))
+    st = (_NATIVE or _native()).matmul(x, w, y, flags, ws, stream)
+    if st:
+        _check(st)
 
 
 def sbp_softmax_xent_workspace_bytes(logits: SbpTensor) -> int:
@@ -420,13 +444,9 @@ def sbp_softmax_xent_workspace_bytes(logits: SbpTensor) -> int:
 def sbp_softmax_xent(logits: SbpTensor, labels: SbpTensor, loss: SbpTensor,
                      row_max: Optional[SbpTensor], row_sum: Optional[SbpTensor],
                      ws: torch.Tensor, stream=None) -> None:
-    a, b, c = logits._c(), labels._c(), loss._c()
-    m = row_max._c() if row_max is not None else None
-    s = row_sum._c() if row_sum is not None else None
-    _check(load_library().sbp_softmax_xent(
-        C.byref(a), C.byref(b), C.byref(c),
-        C.byref(m) if m is not None else None, C.byref(s) if s is not None else None,
-        C.c_void_p(ws.data_ptr()), ws.numel() * ws.element_size(), _stream_ptr(stream)))
+    st = (_NATIVE or _native()).softmax_xent(logits, labels, loss, row_max, row_sum, ws, stream)
+    if st:
+        _check(st)
 
 
 def sbp_matmul_softmax_xent_workspace_bytes(features: SbpTensor, weight: SbpTensor) -> int:
@@ -437,29 +457,24 @@ def sbp_matmul_softmax_xent_workspace_bytes(features: SbpTensor, weight: SbpTens
 def sbp_matmul_softmax_xent(features: SbpTensor, weight: SbpTensor, labels: SbpTensor, loss: SbpTensor,
                             row_max: Optional[SbpTensor], row_sum: Optional[SbpTensor],
                             ws: torch.Tensor, stream=None) -> None:
-    a, b, l, c = features._c(), weight._c(), labels._c(), loss._c()
-    m = row_max._c() if row_max is not None else None
-    s = row_sum._c() if row_sum is not None else None
-    _check(load_library().sbp_matmul_softmax_xent(
-        C.byref(a), C.byref(b), C.byref(l), C.byref(c),
-        C.byref(m) if m is not None else None, C.byref(s) if s is not None else None,
-        C.c_void_p(ws.data_ptr()), ws.numel() * ws.element_size(), _stream_ptr(stream)))
-
+    st = (_NATIVE or _native()).matmul_softmax_xent(features, weight, labels, loss, row_max, row_sum, ws, stream)
+    if st:
+        _check(st)
 
 
 def sbp_matmul_softmax_xent_backward(features: SbpTensor, weight: SbpTensor, labels: SbpTensor, row_max: SbpTensor,
                                      row_sum: SbpTensor, grad_logits: SbpTensor, stream=None) -> None:
     """softmax(F W) - onehot written as S(1) without the logits ever being stored."""
-    a, w, l, m, s, g = (features._c(), weight._c(), labels._c(), row_max._c(), row_sum._c(), grad_logits._c())
-    _check(load_library().sbp_matmul_softmax_xent_backward(C.byref(a), C.byref(w), C.byref(l), C.byref(m), C.byref(s),
-                                                           C.byref(g), _stream_ptr(stream)))
+    st = (_NATIVE or _native()).matmul_softmax_xent_backward(features, weight, labels, row_max, row_sum, grad_logits, stream)
+    if st:
+        _check(st)
 
 
 def sbp_softmax_xent_backward(logits: SbpTensor, labels: SbpTensor, row_max: SbpTensor, row_sum: SbpTensor,
                               grad_logits: SbpTensor, stream=None) -> None:
-    a, b, m, s, g = logits._c(), labels._c(), row_max._c(), row_sum._c(), grad_logits._c()
-    _check(load_library().sbp_softmax_xent_backward(C.byref(a), C.byref(b), C.byref(m), C.byref(s), C.byref(g),
-                                                    _stream_ptr(stream)))
+    st = (_NATIVE or _native()).softmax_xent_backward(logits, labels, row_max, row_sum, grad_logits, stream)
+    if st:
+        _check(st)
 
 
 def sbp_softmax_xent_static(logits: SbpTensor, labels: SbpTensor, loss: SbpTensor,
@@ -468,25 +483,20 @@ def sbp_softmax_xent_static(logits: SbpTensor, labels: SbpTensor, loss: SbpTenso
     """sbp_softmax_xent without a workspace argument: the partial vectors live in an array
     built into the library, for callers that cannot allocate device memory.  See
     include/sbp.h for the size limit and the sharing rules."""
-    a, b, c = logits._c(), labels._c(), loss._c()
-    m = row_max._c() if row_max is not None else None
-    s = row_sum._c() if row_sum is not None else None
-    _check(load_library().sbp_softmax_xent_static(
-        C.byref(a), C.byref(b), C.byref(c),
-        C.byref(m) if m is not None else None, C.byref(s) if s is not None else None,
-        _stream_ptr(stream)))
+    st = (_NATIVE or _native()).softmax_xent_static(logits, labels, loss, row_max, row_sum, stream)
+    if st:
+        _check(st)
 
 
 def sbp_embedding(table: SbpTensor, ids: SbpTensor, out: SbpTensor,
                   oob_count: Optional[torch.Tensor] = None, stream=None) -> None:
-    a, b, c = table._c(), ids._c(), out._c()
-    oob = C.c_void_p(oob_count.data_ptr()) if oob_count is not None else C.c_void_p(0)
-    _check(load_library().sbp_embedding(C.byref(a), C.byref(b), C.byref(c), oob, _stream_ptr(stream)))
+    st = (_NATIVE or _native()).embedding(table, ids, out, oob_count, stream)
+    if st:
+        _check(st)
 
 
 def sbp_embedding_backward(grad_out: SbpTensor, ids: SbpTensor, grad_table: SbpTensor,
                            oob_count: Optional[torch.Tensor] = None, stream=None) -> None:
-    a, b, c = grad_out._c(), ids._c(), grad_table._c()
-    oob = C.c_void_p(oob_count.data_ptr()) if oob_count is not None else C.c_void_p(0)
-    _check(load_library().sbp_embedding_backward(C.byref(a), C.byref(b), C.byref(c), oob, _stream_ptr(stream)))
-
+    st = (_NATIVE or _native()).embedding_backward(grad_out, ids, grad_table, oob_count, stream)
+    if st:
+        _check(st)

@@ -1,4 +1,5 @@
-"""Builds the C-ABI shared library (libsbp_b200.so) in-tree with nvcc for sm_100a.
+"""Builds the C-ABI shared library (libsbp_b200.so) in-tree with nvcc for sm_100a, and the native part
+of the Python binding (_native.so) with the host compiler.
 
 Usage:  python -m paper_2110_15032_b200.build [--force] [--verbose] [--debug-bounds]
 
@@ -20,6 +21,8 @@ CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libsbp_b200.so")
 OBJ_DBG = os.path.join(PKG, "_build", "dbg")
+BINDING_SRC = os.path.join(CSRC, "binding_native.cpp")
+BINDING = os.path.join(PKG, "_native.so")
 LIB_DBG = os.path.join(PKG, "libsbp_b200_dbg.so")
 
 NVCC_FLAGS = [
@@ -43,6 +46,31 @@ def _stale(target: str, deps) -> bool:
         return True
     t = os.path.getmtime(target)
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def build_binding(force: bool = False, verbose: bool = False) -> str:
+    """The extension module the binding makes its hot calls through (CPython and torch C++ interfaces;
+    it is handed the library's entry points at run time, so one build serves either library)."""
+    if not (force or _stale(BINDING, [BINDING_SRC, os.path.join(ROOT, "include", "sbp.h")])):
+        return BINDING
+    import sysconfig
+
+    import torch
+    from torch.utils.cpp_extension import include_paths
+    torch_lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    cuda_inc = os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include")
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", os.path.join(ROOT, "include"), "-isystem", sysconfig.get_paths()["include"], "-isystem", cuda_inc]
+    for d in include_paths():
+        cmd += ["-isystem", d]
+    cmd += [BINDING_SRC, "-o", BINDING, "-L", torch_lib, "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if verbose or r.returncode != 0:
+        sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
+    if r.returncode != 0:
+        raise RuntimeError("the host compiler failed on " + BINDING_SRC)
+    return BINDING
 
 
 def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False) -> str:
@@ -80,6 +108,7 @@ def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False
         if r.returncode != 0:
             sys.stderr.write(r.stdout + r.stderr)
             raise RuntimeError("link failed")
+    build_binding(force, verbose)
     return lib
 
 
