@@ -339,19 +339,24 @@ void sbp_tensor_map_stats(uint64_t* reused, uint64_t* encoded);
  * MMA, the epilogue exposed).  The library picks per product, from the tile count, the length of
  * the contraction and the epilogue, one of: square; tall; or a mixed run -- whole waves of tall
  * tiles, then the rest of the result in the square form as a second launch.  The results do not
- * depend on the choice (same accumulation order per element).  This reports the launches since the
- * library was loaded (process-wide): [0] square, [1] tall, [2] the square launch that ends a mixed run.
+ * depend on the choice between those (same accumulation order per element).  A product with too few
+ * tiles to occupy the device, or with few rows, takes a third kernel, "split": a cluster of CTA pairs
+ * per tile, each pair with its part of the contraction, the parts added in a fixed order (its results
+ * may differ from the other forms' in the last bits, and are the same from call to call).  This reports the launches since the
+ * library was loaded (process-wide): [0] square
+ * or split, [1] tall, [2] the square launch that ends a mixed run.
  * sbp_matmul_set_form overrides the choice for tests and measurements (process-wide, not a tuning
- * knob): form 0 = the library chooses, 1 = square, 2 = tall, 3 = mixed (where a product cannot run
+ * knob): form 0 = the library chooses, 1 = square, 2 = tall, 3 = mixed, 4 = split (where a product cannot run
  * the forced form -- softmax epilogues, results written element-wise, fewer tiles than one wave
  * for "mixed" -- it runs the nearest one that it can); max_pairs > 0 caps the CTA pairs of a
  * launch (0 = all the device holds), which makes small products run many waves.  Until it is
- * called, the environment variables SBP_TC_FORM = square | tall | mixed and SBP_TC_PAIRS, read
+ * called, the environment variables SBP_TC_FORM = square | tall | mixed | split and SBP_TC_PAIRS, read
  * once, give the same two values. */
 #define SBP_TC_FORM_AUTO 0
 #define SBP_TC_FORM_SQUARE 1
 #define SBP_TC_FORM_TALL 2
 #define SBP_TC_FORM_MIXED 3
+#define SBP_TC_FORM_SPLIT 4
 void sbp_matmul_set_form(int32_t form, int32_t max_pairs);
 /* (The paper has no counterpart: this is about how THIS library runs a Table 1 product.)
  * The route the library's cost model picks for ONE bf16 output group of m x n with a contraction of
@@ -359,7 +364,8 @@ void sbp_matmul_set_form(int32_t form, int32_t max_pairs);
  * destinations: returns 0 square, 1 tall, 2 mixed (then *tall_tiles = the 512 x 256 tiles that run
  * in the tall form; 0 for square), -1 for arguments out of range.  Host arithmetic only: no
  * device is touched, overrides set with sbp_matmul_set_form are not applied, and products that
- * cannot leave the square form (softmax epilogues, element-wise stores) are not modelled. */
+ * cannot leave the square form (softmax epilogues, element-wise stores) are not modelled, nor is the split
+ * form. */
 int32_t sbp_matmul_route(int64_t m, int64_t n, int64_t k, int32_t pairs, uint32_t flags, int32_t replicas, int32_t out_f32,
                          int64_t* tall_tiles);
 void sbp_matmul_form_stats(uint64_t launches[3]);

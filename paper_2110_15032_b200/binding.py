@@ -316,7 +316,7 @@ def sbp_tensor_map_stats():
     return int(a.value), int(b.value)
 
 
-SBP_TC_FORM_AUTO, SBP_TC_FORM_SQUARE, SBP_TC_FORM_TALL, SBP_TC_FORM_MIXED = 0, 1, 2, 3
+SBP_TC_FORM_AUTO, SBP_TC_FORM_SQUARE, SBP_TC_FORM_TALL, SBP_TC_FORM_MIXED, SBP_TC_FORM_SPLIT = 0, 1, 2, 3, 4
 
 
 def sbp_matmul_set_form(form: int = 0, max_pairs: int = 0) -> None:

@@ -224,11 +224,18 @@ __device__ __forceinline__ void umma_bf16(unsigned d_tmem, unsigned long long a_
 }
 
 // Arrives on the barrier at this offset in BOTH CTAs of the pair once every tcgen05 operation
-// issued so far by this thread is done.
-__device__ __forceinline__ void umma_commit_pair(unsigned bar) {
-  const unsigned short mask = 3;
+// issued so far by this thread is done.  (mask: the pair's two CTAs inside the cluster.)
+__device__ __forceinline__ void umma_commit_pair(unsigned bar, unsigned short mask = 3) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
                "h"(mask)
+               : "memory");
+}
+
+__device__ __forceinline__ void tmem_ld8(unsigned taddr, float* v) {
+  unsigned* r = reinterpret_cast<unsigned*>(v);
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
                : "memory");
 }
 
@@ -259,13 +266,13 @@ __device__ __forceinline__ unsigned long long desc_pack(unsigned lo, unsigned hi
   return d;
 }
 
-// Instruction descriptor: D fp32, A and B bf16, M = 256 (pair), N = 256.  Bit 15 / bit 16 say
+// Instruction descriptor: D fp32, A and B bf16, M = 256 (pair), N = `n`.  Bit 15 / bit 16 say
 // that A / B lies in shared memory with its M / N index contiguous ("MN-major") instead of its
 // K index.  Operands as given: A [M,K] row-major is K-major, B [K,N] row-major is N-major; a
 // transposed operand is the other way round.
-constexpr unsigned kIdescBase = (1u << 4) | (1u << 7) | (1u << 10) | ((BN >> 3) << 17) | ((BM >> 4) << 24);
-__host__ __device__ constexpr unsigned make_idesc(int a_trans, int b_trans) {
-  return kIdescBase | ((a_trans ? 1u : 0u) << 15) | ((b_trans ? 0u : 1u) << 16);
+constexpr unsigned kIdescBase = (1u << 4) | (1u << 7) | (1u << 10) | ((BM >> 4) << 24);
+__host__ __device__ constexpr unsigned make_idesc(int a_trans, int b_trans, int n = BN) {
+  return kIdescBase | ((unsigned)(n >> 3) << 17) | ((a_trans ? 1u : 0u) << 15) | ((b_trans ? 0u : 1u) << 16);
 }
 
 // erf by the rational approximation 7.1.26 of Abramowitz & Stegun (|error| <= 1.5e-7), which is
@@ -784,6 +791,333 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
   }
 }
 
+// ------------------------------------------------------------------ the split form
+//
+// A product with fewer 256 x 256 tiles than the device has CTA pairs leaves pairs idle for its whole
+// contraction (a fused P(sum) product of 512 x 512 over 2^20 classes: 4 tiles of 16384 K-blocks, 4.6 ms on
+// four of 74 pairs), and one with few rows multiplies padding.  Here a tile belongs to a CLUSTER of
+// `splits` pairs, each of which multiplies its own range of the K-blocks into its own tensor memory; the
+// partial accumulators are then added up through distributed shared memory: the tile's columns are dealt
+// out to the pairs, every other pair pushes its partial sums of those columns into the owner's shared
+// memory (which its ring no longer needs), and the owner adds the slices in ascending order (the same bits
+// every time), applies GeLU and stores.  No workspace and no atomics.
+//   NB  columns of a tile.  A tile is 256 rows x NB; narrower ones give more tiles, or less padding.
+//   SW  the operands are exchanged by the host, Y^T = W^T X^T: the tile's rows are then columns of the
+//       result and its NB columns are rows of it.  A product of few rows so spends its tile on them: the
+//       weight streams through shared memory as the 256-row operand with NB = 32 columns beside it, 18 KiB
+//       a K-block and CTA of which 16 are weight, ten K-blocks deep.
+// One tile per cluster, so nothing is persistent; results leave through shared memory as whole 16-byte
+// pieces of rows (element by element where base or pitch is not aligned).
+struct TcSplitParams {
+  CUtensorMap map_a[SBP_MAX_K];
+  CUtensorMap map_b[SBP_MAX_K];
+  long long m[SBP_MAX_K], n[SBP_MAX_K], row_off[SBP_MAX_K], col_off[SBP_MAX_K], ldy[SBP_MAX_K];
+  void* y_ptr[SBP_MAX_K];
+  void* rep_ptr[SBP_MAX_K];
+  int kblocks[SBP_MAX_K];
+  int tile_begin[SBP_MAX_K + 1];
+  int tiles_m[SBP_MAX_K];
+  int ngroups, nseg, chain, gelu, n_rep, out_f32;
+  int splits;
+  int y_vec;                     // 16-byte stores are possible everywhere
+};
+
+// A ring slot holds kGroup K-blocks behind one pair of barriers: whatever its size, a round of waits, issue and
+// bookkeeping costs either single-issue role some 480 clocks, and a K-block of a narrow tile is worth 64-256
+// clocks of the tensor pipe.
+constexpr int kGroup = 2;
+constexpr int kMaxSplits = 8;         // a cluster has at most 16 CTAs
+template <int NB>
+constexpr int split_block_bytes() { return kStageA + BK * NB; }        // B: 64 x NB/2 elements of 2 bytes per CTA
+constexpr int kSplitRing = 192 * 1024;
+template <int NB>
+constexpr int split_stages() { return kSplitRing / (kGroup * split_block_bytes<NB>()); }      // 3 (NB = 256), 4, 4, 5 (NB = 32)
+constexpr int kSmemSplit = kSplitRing + 1024;                                       // + alignment slack
+
+template <int AT, int BT, int NB, int SW>
+__global__ void __launch_bounds__(kThreadsTc, 1) matmul_tc_split_kernel(const __grid_constant__ TcSplitParams p) {
+  constexpr int kSt = split_stages<NB>(), kBlk = split_block_bytes<NB>(), kBH = NB / 2;
+  static_assert(BT || kBH % 64 == 0, "an N-major B tile comes in boxes of 64 columns");
+  extern __shared__ unsigned char smem_raw[];
+  __shared__ __align__(8) unsigned long long bar_full[kSt], bar_empty[kSt], bar_acc;
+  __shared__ unsigned tmem_base_slot;
+  __shared__ int abort_flag_s;
+  volatile int* abort_flag = &abort_flag_s;
+
+  unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned crank = cluster_ctarank(), rank = crank & 1, even = crank & ~1u;      // `even` issues its pair's MMAs
+  const int S = p.splits, slice = (int)(crank >> 1);
+
+  if (threadIdx.x == 0) {
+    abort_flag_s = 0;
+    for (int i = 0; i < kSt; ++i) {
+      mbar_init(smem_addr(&bar_full[i]), 1);      // used in the even CTA only
+      mbar_init(smem_addr(&bar_empty[i]), 1);
+    }
+    mbar_init(smem_addr(&bar_acc), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_base_slot)), "r"(NB)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  cluster_sync_all();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const unsigned tmem_base = tmem_base_slot;
+  SBP_PDL_WAIT();                                  // everything up to here overlaps the kernel before this one
+
+  // this cluster's tile and this pair's range of its K-blocks
+  const int tile = (int)(blockIdx.x / (unsigned)(2 * S));
+  int g = 0;
+  while (g + 1 < p.ngroups && tile >= p.tile_begin[g + 1]) ++g;
+  const int local = tile - p.tile_begin[g], nt = local / p.tiles_m[g], mt = local - nt * p.tiles_m[g];
+  const int m0 = mt * BM, n0 = nt * NB;
+  const int s_lo = p.chain ? 0 : g, s_hi = p.chain ? p.nseg : g + 1;
+  long long total = 0;
+  for (int s = s_lo; s < s_hi; ++s) total += p.kblocks[s];
+  const int it0 = (int)(total * slice / S), iters = (int)(total * (slice + 1) / S) - it0;
+  bool ok = true;
+
+  if (warp == 0) {
+    // ------------------------------------------------ producer (both CTAs of every pair)
+    const bool leader = elect_one();
+    int seg = s_lo, kb = it0, slot = 0, rounds = 0;
+    unsigned round = 0;
+    while (seg < s_hi && kb >= p.kblocks[seg]) kb -= p.kblocks[seg++];
+    int nkb = seg < s_hi ? p.kblocks[seg] : 0;
+    const int arow = (int)p.row_off[g] + m0 + (int)rank * BMH, bcol = (int)p.col_off[g] + n0 + (int)rank * kBH;
+    for (int left = iters; left > 0; left -= kGroup, ++rounds) {
+      if (!mbar_wait_warp(smem_addr(&bar_empty[slot]), round ^ 1, abort_flag)) break;
+      const unsigned full0 = map_to_cta(smem_addr(&bar_full[slot]), even);
+      if (leader && rank == 0) mbar_expect_tx(smem_addr(&bar_full[slot]), 2 * kBlk * (left < kGroup ? left : kGroup));
+#pragma unroll
+      for (int b = 0; b < kGroup; ++b) {
+        if (b >= left) break;
+        if (leader) {
+          unsigned char* sa = smem + (slot * kGroup + b) * kBlk;
+          unsigned char* sb = sa + kStageA;
+          if constexpr (!AT) {
+            tma_load_2d(smem_addr(sa), &p.map_a[seg], kb * BK, arow, full0);
+          } else {
+#pragma unroll
+            for (int c = 0; c < BMH / 64; ++c) tma_load_2d(smem_addr(sa + c * (BK * 128)), &p.map_a[seg], arow + c * 64, kb * BK, full0);
+          }
+          if constexpr (!BT) {
+#pragma unroll
+            for (int c = 0; c < kBH / 64; ++c) tma_load_2d(smem_addr(sb + c * (BK * 128)), &p.map_b[seg], bcol + c * 64, kb * BK, full0);
+          } else {
+            tma_load_2d(smem_addr(sb), &p.map_b[seg], kb * BK, bcol, full0);
+          }
+        }
+        __syncwarp();
+        if (++kb >= nkb) {
+          kb = 0;
+          do nkb = ++seg < s_hi ? p.kblocks[seg] : 1; while (nkb == 0);      // steps over empty segments
+        }
+      }
+      slot = slot + 1 == kSt ? 0 : slot + 1;
+      round ^= (slot == 0);
+    }
+    if (*abort_flag && rank == 0 && leader) {
+      // give the loads still in flight a bounded chance to land before the CTA goes away
+      for (int i = rounds > kSt ? rounds - kSt : 0; i < rounds; ++i) {
+        const unsigned long long t0 = now_ns();
+        while (!mbar_try(smem_addr(&bar_full[i % kSt]), (unsigned)((i / kSt) & 1)) && now_ns() - t0 < 100000000ull) {
+        }
+      }
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------ MMA issuer (the even CTA of every pair)
+    if (rank == 0) {
+      const bool leader = elect_one();
+      const unsigned short pair_mask = (unsigned short)(3u << even);
+      constexpr unsigned idesc = make_idesc(AT, BT, NB);
+      int slot = 0;
+      unsigned round = 0, accumulate = 0;
+      for (int left = iters; left > 0; left -= kGroup) {
+        if (!mbar_wait_warp(smem_addr(&bar_full[slot]), round, abort_flag)) {
+          ok = false;
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        // a shared-memory address carries the CTA's rank in its high bits; a descriptor takes the offset alone
+        const unsigned s0 = smem_addr(smem + slot * kGroup * kBlk) & 0x3ffffu;
+        if (leader) {
+#pragma unroll
+          for (int b = 0; b < kGroup; ++b) {
+            if (b >= left) break;
+            const unsigned sa = s0 + b * kBlk, sb = sa + kStageA;
+#pragma unroll
+            for (int kk = 0; kk < BK / 16; ++kk) {        // descriptors as in the persistent kernel
+              constexpr unsigned a_lo = desc_lo_fixed(AT ? BK * 128 : 16), b_lo = desc_lo_fixed(BT ? 16 : BK * 128);
+              constexpr unsigned hi = desc_hi_fixed(1024);
+              umma_bf16(tmem_base, desc_pack(a_lo + (sa >> 4) + kk * (AT ? 128 : 2), hi), desc_pack(b_lo + (sb >> 4) + kk * (BT ? 2 : 128), hi),
+                        idesc, (b > 0 || kk > 0) ? 1u : accumulate);
+            }
+          }
+          umma_commit_pair(smem_addr(&bar_empty[slot]), pair_mask);
+        }
+        __syncwarp();
+        accumulate = 1;
+        slot = slot + 1 == kSt ? 0 : slot + 1;
+        round ^= (slot == 0);
+      }
+      if (leader && ok) umma_commit_pair(smem_addr(&bar_acc), pair_mask);
+      __syncwarp();
+    }
+  } else if (warp == 2 && lane == 0) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&p.map_a[s_lo]) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&p.map_b[s_lo]) : "memory");
+  }
+
+  // Epilogue warps 2..9: tensor-memory lanes 32 q .. 32 q + 31.  The tile's columns are dealt to the pairs in groups
+  // of 8, `per` groups each (the last owner may have fewer, the last pairs none); of an owner's groups the first
+  // warp of a lane quadrant takes the first half, the second warp the rest.
+  constexpr int kCg = NB / 8;
+  const int q = warp & 3, half = (warp - 2) >> 2;
+  const long long Mg = p.m[g], Ng = p.n[g];
+  const int row0 = m0 + (int)rank * BMH + q * 32;
+  const int per = (kCg + S - 1) / S;
+  const bool rows_live = warp >= 2 && row0 < Mg;       // warp-uniform
+  const unsigned tq = tmem_base + ((unsigned)(q * 32) << 16);
+  // this warp's column groups of owner o, counted from the owner's first
+  auto mine = [&](int o, int* lo, int* hi) {
+    const int have = kCg - o * per < per ? kCg - o * per : per;
+    *lo = half ? (have + 1) / 2 : 0;
+    *hi = half ? have : (have + 1) / 2;
+  };
+  if (warp >= 2) {
+    ok = lane != 0 || mbar_wait(smem_addr(&bar_acc), 0, abort_flag);
+    ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  }
+  SBP_PDL_RELEASE();
+  if (S > 1) {
+    cluster_sync_all();                                // every pair is done with its ring
+    if (rows_live && ok) {
+      for (int d = 1; d < S; ++d) {
+        const int o = slice + d < S ? slice + d : slice + d - S;
+        int lo, hi;
+        mine(o, &lo, &hi);
+        if (lo >= hi) continue;
+        const int from = slice < o ? slice : slice - 1;              // my place among o's S - 1 sources
+        const unsigned dst = map_to_cta(smem_addr(smem) + (unsigned)(from * per * (BMH * 32)), (unsigned)(2 * o) + rank);
+        for (int c = lo; c < hi; ++c) {
+          float v[8];
+          tmem_ld8(tq + (o * per + c) * 8, v);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          const unsigned at = dst + (unsigned)(2 * c * BMH + q * 32 + lane) * 16u;      // [4-column group][row]
+#pragma unroll
+          for (int e = 0; e < 2; ++e)
+            asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at + e * BMH * 16u), "f"(v[4 * e]), "f"(v[4 * e + 1]),
+                         "f"(v[4 * e + 2]), "f"(v[4 * e + 3])
+                         : "memory");
+        }
+      }
+    }
+    cluster_sync_all();                                // all partial sums have arrived
+  }
+  int lo, hi;
+  mine(slice, &lo, &hi);
+  const int col0 = n0 + (slice * per + lo) * 8;
+  if (rows_live && ok && lo < hi && col0 < Ng) {
+    const int esz = p.out_f32 ? 4 : 2, cols = (hi - lo) * 8;
+    // Staged per warp as rows of the RESULT: 32 rows of `cols` elements, 16 bytes apart so that 32 rows written at
+    // once spread over the banks (SW: `cols` rows of 32 elements).
+    const int pitch = SW ? 32 * esz : cols * esz + 16;
+    unsigned char* stage = smem + (S - 1) * per * (BMH * 32) + (warp - 2) * (32 * ((per + 1) / 2 * 8 * esz + 16));
+    for (int c = lo; c < hi; ++c) {
+      float v[8], own[8];
+      tmem_ld8(tq + (slice * per + c) * 8, own);
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      for (int s = 0; s < S; ++s) {
+        float x[8];
+        if (s == slice) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) x[e] = own[e];
+        } else {
+          const int from = s < slice ? s : s - 1;
+          const unsigned char* at = smem + from * per * (BMH * 32) + (2 * c * BMH + q * 32 + lane) * 16;
+          *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(at);
+          *reinterpret_cast<float4*>(x + 4) = *reinterpret_cast<const float4*>(at + BMH * 16);
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = s == 0 ? x[e] : v[e] + x[e];
+      }
+      if (p.gelu) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = gelu_erf_tc(v[e]);
+      }
+      const int cc = (c - lo) * 8;
+      if constexpr (SW) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          unsigned char* at = stage + (cc + e) * pitch + lane * esz;
+          if (p.out_f32) *reinterpret_cast<float*>(at) = v[e];
+          else *reinterpret_cast<__nv_bfloat16*>(at) = __float2bfloat16_rn(v[e]);
+        }
+      } else {
+        unsigned char* at = stage + lane * pitch + cc * esz;
+        if (p.out_f32) {
+          *reinterpret_cast<float4*>(at) = make_float4(v[0], v[1], v[2], v[3]);
+          *reinterpret_cast<float4*>(at + 16) = make_float4(v[4], v[5], v[6], v[7]);
+        } else {
+          uint4 o;
+          __nv_bfloat162 h;
+          h = __floats2bfloat162_rn(v[0], v[1]); o.x = *reinterpret_cast<unsigned*>(&h);
+          h = __floats2bfloat162_rn(v[2], v[3]); o.y = *reinterpret_cast<unsigned*>(&h);
+          h = __floats2bfloat162_rn(v[4], v[5]); o.z = *reinterpret_cast<unsigned*>(&h);
+          h = __floats2bfloat162_rn(v[6], v[7]); o.w = *reinterpret_cast<unsigned*>(&h);
+          *reinterpret_cast<uint4*>(at) = o;
+        }
+      }
+    }
+    __syncwarp();
+    // out: consecutive lanes take consecutive 16-byte pieces of a row of the result
+    const int el = 16 / esz, pieces = (SW ? 32 : cols) / el, nrows = SW ? cols : 32;
+    const long long yr0 = SW ? col0 : row0, yc0 = SW ? row0 : col0, yrows = SW ? Ng : Mg, ycols = SW ? Mg : Ng;
+    const int n_out = (g == 0 ? p.n_rep : 0) + 1;
+    const long long ld = p.ldy[g];
+    for (int o = 0; o < n_out; ++o) {
+      unsigned char* y = static_cast<unsigned char*>(o == 0 ? p.y_ptr[g] : p.rep_ptr[o - 1]);
+      for (int idx = lane; idx < nrows * pieces; idx += 32) {
+        const int r = idx / pieces, ch = idx - r * pieces;
+        if (yr0 + r >= yrows) continue;
+        const uint4 v = *reinterpret_cast<const uint4*>(stage + r * pitch + ch * 16);
+        const long long c = yc0 + ch * el;
+        unsigned char* at = y + ((yr0 + r) * ld + c) * esz;
+        if (p.y_vec && c + el <= ycols) {
+          if (SBP_GUARD(at, 16)) *reinterpret_cast<uint4*>(at) = v;
+        } else if (p.out_f32) {
+          const float* f = reinterpret_cast<const float*>(&v);
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (c + e < ycols && SBP_GUARD(at + 4 * e, 4)) reinterpret_cast<float*>(at)[e] = f[e];
+        } else {
+          const unsigned short* f = reinterpret_cast<const unsigned short*>(&v);
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            if (c + e < ycols && SBP_GUARD(at + 2 * e, 2)) reinterpret_cast<unsigned short*>(at)[e] = f[e];
+        }
+      }
+    }
+  }
+
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  cluster_sync_all();
+  if (warp == 1) {
+    __syncwarp();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(NB) : "memory");
+  }
+}
+
 // ------------------------------------------------------------------ host side
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -845,14 +1179,14 @@ void tensor_map_cache_stats(unsigned long long* hits, unsigned long long* encode
 static std::atomic<unsigned long long> g_form_launches[3];
 
 // Overrides of the form choice and of the CTA pairs a launch may use (tests and measurements):
-// set by tc_set_form, else taken once from SBP_TC_FORM (square | tall | mixed) and SBP_TC_PAIRS.
+// set by tc_set_form, else taken once from SBP_TC_FORM (square | tall | mixed | split) and SBP_TC_PAIRS.
 static std::atomic<int> g_forced_form{-1}, g_pair_cap{-1};
 
 static int forced_form() {
   int v = g_forced_form.load();
   if (v < 0) {
     const char* e = getenv("SBP_TC_FORM");
-    v = e ? (e[0] == 's' ? 1 : (e[0] == 't' ? 2 : (e[0] == 'm' ? 3 : 0))) : 0;
+    v = e ? (e[0] == 's' ? (e[1] == 'p' ? 4 : 1) : (e[0] == 't' ? 2 : (e[0] == 'm' ? 3 : 0))) : 0;
     g_forced_form.store(v);
   }
   return v;
@@ -869,7 +1203,7 @@ static int pair_cap() {
 }
 
 void tc_set_form(int form, int max_pairs) {
-  g_forced_form.store(form >= 0 && form <= 3 ? form : 0);
+  g_forced_form.store(form >= 0 && form <= 4 ? form : 0);
   g_pair_cap.store(max_pairs > 0 ? max_pairs : 0);
 }
 
@@ -990,6 +1324,7 @@ static sbp_status launch_tc(bool tall, bool a_trans, bool b_trans, const TcParam
 struct FormChoice {
   bool walk_tall;      // tiles are walked 512 rows at a time
   int tall_tiles;      // the first so many walked tiles run in the tall form
+  double cost;         // the model's time for it, without what every launch pays
 };
 
 static FormChoice choose_form(long long tiles_sq, long long tiles_tall, long long kb, int cap_sq, int cap_tall, bool gelu, int n_rep,
@@ -1013,8 +1348,8 @@ static FormChoice choose_form(long long tiles_sq, long long tiles_tall, long lon
     if (cost_mixed < best) { best = cost_mixed; pick = 2; }
   }
   if (pick == 2 && (full == 0 || full == tiles_tall)) pick = full == 0 ? 0 : 1;
-  if (pick == 0) return FormChoice{false, 0};
-  return FormChoice{true, (int)(pick == 1 ? tiles_tall : full)};
+  if (pick == 0) return FormChoice{false, 0, cost_sq};
+  return FormChoice{true, (int)(pick == 1 ? tiles_tall : full), pick == 1 ? cost_tall : cost_mixed};
 }
 
 // choose_form for callers outside this file (the C ABI's planning query): 0 square, 1 tall, 2 mixed.
@@ -1023,6 +1358,199 @@ int tc_route(long long tiles_sq, long long tiles_tall, long long kb, int pairs, 
   const FormChoice f = choose_form(tiles_sq, tiles_tall, kb, pairs, pairs, gelu, n_rep, out_f32, forced);
   if (tall_tiles) *tall_tiles = f.walk_tall ? f.tall_tiles : 0;
   return !f.walk_tall ? 0 : (f.tall_tiles == tiles_tall ? 1 : 2);
+}
+
+// One split product, or, with p == nullptr, only the clusters of this size the device holds at once.
+template <int AT, int BT, int NB, int SW>
+static sbp_status launch_split_form(const TcSplitParams* p, int splits, int tiles, cudaStream_t st, int* capacity) {
+  static std::atomic<unsigned long long> opted{0};      // one bit per device
+  int dev = 0;
+  SBP_CUDA_TRY(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64) return fail(SBP_ERR_UNSUPPORTED, "device ordinal %d out of range", dev);
+  auto* kernel = matmul_tc_split_kernel<AT, BT, NB, SW>;
+  if (!(opted.load(std::memory_order_relaxed) >> dev & 1)) {
+    SBP_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemSplit));
+    SBP_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    opted.fetch_or(1ull << dev, std::memory_order_relaxed);
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(2 * splits * tiles));
+  cfg.blockDim = dim3(kThreadsTc);
+  cfg.dynamicSmemBytes = kSmemSplit;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)(2 * splits);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (capacity) {
+    *capacity = 0;
+    if (cudaOccupancyMaxActiveClusters(capacity, kernel, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      *capacity = 0;
+    }
+    return SBP_OK;
+  }
+  cfg.numAttrs = 2;
+  SBP_BOUNDS_UPLOAD(st);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, *p);
+  if (e != cudaSuccess) return cuda_fail(e, "tensor-core matmul launch");
+  count_launch();
+  g_form_launches[0]++;
+  return SBP_OK;
+}
+
+// How a split product is cut: NB columns a tile, `splits` pairs a tile (0: the persistent kernel runs it),
+// operands exchanged or not.
+struct SplitChoice {
+  int nb, splits, swap;
+};
+
+static sbp_status launch_split_any(bool a_trans, bool b_trans, SplitChoice c, const TcSplitParams* p, int tiles, cudaStream_t st) {
+  const int s = c.splits;
+  if (c.swap) {            // b_trans holds: the exchanged operand is X as given
+    switch (c.nb | (a_trans ? 1 : 0)) {
+      case 32: return launch_split_form<0, 1, 32, 1>(p, s, tiles, st, nullptr);
+      case 33: return launch_split_form<1, 1, 32, 1>(p, s, tiles, st, nullptr);
+      case 64: return launch_split_form<0, 1, 64, 1>(p, s, tiles, st, nullptr);
+      case 65: return launch_split_form<1, 1, 64, 1>(p, s, tiles, st, nullptr);
+      case 128: return launch_split_form<0, 1, 128, 1>(p, s, tiles, st, nullptr);
+      default: return launch_split_form<1, 1, 128, 1>(p, s, tiles, st, nullptr);
+    }
+  }
+  switch (c.nb | (a_trans ? 2 : 0) | (b_trans ? 1 : 0)) {
+    case 128: return launch_split_form<0, 0, 128, 0>(p, s, tiles, st, nullptr);
+    case 129: return launch_split_form<0, 1, 128, 0>(p, s, tiles, st, nullptr);
+    case 130: return launch_split_form<1, 0, 128, 0>(p, s, tiles, st, nullptr);
+    case 131: return launch_split_form<1, 1, 128, 0>(p, s, tiles, st, nullptr);
+    case 256: return launch_split_form<0, 0, 256, 0>(p, s, tiles, st, nullptr);
+    case 257: return launch_split_form<0, 1, 256, 0>(p, s, tiles, st, nullptr);
+    case 258: return launch_split_form<1, 0, 256, 0>(p, s, tiles, st, nullptr);
+    default: return launch_split_form<1, 1, 256, 0>(p, s, tiles, st, nullptr);
+  }
+}
+
+// Clusters of 2 * splits CTAs that the current device holds at once (every instance of the kernel fills an SM).
+static int split_capacity(int splits) {
+  static std::atomic<int> known[64][kMaxSplits + 1];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  int v = known[dev][splits].load(std::memory_order_relaxed);
+  if (v == 0) {
+    if (launch_split_form<0, 0, 256, 0>(nullptr, splits, 1, nullptr, &v) != SBP_OK || v < 1) v = -1;
+    known[dev][splits].store(v, std::memory_order_relaxed);
+  }
+  return v;
+}
+
+// Whether a product runs in the split form, and how it is cut: the smallest estimated time in us.  Per wave of
+// clusters: a K-block takes 0.32 us with 256 columns (the tensor pipe's 512 clocks and a little), 0.19-0.20
+// with 128 and fewer (the single-issue roles); set-up, drain and stores 9.6 / 6.6 us (256 / 128 columns),
+// 6.5 / 5.3 / 4.4 for the exchanged form (128 / 64 / 32).  Fitted to 1208 timings of 54 products (rms error
+// 12 %; the pick within 8 % of the best cut of each).  The persistent kernel keeps what it does as well:
+// `cost_persistent` includes the 5.5 us it takes besides its waves, and a split has to win by 8 %.
+// (us, persistent / split, one product in a row of them: 16 rows [4096 x 16384] 31 / 24 and [16384 x 4096]
+// 79 / 26; 1000 rows [4096 x 1024] written to four replicas 28 / 16; 500 rows [1024 x 4096] + GeLU 15 / 11;
+// 512 x 512 over 2^20 classes 4569 / 621; 64 x 256 over 2^17 578 / 48.)
+static SplitChoice choose_split(const MatmulPlan& plan, const int* kblocks, double cost_persistent, int forced) {
+  long long kb_max = 0, kb_min = -1, chain_kb = 0, m_max = 0;
+  for (int s = 0; s < plan.nseg; ++s) chain_kb += kblocks[s];
+  for (int g = 0; g < plan.ngroups; ++g) {
+    if (plan.m[g] <= 0 || plan.n[g] <= 0) continue;
+    m_max = plan.m[g] > m_max ? plan.m[g] : m_max;
+    const long long kb = plan.chain ? chain_kb : kblocks[g];
+    kb_max = kb > kb_max ? kb : kb_max;
+    kb_min = kb_min < 0 || kb < kb_min ? kb : kb_min;
+  }
+  SplitChoice best{0, 0, 0};
+  double best_cost = forced == 4 ? 1e300 : cost_persistent;
+  for (int swap = 0; swap < 2; ++swap) {
+    if (swap && plan.a_trans) continue;      // X would be the N-major operand: boxes of 64 rows and more
+    if (swap && m_max > 192) continue;       // its tiles read the weight once per 128 rows, the plain ones once per 256
+    for (int nb = swap ? 128 : 256; nb >= (swap ? 32 : 128); nb /= 2) {
+      long long tiles = 0;
+      for (int g = 0; g < plan.ngroups; ++g) {
+        const long long rows = swap ? plan.n[g] : plan.m[g], cols = swap ? plan.m[g] : plan.n[g];
+        if (rows > 0 && cols > 0) tiles += (rows + BM - 1) / BM * ((cols + nb - 1) / nb);
+      }
+      if (tiles > 4096) continue;
+      for (int s = 1; s <= kMaxSplits; ++s) {
+        if (kb_min < s) break;
+        const int cap = split_capacity(s);
+        if (cap < 1) continue;
+        const double waves = (double)((tiles + cap - 1) / cap), kb = (double)((kb_max + s - 1) / s);
+        const double per_kb = nb == 256 ? 0.323 : (nb == 128 ? 0.2 : 0.187);
+        const double per_wave = nb == 256 ? 9.6 : (nb == 128 ? 6.6 : (nb == 64 ? 5.3 : 4.4));
+        const double cost = waves * (kb * per_kb + per_wave + (s > 1 ? 0.8 + 0.08 * s : 0.0) + (plan.gelu ? 0.4 : 0.0) +
+                                     plan.n_rep * 2.0 * nb / (256.0 * s));
+        if (cost < best_cost) {
+          best_cost = cost;
+          best = SplitChoice{nb, s, swap};
+        }
+      }
+    }
+  }
+  return best;
+}
+
+static sbp_status launch_split(const MatmulPlan& given, const int* kblocks, SplitChoice c, bool y_vec, cudaStream_t st, bool* taken) {
+  MatmulPlan plan = given;
+  if (c.swap) {            // Y^T = W^T X^T
+    for (int i = 0; i < SBP_MAX_K; ++i) {
+      std::swap(plan.a[i], plan.b[i]);
+      std::swap(plan.lda[i], plan.ldb[i]);
+      std::swap(plan.m[i], plan.n[i]);
+      std::swap(plan.row_off[i], plan.col_off[i]);
+    }
+    plan.a_trans = !given.b_trans;
+    plan.b_trans = !given.a_trans;
+  }
+  TcSplitParams p;
+  int tiles = 0;
+  for (int g = 0; g < plan.ngroups; ++g) {
+    p.m[g] = plan.m[g];
+    p.n[g] = plan.n[g];
+    p.row_off[g] = plan.row_off[g];
+    p.col_off[g] = plan.col_off[g];
+    p.ldy[g] = plan.ldy[g];
+    p.y_ptr[g] = plan.y[g];
+    p.tile_begin[g] = tiles;
+    const int tm = (int)((plan.m[g] + BM - 1) / BM);
+    p.tiles_m[g] = tm > 0 ? tm : 1;
+    if (plan.m[g] > 0 && plan.n[g] > 0) tiles += tm * (int)((plan.n[g] + c.nb - 1) / c.nb);
+  }
+  for (int g = plan.ngroups; g <= SBP_MAX_K; ++g) p.tile_begin[g] = tiles;
+  for (int r = 0; r < plan.n_rep; ++r) p.rep_ptr[r] = plan.y_rep[r];
+  for (int s = 0; s < plan.nseg; ++s) {
+    p.kblocks[s] = kblocks[s];
+    if (!(plan.chain || s < plan.ngroups) || kblocks[s] == 0) continue;
+    long long rows_a = plan.chain ? 0 : plan.m[s], cols_b = plan.chain ? 0 : plan.n[s];
+    for (int g = 0; plan.chain && g < plan.ngroups; ++g) {
+      rows_a = std::max(rows_a, plan.row_off[g] + plan.m[g]);
+      cols_b = std::max(cols_b, plan.col_off[g] + plan.n[g]);
+    }
+    if (rows_a == 0 || cols_b == 0) continue;
+    const bool ok_a = plan.a_trans ? make_map(&p.map_a[s], plan.a[s], 2, plan.kseg[s], rows_a, plan.lda[s], BK, 64)
+                                   : make_map(&p.map_a[s], plan.a[s], 2, rows_a, plan.kseg[s], plan.lda[s], BMH, BK);
+    const bool ok_b = plan.b_trans ? make_map(&p.map_b[s], plan.b[s], 2, cols_b, plan.kseg[s], plan.ldb[s], c.nb / 2, BK)
+                                   : make_map(&p.map_b[s], plan.b[s], 2, plan.kseg[s], cols_b, plan.ldb[s], BK, 64);
+    if (!ok_a || !ok_b) return fail(SBP_ERR_CUDA, "cuTensorMapEncodeTiled failed for an operand of shard %d", s);
+  }
+  p.ngroups = plan.ngroups;
+  p.nseg = plan.nseg;
+  p.chain = plan.chain;
+  p.gelu = plan.gelu;
+  p.n_rep = plan.n_rep;
+  p.out_f32 = plan.out_dtype == SBP_F32;
+  p.splits = c.splits;
+  p.y_vec = y_vec ? 1 : 0;
+  *taken = true;
+  if (tiles == 0) return SBP_OK;
+  return launch_split_any(plan.a_trans, plan.b_trans, c, &p, tiles, st);
 }
 
 sbp_status launch_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, cudaStream_t st, bool* taken) {
@@ -1055,9 +1583,40 @@ sbp_status launch_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, cudaSt
     if (!aligned16(plan.y_rep[r])) y_direct = true;
   if (!encode_fn()) return SBP_ERR_UNSUPPORTED;
 
+  int kblocks[SBP_MAX_K];
+  long long kb_tile = 0, tiles_sq = 0, tiles_tall = 0;
+  for (int s = 0; s < plan.nseg; ++s) {
+    kblocks[s] = (int)((plan.kseg[s] + BK - 1) / BK);
+    if (plan.chain || s < plan.ngroups) kb_tile = plan.chain ? kb_tile + kblocks[s] : std::max<long long>(kb_tile, kblocks[s]);
+  }
+  for (int g = 0; g < plan.ngroups; ++g) {
+    if (plan.m[g] <= 0 || plan.n[g] <= 0) continue;
+    const long long tn = (plan.n[g] + BN - 1) / BN;
+    tiles_sq += (plan.m[g] + BM - 1) / BM * tn;
+    tiles_tall += (plan.m[g] + 2 * BM - 1) / (2 * BM) * tn;
+  }
+
   static TcParams p;          // large; filled under a lock and copied by value at launch
   static std::mutex mu;
   std::lock_guard<std::mutex> lock(mu);
+
+  // Which form (see choose_form).  The softmax epilogues are written for the square form, and so is
+  // the element-wise store of a result the copy engine cannot address.
+  FormChoice form{false, 0, 0.0};
+  if (!xf && tiles_tall > 0 && tiles_sq <= 0x1fffffffLL) {
+    int cap_sq = 0, cap_tall = 0;
+    sbp_status qs = launch_tc(false, plan.a_trans, plan.b_trans, nullptr, st, &cap_sq);
+    if (qs == SBP_OK) qs = launch_tc(true, plan.a_trans, plan.b_trans, nullptr, st, &cap_tall);
+    if (qs != SBP_OK) return qs;
+    const int forced = forced_form();
+    form = choose_form(tiles_sq, tiles_tall, kb_tile, cap_sq, cap_tall, plan.gelu != 0, plan.n_rep, plan.out_dtype == SBP_F32, forced == 4 ? 0 : forced);
+    if (y_direct) form.walk_tall = false;
+    if (forced == 4 || (forced == 0 && pair_cap() == 0)) {
+      const SplitChoice sc = choose_split(plan, kblocks, 0.92 * (form.cost + 5.5), forced);
+      if (sc.splits > 0) return launch_split(plan, kblocks, sc, !y_direct, st, taken);
+    }
+  }
+
   p.ngroups = plan.ngroups;
   p.nseg = plan.nseg;
   p.chain = plan.chain;
@@ -1069,7 +1628,7 @@ sbp_status launch_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, cudaSt
   p.y_direct = y_direct ? 1 : 0;
 
   for (int s = 0; s < plan.nseg; ++s) {
-    p.kblocks[s] = (int)((plan.kseg[s] + BK - 1) / BK);
+    p.kblocks[s] = kblocks[s];
     const bool used = plan.chain || s < plan.ngroups;
     if (!used || plan.kseg[s] == 0) continue;
     long long rows_a = 0, cols_b = 0;
@@ -1090,25 +1649,6 @@ sbp_status launch_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, cudaSt
     const bool ok_b = plan.b_trans ? make_map(&p.map_b[s], plan.b[s], 2, cols_b, plan.kseg[s], plan.ldb[s], BNH, BK)
                                    : make_map(&p.map_b[s], plan.b[s], 2, plan.kseg[s], cols_b, plan.ldb[s], BK, 64);
     if (!ok_b) return fail(SBP_ERR_CUDA, "cuTensorMapEncodeTiled failed for operand w of shard %d", s);
-  }
-  // Which form (see choose_form).  The softmax epilogues are written for the square form, and so is
-  // the element-wise store of a result the copy engine cannot address.
-  long long kb_tile = 0, tiles_sq = 0, tiles_tall = 0;
-  for (int s = 0; s < plan.nseg; ++s)
-    if (plan.chain || s < plan.ngroups) kb_tile = plan.chain ? kb_tile + p.kblocks[s] : std::max<long long>(kb_tile, p.kblocks[s]);
-  for (int g = 0; g < plan.ngroups; ++g) {
-    if (plan.m[g] <= 0 || plan.n[g] <= 0) continue;
-    const long long tn = (plan.n[g] + BN - 1) / BN;
-    tiles_sq += (plan.m[g] + BM - 1) / BM * tn;
-    tiles_tall += (plan.m[g] + 2 * BM - 1) / (2 * BM) * tn;
-  }
-  FormChoice form{false, 0};
-  if (!xf && !y_direct && tiles_tall > 0 && tiles_sq <= 0x1fffffffLL) {
-    int cap_sq = 0, cap_tall = 0;
-    sbp_status qs = launch_tc(false, plan.a_trans, plan.b_trans, nullptr, st, &cap_sq);
-    if (qs == SBP_OK) qs = launch_tc(true, plan.a_trans, plan.b_trans, nullptr, st, &cap_tall);
-    if (qs != SBP_OK) return qs;
-    form = choose_form(tiles_sq, tiles_tall, kb_tile, cap_sq, cap_tall, plan.gelu != 0, plan.n_rep, plan.out_dtype == SBP_F32, forced_form());
   }
   const int tile_m = form.walk_tall ? 2 * BM : BM;
   p.walk_m = tile_m;
