@@ -22,6 +22,7 @@
 #include "boxing_arith.h"
 #include "boxing_params.h"
 #include "sbp_internal.h"
+#include "boxing_shift.h"
 
 namespace sbp {
 
@@ -169,6 +170,35 @@ __global__ void __launch_bounds__(256) box_tile_kernel(const __grid_constant__ B
   }
 }
 
+// The same tasks over data that is not 16-byte aligned (boxing_shift.h).  us in a row of calls, element-wise tiles /
+// this: fp32 [1021, 1537] over three shards S(0) -> S(1) 12.0 / 3.0, P(sum) -> S(1) 15.5 / 7.9, S(0) -> B 6.2 / 5.3;
+// fp32 [4096, 4097] over two S(0) -> S(1) 87 / 20 (6.6 TB/s); bf16 [4001, 3333] over eight S(1) -> S(0) 62 / 11,
+// P(sum) -> B 97 / 71.
+template <int ESZ, int OP, int KB>
+__global__ void __launch_bounds__(256, shift_ctas(OP, KB, ESZ)) box_shift_kernel(const __grid_constant__ BoxParams p) {
+  constexpr int J = OP == OP_COPY ? kShiftJCopy : shift_j(KB, ESZ);
+  SBP_PDL_RELEASE();
+  const unsigned tile = blockIdx.x / (unsigned)p.ntasks;
+  const int t = (int)(blockIdx.x - tile * (unsigned)p.ntasks);
+  int s = t, d = t;
+  if (p.one_dst) { d = p.dst_shard; if (p.mode == MODE_DIAG) s = p.dst_shard; }
+  else if (p.mode == MODE_PAIRS) { s = t / p.k; d = t - s * p.k; }
+  else if (p.mode == MODE_REDUCE_B) { s = 0; d = 0; }
+  TaskGeom g;
+  task_geometry(p, s, d, 1, &g);
+  SegView v;
+  v.nseg = g.nseg;  v.la = g.la;  v.M = p.M;  v.seg_bytes = g.seg_vecs;      // "vectors" of one byte
+  v.flat = p.A == 1 && p.M == 1;
+  if (v.nseg == 0 || v.seg_bytes == 0) return;
+  const long long cs = p.C * p.esz;
+  v.sm = g.Ps * cs;  v.si = p.M * v.sm;  v.sx = g.Na_s * v.si;  v.s0 = g.aoff_s * v.si + g.boff_s * cs;
+  v.dm = g.Pd * cs;  v.di = p.M * v.dm;  v.dx = g.Na_d * v.di;  v.d0 = g.aoff_d * v.di + g.boff_d * cs;
+  const bool all = p.mode == MODE_GATHER || p.mode == MODE_REDUCE_B;
+  const ShiftPlan sp{p.shift_team_log2, p.shift_chunks};
+  if (OP == OP_COPY) shift_unit<ESZ, OP, J, KB>(v, sp, tile, p.src, p.src_bytes, s, 1, 1, all ? p.dst : p.dst + d, all ? p.n_dst : 1);
+  else shift_unit<ESZ, OP, J, KB>(v, sp, tile, p.src, p.src_bytes, 0, 1, p.k, all ? p.dst : p.dst + d, all ? p.n_dst : 1);
+}
+
 // row = c / per_row and the remainder; 32-bit arithmetic whenever both fit (a 64-bit division
 // costs an order of magnitude more and sits in front of every chunk's loads).
 __device__ __forceinline__ void chunk_row(long long c, long long per_row, long long* row, long long* within) {
@@ -311,6 +341,7 @@ struct Plan {
   int vbytes;
   int ntasks;
   long long grid;
+  bool shift;       // unaligned data in 16-byte vectors (boxing_shift.h)
 };
 
 static int pick_vector_bytes(const BoxParams& p, const sbp_tensor* src, const sbp_tensor* dst, int k) {
@@ -381,6 +412,32 @@ static void launch_v_f32(const Plan& pl, cudaStream_t st) {
 
 constexpr int kJCopy = 4;
 constexpr int kJReduce = 2;
+
+template <int ESZ, int OP>
+static void launch_shift_k(const Plan& pl, cudaStream_t st) {
+  const dim3 g((unsigned)pl.grid), b(256);
+  switch (OP == OP_COPY ? 1 : shift_kb(pl.p.k)) {
+    case 1: launch_dependent(box_shift_kernel<ESZ, OP, 1>, g, b, 0, st, pl.p); break;
+    case 2: if constexpr (OP != OP_COPY) launch_dependent(box_shift_kernel<ESZ, OP, 2>, g, b, 0, st, pl.p); break;
+    case 3: if constexpr (OP != OP_COPY) launch_dependent(box_shift_kernel<ESZ, OP, 3>, g, b, 0, st, pl.p); break;
+    default: if constexpr (OP != OP_COPY) launch_dependent(box_shift_kernel<ESZ, OP, 4>, g, b, 0, st, pl.p); break;
+  }
+}
+
+static void launch_shift(const Plan& pl, cudaStream_t st) {
+  SBP_BOUNDS_UPLOAD(st);
+  switch (pl.op) {
+    case OP_COPY:
+      if (pl.p.esz == 2) launch_shift_k<2, OP_COPY>(pl, st);
+      else if (pl.p.esz == 4) launch_shift_k<4, OP_COPY>(pl, st);
+      else launch_shift_k<8, OP_COPY>(pl, st);
+      break;
+    case OP_SUM_F32: launch_shift_k<4, OP_SUM_F32>(pl, st); break;
+    case OP_MAX_F32: launch_shift_k<4, OP_MAX_F32>(pl, st); break;
+    case OP_SUM_BF16: launch_shift_k<2, OP_SUM_BF16>(pl, st); break;
+    case OP_MAX_BF16: launch_shift_k<2, OP_MAX_BF16>(pl, st); break;
+  }
+}
 
 static sbp_status make_plan(const sbp_tensor* src, const sbp_tensor* dst, int dst_shard, Plan* pl) {
   const int k = placement_k(src);
@@ -506,6 +563,40 @@ static sbp_status make_plan(const sbp_tensor* src, const sbp_tensor* dst, int ds
   const long long lb_max = ((p.src_b || p.dst_b) && p.mode != MODE_SCATTER_P) ? (p.Nb + k - 1) / k : p.Nb;
   const long long nseg_max = p.A * la_max * p.M;
   const long long seg_vecs_max = lb_max * p.C * p.esz / pl->vbytes;
+  pl->ntasks = p.mode == MODE_PAIRS ? k * k : (p.mode == MODE_REDUCE_B ? 1 : k);
+  if (p.one_dst) pl->ntasks = (p.mode == MODE_PAIRS || p.mode == MODE_GATHER) ? k : 1;
+  p.ntasks = pl->ntasks;
+
+  // Unaligned data: 16-byte vectors of the destination with shifted sources, unless the segments are so short
+  // that their incomplete ends are most of them, the tensor so small that the call is all latency (one element
+  // per thread then has the shorter chain), or buffers that share an offset differ modulo 16.
+  const long long seg_bytes_max = lb_max * p.C * p.esz;
+  pl->shift = false;
+  if (pl->vbytes < 16 && p.mode != MODE_SCATTER_P && src->dtype == dst->dtype && seg_bytes_max >= kShiftMinSegment &&
+      numel(src) >= kShiftMinElements) {
+    bool ok = true;
+    for (int q = 1; q < p.n_dst; ++q)
+      ok = ok && (reinterpret_cast<uintptr_t>(p.dst[q]) - reinterpret_cast<uintptr_t>(p.dst[0])) % 16 == 0;
+    if (pl->op != OP_COPY)
+      for (int r = 1; r < k; ++r) ok = ok && (reinterpret_cast<uintptr_t>(p.src[r]) - reinterpret_cast<uintptr_t>(p.src[0])) % 16 == 0;
+    const ShiftPlan sp = shift_plan(seg_bytes_max, pl->op == OP_COPY ? kShiftJCopy : shift_j(shift_kb(k), p.esz));
+    const long long units = nseg_max * sp.chunks, teams = 256 >> sp.team_log2;
+    const long long tiles = std::max(1LL, (units + teams - 1) / teams);
+    if (ok && units < 0x7fffff00LL && tiles * pl->ntasks <= 0x7fffffffLL) {
+      pl->shift = true;
+      p.shift_team_log2 = sp.team_log2;
+      p.shift_chunks = sp.chunks;
+      for (int r = 0; r < k; ++r) {
+        const long long n = local_numel(src, r), pitch = local_pitch(src, r);
+        int64_t shp[SBP_MAX_DIMS];
+        local_shape_nd(src, r, shp);
+        const long long cols = shp[src->ndim - 1];
+        p.src_bytes[r] = n == 0 ? 0 : ((n / cols - 1) * pitch + cols) * p.esz;
+      }
+      pl->grid = tiles * pl->ntasks;
+      return SBP_OK;
+    }
+  }
   const int J = pl->op == OP_COPY ? kJCopy : kJReduce;
   const int tile_vecs = J * 256;
   int cv_log2 = 0;
@@ -515,9 +606,6 @@ static sbp_status make_plan(const sbp_tensor* src, const sbp_tensor* dst, int ds
   p.col_tiles = std::max(1LL, (seg_vecs_max + (1LL << cv_log2) - 1) >> cv_log2);
   const long long row_tiles = std::max(1LL, (nseg_max + p.rows_per_tile - 1) / p.rows_per_tile);
   p.tiles_per_task = p.col_tiles * row_tiles;
-  pl->ntasks = p.mode == MODE_PAIRS ? k * k : (p.mode == MODE_REDUCE_B ? 1 : k);
-  if (p.one_dst) pl->ntasks = (p.mode == MODE_PAIRS || p.mode == MODE_GATHER) ? k : 1;
-  p.ntasks = pl->ntasks;
   pl->grid = p.tiles_per_task * pl->ntasks;
   if (pl->grid > 0x7fffffffLL) return fail(SBP_ERR_UNSUPPORTED, "tensor too large for one launch");
   return SBP_OK;
@@ -730,6 +818,10 @@ static sbp_status boxing_one_axis(const sbp_tensor* src, sbp_tensor* dst, int ds
   const bool want_bulk = engine == 2;
   if (!done && pl.op == OP_COPY && want_bulk && pl.vbytes == 16 && !pl.pitched)
     done = launch_bulk_copy(pl.p, pl.ntasks, stream);
+  if (!done && pl.shift) {
+    launch_shift(pl, stream);
+    done = true;
+  }
   if (!done) {
     switch (pl.op) {
       case OP_COPY: launch_v<OP_COPY, kJCopy>(pl, stream); break;

@@ -18,6 +18,7 @@
 
 #include "bounds_check.h"
 #include "boxing_arith.h"
+#include "boxing_shift.h"
 #include "sbp_internal.h"
 
 namespace sbp {
@@ -46,6 +47,9 @@ struct DisjointParams {
   int one_dst, dst_shard;           // one_dst: only the tasks that produce destination shard dst_shard
   int cv_log2, rows_per_tile, ntasks;
   unsigned char pair_s[kMaxPairs], pair_d[kMaxPairs];
+  long long src_bytes[SBP_MAX_K];   // 16-byte path for unaligned data (boxing_shift.h)
+  int shift_team_log2;
+  unsigned shift_chunks;
   // quotient and remainder of each axis by each side's shard count: the balanced split without a division
   long long a_base_s, a_rem_s, a_base_d, a_rem_d, b_base_s, b_rem_s, b_base_d, b_rem_d;
 };
@@ -79,6 +83,58 @@ __device__ __forceinline__ AxisCut cut_axis(long long n, bool by_src, long long 
   return c;
 }
 
+// Source and destination shard of task t.
+__device__ __forceinline__ void disjoint_task(const DisjointParams& p, int t, int* s, int* d) {
+  *s = 0;
+  *d = 0;
+  switch (p.mode) {
+    case DJ_PAIRS:
+      if (p.n_pairs > 0) { *s = p.pair_s[t]; *d = p.pair_d[t]; }
+      else if (p.one_dst) { *s = t; *d = p.dst_shard; }
+      else { *s = t / p.kd; *d = t - *s * p.kd; }
+      break;
+    case DJ_FROM_REPLICA: *d = p.one_dst ? p.dst_shard : t; *s = *d % p.ks; break;
+    case DJ_TO_ALL: *s = t; break;
+    case DJ_REDUCE: *d = p.one_dst ? p.dst_shard : t; break;
+    default: break;
+  }
+}
+
+// Sources of a reducing task: first, first + stride, ...
+__device__ __forceinline__ void disjoint_sources(const DisjointParams& p, int d, int* first, int* stride, int* count) {
+  *first = 0;
+  *stride = 1;
+  *count = p.ks;
+  if (p.mode == DJ_REDUCE && p.red_by_dst) {
+    *first = d;
+    *stride = p.kd;
+    *count = d < p.ks ? (p.ks - d + p.kd - 1) / p.kd : 0;
+  }
+}
+
+// The same tasks over data that is not 16-byte aligned (boxing_shift.h).
+template <int ESZ, int OP, int KB>
+__global__ void __launch_bounds__(256, shift_ctas(OP, KB, ESZ)) box_disjoint_shift_kernel(const __grid_constant__ DisjointParams p) {
+  constexpr int J = OP == OP_COPY ? kShiftJCopy : shift_j(KB, ESZ);
+  SBP_PDL_RELEASE();
+  const unsigned tile = blockIdx.x / (unsigned)p.ntasks;
+  int s, d;
+  disjoint_task(p, (int)(blockIdx.x - tile * (unsigned)p.ntasks), &s, &d);
+  const AxisCut ca = cut_axis(p.Na, p.src_a, p.a_base_s, p.a_rem_s, s, p.dst_a, p.a_base_d, p.a_rem_d, d, p.dst_full);
+  const AxisCut cb = cut_axis(p.Nb, p.src_b, p.b_base_s, p.b_rem_s, s, p.dst_b, p.b_base_d, p.b_rem_d, d, p.dst_full);
+  if (ca.len <= 0 || cb.len <= 0) return;
+  const long long cs = p.C * p.esz;
+  SegView v;
+  v.nseg = p.A * ca.len * p.M;  v.la = ca.len;  v.M = p.M;  v.seg_bytes = cb.len * cs;
+  v.flat = p.A == 1 && p.M == 1;
+  v.sm = cb.n_s * cs;  v.si = p.M * v.sm;  v.sx = ca.n_s * v.si;  v.s0 = ca.off_s * v.si + cb.off_s * cs;
+  v.dm = cb.n_d * cs;  v.di = p.M * v.dm;  v.dx = ca.n_d * v.di;  v.d0 = ca.off_d * v.di + cb.off_d * cs;
+  int first = s, stride = 1, count = 1;
+  if (OP != OP_COPY) disjoint_sources(p, d, &first, &stride, &count);
+  const bool all = p.mode == DJ_TO_ALL || p.mode == DJ_REDUCE_ALL;
+  shift_unit<ESZ, OP, J, KB>(v, ShiftPlan{p.shift_team_log2, p.shift_chunks}, tile, p.src, p.src_bytes, first, stride, count, all ? p.dst : p.dst + d, all ? p.n_dst : 1);
+}
+
 template <typename V, int OP>
 __global__ void __launch_bounds__(256, OP == OP_COPY ? 4 : 3) box_disjoint_kernel(const __grid_constant__ DisjointParams p) {
   constexpr int J = OP == OP_COPY ? 4 : 2;
@@ -90,19 +146,8 @@ __global__ void __launch_bounds__(256, OP == OP_COPY ? 4 : 3) box_disjoint_kerne
   const long long row_tile = row_tile_u;
   const long long col_tile = rem - row_tile_u * (unsigned)p.col_tiles;
 
-  int s = 0, d = 0;
-  switch (p.mode) {
-    case DJ_PAIRS:
-      if (p.n_pairs > 0) { s = p.pair_s[t]; d = p.pair_d[t]; }
-      else if (p.one_dst) { s = t; d = p.dst_shard; }
-      else { s = t / p.kd; d = t - s * p.kd; }
-      break;
-    case DJ_FROM_REPLICA: d = p.one_dst ? p.dst_shard : t; s = d % p.ks; break;
-    case DJ_TO_ALL: s = t; break;
-    case DJ_REDUCE: d = p.one_dst ? p.dst_shard : t; break;
-    default: break;
-  }
-
+  int s, d;
+  disjoint_task(p, t, &s, &d);
   const AxisCut ca = cut_axis(p.Na, p.src_a, p.a_base_s, p.a_rem_s, s, p.dst_a, p.a_base_d, p.a_rem_d, d, p.dst_full);
   const AxisCut cb = cut_axis(p.Nb, p.src_b, p.b_base_s, p.b_rem_s, s, p.dst_b, p.b_base_d, p.b_rem_d, d, p.dst_full);
   if (ca.len <= 0 || cb.len <= 0) return;
@@ -143,12 +188,8 @@ __global__ void __launch_bounds__(256, OP == OP_COPY ? 4 : 3) box_disjoint_kerne
       if (ok[j] && SBP_GUARD(sp + so[j], sizeof(V))) val[j] = ld_stream(sp + so[j]);
   } else {
     using L = typename Lanes<OP, V>::type;
-    int first = 0, stride = 1, count = p.ks;
-    if (p.mode == DJ_REDUCE && p.red_by_dst) {
-      first = d;
-      stride = p.kd;
-      count = d < p.ks ? (p.ks - d + p.kd - 1) / p.kd : 0;
-    }
+    int first, stride, count;
+    disjoint_sources(p, d, &first, &stride, &count);
     // sources in ascending order, four at a time so that 4 * J loads are in flight per thread
     constexpr int kBatch = 4;
     L acc[J];
@@ -226,6 +267,32 @@ static void launch_disjoint(const DisjointParams& p, int vbytes, long long grid,
       // a 2-byte vector cannot carry an fp32 lane; the fp32 reductions never get here
       if constexpr (OP != OP_SUM_F32 && OP != OP_MAX_F32) launch_dependent(box_disjoint_kernel<uint16_t, OP>, g, b, 0, st, p);
       break;
+  }
+}
+
+template <int ESZ, int OP>
+static void launch_disjoint_shift_k(const DisjointParams& p, long long grid, cudaStream_t st) {
+  const dim3 g((unsigned)grid), b(256);
+  switch (OP == OP_COPY ? 1 : shift_kb(p.ks)) {
+    case 1: launch_dependent(box_disjoint_shift_kernel<ESZ, OP, 1>, g, b, 0, st, p); break;
+    case 2: if constexpr (OP != OP_COPY) launch_dependent(box_disjoint_shift_kernel<ESZ, OP, 2>, g, b, 0, st, p); break;
+    case 3: if constexpr (OP != OP_COPY) launch_dependent(box_disjoint_shift_kernel<ESZ, OP, 3>, g, b, 0, st, p); break;
+    default: if constexpr (OP != OP_COPY) launch_dependent(box_disjoint_shift_kernel<ESZ, OP, 4>, g, b, 0, st, p); break;
+  }
+}
+
+static void launch_disjoint_shift(const DisjointParams& p, int op, long long grid, cudaStream_t st) {
+  SBP_BOUNDS_UPLOAD(st);
+  switch (op) {
+    case OP_COPY:
+      if (p.esz == 2) launch_disjoint_shift_k<2, OP_COPY>(p, grid, st);
+      else if (p.esz == 4) launch_disjoint_shift_k<4, OP_COPY>(p, grid, st);
+      else launch_disjoint_shift_k<8, OP_COPY>(p, grid, st);
+      break;
+    case OP_SUM_F32: launch_disjoint_shift_k<4, OP_SUM_F32>(p, grid, st); break;
+    case OP_MAX_F32: launch_disjoint_shift_k<4, OP_MAX_F32>(p, grid, st); break;
+    case OP_SUM_BF16: launch_disjoint_shift_k<2, OP_SUM_BF16>(p, grid, st); break;
+    default: launch_disjoint_shift_k<2, OP_MAX_BF16>(p, grid, st); break;
   }
 }
 
@@ -381,7 +448,7 @@ sbp_status boxing_disjoint(const sbp_tensor* src, sbp_tensor* dst, int dst_shard
     return m;
   };
   const long long nseg_max = p.A * max_cut(p.Na, p.src_a, p.dst_a) * p.M;
-  const long long seg_vecs_max = max_cut(p.Nb, p.src_b, p.dst_b) * p.C * esz / vbytes;
+  const long long seg_bytes_max = max_cut(p.Nb, p.src_b, p.dst_b) * p.C * esz, seg_vecs_max = seg_bytes_max / vbytes;
   const int tile_vecs = (op == OP_COPY ? 4 : 2) * 256;
   int cv_log2 = 0;
   while ((1 << cv_log2) < tile_vecs && (1LL << cv_log2) < seg_vecs_max) ++cv_log2;
@@ -390,7 +457,27 @@ sbp_status boxing_disjoint(const sbp_tensor* src, sbp_tensor* dst, int dst_shard
   p.col_tiles = std::max(1LL, (seg_vecs_max + (1LL << cv_log2) - 1) >> cv_log2);
   const long long row_tiles = std::max(1LL, (nseg_max + p.rows_per_tile - 1) / p.rows_per_tile);
   p.tiles_per_task = p.col_tiles * row_tiles;
-  const long long grid = p.tiles_per_task * p.ntasks;
+  long long grid = p.tiles_per_task * p.ntasks;
+  // unaligned data in 16-byte vectors, by the rule of the same-placement kernels
+  bool shift = vbytes < 16 && seg_bytes_max >= kShiftMinSegment && numel(src) >= kShiftMinElements;
+  if (op != OP_COPY)
+    for (int r = 1; r < ks; ++r)
+      shift = shift && (reinterpret_cast<uintptr_t>(src->local[r]) - reinterpret_cast<uintptr_t>(src->local[0])) % 16 == 0;
+  for (int q = 1; q < p.n_dst; ++q)
+    shift = shift && (reinterpret_cast<uintptr_t>(p.dst[q]) - reinterpret_cast<uintptr_t>(p.dst[0])) % 16 == 0;
+  if (shift) {
+    const ShiftPlan sp = shift_plan(seg_bytes_max, op == OP_COPY ? kShiftJCopy : shift_j(shift_kb(ks), esz));
+    const long long units = nseg_max * sp.chunks, teams = 256 >> sp.team_log2;
+    const long long tiles = std::max(1LL, (units + teams - 1) / teams);
+    if (units < 0x7fffff00LL && tiles * p.ntasks <= 0x7fffffffLL) {
+      p.shift_team_log2 = sp.team_log2;
+      p.shift_chunks = sp.chunks;
+      for (int r = 0; r < ks; ++r) p.src_bytes[r] = (long long)local_numel(src, r) * esz;
+      grid = tiles * p.ntasks;
+    } else {
+      shift = false;
+    }
+  }
   if (copy_needed && grid > 0x7fffffffLL) return fail(SBP_ERR_UNSUPPORTED, "tensor too large for one launch");
   if (dry) return SBP_OK;   // every refusal lies above this line, every launch below it
   SBP_BOUNDS_RESET();
@@ -426,7 +513,8 @@ sbp_status boxing_disjoint(const sbp_tensor* src, sbp_tensor* dst, int dst_shard
     }
   }
   if (!copy_needed) return SBP_OK;
-  switch (op) {
+  if (shift) launch_disjoint_shift(p, op, grid, stream);
+  else switch (op) {
     case OP_COPY: launch_disjoint<OP_COPY>(p, vbytes, grid, stream); break;
     case OP_SUM_F32: launch_disjoint<OP_SUM_F32>(p, vbytes, grid, stream); break;
     case OP_MAX_F32: launch_disjoint<OP_MAX_F32>(p, vbytes, grid, stream); break;

@@ -32,6 +32,10 @@ struct BoxParams {
   // Row pitch of every local tensor in units of C elements, 0 = dense (the pitch is then the local
   // extent of the Nb axis).  Non-zero only for 2-D tensors with a leading dimension (C == 1).
   long long src_pitch[SBP_MAX_K], dst_pitch[SBP_MAX_K];
+  // 16-byte path for unaligned data (boxing_shift.h): bytes of every source local tensor, how segments are dealt out
+  long long src_bytes[SBP_MAX_K];
+  int shift_team_log2;
+  unsigned shift_chunks;
 };
 
 // Start and length of shard r's piece of an axis whose n / k and n % k are known.
