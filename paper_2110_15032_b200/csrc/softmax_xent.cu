@@ -5,6 +5,7 @@
 //   partial kernel   one CTA per (row, shard, column chunk) streams its piece of the logits
 //                    once and leaves a local max m_p, a local exp-sum s_p = sum exp(z - m_p)
 //                    and the label's logit t_p (0 when the label lies elsewhere);
+//   (or, with many rows, one kernel whose teams of threads finish a row each: xent_rows_kernel)
 //   combine kernel   per row, over the pieces p (one warp per row: the pieces of a lane in
 //                    ascending order, then the lanes by a butterfly):
 //                    m = max_p m_p            (the P(max) -> B boxing of the local maxima)
@@ -16,6 +17,7 @@
 // so results are reproducible for a given shape.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cfloat>
 #include <cmath>
 
@@ -39,8 +41,7 @@ struct XentParams {
   long long rows, classes;
   long long pitch[SBP_MAX_K];   // elements between consecutive rows of shard r's logits
   int k, nsplit;
-  long long chunk;   // elements per chunk (kThreads * kLoadsPerThread * VEC)
-  long long span;    // elements per CTA (chunk * chunks per CTA)
+  long long span;    // elements per CTA
 };
 
 struct XentCombineParams {
@@ -73,24 +74,37 @@ __device__ __forceinline__ void merge(float& m, float& s, float m2, float s2) {
   m = mm;
 }
 
-// ---- chunk policies: how one thread loads, maxes and exp-sums its kLoadsPerThread vectors
+// Loss, max and sum of a finished row, to every replica.
+__device__ __forceinline__ void write_row(const XentCombineParams& p, long long row, float m, float S, float zy) {
+  const float loss = logf(S) + m - zy;
+  for (int j = 0; j < p.n_loss; ++j)
+    if (SBP_GUARD(p.loss[j] + row, 4)) p.loss[j][row] = loss;
+  for (int j = 0; j < p.n_max; ++j)
+    if (SBP_GUARD(p.row_max[j] + row, 4)) p.row_max[j][row] = m;
+  for (int j = 0; j < p.n_sum; ++j)
+    if (SBP_GUARD(p.row_sum[j] + row, 4)) p.row_sum[j][row] = S;
+}
 
-// bf16, 8 elements per 16-byte load; max on packed pairs, exp in fp32.
-struct ChunkBF16x8 {
+// ---- chunk policies: how one thread of a team loads, maxes and exp-sums its kLoadsPerThread vectors of 16 bytes.  z
+// points at the first vector (16-byte aligned), nv counts the vectors there are.
+
+__device__ __forceinline__ uint4 ld_logits(const void* p) {
+  uint4 r;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
+  return r;
+}
+
+// bf16, 8 elements per load; max on packed pairs, exp in fp32.
+struct ChunkBF16 {
   using T = __nv_bfloat16;
   static constexpr int VEC = 8;
   uint4 raw[kLoadsPerThread];
-  __device__ __forceinline__ void load(const T* z, long long n, int tid) {
+  __device__ __forceinline__ void load(const T* z, long long nv, int tid, int team) {
 #pragma unroll
     for (int u = 0; u < kLoadsPerThread; ++u) {
-      const long long e0 = ((long long)u * kThreads + tid) * VEC;
-      if (e0 < n && SBP_GUARD(z + e0, 16)) {
-        asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-                     : "=r"(raw[u].x), "=r"(raw[u].y), "=r"(raw[u].z), "=r"(raw[u].w)
-                     : "l"(z + e0));
-      } else {
-        raw[u] = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);   // -inf, -inf
-      }
+      const long long v = (long long)u * team + tid;
+      if (v < nv && SBP_GUARD(z + v * VEC, 16)) raw[u] = ld_logits(z + v * VEC);
+      else raw[u] = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);   // -inf, -inf
     }
   }
   __device__ __forceinline__ float max() const {
@@ -121,45 +135,128 @@ struct ChunkBF16x8 {
   }
 };
 
-// Generic policy: element type TT, V elements per load (V * sizeof(TT) is 16 or sizeof(TT)).
-template <typename TT, int V>
-struct ChunkGeneric {
-  using T = TT;
-  static constexpr int VEC = V;
-  struct alignas(sizeof(TT) * V) Pack { TT e[V]; };
-  Pack raw[kLoadsPerThread];
-  bool ok[kLoadsPerThread];
-  __device__ __forceinline__ static float f32(float v) { return v; }
-  __device__ __forceinline__ static float f32(__nv_bfloat16 v) { return __bfloat162float(v); }
-  __device__ __forceinline__ void load(const T* z, long long n, int tid) {
+// fp32, 4 elements per load.
+struct ChunkF32 {
+  using T = float;
+  static constexpr int VEC = 4;
+  uint4 raw[kLoadsPerThread];
+  __device__ __forceinline__ void load(const T* z, long long nv, int tid, int team) {
 #pragma unroll
     for (int u = 0; u < kLoadsPerThread; ++u) {
-      const long long e0 = ((long long)u * kThreads + tid) * VEC;
-      ok[u] = e0 < n && SBP_GUARD(z + e0, sizeof(Pack));
-      if (ok[u]) raw[u] = *reinterpret_cast<const Pack*>(z + e0);
+      const long long v = (long long)u * team + tid;
+      if (v < nv && SBP_GUARD(z + v * VEC, 16)) raw[u] = ld_logits(z + v * VEC);
+      else raw[u] = make_uint4(0xFF800000u, 0xFF800000u, 0xFF800000u, 0xFF800000u);   // -inf
     }
   }
   __device__ __forceinline__ float max() const {
     float m = -INFINITY;
 #pragma unroll
-    for (int u = 0; u < kLoadsPerThread; ++u)
-      if (ok[u]) {
+    for (int u = 0; u < kLoadsPerThread; ++u) {
+      const float* f = reinterpret_cast<const float*>(&raw[u]);
 #pragma unroll
-        for (int i = 0; i < VEC; ++i) m = fmaxf(m, f32(raw[u].e[i]));
-      }
+      for (int i = 0; i < 4; ++i) m = fmaxf(m, f[i]);
+    }
     return m;
   }
   __device__ __forceinline__ float expsum(float neg_m_l2e) const {
-    float s = 0.f;
+    float s0 = 0.f, s1 = 0.f;
 #pragma unroll
-    for (int u = 0; u < kLoadsPerThread; ++u)
-      if (ok[u]) {
-#pragma unroll
-        for (int i = 0; i < VEC; ++i) s += ex2(fmaf(f32(raw[u].e[i]), kLog2e, neg_m_l2e));
-      }
-    return s;
+    for (int u = 0; u < kLoadsPerThread; ++u) {
+      const float* f = reinterpret_cast<const float*>(&raw[u]);
+      s0 += ex2(fmaf(f[0], kLog2e, neg_m_l2e));
+      s1 += ex2(fmaf(f[1], kLog2e, neg_m_l2e));
+      s0 += ex2(fmaf(f[2], kLog2e, neg_m_l2e));
+      s1 += ex2(fmaf(f[3], kLog2e, neg_m_l2e));
+    }
+    return s0 + s1;
   }
 };
+
+// Elements before the first 16-byte boundary at or after z, at most n.
+template <typename T>
+__device__ __forceinline__ int to_boundary(const T* z, long long n) {
+  const int h = (int)((0ull - reinterpret_cast<unsigned long long>(z)) & 15) / (int)sizeof(T);
+  return h < n ? h : (int)n;
+}
+
+// A team's pass over the n > 0 logits at z: the running (m, s) of each of its threads.
+// A row starts wherever the class count and the pitch put it: up to 15 bytes on either end of the span are taken
+// element by element, one element a thread, and what lies between as aligned vectors; the loads of the next chunk
+// are issued before the current one is reduced.  (Unaligned rows element by element throughout: fp32 [256, 100003]
+// over four shards 33 us, backward 76; as here 25 and 35: 0.62 and 0.89 of the copy bandwidth.)
+template <typename Chunk>
+__device__ __forceinline__ void walk_span(const typename Chunk::T* z, long long n, int tid, int team, float& m, float& s) {
+  using T = typename Chunk::T;
+  constexpr int VEC = Chunk::VEC;
+  const int head = to_boundary(z, n);
+  const long long nv = (n - head) / VEC;
+  const int tail = (int)(n - head - nv * VEC);
+  const T* zv = z + head;
+  const long long step = (long long)team * kLoadsPerThread;     // vectors per chunk
+  Chunk cur, nxt;
+  if (nv > 0) cur.load(zv, nv, tid, team);
+  const T* lone = tid < head ? z + tid : (tid >= 16 && tid - 16 < tail ? zv + nv * VEC + (tid - 16) : nullptr);
+  if (lone && SBP_GUARD(lone, sizeof(T))) {
+    const float x = static_cast<float>(*lone);
+    if (x != -INFINITY) merge(m, s, x, 1.f);
+  }
+  for (long long off = 0; off < nv; off += step) {
+    const bool more = off + step < nv;
+    if (more) nxt.load(zv + (off + step) * VEC, nv - off - step, tid, team);
+    const float cm = cur.max();
+    if (cm != -INFINITY) {
+      const float mm = fmaxf(m, cm);
+      const float neg = -mm * kLog2e;
+      const float carried = (m == -INFINITY) ? 0.f : s * ex2(fmaf(m, kLog2e, neg));
+      s = carried + cur.expsum(neg);
+      m = mm;
+    }
+    if (more) cur = nxt;
+  }
+}
+
+// Many rows: a team of 1 << team_log2 threads takes a whole row, shard after shard, and finishes it -- no partials,
+// no second kernel.  Taken from 740 rows on (five CTAs an SM), with the team that spreads the rows over the device
+// once.  (us, partial + combine kernels / this: fp32 [4096, 1003] over two shards 24 / 8.5, bf16 [1000, 30000] over
+// four 39 / 24.)
+constexpr long long kRowsForTeams = 740;
+
+template <typename Chunk>
+__global__ void __launch_bounds__(kThreads) xent_rows_kernel(const __grid_constant__ XentParams p, const __grid_constant__ XentCombineParams c,
+                                                            int team_log2) {
+  using T = typename Chunk::T;
+  const int team = 1 << team_log2, tl = threadIdx.x & (team - 1);
+  const long long row = (long long)blockIdx.x * (kThreads >> team_log2) + (threadIdx.x >> team_log2);
+  float m = -INFINITY, s = 0.f, t = 0.f;
+  if (row < p.rows) {
+    const long long y = SBP_GUARD(p.labels + row, 8) ? p.labels[row] : -1;
+    for (int r = 0; r < p.k; ++r) {
+      long long c_start, c_len;
+      split_range(p.classes, p.k, r, (int64_t*)&c_start, (int64_t*)&c_len);
+      const T* z = reinterpret_cast<const T*>(p.logits[r]) + row * p.pitch[r];
+      if (c_len > 0) walk_span<Chunk>(z, c_len, tl, team, m, s);
+      if (tl == 0 && y >= c_start && y < c_start + c_len && SBP_GUARD(z + (y - c_start), sizeof(T))) t = static_cast<float>(z[y - c_start]);
+    }
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    const float m2 = __shfl_xor_sync(0xffffffffu, m, off);
+    const float s2 = __shfl_xor_sync(0xffffffffu, s, off);
+    merge(m, s, m2, s2);
+  }
+  if (team > 32) {
+    __shared__ float sm[kThreads / 32], ss[kThreads / 32];
+    const int w0 = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0) {
+      sm[w0] = m;
+      ss[w0] = s;
+    }
+    __syncthreads();
+    if (tl == 0)
+      for (int w = 1; w < team / 32; ++w) merge(m, s, sm[w0 + w], ss[w0 + w]);
+  }
+  if (tl == 0 && row < p.rows) write_row(c, row, m, s, t);
+}
 
 // One CTA per (row, shard, column span).  Each thread keeps a running (m, s) over the chunks
 // of its span -- the loads of the next chunk are issued before the current one is reduced --
@@ -183,21 +280,7 @@ __global__ void __launch_bounds__(kThreads) xent_partial_kernel(const __grid_con
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   float m = -INFINITY, s = 0.f;
-  Chunk cur, nxt;
-  if (n > 0) cur.load(z, n, tid);
-  for (long long off = 0; off < n; off += p.chunk) {
-    const bool more = off + p.chunk < n;
-    if (more) nxt.load(z + off + p.chunk, n - off - p.chunk, tid);
-    const float cm = cur.max();
-    if (cm != -INFINITY) {
-      const float mm = fmaxf(m, cm);
-      const float neg = -mm * kLog2e;
-      const float carried = (m == -INFINITY) ? 0.f : s * ex2(fmaf(m, kLog2e, neg));
-      s = carried + cur.expsum(neg);
-      m = mm;
-    }
-    if (more) cur = nxt;
-  }
+  if (n > 0) walk_span<Chunk>(z, n, tid, kThreads, m, s);
 
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
@@ -250,46 +333,46 @@ __global__ void __launch_bounds__(kCombineThreads) xent_combine_kernel(const __g
     zy += __shfl_xor_sync(0xffffffffu, zy, off);
     merge(m, S, m2, s2);
   }
-  if (lane == 0) {
-    const float loss = logf(S) + m - zy;
-    for (int j = 0; j < p.n_loss; ++j)
-      if (SBP_GUARD(p.loss[j] + row, 4)) p.loss[j][row] = loss;
-    for (int j = 0; j < p.n_max; ++j)
-      if (SBP_GUARD(p.row_max[j] + row, 4)) p.row_max[j][row] = m;
-    for (int j = 0; j < p.n_sum; ++j)
-      if (SBP_GUARD(p.row_sum[j] + row, 4)) p.row_sum[j][row] = S;
-  }
+  if (lane == 0) write_row(p, row, m, S, zy);
 }
 
-// Elements of one CTA's column span, and how many spans cover the widest shard.
-static void tiling_for(const sbp_tensor* logits, int vec, long long* chunk, long long* span, int* nsplit) {
+// Elements of one CTA's column span, and how many spans cover the widest shard, for loads of `vec` elements.
+static void tiling_for(const sbp_tensor* logits, int vec, long long* span, int* nsplit) {
   const int k = placement_k(logits);
   const long long c_max = (logits->shape[1] + k - 1) / k;
-  *chunk = (long long)kThreads * kLoadsPerThread * vec;
-  long long chunks = (c_max + *chunk - 1) / *chunk;
+  const long long chunk = (long long)kThreads * kLoadsPerThread * vec;
+  long long chunks = (c_max + chunk - 1) / chunk;
   if (chunks < 1) chunks = 1;
   const long long per_cta = chunks < kMaxChunksPerCta ? chunks : kMaxChunksPerCta;
-  *span = *chunk * per_cta;
+  *span = chunk * per_cta;
   *nsplit = (int)((chunks + per_cta - 1) / per_cta);
 }
 
 static int nsplit_for(const sbp_tensor* logits, int vec) {
-  long long chunk, span;
+  long long span;
   int ns;
-  tiling_for(logits, vec, &chunk, &span, &ns);
+  tiling_for(logits, vec, &span, &ns);
   return ns;
 }
 
-// Elements per load: 16 bytes worth when every shard's rows are 16-byte aligned, else 1.
-static int pick_vec(const sbp_tensor* logits) {
-  const int k = placement_k(logits), esz = elem_size(logits->dtype);
-  for (int r = 0; r < k; ++r) {
-    int64_t st, ln;
-    split_range(logits->shape[1], k, r, &st, &ln);
-    if ((ln * esz) % 16 != 0 || (local_pitch(logits, r) * esz) % 16 != 0) return 1;
-    if (logits->local[r] && reinterpret_cast<uintptr_t>(logits->local[r]) % 16 != 0) return 1;
+static int vec_of(const sbp_tensor* logits) { return 16 / elem_size(logits->dtype); }
+
+// The spans a call uses: those of tiling_for, or shorter ones (down to one chunk) when the rows alone do not fill the
+// device four CTAs deep and the scratch has room for the partials.
+static void tiling_in(const sbp_tensor* logits, size_t ws_bytes, long long* span, int* nsplit) {
+  tiling_for(logits, vec_of(logits), span, nsplit);
+  const int k = placement_k(logits);
+  const long long rows = logits->shape[0], c_max = (logits->shape[1] + k - 1) / k;
+  const long long chunk = (long long)kThreads * kLoadsPerThread * vec_of(logits);
+  // (never more scratch than the size query answers or the built-in array holds, so that both entry points cut alike)
+  const size_t most = std::min({ws_bytes, sbp_softmax_xent_workspace_bytes(logits), (size_t)SBP_SOFTMAX_XENT_STATIC_SCRATCH_BYTES});
+  const long long room = (long long)(most / (3 * sizeof(float) * (size_t)k * (size_t)rows));
+  while (*nsplit * rows * k < 148 * 4 && *span > chunk) {
+    const long long sp = (*span / chunk + 1) / 2 * chunk, ns = (c_max + sp - 1) / sp;
+    if (ns > room) break;
+    *span = sp;
+    *nsplit = (int)ns;
   }
-  return 16 / esz;
 }
 
 static int dedup(float** out, const sbp_tensor* t, int k) {
@@ -458,12 +541,18 @@ struct XentBwdParams {
   const float* row_sum;
   long long rows, classes;
   long long lpitch[SBP_MAX_K], gpitch[SBP_MAX_K];   // elements between consecutive rows: logits, gradient
-  int k;
+  int k, team_log2;
 };
+
+// VEC elements of 16 bytes a thread and step where both rows stand alike modulo 16 (always, for dense tensors
+// with aligned bases), the elements before and after the whole vectors one a thread; VEC = 1 otherwise.
+constexpr int kBwdVecs = 4;      // vectors in flight per thread
 
 template <typename T, int VEC>
 __global__ void __launch_bounds__(kThreads) xent_backward_kernel(const __grid_constant__ XentBwdParams p) {
-  const long long row = blockIdx.x;
+  const int team = 1 << p.team_log2, tid = threadIdx.x & (team - 1);      // short rows: several to a CTA
+  const long long row = (long long)blockIdx.x * (kThreads >> p.team_log2) + (threadIdx.x >> p.team_log2);
+  if (row >= p.rows) return;
   const int shard = blockIdx.z;
   long long c_start, c_len;
   split_range(p.classes, p.k, shard, (int64_t*)&c_start, (int64_t*)&c_len);
@@ -473,19 +562,46 @@ __global__ void __launch_bounds__(kThreads) xent_backward_kernel(const __grid_co
   if (!SBP_GUARD(p.row_max + row, 4) || !SBP_GUARD(p.row_sum + row, 4) || !SBP_GUARD(p.labels + row, 8)) return;
   const float neg = -p.row_max[row] * kLog2e - log2f(p.row_sum[row]);
   const long long y = p.labels[row] - c_start;      // label's column inside this shard, if any
+  const int head = VEC > 1 ? to_boundary(z, c_len) : 0;
+  const long long nv = (c_len - head) / VEC;
+  const int tail = (int)(c_len - head - nv * VEC);
   struct alignas(sizeof(T) * VEC) Pack { T e[VEC]; };
-  for (long long e0 = ((long long)blockIdx.y * kThreads + threadIdx.x) * VEC; e0 < c_len;
-       e0 += (long long)gridDim.y * kThreads * VEC) {
-    if (!SBP_GUARD(z + e0, sizeof(Pack)) || !SBP_GUARD(g + e0, sizeof(Pack))) continue;
-    Pack in = *reinterpret_cast<const Pack*>(z + e0), out;
-    const int y_rel = (y >= e0 && y < e0 + VEC) ? (int)(y - e0) : -1;   // the label's place in this vector, if it is here
-#pragma unroll
-    for (int i = 0; i < VEC; ++i) {
-      float v = ex2(fmaf(static_cast<float>(in.e[i]), kLog2e, neg));
-      if (i == y_rel) v -= 1.0f;
-      out.e[i] = static_cast<T>(v);
+  if (VEC > 1 && blockIdx.y == 0) {
+    const long long at = tid < head ? tid : (tid >= 16 && tid - 16 < tail ? head + nv * VEC + (tid - 16) : -1);
+    if (at >= 0 && SBP_GUARD(z + at, sizeof(T)) && SBP_GUARD(g + at, sizeof(T))) {
+      float v = ex2(fmaf(static_cast<float>(z[at]), kLog2e, neg));
+      if (at == y) v -= 1.0f;
+      g[at] = static_cast<T>(v);
     }
-    *reinterpret_cast<Pack*>(g + e0) = out;
+  }
+  const T* zv = z + head;
+  T* gv = g + head;
+  const long long step = (long long)gridDim.y * team;
+  for (long long v0 = (long long)blockIdx.y * team + tid; v0 < nv; v0 += kBwdVecs * step) {
+    Pack in[kBwdVecs];
+#pragma unroll
+    for (int u = 0; u < kBwdVecs; ++u) {
+      const long long v = v0 + u * step;
+      if (v >= nv || !SBP_GUARD(zv + v * VEC, sizeof(Pack))) continue;
+      if constexpr (VEC > 1) *reinterpret_cast<uint4*>(&in[u]) = ld_logits(zv + v * VEC);
+      else in[u] = *reinterpret_cast<const Pack*>(zv + v * VEC);
+    }
+#pragma unroll
+    for (int u = 0; u < kBwdVecs; ++u) {
+      const long long v = v0 + u * step;
+      if (v >= nv || !SBP_GUARD(gv + v * VEC, sizeof(Pack))) continue;
+      const long long rel = y - head - v * VEC;
+      const int y_rel = rel >= 0 && rel < VEC ? (int)rel : -1;   // the label's place in this vector, if it is here
+      Pack out;
+#pragma unroll
+      for (int i = 0; i < VEC; ++i) {
+        float f = ex2(fmaf(static_cast<float>(in[u].e[i]), kLog2e, neg));
+        if (i == y_rel) f -= 1.0f;
+        out.e[i] = static_cast<T>(f);
+      }
+      if constexpr (VEC > 1) __stcs(reinterpret_cast<uint4*>(gv + v * VEC), *reinterpret_cast<const uint4*>(&out));
+      else *reinterpret_cast<Pack*>(gv + v * VEC) = out;
+    }
   }
 }
 
@@ -497,10 +613,10 @@ extern "C" {
 
 size_t sbp_softmax_xent_workspace_bytes(const sbp_tensor* logits) {
   if (check_tensor(logits, "logits", false) != SBP_OK || logits->ndim != 2) return 0;
-  // sized for the element-wise path as well, so the answer does not depend on pointer values
+  // room for spans of a sixteenth of a chunk's elements too: short rows are cut finer when there is room
   const int k = placement_k(logits);
   const int ns = nsplit_for(logits, 1);
-  const int ns_vec = nsplit_for(logits, 16 / elem_size(logits->dtype));
+  const int ns_vec = nsplit_for(logits, vec_of(logits));
   const size_t parts = (size_t)k * (size_t)(ns > ns_vec ? ns : ns_vec);
   return 3 * parts * (size_t)logits->shape[0] * sizeof(float);
 }
@@ -530,13 +646,14 @@ sbp_status sbp_softmax_xent(const sbp_tensor* logits, const sbp_tensor* labels, 
   if (classes < 1) return fail(SBP_ERR_SHAPE, "softmax over zero classes");
   if (rows == 0) return SBP_OK;
 
-  const int vec = pick_vec(logits);
-  const int nsplit = nsplit_for(logits, vec);
-  const int parts = k * nsplit;
-  const size_t need = 3 * (size_t)parts * rows * sizeof(float);
-  if (!ws || ws_bytes < need) return fail(SBP_ERR_WORKSPACE, "workspace of %zu bytes needed, %zu given", need, ws_bytes);
+  const size_t least = 3 * (size_t)k * (size_t)nsplit_for(logits, vec_of(logits)) * rows * sizeof(float);
+  if (!ws || ws_bytes < least) return fail(SBP_ERR_WORKSPACE, "workspace of %zu bytes needed, %zu given", least, ws_bytes);
   if (reinterpret_cast<uintptr_t>(ws) % 4 != 0) return fail(SBP_ERR_ALIGNMENT, "workspace must be 4-byte aligned");
+  long long span;
+  int nsplit;
+  tiling_in(logits, ws_bytes, &span, &nsplit);
   if (rows > 0x7fffffffLL || nsplit > 65535) return fail(SBP_ERR_UNSUPPORTED, "shape too large for one launch");
+  const int parts = k * nsplit;
 
   XentParams p{};
   for (int r = 0; r < k; ++r) {
@@ -551,30 +668,7 @@ sbp_status sbp_softmax_xent(const sbp_tensor* logits, const sbp_tensor* labels, 
   p.classes = classes;
   p.k = k;
   p.nsplit = nsplit;
-  {
-    int ns;
-    tiling_for(logits, vec, &p.chunk, &p.span, &ns);
-  }
-
-  cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-  dim3 grid((unsigned)rows, (unsigned)nsplit, (unsigned)k);
-  SBP_BOUNDS_RESET();
-  SBP_BOUNDS_TENSOR(logits);
-  SBP_BOUNDS_TENSOR(labels);
-  SBP_BOUNDS_TENSOR(loss);
-  SBP_BOUNDS_TENSOR(row_max);
-  SBP_BOUNDS_TENSOR(row_sum);
-  SBP_BOUNDS_ADD(ws, need);
-  SBP_BOUNDS_UPLOAD(stream);
-  if (logits->dtype == SBP_BF16) {
-    if (vec > 1) xent_partial_kernel<ChunkBF16x8><<<grid, kThreads, 0, stream>>>(p);
-    else xent_partial_kernel<ChunkGeneric<__nv_bfloat16, 1>><<<grid, kThreads, 0, stream>>>(p);
-  } else {
-    if (vec > 1) xent_partial_kernel<ChunkGeneric<float, 4>><<<grid, kThreads, 0, stream>>>(p);
-    else xent_partial_kernel<ChunkGeneric<float, 1>><<<grid, kThreads, 0, stream>>>(p);
-  }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_fail(e, "softmax partial launch");
+  p.span = span;
 
   XentCombineParams c{};
   c.part_m = p.part_m;
@@ -585,6 +679,33 @@ sbp_status sbp_softmax_xent(const sbp_tensor* logits, const sbp_tensor* labels, 
   c.n_loss = dedup(c.loss, loss, k);
   c.n_max = row_max ? dedup(c.row_max, row_max, k) : 0;
   c.n_sum = row_sum ? dedup(c.row_sum, row_sum, k) : 0;
+
+  cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+  SBP_BOUNDS_RESET();
+  SBP_BOUNDS_TENSOR(logits);
+  SBP_BOUNDS_TENSOR(labels);
+  SBP_BOUNDS_TENSOR(loss);
+  SBP_BOUNDS_TENSOR(row_max);
+  SBP_BOUNDS_TENSOR(row_sum);
+  SBP_BOUNDS_ADD(ws, 3 * (size_t)parts * rows * sizeof(float));
+  SBP_BOUNDS_UPLOAD(stream);
+  if (rows >= kRowsForTeams) {
+    const int team_log2 = rows < 2 * kRowsForTeams ? 7 : (rows < 4 * kRowsForTeams ? 6 : 5);
+    const int per_cta = kThreads >> team_log2;
+    const dim3 g((unsigned)((rows + per_cta - 1) / per_cta));
+    if (logits->dtype == SBP_BF16) xent_rows_kernel<ChunkBF16><<<g, kThreads, 0, stream>>>(p, c, team_log2);
+    else xent_rows_kernel<ChunkF32><<<g, kThreads, 0, stream>>>(p, c, team_log2);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_fail(e, "softmax launch");
+    count_launch();
+    return SBP_OK;
+  }
+  dim3 grid((unsigned)rows, (unsigned)nsplit, (unsigned)k);
+  if (logits->dtype == SBP_BF16) xent_partial_kernel<ChunkBF16><<<grid, kThreads, 0, stream>>>(p);
+  else xent_partial_kernel<ChunkF32><<<grid, kThreads, 0, stream>>>(p);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(e, "softmax partial launch");
+
   // Launched as the programmatic dependent of the partial kernel: it may be set up while that
   // kernel still runs and waits, on the device, for it to finish before reading the partials.
   cudaLaunchConfig_t cfg{};
@@ -623,7 +744,7 @@ extern "C" sbp_status sbp_softmax_xent_static(const sbp_tensor* logits, const sb
   if (st != SBP_OK) return st;
   if (logits->ndim != 2) return fail(SBP_ERR_SHAPE, "logits must be [rows, classes]");
   const size_t need =
-      3 * (size_t)placement_k(logits) * (size_t)nsplit_for(logits, pick_vec(logits)) * (size_t)logits->shape[0] * sizeof(float);
+      3 * (size_t)placement_k(logits) * (size_t)nsplit_for(logits, vec_of(logits)) * (size_t)logits->shape[0] * sizeof(float);
   if (need > kStaticScratchBytes)
     return fail(SBP_ERR_WORKSPACE,
                 "this shape needs %zu bytes of scratch but the built-in array holds %zu; call sbp_softmax_xent "
@@ -678,13 +799,11 @@ extern "C" sbp_status sbp_softmax_xent_backward(const sbp_tensor* logits, const 
   bool vec_ok = true;
   const int esz = elem_size(logits->dtype);
   for (int r = 0; r < k; ++r) {
-    int64_t s0, ln;
-    split_range(classes, k, r, &s0, &ln);
     p.lpitch[r] = local_pitch(logits, r);
     p.gpitch[r] = local_pitch(grad_logits, r);
-    vec_ok = vec_ok && (ln * esz) % 16 == 0 && reinterpret_cast<uintptr_t>(logits->local[r]) % 16 == 0 &&
-             reinterpret_cast<uintptr_t>(grad_logits->local[r]) % 16 == 0 && (p.lpitch[r] * esz) % 16 == 0 &&
-             (p.gpitch[r] * esz) % 16 == 0;
+    // every row of the gradient stands as the logits' row does, modulo 16 bytes
+    vec_ok = vec_ok && (reinterpret_cast<uintptr_t>(logits->local[r]) - reinterpret_cast<uintptr_t>(grad_logits->local[r])) % 16 == 0 &&
+             ((p.lpitch[r] - p.gpitch[r]) * esz) % 16 == 0;
     p.logits[r] = static_cast<const char*>(logits->local[r]);
     p.grad[r] = static_cast<char*>(grad_logits->local[r]);
   }
@@ -696,10 +815,13 @@ extern "C" sbp_status sbp_softmax_xent_backward(const sbp_tensor* logits, const 
   p.k = k;
   const int vec = vec_ok ? 16 / esz : 1;
   const long long c_max = (classes + k - 1) / k;
-  long long gy = (c_max + (long long)kThreads * vec * 4 - 1) / ((long long)kThreads * vec * 4);   // ~4 vectors per thread
+  long long gy = (c_max + (long long)kThreads * vec * kBwdVecs - 1) / ((long long)kThreads * vec * kBwdVecs);
   if (gy < 1) gy = 1;
   if (gy > 65535) gy = 65535;
-  dim3 grid((unsigned)rows, (unsigned)gy, (unsigned)k);
+  p.team_log2 = 5;
+  while (p.team_log2 < 8 && ((long long)vec * kBwdVecs << p.team_log2) < c_max) ++p.team_log2;
+  const int per_cta = kThreads >> p.team_log2;
+  dim3 grid((unsigned)((rows + per_cta - 1) / per_cta), (unsigned)gy, (unsigned)k);
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   SBP_BOUNDS_RESET();
   SBP_BOUNDS_TENSOR(logits);
