@@ -323,7 +323,10 @@ void sbp_boxing_set_copy_engine(int32_t engine);
  * descriptors and flags (0 when nothing has to be copied; judged from the shapes, so pass 256-byte
  * aligned local tensors or add the operands' sizes yourself); ws must be 256-byte aligned.  Without
  * a large enough workspace such a product runs on the FMA kernel: same results within the stated
- * tolerance, far slower.  sbp_matmul_workspace_bytes is the same query for flags = 0. */
+ * tolerance, far slower.  sbp_matmul_workspace_bytes is the same query for flags = 0.
+ * A 16-byte aligned workspace with more room than that is used as well where it helps: a small result of a
+ * long contraction (the feature gradient of a classifier) is cut along K over the whole device when `ws`
+ * holds at least two fp32 copies of the result. */
 size_t sbp_matmul_workspace_bytes_for(const sbp_tensor* x, const sbp_tensor* w, const sbp_tensor* y, uint32_t flags);
 size_t sbp_matmul_workspace_bytes(const sbp_tensor* x, const sbp_tensor* w, const sbp_tensor* y);
 

@@ -16,8 +16,8 @@ namespace sbp {
 
 // Defined in matmul_tc.cu.  Returns SBP_ERR_UNSUPPORTED (without touching the error text)
 // when the plan does not meet the tensor-core kernel's rules; the caller then falls back
-// to the FMA kernel.
-sbp_status launch_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, cudaStream_t st, bool* taken);
+// to the FMA kernel.  ws: scratch for partial results of a contraction cut over many clusters (may be null).
+sbp_status launch_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, void* ws, size_t ws_bytes, cudaStream_t st, bool* taken);
 // Defined in matmul_f32.cu: fp32 operands and result.
 sbp_status launch_matmul_f32(const MatmulPlan& plan, cudaStream_t st);
 // Defined in softmax_xent.cu: reduces the per-chunk partials left by the fused classifier kernel.
@@ -574,7 +574,7 @@ sbp_status sbp_matmul(const sbp_tensor* x, const sbp_tensor* w, sbp_tensor* y, u
   SBP_BOUNDS_ADD(ws, ws_bytes);
   if (plan.in_dtype == SBP_F32) return launch_matmul_f32(plan, stream);
   bool taken = false;
-  st = launch_matmul_tc(plan, nullptr, stream, &taken);
+  st = launch_matmul_tc(plan, nullptr, ws, ws ? ws_bytes : 0, stream, &taken);
   if (taken) return st;
   // bf16 operands that only miss the copy engine's alignment rules: repack them into the workspace,
   // when the caller gave one that is large enough, and stay on the tensor cores
@@ -583,7 +583,7 @@ sbp_status sbp_matmul(const sbp_tensor* x, const sbp_tensor* w, sbp_tensor* y, u
     MatmulPlan packed = plan;
     st = pack_operands(&packed, need, ws, stream);
     if (st != SBP_OK) return st;
-    st = launch_matmul_tc(packed, nullptr, stream, &taken);
+    st = launch_matmul_tc(packed, nullptr, static_cast<char*>(ws) + need.bytes, ws_bytes - need.bytes, stream, &taken);
     if (taken) return st;
   }
   return launch_fma(plan, stream);
@@ -683,7 +683,7 @@ sbp_status sbp_matmul_softmax_xent(const sbp_tensor* features, const sbp_tensor*
   SBP_BOUNDS_TENSOR(row_sum);
   SBP_BOUNDS_ADD(ws, need);
   bool taken = false;
-  st = launch_matmul_tc(plan, &xf, stream, &taken);
+  st = launch_matmul_tc(plan, &xf, nullptr, 0, stream, &taken);
   if (!taken)
     return fail(SBP_ERR_UNSUPPORTED,
                 "the fused classifier needs the tensor-core path (16-byte aligned operands, feature and per-shard class "
@@ -753,7 +753,7 @@ sbp_status sbp_matmul_softmax_xent_backward(const sbp_tensor* features, const sb
   SBP_BOUNDS_TENSOR(row_sum);
   SBP_BOUNDS_TENSOR(grad_logits);
   bool taken = false;
-  st = launch_matmul_tc(plan, &xf, static_cast<cudaStream_t>(cuda_stream), &taken);
+  st = launch_matmul_tc(plan, &xf, nullptr, 0, static_cast<cudaStream_t>(cuda_stream), &taken);
   if (!taken)
     return fail(SBP_ERR_UNSUPPORTED,
                 "the fused classifier backward needs the tensor-core path (16-byte aligned operands and result, feature "

@@ -800,7 +800,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
 // partial accumulators are then added up through distributed shared memory: the tile's columns are dealt
 // out to the pairs, every other pair pushes its partial sums of those columns into the owner's shared
 // memory (which its ring no longer needs), and the owner adds the slices in ascending order (the same bits
-// every time), applies GeLU and stores.  No workspace and no atomics.
+// every time), applies GeLU and stores.  No workspace and no atomics.  Where even eight pairs a tile leave
+// pairs idle and the caller gave a workspace, the K-blocks are cut further, over several clusters, whose fp32
+// results matmul_parts_kernel adds up in order (512 x 512 over 2^20 classes: 72 pairs instead of 40).
 //   NB  columns of a tile.  A tile is 256 rows x NB; narrower ones give more tiles, or less padding.
 //   SW  the operands are exchanged by the host, Y^T = W^T X^T: the tile's rows are then columns of the
 //       result and its NB columns are rows of it.  A product of few rows so spends its tile on them: the
@@ -820,6 +822,8 @@ struct TcSplitParams {
   int ngroups, nseg, chain, gelu, n_rep, out_f32;
   int splits;
   int y_vec;                     // 16-byte stores are possible everywhere
+  int tiles, outer;              // outer > 1: cluster c works on tile c mod tiles and part c / tiles of its K-blocks ...
+  long long part_bytes;          // ... and writes fp32 partial results this far apart, which a second kernel adds up
 };
 
 // A ring slot holds kGroup K-blocks behind one pair of barriers: whatever its size, a round of waits, issue and
@@ -872,7 +876,8 @@ __global__ void __launch_bounds__(kThreadsTc, 1) matmul_tc_split_kernel(const __
   SBP_PDL_WAIT();                                  // everything up to here overlaps the kernel before this one
 
   // this cluster's tile and this pair's range of its K-blocks
-  const int tile = (int)(blockIdx.x / (unsigned)(2 * S));
+  const int cluster = (int)(blockIdx.x / (unsigned)(2 * S)), part = p.outer > 1 ? cluster / p.tiles : 0;
+  const int tile = cluster - part * p.tiles;
   int g = 0;
   while (g + 1 < p.ngroups && tile >= p.tile_begin[g + 1]) ++g;
   const int local = tile - p.tile_begin[g], nt = local / p.tiles_m[g], mt = local - nt * p.tiles_m[g];
@@ -880,7 +885,8 @@ __global__ void __launch_bounds__(kThreadsTc, 1) matmul_tc_split_kernel(const __
   const int s_lo = p.chain ? 0 : g, s_hi = p.chain ? p.nseg : g + 1;
   long long total = 0;
   for (int s = s_lo; s < s_hi; ++s) total += p.kblocks[s];
-  const int it0 = (int)(total * slice / S), iters = (int)(total * (slice + 1) / S) - it0;
+  const int cuts = S * p.outer, cut = part * S + slice;
+  const int it0 = (int)(total * cut / cuts), iters = (int)(total * (cut + 1) / cuts) - it0;
   bool ok = true;
 
   if (warp == 0) {
@@ -1084,7 +1090,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) matmul_tc_split_kernel(const __
     const int n_out = (g == 0 ? p.n_rep : 0) + 1;
     const long long ld = p.ldy[g];
     for (int o = 0; o < n_out; ++o) {
-      unsigned char* y = static_cast<unsigned char*>(o == 0 ? p.y_ptr[g] : p.rep_ptr[o - 1]);
+      unsigned char* y = static_cast<unsigned char*>(o == 0 ? p.y_ptr[g] : p.rep_ptr[o - 1]) + part * p.part_bytes;
       for (int idx = lane; idx < nrows * pieces; idx += 32) {
         const int r = idx / pieces, ch = idx - r * pieces;
         if (yr0 + r >= yrows) continue;
@@ -1115,6 +1121,74 @@ __global__ void __launch_bounds__(kThreadsTc, 1) matmul_tc_split_kernel(const __
     __syncwarp();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(NB) : "memory");
+  }
+}
+
+// Adds up the fp32 results of a contraction cut over several clusters, in order, applies GeLU and stores the
+// result and its replicas.  Four columns a thread; eight parts are in flight at once.
+struct PartsParams {
+  const float* part[SBP_MAX_K];        // group g's first part: rows of ld[g] floats
+  long long m[SBP_MAX_K], n[SBP_MAX_K], ld[SBP_MAX_K], ldy[SBP_MAX_K];
+  void* y_ptr[SBP_MAX_K];
+  void* rep_ptr[SBP_MAX_K];
+  long long stride;                    // floats between parts
+  int parts, gelu, n_rep, out_f32, y_vec;
+};
+
+__global__ void __launch_bounds__(256) matmul_parts_kernel(const __grid_constant__ PartsParams p) {
+  SBP_PDL_RELEASE();
+  const int g = blockIdx.y;
+  const long long quads = p.ld[g] / 4, total = p.m[g] * quads;
+  SBP_PDL_WAIT();
+  for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < total; i += (long long)gridDim.x * 256) {
+    const long long row = i / quads, c = (i - row * quads) * 4;
+    const float* at = p.part[g] + row * p.ld[g] + c;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int q0 = 0; q0 < p.parts; q0 += 8) {
+      float4 x[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (q0 + q < p.parts && SBP_GUARD(at + (q0 + q) * p.stride, 16)) x[q] = __ldcg(reinterpret_cast<const float4*>(at + (q0 + q) * p.stride));
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        if (q0 + q >= p.parts) continue;
+        if (q0 + q == 0) {
+          v = x[0];
+        } else {
+          v.x += x[q].x; v.y += x[q].y; v.z += x[q].z; v.w += x[q].w;
+        }
+      }
+    }
+    float f[4] = {v.x, v.y, v.z, v.w};
+    if (p.gelu) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) f[e] = gelu_erf_tc(f[e]);
+    }
+    const int n_out = (g == 0 ? p.n_rep : 0) + 1;
+    for (int o = 0; o < n_out; ++o) {
+      void* y = o == 0 ? p.y_ptr[g] : p.rep_ptr[o - 1];
+      if (p.out_f32) {
+        float* d = static_cast<float*>(y) + row * p.ldy[g] + c;
+        if (p.y_vec && c + 4 <= p.n[g]) {
+          if (SBP_GUARD(d, 16)) *reinterpret_cast<float4*>(d) = make_float4(f[0], f[1], f[2], f[3]);
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (c + e < p.n[g] && SBP_GUARD(d + e, 4)) d[e] = f[e];
+        }
+      } else {
+        __nv_bfloat16* d = static_cast<__nv_bfloat16*>(y) + row * p.ldy[g] + c;
+        if (p.y_vec && c + 4 <= p.n[g]) {
+          const __nv_bfloat162 lo = __floats2bfloat162_rn(f[0], f[1]), hi = __floats2bfloat162_rn(f[2], f[3]);
+          if (SBP_GUARD(d, 8))
+            *reinterpret_cast<uint2*>(d) = make_uint2(*reinterpret_cast<const unsigned*>(&lo), *reinterpret_cast<const unsigned*>(&hi));
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (c + e < p.n[g] && SBP_GUARD(d + e, 2)) d[e] = __float2bfloat16_rn(f[e]);
+        }
+      }
+    }
   }
 }
 
@@ -1374,7 +1448,7 @@ static sbp_status launch_split_form(const TcSplitParams* p, int splits, int tile
     opted.fetch_or(1ull << dev, std::memory_order_relaxed);
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(2 * splits * tiles));
+  cfg.gridDim = dim3((unsigned)(2 * splits * tiles * (p ? p->outer : 1)));
   cfg.blockDim = dim3(kThreadsTc);
   cfg.dynamicSmemBytes = kSmemSplit;
   cfg.stream = st;
@@ -1405,10 +1479,19 @@ static sbp_status launch_split_form(const TcSplitParams* p, int splits, int tile
 }
 
 // How a split product is cut: NB columns a tile, `splits` pairs a tile (0: the persistent kernel runs it),
-// operands exchanged or not.
+// operands exchanged or not, `outer` clusters a tile.
 struct SplitChoice {
-  int nb, splits, swap;
+  int nb, splits, swap, outer;
 };
+
+static long long pad4(long long v) { return (v + 3) / 4 * 4; }
+
+// Floats of one set of partial results.
+static long long part_floats(const MatmulPlan& plan) {
+  long long v = 0;
+  for (int g = 0; g < plan.ngroups; ++g) v += plan.m[g] * pad4(plan.n[g]);
+  return v;
+}
 
 static sbp_status launch_split_any(bool a_trans, bool b_trans, SplitChoice c, const TcSplitParams* p, int tiles, cudaStream_t st) {
   const int s = c.splits;
@@ -1456,7 +1539,7 @@ static int split_capacity(int splits) {
 // (us, persistent / split, one product in a row of them: 16 rows [4096 x 16384] 31 / 24 and [16384 x 4096]
 // 79 / 26; 1000 rows [4096 x 1024] written to four replicas 28 / 16; 500 rows [1024 x 4096] + GeLU 15 / 11;
 // 512 x 512 over 2^20 classes 4569 / 621; 64 x 256 over 2^17 578 / 48.)
-static SplitChoice choose_split(const MatmulPlan& plan, const int* kblocks, double cost_persistent, int forced) {
+static SplitChoice choose_split(const MatmulPlan& plan, const int* kblocks, double cost_persistent, int forced, size_t ws_bytes) {
   long long kb_max = 0, kb_min = -1, chain_kb = 0, m_max = 0;
   for (int s = 0; s < plan.nseg; ++s) chain_kb += kblocks[s];
   for (int g = 0; g < plan.ngroups; ++g) {
@@ -1466,7 +1549,9 @@ static SplitChoice choose_split(const MatmulPlan& plan, const int* kblocks, doub
     kb_max = kb > kb_max ? kb : kb_max;
     kb_min = kb_min < 0 || kb < kb_min ? kb : kb_min;
   }
-  SplitChoice best{0, 0, 0};
+  SplitChoice best{0, 0, 0, 1};
+  const long long pf = part_floats(plan);
+  const long long room = pf > 0 ? (long long)(ws_bytes / 4) / pf : 0;      // sets of partial results the workspace holds
   double best_cost = forced == 4 ? 1e300 : cost_persistent;
   for (int swap = 0; swap < 2; ++swap) {
     if (swap && plan.a_trans) continue;      // X would be the N-major operand: boxes of 64 rows and more
@@ -1489,7 +1574,18 @@ static SplitChoice choose_split(const MatmulPlan& plan, const int* kblocks, doub
                                      plan.n_rep * 2.0 * nb / (256.0 * s));
         if (cost < best_cost) {
           best_cost = cost;
-          best = SplitChoice{nb, s, swap};
+          best = SplitChoice{nb, s, swap, 1};
+        }
+        // as many clusters a tile as run at once; adding their results up is a launch, one write and one read
+        const long long outer = std::min({tiles > 0 ? cap / tiles : 0, room, kb_min / (8 * s), 128LL});
+        if (outer >= 2) {
+          const double kbo = (double)((kb_max + s * outer - 1) / (s * outer));
+          const double sum = 4.0 + (double)pf * (8.0 * outer + (plan.out_dtype == SBP_F32 ? 4.0 : 2.0) * (1 + plan.n_rep)) / 5e6;
+          const double co = kbo * per_kb + per_wave + (s > 1 ? 0.8 + 0.08 * s : 0.0) + sum;
+          if (co < best_cost) {
+            best_cost = co;
+            best = SplitChoice{nb, s, swap, (int)outer};
+          }
         }
       }
     }
@@ -1497,7 +1593,7 @@ static SplitChoice choose_split(const MatmulPlan& plan, const int* kblocks, doub
   return best;
 }
 
-static sbp_status launch_split(const MatmulPlan& given, const int* kblocks, SplitChoice c, bool y_vec, cudaStream_t st, bool* taken) {
+static sbp_status launch_split(const MatmulPlan& given, const int* kblocks, SplitChoice c, bool y_vec, float* ws, cudaStream_t st, bool* taken) {
   MatmulPlan plan = given;
   if (c.swap) {            // Y^T = W^T X^T
     for (int i = 0; i < SBP_MAX_K; ++i) {
@@ -1548,12 +1644,50 @@ static sbp_status launch_split(const MatmulPlan& given, const int* kblocks, Spli
   p.out_f32 = plan.out_dtype == SBP_F32;
   p.splits = c.splits;
   p.y_vec = y_vec ? 1 : 0;
+  p.tiles = tiles;
+  p.outer = c.outer;
+  p.part_bytes = 0;
   *taken = true;
   if (tiles == 0) return SBP_OK;
-  return launch_split_any(plan.a_trans, plan.b_trans, c, &p, tiles, st);
+  if (c.outer == 1) return launch_split_any(plan.a_trans, plan.b_trans, c, &p, tiles, st);
+
+  PartsParams q;
+  float* at = ws;
+  long long quads = 0;
+  for (int g = 0; g < given.ngroups; ++g) {
+    q.part[g] = at;
+    q.m[g] = given.m[g];
+    q.n[g] = given.n[g];
+    q.ld[g] = pad4(given.n[g]);
+    q.ldy[g] = given.ldy[g];
+    q.y_ptr[g] = given.y[g];
+    p.y_ptr[g] = at;
+    p.ldy[g] = q.ld[g];
+    at += given.m[g] * q.ld[g];
+    quads = std::max(quads, given.m[g] * q.ld[g] / 4);
+  }
+  for (int r = 0; r < given.n_rep; ++r) q.rep_ptr[r] = given.y_rep[r];
+  q.stride = at - ws;
+  q.parts = c.outer;
+  q.gelu = given.gelu;
+  q.n_rep = given.n_rep;
+  q.out_f32 = p.out_f32;
+  q.y_vec = p.y_vec;
+  p.part_bytes = q.stride * 4;
+  p.gelu = 0;
+  p.n_rep = 0;
+  p.out_f32 = 1;
+  p.y_vec = 1;
+  const sbp_status rs = launch_split_any(plan.a_trans, plan.b_trans, c, &p, tiles, st);
+  if (rs != SBP_OK) return rs;
+  const long long blocks = std::min(148LL * 8, (quads + 255) / 256);
+  const cudaError_t e = launch_dependent(matmul_parts_kernel, dim3((unsigned)blocks, (unsigned)given.ngroups), dim3(256), 0, st, q);
+  if (e != cudaSuccess) return cuda_fail(e, "matmul partial sums launch");
+  count_launch();
+  return SBP_OK;
 }
 
-sbp_status launch_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, cudaStream_t st, bool* taken) {
+sbp_status launch_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, void* ws, size_t ws_bytes, cudaStream_t st, bool* taken) {
   *taken = false;
   if (plan.in_dtype != SBP_BF16) return SBP_ERR_UNSUPPORTED;
   const int oesz = plan.out_dtype == SBP_F32 ? 4 : 2;
@@ -1612,8 +1746,8 @@ sbp_status launch_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, cudaSt
     form = choose_form(tiles_sq, tiles_tall, kb_tile, cap_sq, cap_tall, plan.gelu != 0, plan.n_rep, plan.out_dtype == SBP_F32, forced == 4 ? 0 : forced);
     if (y_direct) form.walk_tall = false;
     if (forced == 4 || (forced == 0 && pair_cap() == 0)) {
-      const SplitChoice sc = choose_split(plan, kblocks, 0.92 * (form.cost + 5.5), forced);
-      if (sc.splits > 0) return launch_split(plan, kblocks, sc, !y_direct, st, taken);
+      const SplitChoice sc = choose_split(plan, kblocks, 0.92 * (form.cost + 5.5), forced, aligned16(ws) ? ws_bytes : 0);
+      if (sc.splits > 0) return launch_split(plan, kblocks, sc, !y_direct, static_cast<float*>(ws), st, taken);
     }
   }
 

@@ -46,6 +46,37 @@ def test_results_the_vector_stores_cannot_address(split):
     _matmul_case(200, 512, 333, 2, BF16, B, S1)
 
 
+@pytest.mark.parametrize("M,K,N,k,ys", [(40, 100000, 72, 1, B), (264, 80001, 136, 8, B), (16, 200000, 100, 3, S1), (130, 100000, 255, 2, S0)])
+@pytest.mark.parametrize("out_dtype", [BF16, F32])
+def test_contraction_cut_over_many_clusters(split, M, K, N, k, ys, out_dtype):
+    """With room in the workspace for several copies of the result; replicas, GeLU, columns that 4 does not divide."""
+    torch.manual_seed(5)
+    X, W = torch.randn(M, K, device="cuda").to(BF16), (torch.randn(K, N, device="cuda") / K ** 0.5).to(BF16)
+    xl = [t.contiguous() for t in torch.tensor_split(X, k, 1)]
+    wl = [t.contiguous() for t in torch.tensor_split(W, k, 0)]
+    x, w = sbp.SbpTensor((M, K), BF16, S1, xl), sbp.SbpTensor((K, N), BF16, S0, wl)
+    y = sbp.empty_global((M, N), out_dtype, ys, k)
+    flags = sbp.SBP_EPILOGUE_GELU if N == 100 else 0
+    need = sbp.sbp_matmul_workspace_bytes(x, w, y, flags)
+    few = torch.empty(max(16, need), dtype=torch.uint8, device="cuda")
+    room = torch.empty(need + 40 * M * (N + 3) * 4, dtype=torch.uint8, device="cuda")
+    ref = X.double() @ W.double()
+    ref = torch.nn.functional.gelu(ref) if flags else ref
+    before = sbp.sbp_launch_count()
+    sbp.sbp_matmul(x, w, y, flags, few)
+    once = sbp.sbp_launch_count() - before
+    for _ in range(2):
+        for t in y.locals:
+            t.fill_(float("nan"))
+        before = sbp.sbp_launch_count()
+        sbp.sbp_matmul(x, w, y, flags, room)
+        assert sbp.sbp_launch_count() - before == once + 1, "the partial results are added up by a kernel of their own"
+        got = y.locals[0].double() if ys == B else torch.cat([t.double() for t in y.locals], 0 if ys == S0 else 1)
+        assert bool(((got - ref).abs() <= 1e-3 + 2e-2 * ref.abs()).all())
+        if ys == B:
+            assert all(torch.equal(y.locals[0], t) for t in y.locals)
+
+
 def test_the_library_takes_the_split_form_for_few_tiles():
     """The same bits every time, and far fewer operand tiles than CTA pairs so that the choice is clear."""
     X, W = torch.randn(16, 8192, device="cuda").to(BF16), torch.randn(8192, 1024, device="cuda").to(BF16)
