@@ -463,9 +463,13 @@ __global__ void __launch_bounds__(256) xent_reduce_parts_kernel(const __grid_con
 
 constexpr int kMaxSlices = 64;
 
-static int slices_for(int parts) {
-  int s = parts / 256;
-  return s < 1 ? 1 : (s > kMaxSlices ? kMaxSlices : s);
+// Enough slices for four CTAs an SM, at least two parts a thread in each; one slice per 256 parts at least.  (1024
+// parts of 64 rows: 8 CTAs with 32 parts a thread before.)
+static int slices_for(int parts, long long rows) {
+  const long long row_ctas = (rows + 31) / 32;
+  long long s = std::min((long long)parts / 16, 592 / row_ctas);
+  s = std::max(s, (long long)parts / 256);
+  return (int)std::max(1LL, std::min(s, (long long)kMaxSlices));
 }
 
 size_t xent_finish_stage_floats(long long rows) { return 3 * (size_t)kMaxSlices * (size_t)rows; }
@@ -488,7 +492,7 @@ sbp_status check_xent_outputs(const sbp_tensor* labels, const sbp_tensor* loss, 
 // parts partials per row in part_* ([parts][rows]) -> loss / row_max / row_sum.
 sbp_status launch_xent_finish(float* part_m, float* part_s, float* part_t, int parts, long long rows, float* stage,
                               sbp_tensor* loss, sbp_tensor* row_max, sbp_tensor* row_sum, int k, cudaStream_t st) {
-  const int slices = slices_for(parts);
+  const int slices = slices_for(parts, rows);
   XentReduceParams r{};
   r.in_m = part_m;
   r.in_s = part_s;
