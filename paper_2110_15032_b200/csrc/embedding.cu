@@ -11,6 +11,8 @@
 // lookups; all id loads, then all row loads, are issued before the first store.
 #include <cuda_bf16.h>
 
+#include <atomic>
+
 #include "bounds_check.h"
 #include "sbp_internal.h"
 
@@ -26,6 +28,8 @@ struct EmbParams {
   long long n_lookups;
   long long vpr;          // vectors per row
   int vpr_log2;           // >= 0 when vpr is a power of two, else -1
+  long long chunk;        // chunked kernel: lookups per chunk
+  unsigned vpr_magic;     // ceil(2^32 / vpr): exact for the at most 4096 pieces of a chunk
   int k, esz;
   int n_dst;              // fused: distinct replicas
   int canon_neg_zero;     // fused and k > 1: write -0.0 as +0.0 (what x + 0 gives)
@@ -102,9 +106,8 @@ __device__ __forceinline__ V canon(V v) {
   return v;
 }
 
-// MINB: resident CTAs per SM the register allocation is held to (see launch_emb).
-template <typename V, int ESZ, int J, bool FUSED, int MINB>
-__global__ void __launch_bounds__(256, MINB) embedding_kernel(const __grid_constant__ EmbParams p) {
+template <typename V, int ESZ, int J, bool FUSED>
+__global__ void __launch_bounds__(256) embedding_kernel(const __grid_constant__ EmbParams p) {
   const long long total = p.n_lookups * p.vpr;
   const long long stride = (long long)gridDim.x * 256;
   const long long base = (long long)blockIdx.x * 256 + threadIdx.x;
@@ -161,22 +164,27 @@ __global__ void __launch_bounds__(256, MINB) embedding_kernel(const __grid_const
   }
 }
 
-// Fused gather with a single destination per row (k = 1, or all B replicas the same buffer).
-// There the element-wise kernel above is bound by the latency of its id -> row -> store chain, not
-// by bandwidth.  This form takes the id load out of the chain.  A persistent CTA walks chunks of
-// 256 * J consecutive 16-byte pieces of the result (for 512-byte rows and J = 8: 64 consecutive
-// lookups).  The ids of a chunk sit in shared memory before its rows are asked for; the ids of the
-// CTA's next chunk are requested first (one coalesced load), then every thread puts J row loads in
-// flight at once (a warp: J whole rows), stores them, and only then parks the next ids in the other
-// half of the shared buffer -- so the id latency hides behind the rows.  The result is written with
-// streaming (evict-first) stores so that the output, which is never read back, does not push the
-// table's hot rows out of L2.  vpr (vectors per row) must be a power of two between 8 and 256 * J, so
-// that a chunk starts on a row boundary and holds at most 256 lookups (one id per thread).
+// Fused gather.  The element-wise kernel above is bound by the latency of its id -> row -> store chain; this form
+// takes the id load out of the chain.  A persistent CTA walks chunks of consecutive lookups, as many as fill 256 * J
+// 16-byte pieces of the result (64 lookups of 512 bytes), 256 at most.  Where a chunk's rows start is in shared memory
+// before they are asked for; the ids of the CTA's next chunk are requested first (one coalesced load, one id per
+// thread), then every thread puts J row loads in flight at once, stores them, and only then resolves the next ids
+// into the other half of the shared buffer -- so the id latency hides behind the rows.  The result is written with
+// streaming (evict-first) stores so that the output, which is never read back, does not push the table's hot
+// rows out of L2.  Any row length up to 256 * J pieces: a piece's lookup is one multiplication by a reciprocal.
+// Four CTAs per SM: with three the [2^24, 128] fp32 gather of 1.7 M lookups is as fast, smaller ones 5-15 % slower;
+// with five the registers no longer hold the J rows in flight (us, floor by unique rows, then 3 / 4 / 5: [2^24, 128]
+// 168, 197 / 202 / 204; [10^6, 64], 213 K lookups 11, 16.6 / 16.1 / 17.2).
+// Launched as a programmatic dependent: launch and first index arithmetic lie under the kernel before, 2 us a call.
+// Measured before (a shift-only form of this kernel for rows of 2^n pieces and one destination, else the element-wise
+// kernel) and now, us: [2^24, 128] 208 -> 200; [300 000, 100], 104 K lookups 19.1 -> 12.1; [3 x 10^6, 44], 520 K
+// lookups 39.1 -> 24.7, to four replicas 78.2 -> 75.6; bf16 [10^7, 100], 780 K lookups 107 -> 53.3; [2^20, 20],
+// 1.7 M lookups 56 -> 41; [4096, 64], 65 K lookups 7.4 -> 4.9.
 template <typename V, int ESZ, int J>
-__global__ void __launch_bounds__(256) embedding_rows_kernel(const __grid_constant__ EmbParams p) {
+__global__ void __launch_bounds__(256, 4) embedding_rows_kernel(const __grid_constant__ EmbParams p) {
   // Per lookup of the chunk: where its table row starts (null for an id outside the table).  The
   // owner of an id -- a division by the shard size -- is worked out once per lookup by the thread
-  // that stages it, a chunk ahead, not by each of the row's 16-byte vectors on its way to the load.
+  // that stages it, a chunk ahead, not by each of the row's pieces on its way to the load.
   __shared__ const char* rows_s[2][256];
   auto resolve = [&](long long id) -> const char* {
     if (id < 0 || id >= p.rows) {
@@ -187,106 +195,101 @@ __global__ void __launch_bounds__(256) embedding_rows_kernel(const __grid_consta
     const int r = owner_of_row(id, p.base, p.rem, p.big, p.narrow, &start);
     return p.table[r] + (id - start) * p.vpr * (long long)sizeof(V);
   };
-  const long long total = p.n_lookups * p.vpr;
-  const long long n_chunks = (total + 256 * J - 1) / (256 * J);
-
-  // first and last lookup of a chunk
-  auto span = [&](long long chunk, long long* look0, int* n_ids) {
-    const long long first = chunk * (256 * J);
-    long long last = first + 256 * J - 1;
-    if (last >= total) last = total - 1;
-    *look0 = first >> p.vpr_log2;
-    *n_ids = (int)((last >> p.vpr_log2) - *look0) + 1;
+  const long long n_chunks = (p.n_lookups + p.chunk - 1) / p.chunk;
+  const unsigned vpr = (unsigned)p.vpr;
+  auto lookups_in = [&](long long chunk) {
+    const long long left = p.n_lookups - chunk * p.chunk;
+    return (int)(left < p.chunk ? left : p.chunk);
   };
 
   long long chunk = blockIdx.x;
   if (chunk >= n_chunks) return;
-  int cur = 0;
-  {
-    long long look0;
-    int n_ids;
-    span(chunk, &look0, &n_ids);
-    if ((int)threadIdx.x < n_ids)
-      rows_s[0][threadIdx.x] = resolve(SBP_GUARD(p.ids[0] + look0 + threadIdx.x, 8) ? __ldcs(p.ids[0] + look0 + threadIdx.x) : -1);
+  SBP_PDL_WAIT();
+  int cur = 0, n_ids = lookups_in(chunk);
+  if ((int)threadIdx.x < n_ids) {
+    const long long* at = p.ids[0] + chunk * p.chunk + threadIdx.x;
+    rows_s[0][threadIdx.x] = resolve(SBP_GUARD(at, 8) ? __ldcs(at) : -1);
   }
   __syncthreads();
 
   for (; chunk < n_chunks; chunk += gridDim.x) {
-    const long long cta_base = chunk * (256 * J);
-    long long look0;
-    int n_ids;
-    span(chunk, &look0, &n_ids);
     // request the next chunk's ids; they are not touched until this chunk's rows are stored
     const long long next = chunk + gridDim.x;
-    long long nlook0 = 0, nid = 0;
-    int nn = 0;
-    if (next < n_chunks) {
-      span(next, &nlook0, &nn);
-      if ((int)threadIdx.x < nn && SBP_GUARD(p.ids[0] + nlook0 + threadIdx.x, 8)) nid = __ldcs(p.ids[0] + nlook0 + threadIdx.x);
-    }
+    const int nn = next < n_chunks ? lookups_in(next) : 0;
+    long long nid = -1;
+    if ((int)threadIdx.x < nn && SBP_GUARD(p.ids[0] + next * p.chunk + threadIdx.x, 8)) nid = __ldcs(p.ids[0] + next * p.chunk + threadIdx.x);
 
+    const unsigned pieces = (unsigned)n_ids * vpr;
+    const long long out0 = chunk * p.chunk * p.vpr;
     V val[J];
-    bool ok[J];
 #pragma unroll
     for (int j = 0; j < J; ++j) {
-      const long long item = cta_base + j * 256 + threadIdx.x;
-      ok[j] = item < total;
+      const unsigned f = j * 256 + threadIdx.x;
       val[j] = zero_vec<V>();
-      if (!ok[j]) continue;
-      const long long look = item >> p.vpr_log2, col = item & (p.vpr - 1);
-      const char* row = rows_s[cur][look - look0];
+      if (f >= pieces) continue;
+      const unsigned look = vpr == 1 ? f : __umulhi(f, p.vpr_magic), col = f - look * vpr;
+      const char* row = rows_s[cur][look];
       if (!row) continue;
       const V* src = reinterpret_cast<const V*>(row) + col;
       if (SBP_GUARD(src, sizeof(V))) val[j] = __ldg(src);
     }
-    V* o = reinterpret_cast<V*>(p.out[0]);
+    for (int q = 0; q < p.n_dst; ++q) {
+      V* o = reinterpret_cast<V*>(p.out[q]) + out0;
 #pragma unroll
-    for (int j = 0; j < J; ++j)
-      if (ok[j] && SBP_GUARD(o + cta_base + j * 256 + threadIdx.x, sizeof(V)))
-        __stcs(o + cta_base + j * 256 + threadIdx.x, p.canon_neg_zero ? canon<V, ESZ>(val[j]) : val[j]);
+      for (int j = 0; j < J; ++j) {
+        const unsigned f = j * 256 + threadIdx.x;
+        if (f < pieces && SBP_GUARD(o + f, sizeof(V))) __stcs(o + f, p.canon_neg_zero ? canon<V, ESZ>(val[j]) : val[j]);
+      }
+    }
 
     if ((int)threadIdx.x < nn) rows_s[cur ^ 1][threadIdx.x] = resolve(nid);
     __syncthreads();
     cur ^= 1;
+    n_ids = nn;
   }
+  SBP_PDL_RELEASE();
 }
 
-// Two shapes of the same kernel.  With several destinations per row the kernel is bound by its
-// stores and runs best with four lookups per thread; with a single destination (aliased
-// replicas, k = 1) it is bound by the latency of the id -> row -> store chain and runs best
-// with more resident warps: two lookups per thread, registers held to eight CTAs per SM
-// (measured on the Zipf workload: 0.347 -> 0.272 ms for one destination, while the same
-// shape costs the eight-replica case 4 %).
+// Pieces per thread of a chunk: eight 16-byte ones, and more of narrower pieces.
+template <typename V>
+constexpr int rows_j() { return sizeof(V) == 16 ? 8 : 16; }
+
+// A fused gather runs the chunked kernel unless one row is longer than a chunk; the unfused one (k outputs, all but one
+// of them zeros) is bound by its stores and runs element by element, four per thread.
 template <typename V, int ESZ>
-static void launch_emb(const EmbParams& p, bool fused, cudaStream_t st) {
-  const long long total = p.n_lookups * p.vpr;
+static void launch_emb(const EmbParams& given, bool fused, cudaStream_t st) {
+  constexpr int J = rows_j<V>();
   SBP_BOUNDS_UPLOAD(st);
-  auto blocks_for = [&](int j) {
-    long long b = (total + 256LL * j - 1) / (256LL * j);
-    return (unsigned)(b < 1 ? 1 : b);
-  };
-  if (fused && p.n_dst == 1 && p.vpr_log2 >= 3 && p.vpr_log2 <= 11) {
+  if (fused && given.vpr <= 256 * J) {
     // persistent: as many CTAs as fit at once
-    static int resident = 0;
-    if (resident == 0) {
+    static std::atomic<int> resident{0};
+    int r = resident.load(std::memory_order_relaxed);
+    if (r == 0) {
       int dev = 0, sms = 148, per_sm = 4;
       cudaGetDevice(&dev);
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, embedding_rows_kernel<V, ESZ, 8>, 256, 0) != cudaSuccess || per_sm < 1) {
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, embedding_rows_kernel<V, ESZ, J>, 256, 0) != cudaSuccess || per_sm < 1) {
         cudaGetLastError();
         per_sm = 4;
       }
-      resident = sms * per_sm;
+      r = sms * per_sm;
+      resident.store(r, std::memory_order_relaxed);
     }
-    const unsigned chunks = blocks_for(8);
-    embedding_rows_kernel<V, ESZ, 8><<<dim3(chunks < (unsigned)resident ? chunks : (unsigned)resident), 256, 0, st>>>(p);
-  } else if (fused && p.n_dst == 1) {
-    embedding_kernel<V, ESZ, 2, true, 8><<<dim3(blocks_for(2)), 256, 0, st>>>(p);
-  } else if (fused) {
-    embedding_kernel<V, ESZ, 4, true, 1><<<dim3(blocks_for(4)), 256, 0, st>>>(p);
-  } else {
-    embedding_kernel<V, ESZ, 4, false, 1><<<dim3(blocks_for(4)), 256, 0, st>>>(p);
+    // Chunks in whole waves of CTAs: a last wave of a few full chunks costs as much as a full one ([4096, 64] with
+    // 65 K lookups 7.4 us with full chunks, 6.4 us so; [50 000, 32] with 2400 5.8 and 4.2 us).
+    EmbParams p = given;
+    const long long most = 256 * J / p.vpr < 256 ? 256 * J / p.vpr : 256;
+    const long long waves = (p.n_lookups + most * r - 1) / (most * r);
+    p.chunk = (p.n_lookups + waves * r - 1) / (waves * r);
+    if (p.chunk < 8) p.chunk = most < 8 ? most : 8;
+    p.vpr_magic = (unsigned)(0xffffffffull / (unsigned long long)p.vpr + 1);
+    const long long chunks = (p.n_lookups + p.chunk - 1) / p.chunk;
+    launch_dependent(embedding_rows_kernel<V, ESZ, J>, dim3((unsigned)(chunks < r ? chunks : r)), dim3(256), 0, st, p);
+    return;
   }
+  const long long blocks = (given.n_lookups * given.vpr + 1023) / 1024;
+  if (fused) embedding_kernel<V, ESZ, 4, true><<<dim3((unsigned)blocks), 256, 0, st>>>(given);
+  else embedding_kernel<V, ESZ, 4, false><<<dim3((unsigned)blocks), 256, 0, st>>>(given);
 }
 
 // ---- table split along the hidden axis: S(1) ("splitting the hidden dimension", Section 6.3).
@@ -443,57 +446,104 @@ struct EmbBwdParams {
   long long rows, base, rem, big;
   int narrow;
   long long n_lookups, vpr;          // float4 vectors per row
-  int k;
+  int k, lanes;
   int* oob;
 };
 
+// 16 KB per CTA, one CTA for each: consecutive CTAs clear consecutive memory.  (Persistent grids were slower: 2 GB with
+// its scatter 344 us so, 362 us with 10 000 CTAs striding, 405 us with 592.)
 __global__ void __launch_bounds__(256) embedding_zero_kernel(const __grid_constant__ EmbBwdParams p) {
+  SBP_PDL_RELEASE();
+  SBP_PDL_WAIT();
+  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
   float4* g = reinterpret_cast<float4*>(p.grad_table[blockIdx.y]);
   const long long n = p.shard_vecs[blockIdx.y];
-  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n; i += (long long)gridDim.x * 256)
-    if (SBP_GUARD(g + i, 16)) g[i] = z;
+  const long long i = (long long)blockIdx.x * 1024 + threadIdx.x;
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+    if (i + u * 256 < n && SBP_GUARD(g + i + u * 256, 16)) g[i + u * 256] = z;
 }
 
-// CHUNK lookups per CTA pass (256 or 1024); key = id * CHUNK + position in the chunk, all ones
-// for a position past the end or an id outside the table (sorted last, skipped).
+// One compare-exchange step of a bitonic sort of CHUNK keys held KPT to a thread (key r of thread t is number t * KPT
+// + r): inside the thread, between lanes of a warp, or through shared memory, by how far apart the partners are.
+template <int KPT>
+__device__ __forceinline__ void sort_step(unsigned long long (&k)[KPT], unsigned long long* smem, int size, int j) {
+  const int t = threadIdx.x;
+  if (j < KPT) {
+#pragma unroll
+    for (int r = 0; r < KPT; ++r) {
+      const int q = r ^ j;
+      if (q > r && q < KPT) {
+        const bool up = ((t * KPT + r) & size) == 0;
+        const unsigned long long a = k[r], b = k[q];
+        const bool swap = (a > b) == up;
+        k[r] = swap ? b : a;
+        k[q] = swap ? a : b;
+      }
+    }
+    return;
+  }
+  const bool low = ((t * KPT) & j) == 0;
+  if (j >= 32 * KPT) {
+#pragma unroll
+    for (int r = 0; r < KPT; ++r) smem[t * KPT + r] = k[r];
+    __syncthreads();
+  }
+#pragma unroll
+  for (int r = 0; r < KPT; ++r) {
+    const unsigned long long other = j < 32 * KPT ? __shfl_xor_sync(0xffffffffu, k[r], j / KPT) : smem[(t * KPT + r) ^ j];
+    const bool up = ((t * KPT + r) & size) == 0;
+    k[r] = (low == up) == (k[r] < other) ? k[r] : other;      // the lower place keeps the smaller key going up
+  }
+  if (j >= 32 * KPT) __syncthreads();
+}
+
+// CHUNK lookups per CTA pass; key = id * CHUNK + position in the chunk, all ones for a position past the end or an id
+// outside the table (sorted last, skipped).  Most of the sort's 36 (45, 55) steps stay inside a thread or a warp: 6
+// at most go through shared memory.  The sorted chunk is then dealt out to teams of `lanes` threads, as many as a
+// row has 16-byte vectors (a power of two, 32 at most), so that short rows leave no lane idle.  Launched as a
+// programmatic dependent of the zero fill: the sort may run under the fill's last CTAs.
+// Zero fill and scatter, us (floor: gradient written and gradient of the output read once), with a warp to each row
+// and every sort step through shared memory, then as here: [10^6, 64], 213 K lookups (48) 78.8, 57; [2 x 10^6, 16],
+// 426 K lookups (24) 90.5, 44.7; [300 000, 100], 104 K (25) 44, 35; [4 x 10^6, 128], 426 K (347) 375, 344; [50 000,
+// 32], 2400 (1) 18.3, 5.9.
 template <int CHUNK>
 __global__ void __launch_bounds__(256, 3) embedding_backward_kernel(const __grid_constant__ EmbBwdParams p) {
-  constexpr int kShift = CHUNK == 1024 ? 10 : 8;
-  constexpr int kPerWarp = CHUNK / 8;     // sorted positions walked by one warp
+  constexpr int kShift = CHUNK == 1024 ? 10 : (CHUNK == 512 ? 9 : 8);
+  constexpr int KPT = CHUNK / 256;
   constexpr int kBatch = 8;               // gradient rows in flight per lane
   constexpr unsigned long long kNone = ~0ull;
   __shared__ unsigned long long key[CHUNK];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
+  const int lanes = p.lanes, tl = tid & (lanes - 1), team = tid / lanes, per_team = CHUNK / (256 / lanes);
   const long long n_chunks = (p.n_lookups + CHUNK - 1) / CHUNK;
   const float4* gout = reinterpret_cast<const float4*>(p.grad_out);
+  bool waited = false;
   for (long long chunk = blockIdx.x; chunk < n_chunks; chunk += gridDim.x) {
     const long long first = chunk * CHUNK;
-    for (int i = tid; i < CHUNK; i += 256) {
-      unsigned long long kv = kNone;
+    unsigned long long k[KPT];
+#pragma unroll
+    for (int r = 0; r < KPT; ++r) {
+      const int i = tid + r * 256;        // any order will do: the keys carry their positions
+      k[r] = kNone;
       if (first + i < p.n_lookups) {
         const long long id = SBP_GUARD(p.ids + first + i, 8) ? __ldg(p.ids + first + i) : -1;
-        if (id >= 0 && id < p.rows) kv = ((unsigned long long)id << kShift) | (unsigned)i;
+        if (id >= 0 && id < p.rows) k[r] = ((unsigned long long)id << kShift) | (unsigned)i;
         else if (p.oob && SBP_GUARD(p.oob, 4)) atomicAdd(p.oob, 1);
       }
-      key[i] = kv;
     }
+#pragma unroll
+    for (int size = 2; size <= CHUNK; size <<= 1)
+#pragma unroll
+      for (int j = size >> 1; j > 0; j >>= 1) sort_step<KPT>(k, key, size, j);
+#pragma unroll
+    for (int r = 0; r < KPT; ++r) key[tid * KPT + r] = k[r];
     __syncthreads();
-    // bitonic sort, ascending
-    for (int size = 2; size <= CHUNK; size <<= 1) {
-      for (int j = size >> 1; j > 0; j >>= 1) {
-        for (int t = tid; t < CHUNK / 2; t += 256) {
-          const int lo = 2 * t - (t & (j - 1)), hi = lo + j;
-          const unsigned long long a = key[lo], b = key[hi];
-          const bool up = (lo & size) == 0;
-          if ((a > b) == up) { key[lo] = b; key[hi] = a; }
-        }
-        __syncthreads();
-      }
-    }
+    if (!waited) SBP_PDL_WAIT();          // the gradient has been cleared from here on
+    waited = true;
     // runs of equal ids -> one atomic row add each
-    for (long long cb = 0; cb < p.vpr; cb += 32) {
-      const long long col = cb + lane;
+    for (long long cb = 0; cb < p.vpr; cb += lanes) {
+      const long long col = cb + tl;
       const bool active = col < p.vpr;
       long long cur = -1;
       float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -505,15 +555,15 @@ __global__ void __launch_bounds__(256, 3) embedding_backward_kernel(const __grid
           if (SBP_GUARD(at, 16)) atomicAdd(at, acc);
         }
       };
-      for (int pos = warp * kPerWarp; pos < (warp + 1) * kPerWarp; pos += kBatch) {
+      for (int pos = team * per_team; pos < (team + 1) * per_team; pos += kBatch) {
         unsigned long long kv[kBatch];
         float4 gv[kBatch];
 #pragma unroll
         for (int j = 0; j < kBatch; ++j) {
-          kv[j] = key[pos + j];
+          kv[j] = pos + j < (team + 1) * per_team ? key[pos + j] : kNone;
           gv[j] = make_float4(0.f, 0.f, 0.f, 0.f);
           if (kv[j] != kNone && active && SBP_GUARD(gout + (first + (long long)(kv[j] & (CHUNK - 1))) * p.vpr + col, 16))
-            gv[j] = __ldg(gout + (first + (long long)(kv[j] & (CHUNK - 1))) * p.vpr + col);
+            gv[j] = __ldcs(gout + (first + (long long)(kv[j] & (CHUNK - 1))) * p.vpr + col);
         }
 #pragma unroll
         for (int j = 0; j < kBatch; ++j) {
@@ -532,6 +582,7 @@ __global__ void __launch_bounds__(256, 3) embedding_backward_kernel(const __grid
     }
     __syncthreads();
   }
+  SBP_PDL_RELEASE();
 }
 
 }  // namespace sbp
@@ -688,22 +739,25 @@ extern "C" sbp_status sbp_embedding_backward(const sbp_tensor* grad_out, const s
     max_vecs = p.shard_vecs[r] > max_vecs ? p.shard_vecs[r] : max_vecs;
   }
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-  long long zb = (max_vecs + 256 * 8 - 1) / (256 * 8);
-  if (zb < 1) zb = 1;
-  if (zb > 148 * 16) zb = 148 * 16;
+  p.lanes = 1;
+  while (p.lanes < 32 && p.lanes < p.vpr) p.lanes *= 2;
+  const long long zb = (max_vecs + 1023) / 1024;
+  if (zb > 0x7fffffffLL) return fail(SBP_ERR_UNSUPPORTED, "gradient too large for one launch");
   SBP_BOUNDS_UPLOAD(stream);
-  embedding_zero_kernel<<<dim3((unsigned)zb, (unsigned)k), 256, 0, stream>>>(p);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_dependent(embedding_zero_kernel, dim3((unsigned)(zb < 1 ? 1 : zb), (unsigned)k), dim3(256), 0, stream, p);
   if (e != cudaSuccess) return cuda_fail(e, "embedding backward launch");
   count_launch();
   if (p.n_lookups > 0) {
-    // 1024-lookup chunks once they fill the GPU a few times over, else 256-lookup chunks
-    const bool big_chunks = p.n_lookups / 1024 >= 148 * 4;
-    const long long chunks = (p.n_lookups + (big_chunks ? 1023 : 255)) / (big_chunks ? 1024 : 256);
-    const unsigned sb = (unsigned)(chunks < 148 * 8 ? chunks : 148 * 8);
-    if (big_chunks) embedding_backward_kernel<1024><<<sb, 256, 0, stream>>>(p);
-    else embedding_backward_kernel<256><<<sb, 256, 0, stream>>>(p);
-    e = cudaGetLastError();
+    // Long chunks catch more repeated ids; a chunk is walked by one CTA, so no longer than 8192 vectors and no fewer
+    // than 1.5 chunks per SM (us for chunks of 256 / 512 / 1024: [2 x 10^6, 16], 426 K lookups 63 / 52 / 47.5;
+    // [10^6, 64], 213 K lookups 68 / 65 / 74; [300 000, 100], 104 K lookups 41 / 48 / 65).
+    int chunk = 1024;
+    while (chunk > 256 && (chunk * p.vpr > 8192 || p.n_lookups < chunk * 222LL)) chunk /= 2;
+    const long long chunks = (p.n_lookups + chunk - 1) / chunk;
+    const dim3 sb((unsigned)(chunks < 148 * 8 ? chunks : 148 * 8)), b(256);
+    if (chunk == 1024) e = launch_dependent(embedding_backward_kernel<1024>, sb, b, 0, stream, p);
+    else if (chunk == 512) e = launch_dependent(embedding_backward_kernel<512>, sb, b, 0, stream, p);
+    else e = launch_dependent(embedding_backward_kernel<256>, sb, b, 0, stream, p);
     if (e != cudaSuccess) return cuda_fail(e, "embedding backward launch");
     count_launch();
   }
