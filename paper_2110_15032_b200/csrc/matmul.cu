@@ -167,6 +167,8 @@ struct PackList {
 
 // One 16-byte store per thread and step: eight consecutive elements of a row, zeros past its end.
 __global__ void __launch_bounds__(256) matmul_pack_kernel(const __grid_constant__ PackList L) {
+  SBP_PDL_RELEASE();
+  SBP_PDL_WAIT();
   const PackBlock& B = L.b[blockIdx.y];
   const long long groups = (B.cols + 7) / 8;
   const long long total = B.rows * groups;
@@ -245,8 +247,7 @@ static sbp_status pack_operands(MatmulPlan* plan, const PackNeed& need, void* ws
     if (gx < 1) gx = 1;
     if (gx > 148 * 8) gx = 148 * 8;
     SBP_BOUNDS_UPLOAD(st);
-    matmul_pack_kernel<<<dim3((unsigned)gx, (unsigned)nb), 256, 0, st>>>(list);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_dependent(matmul_pack_kernel, dim3((unsigned)gx, (unsigned)nb), dim3(256), 0, st, list);
     if (e != cudaSuccess) return cuda_fail(e, "operand repack launch");
     count_launch();
     nb = 0;

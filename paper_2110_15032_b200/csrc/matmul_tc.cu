@@ -409,8 +409,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const unsigned tmem_base = tmem_base_slot;
   // A kernel launched behind this one as its programmatic dependent may be set up from here on;
-  // it waits on the device for this grid to finish before it reads what this grid writes.
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // it waits on the device for this grid to finish before it reads what this grid writes.  This
+  // kernel is launched the same way: barriers and TMEM are set up under the end of the kernel before.
+  SBP_PDL_RELEASE();
+  SBP_PDL_WAIT();
 
   const int first = blockIdx.x >> 1, stride = gridDim.x >> 1;   // tiles are dealt to CTA pairs
 
@@ -1365,8 +1367,7 @@ static sbp_status launch_tc_form(const TcParams* p, cudaStream_t st, int* capaci
   if (!p) return SBP_OK;
   const int pairs = p->total_tiles < max_pairs ? p->total_tiles : max_pairs;
   SBP_BOUNDS_UPLOAD(st);
-  matmul_tc_kernel<AT, BT, MH><<<2 * pairs, kThreadsTc, kSmem, st>>>(*p);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_dependent(matmul_tc_kernel<AT, BT, MH>, dim3((unsigned)(2 * pairs)), dim3(kThreadsTc), kSmem, st, *p);
   if (e != cudaSuccess) return cuda_fail(e, "tensor-core matmul launch");
   count_launch();
   g_form_launches[MH == 2 ? 1 : (p->half_split ? 2 : 0)]++;

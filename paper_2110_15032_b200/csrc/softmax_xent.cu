@@ -227,6 +227,8 @@ __global__ void __launch_bounds__(kThreads) xent_rows_kernel(const __grid_consta
   using T = typename Chunk::T;
   const int team = 1 << team_log2, tl = threadIdx.x & (team - 1);
   const long long row = (long long)blockIdx.x * (kThreads >> team_log2) + (threadIdx.x >> team_log2);
+  SBP_PDL_RELEASE();
+  SBP_PDL_WAIT();
   float m = -INFINITY, s = 0.f, t = 0.f;
   if (row < p.rows) {
     const long long y = SBP_GUARD(p.labels + row, 8) ? p.labels[row] : -1;
@@ -277,7 +279,8 @@ __global__ void __launch_bounds__(kThreads) xent_partial_kernel(const __grid_con
   const int tid = threadIdx.x;
   // The kernel that combines the partials may be set up while this one runs; it waits for
   // this grid to finish before it reads anything.
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  SBP_PDL_RELEASE();
+  SBP_PDL_WAIT();
 
   float m = -INFINITY, s = 0.f;
   if (n > 0) walk_span<Chunk>(z, n, tid, kThreads, m, s);
@@ -315,7 +318,8 @@ constexpr int kCombineThreads = 256;
 __global__ void __launch_bounds__(kCombineThreads) xent_combine_kernel(const __grid_constant__ XentCombineParams p) {
   // When launched as the programmatic dependent of the kernel that writes the partials, wait
   // here until that grid has finished and its writes are visible (a no-op otherwise).
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  SBP_PDL_RELEASE();
+  SBP_PDL_WAIT();
   const long long row = (long long)blockIdx.x * (kCombineThreads / 32) + (threadIdx.x >> 5);
   if (row >= p.rows) return;
   const int lane = threadIdx.x & 31;
@@ -419,8 +423,8 @@ __global__ void __launch_bounds__(256) xent_reduce_parts_kernel(const __grid_con
   // The partials come from the kernel just before this one in the stream; when launched as its
   // programmatic dependent, wait for it here (a no-op otherwise), and let the combine kernel
   // that follows be set up meanwhile.
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  SBP_PDL_RELEASE();
+  SBP_PDL_WAIT();
   float m = -INFINITY, s = 0.f, t = 0.f;
   if (row < p.rows) {
     // four parts (stride 8) are loaded before they are merged, in ascending order
@@ -562,6 +566,8 @@ __global__ void __launch_bounds__(kThreads) xent_backward_kernel(const __grid_co
   split_range(p.classes, p.k, shard, (int64_t*)&c_start, (int64_t*)&c_len);
   const T* z = reinterpret_cast<const T*>(p.logits[shard]) + row * p.lpitch[shard];
   T* g = reinterpret_cast<T*>(p.grad[shard]) + row * p.gpitch[shard];
+  SBP_PDL_RELEASE();
+  SBP_PDL_WAIT();
   // softmax = 2^(z log2e - m log2e - log2 S): the division by the row sum is folded into the exponent
   if (!SBP_GUARD(p.row_max + row, 4) || !SBP_GUARD(p.row_sum + row, 4) || !SBP_GUARD(p.labels + row, 8)) return;
   const float neg = -p.row_max[row] * kLog2e - log2f(p.row_sum[row]);
@@ -697,16 +703,16 @@ sbp_status sbp_softmax_xent(const sbp_tensor* logits, const sbp_tensor* labels, 
     const int team_log2 = rows < 2 * kRowsForTeams ? 7 : (rows < 4 * kRowsForTeams ? 6 : 5);
     const int per_cta = kThreads >> team_log2;
     const dim3 g((unsigned)((rows + per_cta - 1) / per_cta));
-    if (logits->dtype == SBP_BF16) xent_rows_kernel<ChunkBF16><<<g, kThreads, 0, stream>>>(p, c, team_log2);
-    else xent_rows_kernel<ChunkF32><<<g, kThreads, 0, stream>>>(p, c, team_log2);
+    if (logits->dtype == SBP_BF16) launch_dependent(xent_rows_kernel<ChunkBF16>, g, dim3(kThreads), 0, stream, p, c, team_log2);
+    else launch_dependent(xent_rows_kernel<ChunkF32>, g, dim3(kThreads), 0, stream, p, c, team_log2);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "softmax launch");
     count_launch();
     return SBP_OK;
   }
   dim3 grid((unsigned)rows, (unsigned)nsplit, (unsigned)k);
-  if (logits->dtype == SBP_BF16) xent_partial_kernel<ChunkBF16><<<grid, kThreads, 0, stream>>>(p);
-  else xent_partial_kernel<ChunkF32><<<grid, kThreads, 0, stream>>>(p);
+  if (logits->dtype == SBP_BF16) launch_dependent(xent_partial_kernel<ChunkBF16>, grid, dim3(kThreads), 0, stream, p);
+  else launch_dependent(xent_partial_kernel<ChunkF32>, grid, dim3(kThreads), 0, stream, p);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "softmax partial launch");
 
@@ -835,11 +841,11 @@ extern "C" sbp_status sbp_softmax_xent_backward(const sbp_tensor* logits, const 
   SBP_BOUNDS_TENSOR(grad_logits);
   SBP_BOUNDS_UPLOAD(stream);
   if (logits->dtype == SBP_BF16) {
-    if (vec > 1) xent_backward_kernel<__nv_bfloat16, 8><<<grid, kThreads, 0, stream>>>(p);
-    else xent_backward_kernel<__nv_bfloat16, 1><<<grid, kThreads, 0, stream>>>(p);
+    if (vec > 1) launch_dependent(xent_backward_kernel<__nv_bfloat16, 8>, grid, dim3(kThreads), 0, stream, p);
+    else launch_dependent(xent_backward_kernel<__nv_bfloat16, 1>, grid, dim3(kThreads), 0, stream, p);
   } else {
-    if (vec > 1) xent_backward_kernel<float, 4><<<grid, kThreads, 0, stream>>>(p);
-    else xent_backward_kernel<float, 1><<<grid, kThreads, 0, stream>>>(p);
+    if (vec > 1) launch_dependent(xent_backward_kernel<float, 4>, grid, dim3(kThreads), 0, stream, p);
+    else launch_dependent(xent_backward_kernel<float, 1>, grid, dim3(kThreads), 0, stream, p);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "softmax backward launch");
