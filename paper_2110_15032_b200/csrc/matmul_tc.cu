@@ -824,6 +824,11 @@ struct TcSplitParams {
   int ngroups, nseg, chain, gelu, n_rep, out_f32;
   int splits;
   int y_vec;                     // 16-byte stores are possible everywhere
+  // row blocks of one fused result, as S(0) cuts it: multiplied as one product (group 0), block b's rows from
+  // block_row[b] on stored to block_y[b].  0: every group has a result of its own
+  int blocks;
+  long long block_row[SBP_MAX_K + 1];
+  void* block_y[SBP_MAX_K];
   int tiles, outer;              // outer > 1: cluster c works on tile c mod tiles and part c / tiles of its K-blocks ...
   long long part_bytes;          // ... and writes fp32 partial results this far apart, which a second kernel adds up
 };
@@ -1091,14 +1096,21 @@ __global__ void __launch_bounds__(kThreadsTc, 1) matmul_tc_split_kernel(const __
     const long long yr0 = SW ? col0 : row0, yc0 = SW ? row0 : col0, yrows = SW ? Ng : Mg, ycols = SW ? Mg : Ng;
     const int n_out = (g == 0 ? p.n_rep : 0) + 1;
     const long long ld = p.ldy[g];
-    for (int o = 0; o < n_out; ++o) {
-      unsigned char* y = static_cast<unsigned char*>(o == 0 ? p.y_ptr[g] : p.rep_ptr[o - 1]) + part * p.part_bytes;
+    auto store = [&](unsigned char* y, auto blocks) {
       for (int idx = lane; idx < nrows * pieces; idx += 32) {
         const int r = idx / pieces, ch = idx - r * pieces;
         if (yr0 + r >= yrows) continue;
         const uint4 v = *reinterpret_cast<const uint4*>(stage + r * pitch + ch * 16);
         const long long c = yc0 + ch * el;
-        unsigned char* at = y + ((yr0 + r) * ld + c) * esz;
+        long long row = yr0 + r;
+        unsigned char* base = y;
+        if constexpr (decltype(blocks)::value) {
+          int b = 0;
+          while (b + 1 < p.blocks && row >= p.block_row[b + 1]) ++b;
+          base = static_cast<unsigned char*>(p.block_y[b]);
+          row -= p.block_row[b];
+        }
+        unsigned char* at = base + (row * ld + c) * esz;
         if (p.y_vec && c + el <= ycols) {
           if (SBP_GUARD(at, 16)) *reinterpret_cast<uint4*>(at) = v;
         } else if (p.out_f32) {
@@ -1113,7 +1125,11 @@ __global__ void __launch_bounds__(kThreadsTc, 1) matmul_tc_split_kernel(const __
             if (c + e < ycols && SBP_GUARD(at + 2 * e, 2)) reinterpret_cast<unsigned short*>(at)[e] = f[e];
         }
       }
-    }
+    };
+    if (p.blocks) store(nullptr, std::true_type{});
+    else
+      for (int o = 0; o < n_out; ++o)
+        store(static_cast<unsigned char*>(o == 0 ? p.y_ptr[g] : p.rep_ptr[o - 1]) + part * p.part_bytes, std::false_type{});
   }
 
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1402,10 +1418,32 @@ struct FormChoice {
   double cost;         // the model's time for it, without what every launch pays
 };
 
+// What the copy engine needs for the rows of 128 bytes that a CTA loads per K-block, us: 64 bytes a clock, and a
+// row that starts off a 128-byte boundary of memory is two requests (a [5696 x 2280]^T [5696 x 632] product took
+// 44.7 us where [5696 x 2304]^T [5696 x 640] took 28.1).  A long product of such pitches wants wide tiles; the first
+// K-blocks only fill the ring.
+struct OperandRows {
+  double a = 1.0e-3, b = 1.0e-3;      // us per row
+  // time of kb K-blocks beyond `per_kb` each, which they take otherwise
+  double extra(int rows_a, int rows_b, double kb, double per_kb) const {
+    return std::max(0.0, kb - 8.0) * std::max(0.0, a * rows_a + b * rows_b - per_kb);
+  }
+};
+
+static OperandRows operand_rows(const MatmulPlan& p) {
+  OperandRows r;
+  for (int s = 0; s < p.nseg; ++s) {
+    if ((!p.chain && s >= p.ngroups) || p.kseg[s] == 0) continue;
+    if (p.lda[s] % 64 != 0 || reinterpret_cast<uintptr_t>(p.a[s]) % 128 != 0) r.a = 1.9e-3;
+    if (p.ldb[s] % 64 != 0 || reinterpret_cast<uintptr_t>(p.b[s]) % 128 != 0) r.b = 1.9e-3;
+  }
+  return r;
+}
+
 static FormChoice choose_form(long long tiles_sq, long long tiles_tall, long long kb, int cap_sq, int cap_tall, bool gelu, int n_rep,
-                              bool out_f32, int forced) {
-  const double wave_sq = 0.388 * kb + (gelu ? 1.3 : 0.0) + 1.2 * n_rep + (out_f32 ? 1.0 : 0.0);
-  const double wave_tall = 0.70 * kb + 2.6 + (gelu ? 8.6 : 0.0) + 2.5 * n_rep + (out_f32 ? 3.0 : 0.0);
+                              bool out_f32, const OperandRows& rows, int forced) {
+  const double wave_sq = 0.388 * kb + rows.extra(BMH, BNH, (double)kb, 0.388) + (gelu ? 1.3 : 0.0) + 1.2 * n_rep + (out_f32 ? 1.0 : 0.0);
+  const double wave_tall = 0.70 * kb + rows.extra(2 * BMH, BNH, (double)kb, 0.70) + 2.6 + (gelu ? 8.6 : 0.0) + 2.5 * n_rep + (out_f32 ? 3.0 : 0.0);
   const double kRelaunch = 5.0;
   auto waves = [](long long tiles, int cap) { return (double)((tiles + cap - 1) / cap); };
   const double cost_sq = waves(tiles_sq, cap_sq) * wave_sq;
@@ -1430,7 +1468,7 @@ static FormChoice choose_form(long long tiles_sq, long long tiles_tall, long lon
 // choose_form for callers outside this file (the C ABI's planning query): 0 square, 1 tall, 2 mixed.
 int tc_route(long long tiles_sq, long long tiles_tall, long long kb, int pairs, bool gelu, int n_rep, bool out_f32, int forced,
              long long* tall_tiles) {
-  const FormChoice f = choose_form(tiles_sq, tiles_tall, kb, pairs, pairs, gelu, n_rep, out_f32, forced);
+  const FormChoice f = choose_form(tiles_sq, tiles_tall, kb, pairs, pairs, gelu, n_rep, out_f32, OperandRows{}, forced);
   if (tall_tiles) *tall_tiles = f.walk_tall ? f.tall_tiles : 0;
   return !f.walk_tall ? 0 : (f.tall_tiles == tiles_tall ? 1 : 2);
 }
@@ -1551,6 +1589,7 @@ static SplitChoice choose_split(const MatmulPlan& plan, const int* kblocks, doub
     kb_min = kb_min < 0 || kb < kb_min ? kb : kb_min;
   }
   SplitChoice best{0, 0, 0, 1};
+  const OperandRows rows = operand_rows(plan);
   const long long pf = part_floats(plan);
   const long long room = pf > 0 ? (long long)(ws_bytes / 4) / pf : 0;      // sets of partial results the workspace holds
   double best_cost = forced == 4 ? 1e300 : cost_persistent;
@@ -1570,8 +1609,9 @@ static SplitChoice choose_split(const MatmulPlan& plan, const int* kblocks, doub
         if (cap < 1) continue;
         const double waves = (double)((tiles + cap - 1) / cap), kb = (double)((kb_max + s - 1) / s);
         const double per_kb = nb == 256 ? 0.323 : (nb == 128 ? 0.2 : 0.187);
+        auto k_time = [&](double kbs) { return kbs * per_kb + (swap ? rows.extra(nb / 2, BMH, kbs, per_kb) : rows.extra(BMH, nb / 2, kbs, per_kb)); };
         const double per_wave = nb == 256 ? 9.6 : (nb == 128 ? 6.6 : (nb == 64 ? 5.3 : 4.4));
-        const double cost = waves * (kb * per_kb + per_wave + (s > 1 ? 0.8 + 0.08 * s : 0.0) + (plan.gelu ? 0.4 : 0.0) +
+        const double cost = waves * (k_time(kb) + per_wave + (s > 1 ? 0.8 + 0.08 * s : 0.0) + (plan.gelu ? 0.4 : 0.0) +
                                      plan.n_rep * 2.0 * nb / (256.0 * s));
         if (cost < best_cost) {
           best_cost = cost;
@@ -1582,7 +1622,7 @@ static SplitChoice choose_split(const MatmulPlan& plan, const int* kblocks, doub
         if (outer >= 2) {
           const double kbo = (double)((kb_max + s * outer - 1) / (s * outer));
           const double sum = 4.0 + (double)pf * (8.0 * outer + (plan.out_dtype == SBP_F32 ? 4.0 : 2.0) * (1 + plan.n_rep)) / 5e6;
-          const double co = kbo * per_kb + per_wave + (s > 1 ? 0.8 + 0.08 * s : 0.0) + sum;
+          const double co = k_time(kbo) + per_wave + (s > 1 ? 0.8 + 0.08 * s : 0.0) + sum;
           if (co < best_cost) {
             best_cost = co;
             best = SplitChoice{nb, s, swap, (int)outer};
@@ -1594,8 +1634,26 @@ static SplitChoice choose_split(const MatmulPlan& plan, const int* kblocks, doub
   return best;
 }
 
-static sbp_status launch_split(const MatmulPlan& given, const int* kblocks, SplitChoice c, bool y_vec, float* ws, cudaStream_t st, bool* taken) {
-  MatmulPlan plan = given;
+// The row blocks of one fused result as one product, where their results share a pitch; false where they are none.
+// (A block of 34 rows has a tile of 256 to itself otherwise, and one that starts off a multiple of 8 rows of a
+// transposed X needs a repacked copy.  us, separate and repacked / as one: [6838 x 136]^T [6838 x 1808] over four
+// devices 37.6 / 15.4; [5293 x 2488]^T [5293 x 544] over two 38 / 26.)
+static bool merge_row_blocks(const MatmulPlan& plan, MatmulPlan* merged) {
+  if (!plan.chain || plan.ngroups < 2 || plan.n_rep != 0) return false;
+  long long rows = 0;
+  for (int g = 0; g < plan.ngroups; ++g) {
+    if (plan.row_off[g] != rows || plan.col_off[g] != 0 || plan.n[g] != plan.n[0] || plan.ldy[g] != plan.ldy[0]) return false;
+    rows += plan.m[g];
+  }
+  *merged = plan;
+  merged->ngroups = 1;
+  merged->m[0] = rows;
+  return true;
+}
+
+static sbp_status launch_split(const MatmulPlan& given, const MatmulPlan* merged, const int* kblocks, SplitChoice c, bool y_vec, float* ws,
+                               cudaStream_t st, bool* taken) {
+  MatmulPlan plan = merged ? *merged : given;
   if (c.swap) {            // Y^T = W^T X^T
     for (int i = 0; i < SBP_MAX_K; ++i) {
       std::swap(plan.a[i], plan.b[i]);
@@ -1607,6 +1665,14 @@ static sbp_status launch_split(const MatmulPlan& given, const int* kblocks, Spli
     plan.b_trans = !given.a_trans;
   }
   TcSplitParams p;
+  p.blocks = 0;
+  if (merged && c.outer == 1) {
+    p.blocks = given.ngroups;
+    for (int g = 0; g < given.ngroups; ++g) {
+      p.block_row[g] = given.row_off[g];
+      p.block_y[g] = given.y[g];
+    }
+  }
   int tiles = 0;
   for (int g = 0; g < plan.ngroups; ++g) {
     p.m[g] = plan.m[g];
@@ -1662,7 +1728,7 @@ static sbp_status launch_split(const MatmulPlan& given, const int* kblocks, Spli
     q.ld[g] = pad4(given.n[g]);
     q.ldy[g] = given.ldy[g];
     q.y_ptr[g] = given.y[g];
-    p.y_ptr[g] = at;
+    p.y_ptr[g] = at;          // of row blocks multiplied as one, the first: the others follow it
     p.ldy[g] = q.ld[g];
     at += given.m[g] * q.ld[g];
     quads = std::max(quads, given.m[g] * q.ld[g] / 4);
@@ -1702,14 +1768,16 @@ sbp_status launch_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, void* 
     if (plan.lda[s] % 8 != 0 || plan.ldb[s] % 8 != 0) return SBP_ERR_UNSUPPORTED;
     if (plan.lda[s] == 0 || plan.ldb[s] == 0) return SBP_ERR_UNSUPPORTED;
   }
-  bool y_direct = false;
+  MatmulPlan merged;
+  const bool as_one = merge_row_blocks(plan, &merged);
+  bool y_direct = false, rows_aligned = true;
   long long ktotal_chain = 0;
   for (int s = 0; s < plan.nseg; ++s) ktotal_chain += plan.kseg[s];
   for (int g = 0; g < plan.ngroups; ++g) {
     if (plan.m[g] == 0 || plan.n[g] == 0) continue;
     if (stores_y && (!aligned16(plan.y[g]) || (plan.ldy[g] * oesz) % 16 != 0)) y_direct = true;
     if (!plan.b_trans && plan.col_off[g] % 8 != 0) return SBP_ERR_UNSUPPORTED;   // the x coordinate of a TMA load
-    if (plan.a_trans && plan.row_off[g] % 8 != 0) return SBP_ERR_UNSUPPORTED;
+    if (plan.a_trans && plan.row_off[g] % 8 != 0) rows_aligned = false;
     const long long kg = plan.chain ? ktotal_chain : plan.kseg[g];
     if (kg == 0) return SBP_ERR_UNSUPPORTED;   // an all-zero result: left to the FMA kernel
     if (plan.m[g] > 0x7fffffffLL || plan.n[g] > 0x7fffffffLL) return SBP_ERR_UNSUPPORTED;
@@ -1717,6 +1785,7 @@ sbp_status launch_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, void* 
   for (int r = 0; r < plan.n_rep; ++r)
     if (!aligned16(plan.y_rep[r])) y_direct = true;
   if (!encode_fn()) return SBP_ERR_UNSUPPORTED;
+  if (!rows_aligned && !as_one) return SBP_ERR_UNSUPPORTED;
 
   int kblocks[SBP_MAX_K];
   long long kb_tile = 0, tiles_sq = 0, tiles_tall = 0;
@@ -1744,13 +1813,25 @@ sbp_status launch_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, void* 
     if (qs == SBP_OK) qs = launch_tc(true, plan.a_trans, plan.b_trans, nullptr, st, &cap_tall);
     if (qs != SBP_OK) return qs;
     const int forced = forced_form();
-    form = choose_form(tiles_sq, tiles_tall, kb_tile, cap_sq, cap_tall, plan.gelu != 0, plan.n_rep, plan.out_dtype == SBP_F32, forced == 4 ? 0 : forced);
+    OperandRows rows = operand_rows(plan);
+    if (!rows_aligned) {      // it would run on a repacked copy of X, whose pitch is another
+      long long pitch = 0;
+      for (int g = 0; g < plan.ngroups; ++g) pitch += (plan.m[g] + 7) / 8 * 8;
+      rows.a = pitch % 64 != 0 ? 1.9e-3 : 1.0e-3;
+    }
+    form = choose_form(tiles_sq, tiles_tall, kb_tile, cap_sq, cap_tall, plan.gelu != 0, plan.n_rep, plan.out_dtype == SBP_F32, rows,
+                       forced == 4 ? 0 : forced);
     if (y_direct) form.walk_tall = false;
+    if (!rows_aligned) {      // the copy: a launch, one read and one write
+      form.cost += 4.0;
+      for (int s = 0; s < plan.nseg; ++s) form.cost += (double)plan.kseg[s] * merged.m[0] * 4.0 / 4e6;
+    }
     if (forced == 4 || (forced == 0 && pair_cap() == 0)) {
-      const SplitChoice sc = choose_split(plan, kblocks, 0.92 * (form.cost + 5.5), forced, aligned16(ws) ? ws_bytes : 0);
-      if (sc.splits > 0) return launch_split(plan, kblocks, sc, !y_direct, static_cast<float*>(ws), st, taken);
+      const SplitChoice sc = choose_split(as_one ? merged : plan, kblocks, 0.92 * (form.cost + 5.5), forced, aligned16(ws) ? ws_bytes : 0);
+      if (sc.splits > 0) return launch_split(plan, as_one ? &merged : nullptr, kblocks, sc, !y_direct, static_cast<float*>(ws), st, taken);
     }
   }
+  if (!rows_aligned) return SBP_ERR_UNSUPPORTED;
 
   p.ngroups = plan.ngroups;
   p.nseg = plan.nseg;
