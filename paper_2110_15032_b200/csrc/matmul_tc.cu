@@ -38,6 +38,7 @@
 #include <mutex>
 #include <type_traits>
 
+#include "boxing_shift.h"
 #include "bounds_check.h"
 #include "matmul_plan.h"
 #include "sbp_internal.h"
@@ -366,6 +367,26 @@ __device__ __forceinline__ TileCoord tile_coord(const TcParams& p, int tile) {
 // (untransposed) form carries no trace of the other three: as run-time switches they cost the
 // MMA-issuing thread and the producer enough to slow every product by 6 %.
 // MH: m-halves of 256 rows per pair tile (1 = square form, 2 = tall form, see kStageBytesTall).
+// Part `lane` of `lanes` of a row of `bytes` bytes that starts at dst, which need not be 16-byte aligned, from shared
+// memory (`at`: where a byte of the row lies; 16-byte chunks are whole): a whole aligned vector of the destination, two
+// chunks shifted together, and every lanes-th element of those before the first and after the last such vector.
+// (A result [1500 x 4832] over eight devices, rows of 604: 40.0 us so, 45.8 with an element a lane and store; [585 x 1204] over four 14.2, 17.9; [4000 x 4091] 60, 73.)
+template <int ESZ, typename At>
+__device__ __forceinline__ void store_shifted(unsigned char* dst, int bytes, int lane, int lanes, At at) {
+  const int to_line = (int)(-reinterpret_cast<long long>(dst) & 15), head = to_line < bytes ? to_line : bytes;
+  const int nvec = (bytes - head) >> 4;
+  if (lane < nvec && SBP_GUARD(dst + head + lane * 16, 16)) {
+    uint4 v = *reinterpret_cast<const uint4*>(at(lane * 16));
+    if (head) v = shift_pair<ESZ>(v, *reinterpret_cast<const uint4*>(at(lane * 16 + 16)), (unsigned)head);
+    *reinterpret_cast<uint4*>(dst + head + lane * 16) = v;
+  }
+  using E = typename ShiftElem<ESZ>::type;
+  for (int e = lane * ESZ; e < bytes - nvec * 16; e += lanes * ESZ) {
+    const int off = e < head ? e : nvec * 16 + e;
+    if (SBP_GUARD(dst + off, ESZ)) *reinterpret_cast<E*>(dst + off) = *reinterpret_cast<const E*>(at(off));
+  }
+}
+
 template <int AT, int BT, int MH>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
     matmul_tc_kernel(const __grid_constant__ TcParams p) {
@@ -732,28 +753,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
               __syncwarp();
             }
             if (p.y_direct) {
-              // rows of the slab, one after the other; the lanes take consecutive elements of a row
+              // eight lanes to a row of the slab, four rows at a time
               __syncwarp();
-              const int n_out = (tc.g == 0 ? p.n_rep : 0) + 1;
+              const int n_out = (tc.g == 0 ? p.n_rep : 0) + 1, esz = p.out_f32 ? 4 : 2;
+              const int bytes = (int)min((long long)cols_per_slab, Ng - col0) * esz;
               for (int o = 0; o < n_out; ++o) {
-                unsigned char* yb = static_cast<unsigned char*>(o == 0 ? p.y_ptr[tc.g] : p.rep_ptr[o - 1]);
+                unsigned char* yb = static_cast<unsigned char*>(o == 0 ? p.y_ptr[tc.g] : p.rep_ptr[o - 1]) + col0 * esz;
                 const long long ld = p.ldy[tc.g];
-                for (int r = 0; r < 32 && row0 + r < Mg; ++r) {
-                  const unsigned char* srow = buf + r * 128;
-                  if (p.out_f32) {
-                    const int c = lane;
-                    if (col0 + c < Ng && SBP_GUARD(reinterpret_cast<float*>(yb) + (row0 + r) * ld + col0 + c, 4))
-                      reinterpret_cast<float*>(yb)[(row0 + r) * ld + col0 + c] =
-                          *reinterpret_cast<const float*>(srow + ((((c >> 2) ^ (r & 7)) << 4) | ((c & 3) << 2)));
-                  } else {
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                      const int c = lane + 32 * h;
-                      if (col0 + c < Ng && SBP_GUARD(reinterpret_cast<unsigned short*>(yb) + (row0 + r) * ld + col0 + c, 2))
-                        reinterpret_cast<unsigned short*>(yb)[(row0 + r) * ld + col0 + c] =
-                            *reinterpret_cast<const unsigned short*>(srow + ((((c >> 3) ^ (r & 7)) << 4) | ((c & 7) << 1)));
-                    }
-                  }
+#pragma unroll 4
+                for (int r = lane >> 3; r < 32; r += 4) {
+                  if (row0 + r >= Mg) break;
+                  auto at = [&](int off) { return buf + r * 128 + ((((off >> 4) ^ (r & 7)) << 4) | (off & 15)); };
+                  if (p.out_f32) store_shifted<4>(yb + (row0 + r) * ld * 4, bytes, lane & 7, 8, at);
+                  else store_shifted<2>(yb + (row0 + r) * ld * 2, bytes, lane & 7, 8, at);
                 }
               }
               __syncwarp();      // the buffer is rewritten two slabs from now
@@ -1096,40 +1108,63 @@ __global__ void __launch_bounds__(kThreadsTc, 1) matmul_tc_split_kernel(const __
     const long long yr0 = SW ? col0 : row0, yc0 = SW ? row0 : col0, yrows = SW ? Ng : Mg, ycols = SW ? Mg : Ng;
     const int n_out = (g == 0 ? p.n_rep : 0) + 1;
     const long long ld = p.ldy[g];
-    auto store = [&](unsigned char* y, auto blocks) {
+    const long long left = ycols - yc0;                  // columns of the result from this warp's first on
+    unsigned char* y0 = static_cast<unsigned char*>(p.y_ptr[g]) + part * p.part_bytes + (yr0 * ld + yc0) * esz;
+    const long long row_bytes = ld * esz;
+    // where row r of this warp's lies in destination o
+    auto row_at = [&](int r, int o, auto blocks) -> unsigned char* {
+      if constexpr (decltype(blocks)::value) {
+        int b = 0;
+        while (b + 1 < p.blocks && yr0 + r >= p.block_row[b + 1]) ++b;
+        return static_cast<unsigned char*>(p.block_y[b]) + (yr0 + r - p.block_row[b]) * row_bytes + yc0 * esz;
+      } else {
+        return (o == 0 ? y0 : static_cast<unsigned char*>(p.rep_ptr[o - 1]) + yr0 * row_bytes + yc0 * esz) + r * row_bytes;
+      }
+    };
+    auto store = [&](auto blocks, auto one) {
+#pragma unroll 4
       for (int idx = lane; idx < nrows * pieces; idx += 32) {
         const int r = idx / pieces, ch = idx - r * pieces;
-        if (yr0 + r >= yrows) continue;
+        if (yr0 + r >= yrows || ch * el >= left) continue;
         const uint4 v = *reinterpret_cast<const uint4*>(stage + r * pitch + ch * 16);
-        const long long c = yc0 + ch * el;
-        long long row = yr0 + r;
-        unsigned char* base = y;
-        if constexpr (decltype(blocks)::value) {
-          int b = 0;
-          while (b + 1 < p.blocks && row >= p.block_row[b + 1]) ++b;
-          base = static_cast<unsigned char*>(p.block_y[b]);
-          row -= p.block_row[b];
-        }
-        unsigned char* at = base + (row * ld + c) * esz;
-        if (p.y_vec && c + el <= ycols) {
-          if (SBP_GUARD(at, 16)) *reinterpret_cast<uint4*>(at) = v;
-        } else if (p.out_f32) {
-          const float* f = reinterpret_cast<const float*>(&v);
+        for (int o = 0; o < (decltype(one)::value ? 1 : n_out); ++o) {
+          unsigned char* at = row_at(r, o, blocks) + ch * 16;
+          if ((ch + 1) * el <= left) {
+            if (SBP_GUARD(at, 16)) *reinterpret_cast<uint4*>(at) = v;
+          } else if (p.out_f32) {
+            const float* f = reinterpret_cast<const float*>(&v);
 #pragma unroll
-          for (int e = 0; e < 4; ++e)
-            if (c + e < ycols && SBP_GUARD(at + 4 * e, 4)) reinterpret_cast<float*>(at)[e] = f[e];
-        } else {
-          const unsigned short* f = reinterpret_cast<const unsigned short*>(&v);
+            for (int e = 0; e < 3; ++e)
+              if (ch * el + e < left && SBP_GUARD(at + 4 * e, 4)) reinterpret_cast<float*>(at)[e] = f[e];
+          } else {
+            const unsigned short* f = reinterpret_cast<const unsigned short*>(&v);
 #pragma unroll
-          for (int e = 0; e < 8; ++e)
-            if (c + e < ycols && SBP_GUARD(at + 2 * e, 2)) reinterpret_cast<unsigned short*>(at)[e] = f[e];
+            for (int e = 0; e < 7; ++e)
+              if (ch * el + e < left && SBP_GUARD(at + 2 * e, 2)) reinterpret_cast<unsigned short*>(at)[e] = f[e];
+          }
         }
       }
     };
-    if (p.blocks) store(nullptr, std::true_type{});
-    else
-      for (int o = 0; o < n_out; ++o)
-        store(static_cast<unsigned char*>(o == 0 ? p.y_ptr[g] : p.rep_ptr[o - 1]) + part * p.part_bytes, std::false_type{});
+    auto store_unaligned = [&](auto blocks) {
+      const int bytes = (int)(left < pieces * el ? left : pieces * el) * esz;
+      for (int idx = lane; idx < nrows * pieces; idx += 32) {
+        const int r = idx / pieces, ch = idx - r * pieces;
+        if (yr0 + r >= yrows) continue;
+        auto in = [&](int off) { return stage + r * pitch + off; };
+        for (int o = 0; o < n_out; ++o) {
+          if (p.out_f32) store_shifted<4>(row_at(r, o, blocks), bytes, ch, pieces, in);
+          else store_shifted<2>(row_at(r, o, blocks), bytes, ch, pieces, in);
+        }
+      }
+    };
+    if (p.y_vec) {
+      if (p.blocks) store(std::true_type{}, std::true_type{});
+      else if (n_out == 1) store(std::false_type{}, std::true_type{});
+      else store(std::false_type{}, std::false_type{});
+    } else {
+      if (p.blocks) store_unaligned(std::true_type{});
+      else store_unaligned(std::false_type{});
+    }
   }
 
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
