@@ -361,12 +361,6 @@ __device__ __forceinline__ TileCoord tile_coord(const TcParams& p, int tile) {
   return TileCoord{g, mt * p.walk_m + half_m, nt * BN};
 }
 
-// ------------------------------------------------------------------ the kernel
-
-// AT / BT: operand A / B is stored transposed.  They are compile-time so that the usual
-// (untransposed) form carries no trace of the other three: as run-time switches they cost the
-// MMA-issuing thread and the producer enough to slow every product by 6 %.
-// MH: m-halves of 256 rows per pair tile (1 = square form, 2 = tall form, see kStageBytesTall).
 // Part `lane` of `lanes` of a row of `bytes` bytes that starts at dst, which need not be 16-byte aligned, from shared
 // memory (`at`: where a byte of the row lies; 16-byte chunks are whole): a whole aligned vector of the destination, two
 // chunks shifted together, and every lanes-th element of those before the first and after the last such vector.
@@ -387,6 +381,12 @@ __device__ __forceinline__ void store_shifted(unsigned char* dst, int bytes, int
   }
 }
 
+// ------------------------------------------------------------------ the kernel
+
+// AT / BT: operand A / B is stored transposed.  They are compile-time so that the usual
+// (untransposed) form carries no trace of the other three: as run-time switches they cost the
+// MMA-issuing thread and the producer enough to slow every product by 6 %.
+// MH: m-halves of 256 rows per pair tile (1 = square form, 2 = tall form, see kStageBytesTall).
 template <int AT, int BT, int MH>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
     matmul_tc_kernel(const __grid_constant__ TcParams p) {
@@ -1245,6 +1245,307 @@ __global__ void __launch_bounds__(256) matmul_parts_kernel(const __grid_constant
   }
 }
 
+// ------------------------------------------------------------------ the fused classifier for few rows
+//
+// Softmax partials or gradient of the class-split logits, operands exchanged: a tile is 256 CLASSES (128 per CTA of the
+// pair) by all NB >= rows rows.  The weight is read once whatever is done, 2 * feat bytes a class, and is the floor for
+// few rows; in the persistent kernel above a tile of 256 rows costs its epilogue all the same, of whose warps only
+// those that hold the few rows work (14 rows, 176 features, 475 696 classes: 77 us forward, 83 backward, where the
+// weight takes 26; here 40 and 39 with what follows the product).  Here the features stay in shared memory, the weight streams past them in K-blocks of
+// 16 KB a CTA, and every epilogue warp has 32 classes.
+//   forward   a warp turns its 32 classes x 32 rows over in shared memory, so that a lane holds a row: maximum, sum and
+//             the label's logit without a shuffle; the four warps of a 128-class chunk are merged through shared memory.
+//   backward  a lane is a class; four lanes exchange their rows so that each stores four classes of one.
+// With many rows and few features the epilogue is the bound again (its shared-memory and exponential phases, some 1850
+// clocks a batch): 192 features, 161 472 classes, forward / backward: 32 rows 20.5 / 17.9 (persistent kernel 35.7 / 36.2),
+// 64 rows 23.5 / 21.4 (36 / 37), 128 rows 33 / 30 (37 / 38.5), where the line is; above it the rows need a second tile.
+// 512 features, 2^20 classes, 64 rows: 171 / 192 (223 / 225), the weight's 164 us and the gradient's 21.
+struct NarrowParams {
+  CUtensorMap map_w[SBP_MAX_K];       // [feat, classes of shard g], boxes of 64 x 64
+  CUtensorMap map_f;                  // [rows, feat], boxes of NB / 2 rows x 64
+  long long n[SBP_MAX_K], ldy[SBP_MAX_K], class_start[SBP_MAX_K];
+  void* y[SBP_MAX_K];
+  int tile_begin[SBP_MAX_K + 1];
+  int ngroups, kblocks, rows, out_f32, stages;
+  int y_quads;                        // bf16 gradient whose rows take 8-byte stores, classes by the four
+  XentFusion xf;
+};
+
+constexpr int kNarrowRows = 128;
+constexpr int kNarrowMaxStages = 12;
+constexpr int kNarrowAccs = 4;                                 // accumulators of NB columns in flight
+constexpr int kNarrowFeatures = 64 * 1024;                     // most shared memory the features may take
+constexpr int kNarrowPitch = 36;                               // floats between the staged classes of a warp
+constexpr int kNarrowStageBytes = kEpiWarps * 32 * kNarrowPitch * 4;
+constexpr int kNarrowRedBytes = 2 * 2 * 4 * 3 * 32 * 4;        // [half][parity][quadrant][m, s, t][row]
+constexpr int kNarrowSmem = 220 * 1024;
+template <int NB>
+constexpr int narrow_feature_block() { return NB / 2 * 128; }  // one CTA's half of the rows, 64 features
+
+template <int NB, int MODE>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1) xent_narrow_kernel(const __grid_constant__ NarrowParams p) {
+  constexpr int kFb = narrow_feature_block<NB>();
+  extern __shared__ unsigned char smem_raw[];
+  __shared__ __align__(8) unsigned long long bar_full[kNarrowMaxStages], bar_empty[kNarrowMaxStages], bar_feat, bar_acc_full[kNarrowAccs],
+      bar_acc_empty[kNarrowAccs];
+  __shared__ unsigned tmem_base_slot;
+  __shared__ int abort_flag_s;
+  __shared__ __align__(16) float neg_s[MODE == 2 ? NB : 4];
+  __shared__ long long lab_s[NB];
+  volatile int* abort_flag = &abort_flag_s;
+
+  unsigned char* feat = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  unsigned char* ring = feat + (p.kblocks * kFb + 1023) / 1024 * 1024;
+  float* staging = reinterpret_cast<float*>(ring + p.stages * kStageA);
+  float* red = staging + kEpiWarps * 32 * kNarrowPitch;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned rank = cluster_ctarank();
+
+  if (threadIdx.x == 0) {
+    abort_flag_s = 0;
+    for (int i = 0; i < p.stages; ++i) {
+      mbar_init(smem_addr(&bar_full[i]), 1);
+      mbar_init(smem_addr(&bar_empty[i]), 1);
+    }
+    mbar_init(smem_addr(&bar_feat), 1);
+    for (int i = 0; i < kNarrowAccs; ++i) {
+      mbar_init(smem_addr(&bar_acc_full[i]), 1);
+      mbar_init(smem_addr(&bar_acc_empty[i]), NB == 32 ? kEpiWarps : 2 * kEpiWarps);      // used in CTA 0: both CTAs' warps
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_base_slot)),
+                 "r"(kNarrowAccs * NB)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  SBP_PDL_RELEASE();
+  SBP_PDL_WAIT();
+  if (threadIdx.x < NB) {
+    const int row = threadIdx.x;
+    lab_s[row] = row < p.rows && SBP_GUARD(p.xf.labels + row, 8) ? p.xf.labels[row] : -1;
+    // softmax = 2^(z log2e - m log2e - log2 S): the division by the row sum is folded into the exponent
+    if (MODE == 2 && row < p.rows && SBP_GUARD(p.xf.row_max + row, 4) && SBP_GUARD(p.xf.row_sum + row, 4))
+      neg_s[row] = -p.xf.row_max[row] * 1.4426950408889634f - log2f(p.xf.row_sum[row]);
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  cluster_sync_all();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const unsigned tmem_base = tmem_base_slot;
+
+  const int first = blockIdx.x >> 1, stride = gridDim.x >> 1, tiles = p.tile_begin[p.ngroups];
+  if (warp == 0) {
+    // ------------------------------------------------ producer (both CTAs)
+    const bool leader = elect_one();
+    if (leader) {
+      if (rank == 0) mbar_expect_tx(smem_addr(&bar_feat), 2 * p.kblocks * kFb);
+      const unsigned feat0 = map_to_cta(smem_addr(&bar_feat), 0);
+      for (int kb = 0; kb < p.kblocks; ++kb) tma_load_2d(smem_addr(feat + kb * kFb), &p.map_f, kb * BK, (int)rank * (NB / 2), feat0);
+    }
+    __syncwarp();
+    int slot = 0, rounds = 0, g = 0;
+    unsigned round = 0;
+    for (int tile = first; tile < tiles && !*abort_flag; tile += stride) {
+      while (tile >= p.tile_begin[g + 1]) ++g;
+      const int col = (tile - p.tile_begin[g]) * BM + (int)rank * BMH;
+      for (int kb = 0; kb < p.kblocks; ++kb, ++rounds) {
+        if (!mbar_wait_warp(smem_addr(&bar_empty[slot]), round ^ 1, abort_flag)) break;
+        if (leader) {
+          const unsigned full0 = map_to_cta(smem_addr(&bar_full[slot]), 0);
+          if (rank == 0) mbar_expect_tx(smem_addr(&bar_full[slot]), 2 * kStageA);
+#pragma unroll
+          for (int c = 0; c < BMH / 64; ++c)
+            tma_load_2d(smem_addr(ring + slot * kStageA + c * (BK * 128)), &p.map_w[g], col + c * 64, kb * BK, full0);
+        }
+        __syncwarp();
+        slot = slot + 1 == p.stages ? 0 : slot + 1;
+        round ^= (slot == 0);
+      }
+    }
+    if (*abort_flag && rank == 0 && leader) {
+      // give the loads still in flight a bounded chance to land before the CTA goes away
+      for (int i = rounds > p.stages ? rounds - p.stages : 0; i < rounds; ++i) {
+        const unsigned long long t0 = now_ns();
+        while (!mbar_try(smem_addr(&bar_full[i % p.stages]), (unsigned)((i / p.stages) & 1)) && now_ns() - t0 < 100000000ull) {
+        }
+      }
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------ MMA issuer (CTA 0)
+    if (rank == 0) {
+      const bool leader = elect_one();
+      constexpr unsigned idesc = make_idesc(1, 1, NB);
+      bool ok = mbar_wait_warp(smem_addr(&bar_feat), 0, abort_flag);
+      int slot = 0, it = 0;
+      unsigned round = 0;
+      for (int tile = first; tile < tiles && ok; tile += stride, ++it) {
+        const int buf = it % kNarrowAccs;
+        ok = mbar_wait_warp(smem_addr(&bar_acc_empty[buf]), (unsigned)((it / kNarrowAccs) & 1) ^ 1, abort_flag);
+        for (int kb = 0; kb < p.kblocks && ok; ++kb) {
+          ok = mbar_wait_warp(smem_addr(&bar_full[slot]), round, abort_flag);
+          if (!ok) break;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          if (leader) {
+            const unsigned sa = smem_addr(ring + slot * kStageA) & 0x3ffffu, sb = smem_addr(feat + kb * kFb) & 0x3ffffu;
+#pragma unroll
+            for (int kk = 0; kk < BK / 16; ++kk) {
+              constexpr unsigned a_lo = desc_lo_fixed(BK * 128), b_lo = desc_lo_fixed(16), hi = desc_hi_fixed(1024);
+              umma_bf16(tmem_base + buf * NB, desc_pack(a_lo + (sa >> 4) + kk * 128, hi), desc_pack(b_lo + (sb >> 4) + kk * 2, hi), idesc,
+                        (kb > 0 || kk > 0) ? 1u : 0u);
+            }
+            umma_commit_pair(smem_addr(&bar_empty[slot]));
+          }
+          __syncwarp();
+          slot = slot + 1 == p.stages ? 0 : slot + 1;
+          round ^= (slot == 0);
+        }
+        if (leader && ok) umma_commit_pair(smem_addr(&bar_acc_full[buf]));
+        __syncwarp();
+      }
+    }
+  } else {
+    // ------------------------------------------------ epilogue (both CTAs): 32 classes and 32 rows a warp and batch
+    // After a wait that ran out the warps go on without waiting: they still meet at their barriers.
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    const unsigned tq = tmem_base + ((unsigned)(q * 32) << 16);
+    float* mine = staging + (warp - 2) * (32 * kNarrowPitch);
+    int it = 0, g = 0, met = 0;
+    for (int tile = first; tile < tiles; tile += stride, ++it) {
+      if (NB == 32 && (it & 1) != half) continue;      // one batch a tile: the two warps of a quadrant take turns
+      while (tile >= p.tile_begin[g + 1]) ++g;
+      const int buf = it % kNarrowAccs;
+      bool ok = !*abort_flag;
+      if (ok && lane == 0) ok = mbar_wait(smem_addr(&bar_acc_full[buf]), (unsigned)((it / kNarrowAccs) & 1), abort_flag);
+      __syncwarp();
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const long long chunk0 = (long long)(tile - p.tile_begin[g]) * BM + rank * BMH;      // this CTA's first class in the shard
+      const long long cls = chunk0 + q * 32 + lane, Ng = p.n[g];
+      constexpr int kBatches = NB / 32, kStep = NB == 32 ? 1 : 2;
+#pragma unroll(MODE == 1 ? 2 : 1)
+      for (int b0 = 0; b0 < kBatches; b0 += kStep) {
+        const int b = NB == 32 ? 0 : b0 + half, r0 = b * 32;
+        float v[32];
+        tmem_ld32(tq + buf * NB + r0, v);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (b0 + kStep >= kBatches) {                  // the accumulator is free again
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(map_to_cta(smem_addr(&bar_acc_empty[buf]), 0));
+        }
+        if (r0 >= p.rows || chunk0 >= Ng) continue;    // the same for the four warps of a half
+        if constexpr (MODE == 1) {
+          constexpr float kL2e = 1.4426950408889634f;
+#pragma unroll
+          for (int c = 0; c < 8; ++c) {
+            float4 f = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+            if (cls >= Ng) f = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+            *reinterpret_cast<float4*>(mine + lane * kNarrowPitch + 4 * c) = f;
+          }
+          __syncwarp();
+          float x[32];                                  // this lane's row, 32 classes
+#pragma unroll
+          for (int i = 0; i < 32; ++i) x[i] = mine[i * kNarrowPitch + lane];
+          float top[4] = {x[0], x[1], x[2], x[3]};
+#pragma unroll
+          for (int i = 4; i < 32; ++i) top[i & 3] = fmaxf(top[i & 3], x[i]);
+          const float m = fmaxf(fmaxf(top[0], top[1]), fmaxf(top[2], top[3]));
+          const float neg = m == -INFINITY ? 0.f : -m * kL2e;      // no class of the shard here: sum 0
+          float sum[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            float e;
+            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(fmaf(x[i], kL2e, neg)));
+            sum[i & 3] += e;
+          }
+          const long long want = lab_s[r0 + lane] - p.class_start[g] - chunk0 - q * 32;
+          const float t = want >= 0 && want < 32 && want < Ng - chunk0 - q * 32 ? mine[(int)want * kNarrowPitch + lane] : 0.f;
+          float* out = red + ((half * 2 + (met & 1)) * 4) * 96 + lane;
+          out[q * 96] = m;
+          out[q * 96 + 32] = (sum[0] + sum[1]) + (sum[2] + sum[3]);
+          out[q * 96 + 64] = t;
+          asm volatile("bar.sync %0, 128;" ::"r"(1 + half) : "memory");
+          if (q == (met & 3) && r0 + lane < p.rows) {
+            float M = fmaxf(fmaxf(out[0], out[96]), fmaxf(out[192], out[288])), S = 0.f, T = 0.f;
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+              float e;
+              asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"((out[w * 96] - M) * kL2e));
+              S = fmaf(out[w * 96 + 32], e, S);
+              T += out[w * 96 + 64];
+            }
+            const long long at = (long long)(p.xf.part_base[g] + chunk0 / BMH) * p.rows + r0 + lane;
+            if (SBP_GUARD(p.xf.part_m + at, 4)) p.xf.part_m[at] = M;
+            if (SBP_GUARD(p.xf.part_s + at, 4)) p.xf.part_s[at] = S;
+            if (SBP_GUARD(p.xf.part_t + at, 4)) p.xf.part_t[at] = T;
+          }
+          ++met;
+        } else {
+          const long long first_class = p.class_start[g] + chunk0 + q * 32, step = p.ldy[g];
+#pragma unroll
+          for (int c = 0; c < 32; c += 4) {
+            const float4 neg = *reinterpret_cast<const float4*>(neg_s + r0 + c);
+            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(v[c]) : "f"(fmaf(v[c], 1.4426950408889634f, neg.x)));
+            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(v[c + 1]) : "f"(fmaf(v[c + 1], 1.4426950408889634f, neg.y)));
+            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(v[c + 2]) : "f"(fmaf(v[c + 2], 1.4426950408889634f, neg.z)));
+            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(v[c + 3]) : "f"(fmaf(v[c + 3], 1.4426950408889634f, neg.w)));
+          }
+          // rows whose label is one of this warp's 32 classes are rare
+          const long long want = lab_s[r0 + lane] - first_class;
+          if (__any_sync(0xffffffffu, want >= 0 && want < 32)) {
+#pragma unroll
+            for (int c = 0; c < 32; ++c)
+              if (lab_s[r0 + c] == first_class + lane) v[c] -= 1.0f;
+          }
+          if (p.y_quads) {
+            // bf16 in pieces of four classes: lanes 4 i .. 4 i + 3 hold 4 x 4 elements of four rows, and after two
+            // exchanges lane 4 i + r has row r's four
+            const bool odd = lane & 1, high = lane & 2;
+            unsigned char* at = static_cast<unsigned char*>(p.y[g]) + ((r0 + (lane & 3)) * step + (cls & ~3ll)) * 2;
+#pragma unroll
+            for (int c = 0; c < 32; c += 4, at += 8 * step) {
+              if (r0 + c >= p.rows) break;
+              unsigned w[2];
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                const __nv_bfloat162 two = __floats2bfloat162_rn(v[c + 2 * h], v[c + 2 * h + 1]);
+                const unsigned own = *reinterpret_cast<const unsigned*>(&two), other = __shfl_xor_sync(0xffffffffu, own, 1);
+                w[h] = odd ? __byte_perm(other, own, 0x7632) : __byte_perm(own, other, 0x5410);      // row 2 h + odd, two classes
+              }
+              const unsigned other = __shfl_xor_sync(0xffffffffu, high ? w[0] : w[1], 2);
+              const uint2 o = high ? make_uint2(other, w[1]) : make_uint2(w[0], other);
+              if (cls < Ng && r0 + c + (lane & 3) < p.rows && SBP_GUARD(at, 8)) *reinterpret_cast<uint2*>(at) = o;
+            }
+          } else if (cls < Ng) {
+            const int esz = p.out_f32 ? 4 : 2;
+            unsigned char* at = static_cast<unsigned char*>(p.y[g]) + (r0 * step + cls) * esz;
+#pragma unroll
+            for (int c = 0; c < 32; ++c, at += step * esz) {
+              if (r0 + c >= p.rows) break;
+              if (p.out_f32) {
+                if (SBP_GUARD(at, 4)) *reinterpret_cast<float*>(at) = v[c];
+              } else {
+                if (SBP_GUARD(at, 2)) *reinterpret_cast<__nv_bfloat16*>(at) = __float2bfloat16_rn(v[c]);
+              }
+            }
+          }
+        }
+      }
+    }
+  }
+
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  cluster_sync_all();
+  if (warp == 1) {
+    __syncwarp();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kNarrowAccs * NB) : "memory");
+  }
+}
+
 // ------------------------------------------------------------------ host side
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -1789,6 +2090,88 @@ static sbp_status launch_split(const MatmulPlan& given, const MatmulPlan* merged
   return SBP_OK;
 }
 
+template <int NB, int MODE>
+static sbp_status launch_narrow_form(NarrowParams& p, cudaStream_t st) {
+  static std::atomic<int> pairs_on_device[64];
+  int dev = 0;
+  SBP_CUDA_TRY(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64) return fail(SBP_ERR_UNSUPPORTED, "device ordinal %d out of range", dev);
+  auto* kernel = xent_narrow_kernel<NB, MODE>;
+  int pairs = pairs_on_device[dev].load(std::memory_order_relaxed);
+  if (pairs == 0) {
+    SBP_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kNarrowSmem));
+    int sms = 0;
+    SBP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    cudaLaunchConfig_t probe = {};
+    probe.gridDim = dim3((unsigned)(2 * (sms / 2)));
+    probe.blockDim = dim3(kThreadsTc);
+    probe.dynamicSmemBytes = kNarrowSmem;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 2;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    probe.attrs = &attr;
+    probe.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&pairs, kernel, &probe) != cudaSuccess || pairs < 1) {
+      cudaGetLastError();
+      pairs = sms / 2;
+    }
+    pairs_on_device[dev].store(pairs, std::memory_order_relaxed);
+  }
+  const int features = (p.kblocks * narrow_feature_block<NB>() + 1023) / 1024 * 1024;
+  const int room = kNarrowSmem - 1024 - features - (MODE == 1 ? kNarrowStageBytes + kNarrowRedBytes : 0);
+  p.stages = std::min(kNarrowMaxStages, room / kStageA);
+  const int tiles = p.tile_begin[p.ngroups];
+  SBP_BOUNDS_UPLOAD(st);
+  const cudaError_t e = launch_dependent(kernel, dim3((unsigned)(2 * std::min(tiles, pairs))), dim3(kThreadsTc), kNarrowSmem, st, p);
+  if (e != cudaSuccess) return cuda_fail(e, "fused classifier launch");
+  count_launch();
+  return SBP_OK;
+}
+
+// The fused classifier for at most kNarrowRows rows; *taken stays false where the features do not fit.
+static sbp_status launch_narrow(const MatmulPlan& plan, const XentFusion& xf, cudaStream_t st, bool* taken) {
+  const int nb = xf.rows <= 32 ? 32 : (xf.rows <= 64 ? 64 : 128);
+  const long long kb = (plan.kseg[0] + BK - 1) / BK;
+  if (xf.rows > kNarrowRows || kb * (nb / 2 * 128) > kNarrowFeatures) return SBP_OK;
+  NarrowParams p;
+  p.ngroups = plan.ngroups;
+  p.kblocks = (int)kb;
+  p.rows = (int)xf.rows;
+  p.out_f32 = plan.out_dtype == SBP_F32;
+  p.y_quads = !p.out_f32;
+  p.xf = xf;
+  int tiles = 0;
+  for (int g = 0; g < plan.ngroups; ++g) {
+    p.tile_begin[g] = tiles;
+    p.n[g] = plan.n[g];
+    p.ldy[g] = plan.ldy[g];
+    p.y[g] = plan.y[g];
+    p.class_start[g] = xf.class_start[g];
+    if (plan.n[g] % 4 != 0 || plan.ldy[g] % 4 != 0 || reinterpret_cast<uintptr_t>(plan.y[g]) % 8 != 0) p.y_quads = 0;
+    if (plan.n[g] <= 0) continue;
+    if (plan.n[g] / BM + tiles > 0x3fffffffLL) return SBP_OK;
+    tiles += (int)((plan.n[g] + BM - 1) / BM);
+    if (!make_map(&p.map_w[g], plan.b[g], 2, plan.kseg[g], plan.n[g], plan.ldb[g], BK, 64))
+      return fail(SBP_ERR_CUDA, "cuTensorMapEncodeTiled failed for the weight of shard %d", g);
+  }
+  for (int g = plan.ngroups; g <= SBP_MAX_K; ++g) p.tile_begin[g] = tiles;
+  // the replicas of the features are equal: the first serves every shard
+  if (!make_map(&p.map_f, plan.a[0], 2, xf.rows, plan.kseg[0], plan.lda[0], nb / 2, BK))
+    return fail(SBP_ERR_CUDA, "cuTensorMapEncodeTiled failed for the features");
+  *taken = true;
+  if (tiles == 0) return SBP_OK;
+  switch (nb | (xf.grad ? 1 : 0)) {
+    case 32: return launch_narrow_form<32, 1>(p, st);
+    case 33: return launch_narrow_form<32, 2>(p, st);
+    case 64: return launch_narrow_form<64, 1>(p, st);
+    case 65: return launch_narrow_form<64, 2>(p, st);
+    case 128: return launch_narrow_form<128, 1>(p, st);
+    default: return launch_narrow_form<128, 2>(p, st);
+  }
+}
+
 sbp_status launch_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, void* ws, size_t ws_bytes, cudaStream_t st, bool* taken) {
   *taken = false;
   if (plan.in_dtype != SBP_BF16) return SBP_ERR_UNSUPPORTED;
@@ -1838,6 +2221,11 @@ sbp_status launch_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, void* 
   static TcParams p;          // large; filled under a lock and copied by value at launch
   static std::mutex mu;
   std::lock_guard<std::mutex> lock(mu);
+
+  if (xf && forced_form() == 0 && pair_cap() == 0) {
+    const sbp_status ns = launch_narrow(plan, *xf, st, taken);
+    if (ns != SBP_OK || *taken) return ns;
+  }
 
   // Which form (see choose_form).  The softmax epilogues are written for the square form, and so is
   // the element-wise store of a result the copy engine cannot address.
