@@ -70,6 +70,13 @@ constexpr int kStagesTall = 4;
 constexpr int kStageBytesTall = 2 * kStageA + kStageB;     // 48 KiB per CTA
 constexpr int kEpiBufsTall = 1;
 constexpr int kSmemBytesTall = kStagesTall * kStageBytesTall + kEpiWarps * kEpiBufsTall * kSlabBytes + 1024;
+// The short form (MH = 3): the square tile with four ring slots and three staging slabs a warp.  Where the contraction is
+// short the tile is its epilogue: with one slab a warp waits for each store to have read it before it stages the next.
+// (us, square / short, products over 2^19 to 2^20 classes: 1 K-block, 176 rows 56 / 50, 232 rows 108 / 103; gradient with 2
+// K-blocks 137 / 129; 3 K-blocks 39 / 35; softmax partials with 2 K-blocks 132 / 125, 3 37.7 / 35.9, 4 89 / 84.  With 5 and
+// 8 K-blocks four slots are too few: 29.0 / 32.4, 521 / 544.)
+constexpr int kStagesShort = 4, kEpiBufsShort = 3, kShortBlocks = 4;
+static_assert(kStagesShort * kStageBytes + kEpiWarps * kEpiBufsShort * kSlabBytes + 1024 <= kSmemBytes, "the short form fits where the square one does");
 constexpr int kMaxStages = kStages > kStagesTall ? kStages : kStagesTall;
 constexpr int kThreadsTc = 32 * (2 + kEpiWarps);
 constexpr int kTmemCols = 512;
@@ -386,14 +393,15 @@ __device__ __forceinline__ void store_shifted(unsigned char* dst, int bytes, int
 // AT / BT: operand A / B is stored transposed.  They are compile-time so that the usual
 // (untransposed) form carries no trace of the other three: as run-time switches they cost the
 // MMA-issuing thread and the producer enough to slow every product by 6 %.
-// MH: m-halves of 256 rows per pair tile (1 = square form, 2 = tall form, see kStageBytesTall).
+// MH: 1 = square form, 2 = tall form (two m-halves of 256 rows per pair tile, see kStageBytesTall), 3 = short form.
 template <int AT, int BT, int MH>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
     matmul_tc_kernel(const __grid_constant__ TcParams p) {
-  constexpr int kSt = MH == 2 ? kStagesTall : kStages;                  // ring depth
-  constexpr int kStA = MH * kStageA;                                    // bytes of A per ring slot
+  constexpr int kHalves = MH == 2 ? 2 : 1;
+  constexpr int kSt = MH == 2 ? kStagesTall : (MH == 3 ? kStagesShort : kStages);      // ring depth
+  constexpr int kStA = kHalves * kStageA;                                    // bytes of A per ring slot
   constexpr int kStBytes = kStA + kStageB;
-  constexpr int kEB = MH == 2 ? kEpiBufsTall : kEpiBufs;                // staging slabs per epilogue warp
+  constexpr int kEB = MH == 2 ? kEpiBufsTall : (MH == 3 ? kEpiBufsShort : kEpiBufs);                // staging slabs per epilogue warp
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long bar_full[kMaxStages], bar_empty[kMaxStages], bar_acc_full[2], bar_acc_empty[2];
   __shared__ unsigned tmem_base_slot;
@@ -468,7 +476,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
             unsigned char* sb = sa0 + kStA;
             const int bcol = (int)p.col_off[tc.g] + tc.n0 + (int)rank * BNH;
 #pragma unroll
-            for (int h = 0; h < MH; ++h) {       // this CTA's 128 rows of every m-half
+            for (int h = 0; h < kHalves; ++h) {       // this CTA's 128 rows of every m-half
               unsigned char* sa = sa0 + h * kStageA;
               const int arow = (int)p.row_off[tc.g] + tc.m0 + h * BM + (int)rank * BMH;
               if constexpr (!AT) {   // [rows, K] in memory: one box of 128 rows x 64 K
@@ -532,7 +540,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
             const unsigned sa0 = smem_addr(smem + slot * kStBytes);
             const unsigned sb = sa0 + kStA;
 #pragma unroll
-            for (int h = 0; h < MH; ++h) {
+            for (int h = 0; h < kHalves; ++h) {
               if (MH == 2 && h == 1 && accumulate == 0) {      // first K-block of the tile: the second accumulator must be free too
                 if (!mbar_wait_warp(smem_addr(&bar_acc_empty[1]), empty_parity, abort_flag)) {
                   ok = false;
@@ -595,7 +603,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
       const long long Mg = p.m[tc.g], Ng = p.n[tc.g];
       // tall form: the accumulator of the first m-half is drained (and handed back) before the second
 #pragma unroll 1
-      for (int h = 0; h < MH; ++h) {
+      for (int h = 0; h < kHalves; ++h) {
       const int acc = MH == 2 ? h : facc;
       const int row0 = tc.m0 + h * BM + (int)rank * BMH + q * 32;
       const unsigned taddr = tmem_base + ((unsigned)(q * 32) << 16) + acc * BN + half * (BN / 2);
@@ -1726,12 +1734,18 @@ static sbp_status launch_tc_form(const TcParams* p, cudaStream_t st, int* capaci
   return SBP_OK;
 }
 
-static sbp_status launch_tc(bool tall, bool a_trans, bool b_trans, const TcParams* p, cudaStream_t st, int* capacity) {
-  switch ((tall ? 4 : 0) | (a_trans ? 2 : 0) | (b_trans ? 1 : 0)) {
+enum TcForm { kFormSquare = 0, kFormTall = 1, kFormShort = 2 };
+
+static sbp_status launch_tc(TcForm form, bool a_trans, bool b_trans, const TcParams* p, cudaStream_t st, int* capacity) {
+  switch (4 * form + ((a_trans ? 2 : 0) | (b_trans ? 1 : 0))) {
     case 0: return launch_tc_form<0, 0, 1>(p, st, capacity);
     case 1: return launch_tc_form<0, 1, 1>(p, st, capacity);
     case 2: return launch_tc_form<1, 0, 1>(p, st, capacity);
     case 3: return launch_tc_form<1, 1, 1>(p, st, capacity);
+    case 8: return launch_tc_form<0, 0, 3>(p, st, capacity);
+    case 9: return launch_tc_form<0, 1, 3>(p, st, capacity);
+    case 10: return launch_tc_form<1, 0, 3>(p, st, capacity);
+    case 11: return launch_tc_form<1, 1, 3>(p, st, capacity);
     case 4: return launch_tc_form<0, 0, 2>(p, st, capacity);
     case 5: return launch_tc_form<0, 1, 2>(p, st, capacity);
     case 6: return launch_tc_form<1, 0, 2>(p, st, capacity);
@@ -2232,8 +2246,8 @@ sbp_status launch_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, void* 
   FormChoice form{false, 0, 0.0};
   if (!xf && tiles_tall > 0 && tiles_sq <= 0x1fffffffLL) {
     int cap_sq = 0, cap_tall = 0;
-    sbp_status qs = launch_tc(false, plan.a_trans, plan.b_trans, nullptr, st, &cap_sq);
-    if (qs == SBP_OK) qs = launch_tc(true, plan.a_trans, plan.b_trans, nullptr, st, &cap_tall);
+    sbp_status qs = launch_tc(kFormSquare, plan.a_trans, plan.b_trans, nullptr, st, &cap_sq);
+    if (qs == SBP_OK) qs = launch_tc(kFormTall, plan.a_trans, plan.b_trans, nullptr, st, &cap_tall);
     if (qs != SBP_OK) return qs;
     const int forced = forced_form();
     OperandRows rows = operand_rows(plan);
@@ -2341,16 +2355,16 @@ sbp_status launch_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, void* 
   *taken = true;
   if (tiles == 0) return SBP_OK;
 
-  if (!form.walk_tall) return launch_tc(false, plan.a_trans, plan.b_trans, &p, st, nullptr);
+  if (!form.walk_tall) return launch_tc(kb_tile <= kShortBlocks ? kFormShort : kFormSquare, plan.a_trans, plan.b_trans, &p, st, nullptr);
   // tall form over the first walked tiles, then (mixed run) the square form over the halves of the rest
   const int tall_tiles = std::min(form.tall_tiles, tiles);
   p.total_tiles = tall_tiles;
-  sbp_status rs = launch_tc(true, plan.a_trans, plan.b_trans, &p, st, nullptr);
+  sbp_status rs = launch_tc(kFormTall, plan.a_trans, plan.b_trans, &p, st, nullptr);
   if (rs != SBP_OK || tall_tiles == tiles) return rs;
   p.tile_first = tall_tiles;
   p.half_split = 1;
   p.total_tiles = 2 * (tiles - tall_tiles);
-  return launch_tc(false, plan.a_trans, plan.b_trans, &p, st, nullptr);
+  return launch_tc(kFormSquare, plan.a_trans, plan.b_trans, &p, st, nullptr);
 }
 
 sbp_status read_and_clear_tc_timeout(bool* timed_out) {
