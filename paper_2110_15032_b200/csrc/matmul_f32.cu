@@ -107,7 +107,6 @@ __global__ void __launch_bounds__(kThreads, TM == 8 ? 2 : 3) matmul_f32_kernel(c
   const int splits = P.splits, slice = (int)(blockIdx.x % (unsigned)splits);
   const long long M = p.m[g], N = p.n[g];
   const long long m0 = (long long)blockIdx.y * BM, n0 = (long long)(blockIdx.x / (unsigned)splits) * BN;
-  SBP_PDL_WAIT();
   if (m0 >= M || n0 >= N) return;                  // the whole cluster
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int ty = (warp >> 1) * 4 + (lane >> 3), tx = (warp & 1) * 8 + (lane & 7);
@@ -150,6 +149,7 @@ __global__ void __launch_bounds__(kThreads, TM == 8 ? 2 : 3) matmul_f32_kernel(c
 #pragma unroll
     for (int j = 0; j < TN / 2; ++j) acc[i][j] = 0ull;
 
+  SBP_PDL_WAIT();                                  // everything up to here overlaps the kernel before this one
 #pragma unroll
   for (int st = 0; st < kStages - 1; ++st) {
     if (st < iters) load_next(st);
