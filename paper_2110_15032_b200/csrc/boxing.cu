@@ -171,12 +171,11 @@ __global__ void __launch_bounds__(256) box_tile_kernel(const __grid_constant__ B
 }
 
 // The same tasks over data that is not 16-byte aligned (boxing_shift.h).  us in a row of calls, element-wise tiles /
-// this: fp32 [1021, 1537] over three shards S(0) -> S(1) 12.0 / 3.0, P(sum) -> S(1) 15.5 / 7.9, S(0) -> B 6.2 / 5.3;
-// fp32 [4096, 4097] over two S(0) -> S(1) 87 / 20 (6.6 TB/s); bf16 [4001, 3333] over eight S(1) -> S(0) 62 / 11,
-// P(sum) -> B 97 / 71.
+// this: fp32 [1021, 1537] over three shards S(0) -> S(1) 12.0 / 3.0, P(sum) -> S(1) 15.5 / 6.4, S(0) -> B 6.2 / 5.5;
+// fp32 [4096, 4097] over two S(0) -> S(1) 87 / 20 (6.6 TB/s); bf16 [4001, 3333] over eight S(1) -> S(0) 62 / 11;
+// bf16 [7894, 4206] over eight P(sum) -> S(1) 280 with every source shifted, 126 with the sums shifted (floor 91).
 template <int ESZ, int OP, int KB>
-__global__ void __launch_bounds__(256, shift_ctas(OP, KB, ESZ)) box_shift_kernel(const __grid_constant__ BoxParams p) {
-  constexpr int J = OP == OP_COPY ? kShiftJCopy : shift_j(KB, ESZ);
+__global__ void __launch_bounds__(256, shift_ctas(OP, KB)) box_shift_kernel(const __grid_constant__ BoxParams p) {
   SBP_PDL_RELEASE();
   const unsigned tile = blockIdx.x / (unsigned)p.ntasks;
   const int t = (int)(blockIdx.x - tile * (unsigned)p.ntasks);
@@ -195,8 +194,8 @@ __global__ void __launch_bounds__(256, shift_ctas(OP, KB, ESZ)) box_shift_kernel
   v.dm = g.Pd * cs;  v.di = p.M * v.dm;  v.dx = g.Na_d * v.di;  v.d0 = g.aoff_d * v.di + g.boff_d * cs;
   const bool all = p.mode == MODE_GATHER || p.mode == MODE_REDUCE_B;
   const ShiftPlan sp{p.shift_team_log2, p.shift_chunks};
-  if (OP == OP_COPY) shift_unit<ESZ, OP, J, KB>(v, sp, tile, p.src, p.src_bytes, s, 1, 1, all ? p.dst : p.dst + d, all ? p.n_dst : 1);
-  else shift_unit<ESZ, OP, J, KB>(v, sp, tile, p.src, p.src_bytes, 0, 1, p.k, all ? p.dst : p.dst + d, all ? p.n_dst : 1);
+  if constexpr (OP == OP_COPY) shift_copy_unit<ESZ>(v, sp, tile, p.src[s], p.src_bytes[s], all ? p.dst : p.dst + d, all ? p.n_dst : 1);
+  else shift_reduce_unit<ESZ, OP, shift_j(KB), KB>(v, sp, tile, p.src, p.src_bytes, 0, 1, p.k, all ? p.dst : p.dst + d, all ? p.n_dst : 1);
 }
 
 // row = c / per_row and the remainder; 32-bit arithmetic whenever both fit (a 64-bit division
@@ -579,7 +578,7 @@ static sbp_status make_plan(const sbp_tensor* src, const sbp_tensor* dst, int ds
       ok = ok && (reinterpret_cast<uintptr_t>(p.dst[q]) - reinterpret_cast<uintptr_t>(p.dst[0])) % 16 == 0;
     if (pl->op != OP_COPY)
       for (int r = 1; r < k; ++r) ok = ok && (reinterpret_cast<uintptr_t>(p.src[r]) - reinterpret_cast<uintptr_t>(p.src[0])) % 16 == 0;
-    const ShiftPlan sp = shift_plan(seg_bytes_max, pl->op == OP_COPY ? kShiftJCopy : shift_j(shift_kb(k), p.esz));
+    const ShiftPlan sp = pl->op == OP_COPY ? shift_plan_copy(seg_bytes_max) : shift_plan_reduce(seg_bytes_max, shift_j(shift_kb(k)));
     const long long units = nseg_max * sp.chunks, teams = 256 >> sp.team_log2;
     const long long tiles = std::max(1LL, (units + teams - 1) / teams);
     if (ok && units < 0x7fffff00LL && tiles * pl->ntasks <= 0x7fffffffLL) {

@@ -114,8 +114,7 @@ __device__ __forceinline__ void disjoint_sources(const DisjointParams& p, int d,
 
 // The same tasks over data that is not 16-byte aligned (boxing_shift.h).
 template <int ESZ, int OP, int KB>
-__global__ void __launch_bounds__(256, shift_ctas(OP, KB, ESZ)) box_disjoint_shift_kernel(const __grid_constant__ DisjointParams p) {
-  constexpr int J = OP == OP_COPY ? kShiftJCopy : shift_j(KB, ESZ);
+__global__ void __launch_bounds__(256, shift_ctas(OP, KB)) box_disjoint_shift_kernel(const __grid_constant__ DisjointParams p) {
   SBP_PDL_RELEASE();
   const unsigned tile = blockIdx.x / (unsigned)p.ntasks;
   int s, d;
@@ -132,7 +131,9 @@ __global__ void __launch_bounds__(256, shift_ctas(OP, KB, ESZ)) box_disjoint_shi
   int first = s, stride = 1, count = 1;
   if (OP != OP_COPY) disjoint_sources(p, d, &first, &stride, &count);
   const bool all = p.mode == DJ_TO_ALL || p.mode == DJ_REDUCE_ALL;
-  shift_unit<ESZ, OP, J, KB>(v, ShiftPlan{p.shift_team_log2, p.shift_chunks}, tile, p.src, p.src_bytes, first, stride, count, all ? p.dst : p.dst + d, all ? p.n_dst : 1);
+  const ShiftPlan sp{p.shift_team_log2, p.shift_chunks};
+  if constexpr (OP == OP_COPY) shift_copy_unit<ESZ>(v, sp, tile, p.src[first], p.src_bytes[first], all ? p.dst : p.dst + d, all ? p.n_dst : 1);
+  else shift_reduce_unit<ESZ, OP, shift_j(KB), KB>(v, sp, tile, p.src, p.src_bytes, first, stride, count, all ? p.dst : p.dst + d, all ? p.n_dst : 1);
 }
 
 template <typename V, int OP>
@@ -466,7 +467,7 @@ sbp_status boxing_disjoint(const sbp_tensor* src, sbp_tensor* dst, int dst_shard
   for (int q = 1; q < p.n_dst; ++q)
     shift = shift && (reinterpret_cast<uintptr_t>(p.dst[q]) - reinterpret_cast<uintptr_t>(p.dst[0])) % 16 == 0;
   if (shift) {
-    const ShiftPlan sp = shift_plan(seg_bytes_max, op == OP_COPY ? kShiftJCopy : shift_j(shift_kb(ks), esz));
+    const ShiftPlan sp = op == OP_COPY ? shift_plan_copy(seg_bytes_max) : shift_plan_reduce(seg_bytes_max, shift_j(shift_kb(ks)));
     const long long units = nseg_max * sp.chunks, teams = 256 >> sp.team_log2;
     const long long tiles = std::max(1LL, (units + teams - 1) / teams);
     if (units < 0x7fffff00LL && tiles * p.ntasks <= 0x7fffffffLL) {

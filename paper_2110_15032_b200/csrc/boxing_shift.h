@@ -9,6 +9,7 @@
 // destination.  The 16 source bytes under one lie in two aligned source vectors (one when the two sides agree
 // modulo 16), which are read and shifted together.  The up to 31 bytes before the first and after the last such
 // vector are moved element by element, one element a thread, beside the vectors.
+// A reduction adds up the sources' own aligned vectors and shifts the sums (shift_reduce_unit).
 // Values and their order are those of the plain kernels, so the results are the same bits.
 #pragma once
 
@@ -42,16 +43,35 @@ struct ShiftPlan {
 // Vectors per thread and sources at once: 4 to 8 loads of 16 bytes in flight whatever the transform.
 constexpr int kShiftJCopy = 4;
 constexpr int shift_kb(int k) { return k <= 2 ? 2 : (k == 3 ? 3 : 4); }
-constexpr int shift_j(int kb, int esz) { return (kb == 2 ? 2 : 1) * (esz == 4 ? 2 : 1); }
-// CTAs per SM the registers are held to (fp32 [4096, 4097] P(sum) -> S(1) over two shards 50 us with two, 68 with
-// three, 76 with four; bf16 [4001, 3333] over eight 84 us with four, 94 with three, 124 with two).
-constexpr int shift_ctas(int op, int kb, int esz) { return op == OP_COPY || esz != 4 ? 4 : (kb == 2 ? 2 : 3); }
+constexpr int shift_j(int kb) { return kb == 2 ? 4 : 2; }
+// CTAs per SM the registers are held to (P(sum) -> S(1), us with 2 / 3 / 4: bf16 [1429, 4727] over two shards, four
+// vectors a thread, 13.2 / 11.9, with two vectors and four CTAs 12.0; bf16 [1249, 6988] over three 19.4 / 19.7 / 17.3; bf16
+// [7894, 4206] over eight 169 / 136 / 128).
+constexpr int shift_ctas(int op, int kb) { return op != OP_COPY && kb == 2 ? 3 : 4; }
 
-inline ShiftPlan shift_plan(long long seg_bytes, int J) {
+// How the segments of a copy are dealt out.
+inline ShiftPlan shift_plan_copy(long long seg_bytes) {
+  constexpr int J = kShiftJCopy;
   const long long nv = seg_bytes / 16 > 0 ? seg_bytes / 16 : 1;
   int t = 4;      // at least as many threads as elements beside the whole vectors
   while (t < 8 && (J << t) < nv) ++t;
   return ShiftPlan{t, (unsigned)((nv + ((long long)J << t) - 1) / ((long long)J << t))};
+}
+
+// The same for a reduction: the team whose lanes are busiest on segments of this length, the largest of equals.
+inline ShiftPlan shift_plan_reduce(long long seg_bytes, int J) {
+  const long long nv = seg_bytes / 16 + 2;      // destination vectors, incomplete ones included
+  ShiftPlan best{4, 1};
+  double best_use = 0.0;
+  for (int t = 4; t <= 8; ++t) {
+    const long long T = 1 << t, W = T < 32 ? T : 32, per = (long long)J * (T / W) * (W - 1), chunks = (nv + per - 1) / per;
+    const double use = (double)nv / (double)(chunks * J * T);
+    if (use >= best_use) {
+      best_use = use;
+      best = ShiftPlan{t, (unsigned)chunks};
+    }
+  }
+  return best;
 }
 
 template <int ESZ>
@@ -84,12 +104,11 @@ __device__ __forceinline__ uint4 shift_pair(uint4 a, uint4 b, unsigned sh) {
   return make_uint4(w0, w1, w2, w3);
 }
 
-// One unit of a task (a team of threads and J vectors for each of them).  Sources first, first + stride, ...
-// (`count` of them, one for a copy), KB at a time, combined in that order; those of a reduction have one size and
-// bases that agree modulo 16.  The result goes to n_dst destinations whose bases agree modulo 16.
-template <int ESZ, int OP, int J, int KB>
-__device__ __forceinline__ void shift_unit(const SegView& g, ShiftPlan sp, unsigned tile, const char* const* src, const long long* src_bytes,
-                                           int first, int stride, int count, char* const* dst, int n_dst) {
+// One unit of a copy (a team of threads and J vectors for each of them) to n_dst destinations whose bases agree modulo 16.
+template <int ESZ>
+__device__ __forceinline__ void shift_copy_unit(const SegView& g, ShiftPlan sp, unsigned tile, const char* src, long long src_bytes,
+                                                char* const* dst, int n_dst) {
+  constexpr int J = kShiftJCopy;
   using E = typename ShiftElem<ESZ>::type;
   const unsigned T = 1u << sp.team_log2, tl = threadIdx.x & (T - 1);
   const unsigned unit = tile * (256u >> sp.team_log2) + (threadIdx.x >> sp.team_log2);
@@ -108,12 +127,12 @@ __device__ __forceinline__ void shift_unit(const SegView& g, ShiftPlan sp, unsig
   long long nbody = (g.seg_bytes - head) >> 4;
   // where the source stands under a whole vector; a first or last one whose aligned source pair would reach beyond
   // the tensor joins the elements before or after the whole vectors
-  const unsigned sh = (unsigned)((reinterpret_cast<unsigned long long>(src[first]) + (unsigned long long)(so + head)) & 15);
+  const unsigned sh = (unsigned)((reinterpret_cast<unsigned long long>(src) + (unsigned long long)(so + head)) & 15);
   if (sh != 0 && nbody > 0 && so + head - (int)sh < 0) {
     head += 16;
     --nbody;
   }
-  if (sh != 0 && nbody > 0 && so + head - (int)sh + nbody * 16 + 16 > src_bytes[first]) --nbody;
+  if (sh != 0 && nbody > 0 && so + head - (int)sh + nbody * 16 + 16 > src_bytes) --nbody;
   const int tail = (int)(g.seg_bytes - head - nbody * 16);
   const long long v0 = (long long)c * (J * T) + tl;
   // this thread's elements before the first and after the last whole vector (offsets in the segment, -1: none)
@@ -126,111 +145,181 @@ __device__ __forceinline__ void shift_unit(const SegView& g, ShiftPlan sp, unsig
 
   SBP_PDL_WAIT();      // the kernel before this one has finished
 
-  if constexpr (OP == OP_COPY) {
-    const char* base = src[first] + so;
-    E ev[2];
+  const char* base = src + so;
+  E ev[2];
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      ev[e] = E{};
-      if (eo[e] >= 0 && SBP_GUARD(base + eo[e], ESZ)) ev[e] = *reinterpret_cast<const E*>(base + eo[e]);
-    }
-    const char* at = base + head + v0 * 16;
-    uint4 val[J];
-    if (sh == 0) {
-#pragma unroll
-      for (int j = 0; j < J; ++j)
-        if (in[j] && SBP_GUARD(at + j * T * 16, 16)) val[j] = ld_stream(reinterpret_cast<const uint4*>(at + j * T * 16));
-    } else {
-      uint4 a[J], b[J];
-#pragma unroll
-      for (int j = 0; j < J; ++j)
-        if (in[j] && SBP_GUARD(at - sh + j * T * 16, 32)) {
-          a[j] = ld_keep(at - sh + j * T * 16);
-          b[j] = ld_keep(at - sh + j * T * 16 + 16);
-        }
-#pragma unroll
-      for (int j = 0; j < J; ++j)
-        if (in[j]) val[j] = shift_pair<ESZ>(a[j], b[j], sh);
-    }
-    for (int r = 0; r < n_dst; ++r) {
-      char* d = dst[r] + dofs;
-#pragma unroll
-      for (int j = 0; j < J; ++j)
-        if (in[j] && SBP_GUARD(d + head + (v0 + j * T) * 16, 16)) st_stream(reinterpret_cast<uint4*>(d + head + (v0 + j * T) * 16), val[j]);
-#pragma unroll
-      for (int e = 0; e < 2; ++e)
-        if (eo[e] >= 0 && SBP_GUARD(d + eo[e], ESZ)) *reinterpret_cast<E*>(d + eo[e]) = ev[e];
-    }
-  } else {
-    using L = typename Lanes<OP, uint4>::type;
-    using LE = typename Lanes<OP, E>::type;
-    L acc[J];
-    const long long off = so + head + v0 * 16;
-    for (int r0 = 0; r0 < count; r0 += KB) {
-      uint4 a[KB][J], b[KB][J];
-#pragma unroll
-      for (int i = 0; i < KB; ++i) {
-        if (r0 + i >= count) continue;
-        const char* at = src[first + (r0 + i) * stride] + off;
-#pragma unroll
-        for (int j = 0; j < J; ++j) {
-          if (!in[j]) continue;
-          if (sh == 0) {
-            if (SBP_GUARD(at + j * T * 16, 16)) a[i][j] = ld_stream(reinterpret_cast<const uint4*>(at + j * T * 16));
-          } else if (SBP_GUARD(at - sh + j * T * 16, 32)) {
-            a[i][j] = ld_keep(at - sh + j * T * 16);
-            b[i][j] = ld_keep(at - sh + j * T * 16 + 16);
-          }
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < KB; ++i) {
-        if (r0 + i >= count) continue;
-#pragma unroll
-        for (int j = 0; j < J; ++j) {
-          if (!in[j]) continue;
-          L t;
-          t.load(sh != 0 ? shift_pair<ESZ>(a[i][j], b[i][j], sh) : a[i][j]);
-          if (r0 + i == 0) acc[j] = t;
-          else combine<OP>(acc[j], t);
-        }
-      }
-    }
-    uint4 val[J];
+  for (int e = 0; e < 2; ++e) {
+    ev[e] = E{};
+    if (eo[e] >= 0 && SBP_GUARD(base + eo[e], ESZ)) ev[e] = *reinterpret_cast<const E*>(base + eo[e]);
+  }
+  const char* at = base + head + v0 * 16;
+  uint4 val[J];
+  if (sh == 0) {
 #pragma unroll
     for (int j = 0; j < J; ++j)
-      if (in[j]) val[j] = count > 0 ? acc[j].store() : make_uint4(0u, 0u, 0u, 0u);
-    for (int r = 0; r < n_dst; ++r) {
-      char* d = dst[r] + dofs + head + v0 * 16;
+      if (in[j] && SBP_GUARD(at + j * T * 16, 16)) val[j] = ld_stream(reinterpret_cast<const uint4*>(at + j * T * 16));
+  } else {
+    uint4 a[J], b[J];
 #pragma unroll
-      for (int j = 0; j < J; ++j)
-        if (in[j] && SBP_GUARD(d + j * T * 16, 16)) st_stream(reinterpret_cast<uint4*>(d + j * T * 16), val[j]);
+    for (int j = 0; j < J; ++j)
+      if (in[j] && SBP_GUARD(at - sh + j * T * 16, 32)) {
+        a[j] = ld_keep(at - sh + j * T * 16);
+        b[j] = ld_keep(at - sh + j * T * 16 + 16);
+      }
+#pragma unroll
+    for (int j = 0; j < J; ++j)
+      if (in[j]) val[j] = shift_pair<ESZ>(a[j], b[j], sh);
+  }
+  for (int r = 0; r < n_dst; ++r) {
+    char* d = dst[r] + dofs;
+#pragma unroll
+    for (int j = 0; j < J; ++j)
+      if (in[j] && SBP_GUARD(d + head + (v0 + j * T) * 16, 16)) st_stream(reinterpret_cast<uint4*>(d + head + (v0 + j * T) * 16), val[j]);
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+      if (eo[e] >= 0 && SBP_GUARD(d + eo[e], ESZ)) *reinterpret_cast<E*>(d + eo[e]) = ev[e];
+  }
+}
+
+// Bytes lo .. hi - 1 of the 16 at p, the others zero.
+template <int ESZ>
+__device__ __forceinline__ uint4 load_part(const char* p, int lo, int hi) {
+  using E = typename ShiftElem<ESZ>::type;
+  unsigned long long w[2] = {0ull, 0ull};
+#pragma unroll 1
+  for (int e = lo; e < hi; e += ESZ) {
+    if (!SBP_GUARD(p + e, ESZ)) continue;
+    const E x = *reinterpret_cast<const E*>(p + e);
+    unsigned long long v;
+    if constexpr (ESZ == 8) v = ((unsigned long long)x.y << 32) | x.x;
+    else v = x;
+    if (e < 8) w[0] |= v << (8 * e);
+    else w[1] |= v << (8 * (e - 8));
+  }
+  return make_uint4((unsigned)w[0], (unsigned)(w[0] >> 32), (unsigned)w[1], (unsigned)(w[1] >> 32));
+}
+
+// One vector of a unit whose sources reach beyond their tensors, which hold `bytes` bytes: 16 at `at`.
+template <int ESZ, int OP>
+__device__ __noinline__ uint4 shift_part(const char* const* src, int first, int stride, int count, long long at, long long bytes) {
+  const int lo = at < 0 ? (int)-at : 0, hi = at + 16 <= bytes ? 16 : (int)(bytes - at);
+  typename Lanes<OP, uint4>::type acc, t;
+#pragma unroll 1
+  for (int r = 0; r < count; ++r) {
+    t.load(load_part<ESZ>(src[first + r * stride] + at, lo, hi));
+    if (r == 0) acc = t;
+    else combine<OP>(acc, t);
+  }
+  return count > 0 ? acc.store() : make_uint4(0u, 0u, 0u, 0u);
+}
+
+template <int ESZ>
+__device__ __noinline__ void store_part(char* p, uint4 v, int lo, int hi) {
+  using E = typename ShiftElem<ESZ>::type;
+  const unsigned long long w[2] = {((unsigned long long)v.y << 32) | v.x, ((unsigned long long)v.w << 32) | v.z};
+#pragma unroll 1
+  for (int e = lo; e < hi; e += ESZ) {
+    const unsigned long long x = e < 8 ? w[0] >> (8 * e) : w[1] >> (8 * (e - 8));
+    if (!SBP_GUARD(p + e, ESZ)) continue;
+    if constexpr (ESZ == 8) *reinterpret_cast<E*>(p + e) = make_uint2((unsigned)x, (unsigned)(x >> 32));
+    else *reinterpret_cast<E*>(p + e) = (E)x;
+  }
+}
+
+// One unit of a reduction (a team of threads and J vectors for each of them).  Sources first, first + stride, ...
+// (`count` of them) have one size and bases that agree modulo 16, and are combined KB at a time in that order, as aligned
+// vectors of the SOURCES: each is loaded once, by one lane.  The sums are shifted, not the sources: a lane gets the vector
+// after its own from the next lane, so of W lanes W - 1 store.  Incomplete vectors at a segment's ends are summed like the
+// others and stored element by element.  The result goes to n_dst destinations whose bases agree modulo 16.
+template <int ESZ, int OP, int J, int KB>
+__device__ __forceinline__ void shift_reduce_unit(const SegView& g, ShiftPlan sp, unsigned tile, const char* const* src, const long long* src_bytes,
+                                           int first, int stride, int count, char* const* dst, int n_dst) {
+  const unsigned T = 1u << sp.team_log2, tl = threadIdx.x & (T - 1), W = T < 32 ? T : 32, lw = tl & (W - 1);
+  const unsigned unit = tile * (256u >> sp.team_log2) + (threadIdx.x >> sp.team_log2);
+  unsigned seg = sp.chunks == 1 ? unit : unit / sp.chunks;
+  const unsigned c = unit - seg * sp.chunks;
+  const bool live = seg < g.nseg;              // a warp may hold teams on both sides of the end
+  if (!live) seg = 0;
+  unsigned x = 0, ia = seg, m = 0;
+  if (!g.flat) {
+    const unsigned q = seg / (unsigned)g.M;
+    m = seg - q * (unsigned)g.M;
+    x = q / (unsigned)g.la;
+    ia = q - x * (unsigned)g.la;
+  }
+  const long long so = g.s0 + x * g.sx + ia * g.si + m * g.sm, dofs = g.d0 + x * g.dx + ia * g.di + m * g.dm;
+  // the segment begins `lead` bytes into the first aligned vector of the destination; the source bytes under that
+  // vector begin `sh` into an aligned vector of the source, `from` bytes from the source's base
+  const int lead = (int)((reinterpret_cast<unsigned long long>(dst[0]) + (unsigned long long)dofs) & 15);
+  const unsigned sh = (unsigned)((reinterpret_cast<unsigned long long>(src[first]) + (unsigned long long)(so - lead)) & 15);
+  const long long from = so - lead - sh, end = lead + g.seg_bytes, bytes = src_bytes[first];
+  const long long nv = live ? (end + 15) >> 4 : 0;
+  const unsigned per_sub = W - 1, subs = T / W;
+  const long long v0 = (long long)(c * J * subs + tl / W) * per_sub + lw;      // and subs * per_sub further for each j
+  const int step = (int)(subs * per_sub);
+  const long long at0 = from + v0 * 16;        // where source vector 0's bytes begin
+  bool in[J], part[J];
+#pragma unroll
+  for (int j = 0; j < J; ++j) {
+    const long long at = at0 + (long long)j * step * 16;
+    const bool wanted = v0 + (long long)j * step < nv + (sh != 0 ? 1 : 0) && at < bytes && at + 16 > 0;
+    in[j] = wanted && at >= 0 && at + 16 <= bytes;
+    part[j] = wanted && !in[j];
+  }
+
+  SBP_PDL_WAIT();      // the kernel before this one has finished
+
+  uint4 val[J];
+  using L = typename Lanes<OP, uint4>::type;
+  L acc[J];
+  for (int r0 = 0; r0 < count; r0 += KB) {
+    uint4 a[KB][J];
+#pragma unroll
+    for (int i = 0; i < KB; ++i) {
+      if (r0 + i >= count) continue;
+      const char* base = src[first + (r0 + i) * stride] + at0;
+#pragma unroll
+      for (int j = 0; j < J; ++j) {
+        a[i][j] = make_uint4(0u, 0u, 0u, 0u);
+        if (in[j] && SBP_GUARD(base + j * step * 16, 16)) a[i][j] = ld_keep(base + j * step * 16);
+      }
     }
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      if (eo[e] < 0) continue;
-      LE acc;
-      for (int r0 = 0; r0 < count; r0 += KB) {
-        E xs[KB];
+    for (int i = 0; i < KB; ++i) {
+      if (r0 + i >= count) continue;
 #pragma unroll
-        for (int i = 0; i < KB; ++i) {
-          xs[i] = E{};
-          const char* at = r0 + i < count ? src[first + (r0 + i) * stride] + so + eo[e] : nullptr;
-          if (at && SBP_GUARD(at, ESZ)) xs[i] = *reinterpret_cast<const E*>(at);
-        }
-#pragma unroll
-        for (int i = 0; i < KB; ++i) {
-          if (r0 + i >= count) continue;
-          LE t;
-          t.load(xs[i]);
-          if (r0 + i == 0) acc = t;
-          else combine<OP>(acc, t);
-        }
+      for (int j = 0; j < J; ++j) {
+        L t;
+        t.load(a[i][j]);
+        if (r0 + i == 0) acc[j] = t;
+        else combine<OP>(acc[j], t);
       }
-      const E val = count > 0 ? acc.store() : E{};
-      for (int r = 0; r < n_dst; ++r) {
-        E* d = reinterpret_cast<E*>(dst[r] + dofs + eo[e]);
-        if (SBP_GUARD(d, ESZ)) *d = val;
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < J; ++j) val[j] = count > 0 ? acc[j].store() : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+  for (int j = 0; j < J; ++j)
+    if (part[j]) val[j] = shift_part<ESZ, OP>(src, first, stride, count, at0 + (long long)j * step * 16, bytes);
+#pragma unroll
+  for (int j = 0; j < J; ++j) {
+    uint4 next;                                // the vector after this lane's
+    next.x = __shfl_down_sync(0xffffffffu, val[j].x, 1, W);
+    next.y = __shfl_down_sync(0xffffffffu, val[j].y, 1, W);
+    next.z = __shfl_down_sync(0xffffffffu, val[j].z, 1, W);
+    next.w = __shfl_down_sync(0xffffffffu, val[j].w, 1, W);
+    if (sh != 0) val[j] = shift_pair<ESZ>(val[j], next, sh);
+  }
+  for (int r = 0; r < n_dst; ++r) {
+    char* d = dst[r] + dofs - lead;
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+      const long long v = v0 + (long long)j * step, o = v * 16;
+      if (v >= nv || lw == per_sub) continue;
+      if (o >= lead && o + 16 <= end) {
+        if (SBP_GUARD(d + o, 16)) st_stream(reinterpret_cast<uint4*>(d + o), val[j]);
+      } else {
+        store_part<ESZ>(d + o, val[j], o < lead ? (int)(lead - o) : 0, o + 16 <= end ? 16 : (int)(end - o));
       }
     }
   }
