@@ -559,9 +559,9 @@ constexpr int kBwdVecs = 4;      // vectors in flight per thread
 template <typename T, int VEC>
 __global__ void __launch_bounds__(kThreads) xent_backward_kernel(const __grid_constant__ XentBwdParams p) {
   const int team = 1 << p.team_log2, tid = threadIdx.x & (team - 1);      // short rows: several to a CTA
-  const long long row = (long long)blockIdx.x * (kThreads >> p.team_log2) + (threadIdx.x >> p.team_log2);
+  const long long row = (long long)(gridDim.x - 1 - blockIdx.x) * (kThreads >> p.team_log2) + (threadIdx.x >> p.team_log2);
   if (row >= p.rows) return;
-  const int shard = blockIdx.z;
+  const int shard = p.k - 1 - (int)blockIdx.z;
   long long c_start, c_len;
   split_range(p.classes, p.k, shard, (int64_t*)&c_start, (int64_t*)&c_len);
   const T* z = reinterpret_cast<const T*>(p.logits[shard]) + row * p.lpitch[shard];
