@@ -56,7 +56,7 @@ __device__ __forceinline__ void task_geometry(const BoxParams& p, int s, int d, 
 // V: vector type moved by one thread access.  OP: BoxOp.  J: vectors per thread.
 // KT: compile-time number of source shards of a reduction (0 = read p.k at run time).
 template <typename V, int OP, int J, int KT>
-__global__ void __launch_bounds__(256) box_tile_kernel(const __grid_constant__ BoxParams p) {
+__device__ __forceinline__ void box_tile(const BoxParams& p) {
   // Task index varies fastest: CTAs that run together then touch the same rows of every shard
   // (whole DRAM pages) instead of one column stripe of one shard.  The grid is below 2^31 tiles,
   // so this is 32-bit arithmetic.
@@ -170,12 +170,27 @@ __global__ void __launch_bounds__(256) box_tile_kernel(const __grid_constant__ B
   }
 }
 
+template <typename V, int OP, int J, int KT>
+__global__ void __launch_bounds__(256) box_tile_kernel(const __grid_constant__ BoxParams p) { box_tile<V, OP, J, KT>(p); }
+
+// One transform for each blockIdx.y: the groups of a two-axis placement, planned alike.
+constexpr int kBoxGroups = 4;
+struct BoxGroups {
+  BoxParams p[kBoxGroups];
+  unsigned grid[kBoxGroups];
+};
+
+template <typename V, int OP, int J, int KT>
+__global__ void __launch_bounds__(256) box_tile_groups_kernel(const __grid_constant__ BoxGroups g) {
+  if (blockIdx.x < g.grid[blockIdx.y]) box_tile<V, OP, J, KT>(g.p[blockIdx.y]);
+}
+
 // The same tasks over data that is not 16-byte aligned (boxing_shift.h).  us in a row of calls, element-wise tiles /
 // this: fp32 [1021, 1537] over three shards S(0) -> S(1) 12.0 / 3.0, P(sum) -> S(1) 15.5 / 6.4, S(0) -> B 6.2 / 5.5;
 // fp32 [4096, 4097] over two S(0) -> S(1) 87 / 20 (6.6 TB/s); bf16 [4001, 3333] over eight S(1) -> S(0) 62 / 11;
 // bf16 [7894, 4206] over eight P(sum) -> S(1) 280 with every source shifted, 126 with the sums shifted (floor 91).
 template <int ESZ, int OP, int KB>
-__global__ void __launch_bounds__(256, shift_ctas(OP, KB)) box_shift_kernel(const __grid_constant__ BoxParams p) {
+__device__ __forceinline__ void box_shift(const BoxParams& p) {
   SBP_PDL_RELEASE();
   const unsigned tile = blockIdx.x / (unsigned)p.ntasks;
   const int t = (int)(blockIdx.x - tile * (unsigned)p.ntasks);
@@ -196,6 +211,14 @@ __global__ void __launch_bounds__(256, shift_ctas(OP, KB)) box_shift_kernel(cons
   const ShiftPlan sp{p.shift_team_log2, p.shift_chunks};
   if constexpr (OP == OP_COPY) shift_copy_unit<ESZ>(v, sp, tile, p.src[s], p.src_bytes[s], all ? p.dst : p.dst + d, all ? p.n_dst : 1);
   else shift_reduce_unit<ESZ, OP, shift_j(KB), KB>(v, sp, tile, p.src, p.src_bytes, 0, 1, p.k, all ? p.dst : p.dst + d, all ? p.n_dst : 1);
+}
+
+template <int ESZ, int OP, int KB>
+__global__ void __launch_bounds__(256, shift_ctas(OP, KB)) box_shift_kernel(const __grid_constant__ BoxParams p) { box_shift<ESZ, OP, KB>(p); }
+
+template <int ESZ, int OP, int KB>
+__global__ void __launch_bounds__(256, shift_ctas(OP, KB)) box_shift_groups_kernel(const __grid_constant__ BoxGroups g) {
+  if (blockIdx.x < g.grid[blockIdx.y]) box_shift<ESZ, OP, KB>(g.p[blockIdx.y]);
 }
 
 // row = c / per_row and the remainder; 32-bit arithmetic whenever both fit (a 64-bit division
@@ -341,6 +364,8 @@ struct Plan {
   int ntasks;
   long long grid;
   bool shift;       // unaligned data in 16-byte vectors (boxing_shift.h)
+  const BoxGroups* groups;      // several transforms planned like this one, `ngroups` of them, in one launch; null: this one
+  int ngroups;
 };
 
 static int pick_vector_bytes(const BoxParams& p, const sbp_tensor* src, const sbp_tensor* dst, int k) {
@@ -371,7 +396,8 @@ static int pick_vector_bytes(const BoxParams& p, const sbp_tensor* src, const sb
 template <typename V, int OP, int J, int KT>
 static void launch_tile(const Plan& pl, cudaStream_t st) {
   SBP_BOUNDS_UPLOAD(st);
-  launch_dependent(box_tile_kernel<V, OP, J, KT>, dim3((unsigned)pl.grid), dim3(256), 0, st, pl.p);   // errors are picked up by the caller's cudaGetLastError
+  if (pl.groups) launch_dependent(box_tile_groups_kernel<V, OP, J, KT>, dim3((unsigned)pl.grid, (unsigned)pl.ngroups), dim3(256), 0, st, *pl.groups);
+  else launch_dependent(box_tile_kernel<V, OP, J, KT>, dim3((unsigned)pl.grid), dim3(256), 0, st, pl.p);   // errors are picked up by the caller's cudaGetLastError
 }
 
 template <typename V, int OP, int J>
@@ -412,14 +438,19 @@ static void launch_v_f32(const Plan& pl, cudaStream_t st) {
 constexpr int kJCopy = 4;
 constexpr int kJReduce = 2;
 
+template <int ESZ, int OP, int KB>
+static void launch_shift_kb(const Plan& pl, cudaStream_t st) {
+  if (pl.groups) launch_dependent(box_shift_groups_kernel<ESZ, OP, KB>, dim3((unsigned)pl.grid, (unsigned)pl.ngroups), dim3(256), 0, st, *pl.groups);
+  else launch_dependent(box_shift_kernel<ESZ, OP, KB>, dim3((unsigned)pl.grid), dim3(256), 0, st, pl.p);
+}
+
 template <int ESZ, int OP>
 static void launch_shift_k(const Plan& pl, cudaStream_t st) {
-  const dim3 g((unsigned)pl.grid), b(256);
   switch (OP == OP_COPY ? 1 : shift_kb(pl.p.k)) {
-    case 1: launch_dependent(box_shift_kernel<ESZ, OP, 1>, g, b, 0, st, pl.p); break;
-    case 2: if constexpr (OP != OP_COPY) launch_dependent(box_shift_kernel<ESZ, OP, 2>, g, b, 0, st, pl.p); break;
-    case 3: if constexpr (OP != OP_COPY) launch_dependent(box_shift_kernel<ESZ, OP, 3>, g, b, 0, st, pl.p); break;
-    default: if constexpr (OP != OP_COPY) launch_dependent(box_shift_kernel<ESZ, OP, 4>, g, b, 0, st, pl.p); break;
+    case 1: launch_shift_kb<ESZ, OP, 1>(pl, st); break;
+    case 2: if constexpr (OP != OP_COPY) launch_shift_kb<ESZ, OP, 2>(pl, st); break;
+    case 3: if constexpr (OP != OP_COPY) launch_shift_kb<ESZ, OP, 3>(pl, st); break;
+    default: if constexpr (OP != OP_COPY) launch_shift_kb<ESZ, OP, 4>(pl, st); break;
   }
 }
 
@@ -438,11 +469,23 @@ static void launch_shift(const Plan& pl, cudaStream_t st) {
   }
 }
 
+static void launch_planned(const Plan& pl, cudaStream_t stream) {
+  if (pl.shift) return launch_shift(pl, stream);
+  switch (pl.op) {
+    case OP_COPY: launch_v<OP_COPY, kJCopy>(pl, stream); break;
+    case OP_SUM_F32: launch_v_f32<OP_SUM_F32, kJReduce>(pl, stream); break;
+    case OP_MAX_F32: launch_v_f32<OP_MAX_F32, kJReduce>(pl, stream); break;
+    case OP_SUM_BF16: launch_v<OP_SUM_BF16, kJReduce>(pl, stream); break;
+    case OP_MAX_BF16: launch_v<OP_MAX_BF16, kJReduce>(pl, stream); break;
+  }
+}
+
 static sbp_status make_plan(const sbp_tensor* src, const sbp_tensor* dst, int dst_shard, Plan* pl) {
   const int k = placement_k(src);
   const sbp_sig ss = src->sbp[0], ds = dst->sbp[0];
   BoxParams& p = pl->p;
   p = BoxParams{};
+  pl->groups = nullptr;
   p.k = k;
   p.esz = elem_size(src->dtype);
   p.one_dst = dst_shard >= 0 ? 1 : 0;
@@ -663,6 +706,52 @@ static bool is_partial(sbp_sig s) { return s.kind == SBP_PARTIAL_SUM || s.kind =
 // dry: every check is made (descriptors, signature pair, sizes) and nothing is launched.
 static sbp_status boxing_one_axis(const sbp_tensor* src, sbp_tensor* dst, int dst_shard, void* cuda_stream, bool dry);
 
+// The groups' transforms (already checked), up to kBoxGroups in one launch where they are planned alike: a call then
+// costs one launch, not one per group (P(sum) -> B of three groups of 1 x 952 over two 8.4 us with three launches, 4.7 so; of two of 500 x 1024 over four 10.0, 8.6).
+struct TwoAxisBatch {
+  cudaStream_t stream;
+  int n = 0;
+  sbp_tensor s[kBoxGroups], d[kBoxGroups];
+  Plan first;
+  BoxGroups groups;
+
+  sbp_status add(const sbp_tensor* src, const sbp_tensor* dst) {
+    if (numel(src) == 0) return SBP_OK;
+    Plan pl;
+    sbp_status st = make_plan(src, dst, -1, &pl);
+    if (st != SBP_OK) return st;
+    if (pl.p.mode == MODE_SCATTER_P || pl.pitched || g_copy_engine.load() == 2)
+      return (st = flush()) != SBP_OK ? st : boxing_one_axis(src, const_cast<sbp_tensor*>(dst), -1, stream, false);
+    const bool alike = n > 0 && n < kBoxGroups && pl.op == first.op && pl.vbytes == first.vbytes && pl.shift == first.shift &&
+                       pl.p.mode == first.p.mode && pl.p.k == first.p.k;
+    if (n > 0 && !alike && (st = flush()) != SBP_OK) return st;
+    if (n == 0) first = pl;
+    first.grid = std::max(first.grid, pl.grid);
+    s[n] = *src;
+    d[n] = *dst;
+    groups.p[n] = pl.p;
+    groups.grid[n++] = (unsigned)pl.grid;
+    return SBP_OK;
+  }
+
+  sbp_status flush() {
+    if (n == 0) return SBP_OK;
+    SBP_BOUNDS_RESET();
+    for (int i = 0; i < n; ++i) {
+      SBP_BOUNDS_TENSOR(&s[i]);
+      SBP_BOUNDS_TENSOR(&d[i]);
+    }
+    first.groups = n > 1 ? &groups : nullptr;
+    first.ngroups = n;
+    n = 0;
+    launch_planned(first, stream);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_fail(e, "boxing launch");
+    count_launch();
+    return SBP_OK;
+  }
+};
+
 static sbp_status boxing_2d(const sbp_tensor* src, sbp_tensor* dst, void* cuda_stream, bool dry) {
   sbp_status st = check_tensor_nd(src, "src", true);
   if (st != SBP_OK) return st;
@@ -683,6 +772,7 @@ static sbp_status boxing_2d(const sbp_tensor* src, sbp_tensor* dst, void* cuda_s
   if (ch0 && ch1)
     return fail(SBP_ERR_UNSUPPORTED, "change one placement axis per boxing call (two calls for both)");
 
+  TwoAxisBatch batch{static_cast<cudaStream_t>(cuda_stream)};
   sbp_tensor s1 = *src, d1 = *dst;
   s1.pdims = d1.pdims = 1;
   s1.pshape[1] = d1.pshape[1] = 1;
@@ -702,10 +792,10 @@ static sbp_status boxing_2d(const sbp_tensor* src, sbp_tensor* dst, void* cuda_s
         s1.local[j] = src->local[i * k1 + j];
         d1.local[j] = dst->local[i * k1 + j];
       }
-      st = boxing_one_axis(&s1, &d1, -1, cuda_stream, dry);
+      st = dry ? boxing_one_axis(&s1, &d1, -1, cuda_stream, true) : batch.add(&s1, &d1);
       if (st != SBP_OK) return st;
     }
-    return SBP_OK;
+    return batch.flush();
   }
   // axis 0 changes, axis 1 keeps signature c
   const sbp_sig c = src->sbp[1];
@@ -730,10 +820,10 @@ static sbp_status boxing_2d(const sbp_tensor* src, sbp_tensor* dst, void* cuda_s
       s1.local[i] = src->local[i * k1 + j];
       d1.local[i] = dst->local[i * k1 + j];
     }
-    st = boxing_one_axis(&s1, &d1, -1, cuda_stream, dry);
+    st = dry ? boxing_one_axis(&s1, &d1, -1, cuda_stream, true) : batch.add(&s1, &d1);
     if (st != SBP_OK) return st;
   }
-  return SBP_OK;
+  return batch.flush();
 }
 
 static sbp_status boxing_one_axis(const sbp_tensor* src, sbp_tensor* dst, int dst_shard, void* cuda_stream, bool dry) {
@@ -817,19 +907,7 @@ static sbp_status boxing_one_axis(const sbp_tensor* src, sbp_tensor* dst, int ds
   const bool want_bulk = engine == 2;
   if (!done && pl.op == OP_COPY && want_bulk && pl.vbytes == 16 && !pl.pitched)
     done = launch_bulk_copy(pl.p, pl.ntasks, stream);
-  if (!done && pl.shift) {
-    launch_shift(pl, stream);
-    done = true;
-  }
-  if (!done) {
-    switch (pl.op) {
-      case OP_COPY: launch_v<OP_COPY, kJCopy>(pl, stream); break;
-      case OP_SUM_F32: launch_v_f32<OP_SUM_F32, kJReduce>(pl, stream); break;
-      case OP_MAX_F32: launch_v_f32<OP_MAX_F32, kJReduce>(pl, stream); break;
-      case OP_SUM_BF16: launch_v<OP_SUM_BF16, kJReduce>(pl, stream); break;
-      case OP_MAX_BF16: launch_v<OP_MAX_BF16, kJReduce>(pl, stream); break;
-    }
-  }
+  if (!done) launch_planned(pl, stream);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "boxing launch");
   count_launch();
