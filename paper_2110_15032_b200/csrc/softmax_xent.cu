@@ -184,7 +184,7 @@ __device__ __forceinline__ int to_boundary(const T* z, long long n) {
 // element by element, one element a thread, and what lies between as aligned vectors; the loads of the next chunk
 // are issued before the current one is reduced.  (Unaligned rows element by element throughout: fp32 [256, 100003]
 // over four shards 33 us, backward 76; as here 25 and 35: 0.62 and 0.89 of the copy bandwidth.)
-template <typename Chunk>
+template <typename Chunk, bool UNITS>
 __device__ __forceinline__ void walk_span(const typename Chunk::T* z, long long n, int tid, int team, float& m, float& s) {
   using T = typename Chunk::T;
   constexpr int VEC = Chunk::VEC;
@@ -200,26 +200,54 @@ __device__ __forceinline__ void walk_span(const typename Chunk::T* z, long long 
     const float x = static_cast<float>(*lone);
     if (x != -INFINITY) merge(m, s, x, 1.f);
   }
+  // UNITS: inside the loop s counts in units of 2^e, e the integer above m log2 e.  Without, the rounding of m log2 e
+  // scales what a thread has so far once more with every chunk, which only many threads to a row average out.
+  float e = 0.f;
+  if constexpr (UNITS) {
+    e = ceilf(m * kLog2e);      // -inf as long as there is nothing
+    if (m != -INFINITY) s *= ex2(fmaf(m, kLog2e, -e));
+  }
   for (long long off = 0; off < nv; off += step) {
     const bool more = off + step < nv;
     if (more) nxt.load(zv + (off + step) * VEC, nv - off - step, tid, team);
     const float cm = cur.max();
     if (cm != -INFINITY) {
       const float mm = fmaxf(m, cm);
-      const float neg = -mm * kLog2e;
-      const float carried = (m == -INFINITY) ? 0.f : s * ex2(fmaf(m, kLog2e, neg));
-      s = carried + cur.expsum(neg);
+      if constexpr (UNITS) {
+        const float ee = ceilf(mm * kLog2e);
+        const float carried = e == ee ? s : (e == -INFINITY ? 0.f : s * ex2(e - ee));
+        s = carried + cur.expsum(-ee);
+        e = ee;
+      } else {
+        const float neg = -mm * kLog2e;
+        const float carried = (m == -INFINITY) ? 0.f : s * ex2(fmaf(m, kLog2e, neg));
+        s = carried + cur.expsum(neg);
+      }
       m = mm;
     }
     if (more) cur = nxt;
   }
+  if (UNITS && m != -INFINITY) s *= ex2(fmaf(-m, kLog2e, e));
 }
 
 // Many rows: a team of 1 << team_log2 threads takes a whole row, shard after shard, and finishes it -- no partials,
 // no second kernel.  Taken from 740 rows on (five CTAs an SM), with the team that spreads the rows over the device
 // once.  (us, partial + combine kernels / this: fp32 [4096, 1003] over two shards 24 / 8.5, bf16 [1000, 30000] over
-// four 39 / 24.)
+// four 39 / 24.)  The team grows with the row, so that a thread adds up no more elements than in the partial kernel;
+// rows that take more than 128 threads so are left to that kernel, which is as fast for them or faster (fp32 [2000,
+// 134217] over four 254 us with teams of 64, 168 there; [3000, 30000] over two 73 either way; bf16 [2000, 100000] over
+// two 92 with teams of 256, 75 there).  Relative error of the row sums with 64 threads and 9000 fp32 classes 3.3e-7, with no
+// bound on the team's share and without UNITS 3e-6 to 9e-6, in the partial kernel 3e-7 to 4e-7.
 constexpr long long kRowsForTeams = 740;
+
+// log2 of the team for this many rows and classes in vectors of `vec` elements; 0: the partial kernel
+static int team_for(long long rows, long long classes, int vec) {
+  if (rows < kRowsForTeams) return 0;
+  int t = rows < 2 * kRowsForTeams ? 7 : (rows < 4 * kRowsForTeams ? 6 : 5);
+  const long long most = (long long)kMaxChunksPerCta * kLoadsPerThread * vec;
+  while (t <= 7 && (classes >> t) > most) ++t;
+  return t <= 7 ? t : 0;
+}
 
 template <typename Chunk>
 __global__ void __launch_bounds__(kThreads) xent_rows_kernel(const __grid_constant__ XentParams p, const __grid_constant__ XentCombineParams c,
@@ -236,7 +264,7 @@ __global__ void __launch_bounds__(kThreads) xent_rows_kernel(const __grid_consta
       long long c_start, c_len;
       split_range(p.classes, p.k, r, (int64_t*)&c_start, (int64_t*)&c_len);
       const T* z = reinterpret_cast<const T*>(p.logits[r]) + row * p.pitch[r];
-      if (c_len > 0) walk_span<Chunk>(z, c_len, tl, team, m, s);
+      if (c_len > 0) walk_span<Chunk, true>(z, c_len, tl, team, m, s);
       if (tl == 0 && y >= c_start && y < c_start + c_len && SBP_GUARD(z + (y - c_start), sizeof(T))) t = static_cast<float>(z[y - c_start]);
     }
   }
@@ -283,7 +311,7 @@ __global__ void __launch_bounds__(kThreads) xent_partial_kernel(const __grid_con
   SBP_PDL_WAIT();
 
   float m = -INFINITY, s = 0.f;
-  if (n > 0) walk_span<Chunk>(z, n, tid, kThreads, m, s);
+  if (n > 0) walk_span<Chunk, false>(z, n, tid, kThreads, m, s);
 
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
@@ -699,8 +727,8 @@ sbp_status sbp_softmax_xent(const sbp_tensor* logits, const sbp_tensor* labels, 
   SBP_BOUNDS_TENSOR(row_sum);
   SBP_BOUNDS_ADD(ws, 3 * (size_t)parts * rows * sizeof(float));
   SBP_BOUNDS_UPLOAD(stream);
-  if (rows >= kRowsForTeams) {
-    const int team_log2 = rows < 2 * kRowsForTeams ? 7 : (rows < 4 * kRowsForTeams ? 6 : 5);
+  const int team_log2 = team_for(rows, classes, logits->dtype == SBP_BF16 ? 8 : 4);
+  if (team_log2 > 0) {
     const int per_cta = kThreads >> team_log2;
     const dim3 g((unsigned)((rows + per_cta - 1) / per_cta));
     if (logits->dtype == SBP_BF16) launch_dependent(xent_rows_kernel<ChunkBF16>, g, dim3(kThreads), 0, stream, p, c, team_log2);
