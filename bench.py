@@ -175,22 +175,21 @@ NCU_TRAFFIC = {
     # profiles/box_kernels_sweep_bf16_8192x8192_k4.md (full size)
     "P(sum)->B": 1024.0e6, "P(sum)->S(0)": 647.0e6, "P(sum)->S(1)": 648.1e6, "S(0)->B": 614.1e6,
     "S(0)->S(1)": 219.2e6, "S(1)->S(0)": 217.3e6, "B->S(1)": 217.8e6,
-    # profiles/xent_partial_bf16_512x1048576_k8.md (full size)
-    "softmax-xent on bf16 logits (partial + combine)": 1077.2e6,
-    "softmax-xent backward (softmax - onehot, S(1))": 2099.7e6,
-    # profiles/matmul_tc_classifier_bf16_512x512x1048576_k8.md (full size)
-    "classifier GEMM (B,S(1))->S(1), bf16 logits": 2104.3e6,
-    "classifier GEMM fused with softmax-xent (no logits stored)": 1127.8e6 + 50.5e6,
-    "classifier GEMM fused with the softmax-xent backward (grad S(1), no logits stored)": 2103.8e6,
-    # profiles/matmul_tc_mlp_bf16_8192x4096x16384_k8.md (full size; a mixed run is the sum of its two launches)
-    "MLP GEMM1 (B,S(1))->S(1) + GeLU": 1003.3e6,
-    "MLP GEMM2 (S(1),S(0))->P(sum), bf16 partials": 914.0e6,
-    "MLP GEMM2 fused (S(1),S(0))->B": 1195.4e6 + 194.6e6,
-    "MLP GEMM1 with W1 stored transposed (SBP_TRANS_W) + GeLU": 1003.4e6,
-    "MLP GEMM2 fused (S(1),S(0))->B with W2 stored transposed (SBP_TRANS_W)": 1195.2e6 + 194.4e6,
-    "DP layer backward dW = X^T dY, (S(1),S(0))->S(0) fused": 872.6e6,
-    "DP layer backward dW = X^T dY, (S(1),S(0))->B fused (8 replicas written)": 1774.9e6,
-    "DP layer backward dX = dY W^T, (S(0),B)->S(0)": 747.1e6 + 206.0e6,
+    # the softmax and tensor-core MatMul kernels have changed since profiles/xent_partial_..., matmul_tc_classifier_... and
+    # matmul_tc_mlp_... were captured
+    "softmax-xent on bf16 logits (partial + combine)": None,
+    "softmax-xent backward (softmax - onehot, S(1))": None,
+    "classifier GEMM (B,S(1))->S(1), bf16 logits": None,
+    "classifier GEMM fused with softmax-xent (no logits stored)": None,
+    "classifier GEMM fused with the softmax-xent backward (grad S(1), no logits stored)": None,
+    "MLP GEMM1 (B,S(1))->S(1) + GeLU": None,
+    "MLP GEMM2 (S(1),S(0))->P(sum), bf16 partials": None,
+    "MLP GEMM2 fused (S(1),S(0))->B": None,
+    "MLP GEMM1 with W1 stored transposed (SBP_TRANS_W) + GeLU": None,
+    "MLP GEMM2 fused (S(1),S(0))->B with W2 stored transposed (SBP_TRANS_W)": None,
+    "DP layer backward dW = X^T dY, (S(1),S(0))->S(0) fused": None,
+    "DP layer backward dW = X^T dY, (S(1),S(0))->B fused (8 replicas written)": None,
+    "DP layer backward dX = dY W^T, (S(0),B)->S(0)": None,
     # profiles/extras_bf16_8192x8192_p4_and_embedding_fp32_4194304x128_batch16384_k8.md (full size)
     "S(0)->P(sum) bf16 [8192,8192] k=4": 619.4e6,
     "B->P(sum) bf16 [8192,8192] k=4": 611.7e6,
@@ -201,15 +200,13 @@ NCU_TRAFFIC = {
     "disjoint placements: P(sum)[4] -> S(0)[8] bf16 [8192,8192]": 616.9e6,
     "disjoint placements: P(sum)[4] -> B[2] bf16 [8192,8192]": 752.2e6,
     "disjoint placements: S(0)[4] -> P(sum)[8] bf16 [8192,8192]": 1015.0e6 + 216.1e6,
-    # profiles/embedding_fused_fp32_config5_full_size_and_quarter_batch.md (full size, one-pass DRAM counters)
-    "embedding fused gather -> B (8 replicas written)": 7308.8e6,
-    "embedding fused gather -> B (replicas aliased, 1 write)": 1096.1e6,
+    # the gather kernel has changed since profiles/embedding_fused_fp32_... was captured
+    "embedding fused gather -> B (8 replicas written)": None,
+    "embedding fused gather -> B (replicas aliased, 1 write)": None,
 }
-# The commits whose kernels the captures above were taken on (the tensor-core MatMul lines were
-# taken again after the kernel got its tall and mixed forms; the other kernels have not changed
-# since the first).  A kernel that changes afterwards gets its entry set to None (or recaptured)
-# in the same commit: a stale figure is worse than none.
-NCU_TRAFFIC_CAPTURED_AT = "a61a16e (boxing, softmax, embedding to several replicas); 073ea77 (matmul_tc_kernel); 68937c6 (embedding_rows_kernel)"
+# The commit whose kernels the captures above were taken on.  A kernel that changes afterwards gets its entry set to None
+# (or recaptured): a stale figure is worse than none.
+NCU_TRAFFIC_CAPTURED_AT = "a61a16e (boxing)"
 
 
 def ncu_traffic(name):
