@@ -1774,7 +1774,8 @@ struct FormChoice {
 // What the copy engine needs for the rows of 128 bytes that a CTA loads per K-block, us: 64 bytes a clock, and a
 // row that starts off a 128-byte boundary of memory is two requests (a [5696 x 2280]^T [5696 x 632] product took
 // 44.7 us where [5696 x 2304]^T [5696 x 640] took 28.1).  A long product of such pitches wants wide tiles; the first
-// K-blocks only fill the ring.
+// K-blocks only fill the ring.  Operands whose rows lie along K do not pay it: the next K-block finds the other half of the
+// line in L2 (dX of [6000 x 4000] by [2000 x 4000], both pitches misaligned: 72.8 us, 79.5 where the square form paid it).
 struct OperandRows {
   double a = 1.0e-3, b = 1.0e-3;      // us per row
   // time of kb K-blocks beyond `per_kb` each, which they take otherwise
@@ -1787,8 +1788,8 @@ static OperandRows operand_rows(const MatmulPlan& p) {
   OperandRows r;
   for (int s = 0; s < p.nseg; ++s) {
     if ((!p.chain && s >= p.ngroups) || p.kseg[s] == 0) continue;
-    if (p.lda[s] % 64 != 0 || reinterpret_cast<uintptr_t>(p.a[s]) % 128 != 0) r.a = 1.9e-3;
-    if (p.ldb[s] % 64 != 0 || reinterpret_cast<uintptr_t>(p.b[s]) % 128 != 0) r.b = 1.9e-3;
+    if (p.a_trans && (p.lda[s] % 64 != 0 || reinterpret_cast<uintptr_t>(p.a[s]) % 128 != 0)) r.a = 1.9e-3;
+    if (!p.b_trans && (p.ldb[s] % 64 != 0 || reinterpret_cast<uintptr_t>(p.b[s]) % 128 != 0)) r.b = 1.9e-3;
   }
   return r;
 }
