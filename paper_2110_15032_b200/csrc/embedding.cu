@@ -453,8 +453,8 @@ struct EmbBwdParams {
 // 16 KB per CTA, one CTA for each: consecutive CTAs clear consecutive memory.  (Persistent grids were slower: 2 GB with
 // its scatter 344 us so, 362 us with 10 000 CTAs striding, 405 us with 592.)
 __global__ void __launch_bounds__(256) embedding_zero_kernel(const __grid_constant__ EmbBwdParams p) {
-  SBP_PDL_RELEASE();
   SBP_PDL_WAIT();
+  SBP_PDL_RELEASE();      // not before the wait: the scatter reads the ids ahead of its own
   const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
   float4* g = reinterpret_cast<float4*>(p.grad_table[blockIdx.y]);
   const long long n = p.shard_vecs[blockIdx.y];
@@ -502,7 +502,8 @@ __device__ __forceinline__ void sort_step(unsigned long long (&k)[KPT], unsigned
 // outside the table (sorted last, skipped).  Most of the sort's 36 (45, 55) steps stay inside a thread or a warp: 6
 // at most go through shared memory.  The sorted chunk is then dealt out to teams of `lanes` threads, as many as a
 // row has 16-byte vectors (a power of two, 32 at most), so that short rows leave no lane idle.  Launched as a
-// programmatic dependent of the zero fill: the sort may run under the fill's last CTAs.
+// programmatic dependent of the zero fill, which lets it in only after everything before the fill has finished: the ids
+// may be read and sorted under the fill's last CTAs, the gradient is touched after the wait.
 // Zero fill and scatter, us (floor: gradient written and gradient of the output read once), with a warp to each row
 // and every sort step through shared memory, then as here: [10^6, 64], 213 K lookups (48) 78.8, 57; [2 x 10^6, 16],
 // 426 K lookups (24) 90.5, 44.7; [300 000, 100], 104 K (25) 44, 35; [4 x 10^6, 128], 426 K (347) 375, 344; [50 000,

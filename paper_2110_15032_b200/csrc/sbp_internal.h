@@ -96,6 +96,10 @@ sbp_status cuda_fail(cudaError_t e, const char* what);
 // reads and then writes one buffer must use plain loads.  tests/test_boxing_gpu.py
 // (test_ping_pong_between_two_buffers_without_a_host_sync) rewrites a source between two reads of
 // it with no synchronisation in between.
+// The wait is for the ONE grid before, so the order of the stream rests on a chain: a grid that has finished must itself
+// have waited.  A kernel some of whose grids would wait in no thread (all of its CTAs leave early) is not launched at
+// all, and a kernel whose dependent reads anything ahead of its own wait (the scatter of the embedding gradient reads the
+// ids) releases it only after it has waited itself.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                     Args&&... args) {
