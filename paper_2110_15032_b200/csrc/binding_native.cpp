@@ -174,10 +174,18 @@ struct Call {
 };
 
 #define ENTRY(name) PyObject* py_##name(PyObject*, PyObject* const* args, Py_ssize_t n)
-#define RUN(expr)                       \
-  sbp_status st;                        \
-  Py_BEGIN_ALLOW_THREADS st = (expr);   \
-  Py_END_ALLOW_THREADS return PyLong_FromLong((long)st)
+// Other Python threads run during a library call; the lock is held again however the call ends.
+struct Unlocked {
+  PyThreadState* state = PyEval_SaveThread();
+  ~Unlocked() { PyEval_RestoreThread(state); }
+};
+#define RUN(expr)           \
+  sbp_status st;            \
+  {                         \
+    Unlocked other_threads; \
+    st = (expr);            \
+  }                         \
+  return PyLong_FromLong((long)st)
 #define GUARDED(body)                                \
   try {                                              \
     body                                             \
