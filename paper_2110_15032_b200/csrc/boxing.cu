@@ -189,6 +189,7 @@ __global__ void __launch_bounds__(256) box_tile_groups_kernel(const __grid_const
 // this: fp32 [1021, 1537] over three shards S(0) -> S(1) 12.0 / 3.0, P(sum) -> S(1) 15.5 / 6.4, S(0) -> B 6.2 / 5.5;
 // fp32 [4096, 4097] over two S(0) -> S(1) 87 / 20 (6.6 TB/s); bf16 [4001, 3333] over eight S(1) -> S(0) 62 / 11;
 // bf16 [7894, 4206] over eight P(sum) -> S(1) 280 with every source shifted, 126 with the sums shifted (floor 91).
+// KB: sources of a reduction at once, vectors a thread of a copy.
 template <int ESZ, int OP, int KB>
 __device__ __forceinline__ void box_shift(const BoxParams& p) {
   SBP_PDL_RELEASE();
@@ -209,7 +210,7 @@ __device__ __forceinline__ void box_shift(const BoxParams& p) {
   v.dm = g.Pd * cs;  v.di = p.M * v.dm;  v.dx = g.Na_d * v.di;  v.d0 = g.aoff_d * v.di + g.boff_d * cs;
   const bool all = p.mode == MODE_GATHER || p.mode == MODE_REDUCE_B;
   const ShiftPlan sp{p.shift_team_log2, p.shift_chunks};
-  if constexpr (OP == OP_COPY) shift_copy_unit<ESZ>(v, sp, tile, p.src[s], p.src_bytes[s], all ? p.dst : p.dst + d, all ? p.n_dst : 1);
+  if constexpr (OP == OP_COPY) shift_copy_unit<ESZ, KB>(v, sp, tile, p.src[s], p.src_bytes[s], all ? p.dst : p.dst + d, all ? p.n_dst : 1);
   else shift_reduce_unit<ESZ, OP, shift_j(KB), KB>(v, sp, tile, p.src, p.src_bytes, 0, 1, p.k, all ? p.dst : p.dst + d, all ? p.n_dst : 1);
 }
 
@@ -364,6 +365,7 @@ struct Plan {
   int ntasks;
   long long grid;
   bool shift;       // unaligned data in 16-byte vectors (boxing_shift.h)
+  int copy_j;       // vectors a thread of a shifted copy
   const BoxGroups* groups;      // several transforms planned like this one, `ngroups` of them, in one launch; null: this one
   int ngroups;
 };
@@ -446,11 +448,11 @@ static void launch_shift_kb(const Plan& pl, cudaStream_t st) {
 
 template <int ESZ, int OP>
 static void launch_shift_k(const Plan& pl, cudaStream_t st) {
-  switch (OP == OP_COPY ? 1 : shift_kb(pl.p.k)) {
-    case 1: launch_shift_kb<ESZ, OP, 1>(pl, st); break;
+  switch (OP == OP_COPY ? pl.copy_j : shift_kb(pl.p.k)) {
+    case 1: if constexpr (OP == OP_COPY) launch_shift_kb<ESZ, OP, 1>(pl, st); break;
     case 2: if constexpr (OP != OP_COPY) launch_shift_kb<ESZ, OP, 2>(pl, st); break;
     case 3: if constexpr (OP != OP_COPY) launch_shift_kb<ESZ, OP, 3>(pl, st); break;
-    default: if constexpr (OP != OP_COPY) launch_shift_kb<ESZ, OP, 4>(pl, st); break;
+    default: launch_shift_kb<ESZ, OP, 4>(pl, st); break;
   }
 }
 
@@ -609,19 +611,19 @@ static sbp_status make_plan(const sbp_tensor* src, const sbp_tensor* dst, int ds
   if (p.one_dst) pl->ntasks = (p.mode == MODE_PAIRS || p.mode == MODE_GATHER) ? k : 1;
   p.ntasks = pl->ntasks;
 
-  // Unaligned data: 16-byte vectors of the destination with shifted sources, unless the segments are so short
-  // that their incomplete ends are most of them, the tensor so small that the call is all latency (one element
-  // per thread then has the shorter chain), or buffers that share an offset differ modulo 16.
+  // Unaligned data: 16-byte vectors of the destination with shifted sources where that pays, unless buffers that share
+  // an offset differ modulo 16.
   const long long seg_bytes_max = lb_max * p.C * p.esz;
   pl->shift = false;
-  if (pl->vbytes < 16 && p.mode != MODE_SCATTER_P && src->dtype == dst->dtype && seg_bytes_max >= kShiftMinSegment &&
-      numel(src) >= kShiftMinElements) {
+  pl->copy_j = shift_copy_j(p.esz, p.n_dst, numel(src));
+  if (p.mode != MODE_SCATTER_P && src->dtype == dst->dtype &&
+      shift_pays(pl->op == OP_COPY, p.esz, pl->vbytes, k, p.n_dst, seg_bytes_max, numel(src))) {
     bool ok = true;
     for (int q = 1; q < p.n_dst; ++q)
       ok = ok && (reinterpret_cast<uintptr_t>(p.dst[q]) - reinterpret_cast<uintptr_t>(p.dst[0])) % 16 == 0;
     if (pl->op != OP_COPY)
       for (int r = 1; r < k; ++r) ok = ok && (reinterpret_cast<uintptr_t>(p.src[r]) - reinterpret_cast<uintptr_t>(p.src[0])) % 16 == 0;
-    const ShiftPlan sp = pl->op == OP_COPY ? shift_plan_copy(seg_bytes_max) : shift_plan_reduce(seg_bytes_max, shift_j(shift_kb(k)));
+    const ShiftPlan sp = pl->op == OP_COPY ? shift_plan_copy(seg_bytes_max, pl->copy_j) : shift_plan_reduce(seg_bytes_max, shift_j(shift_kb(k)));
     const long long units = nseg_max * sp.chunks, teams = 256 >> sp.team_log2;
     const long long tiles = std::max(1LL, (units + teams - 1) / teams);
     if (ok && units < 0x7fffff00LL && tiles * pl->ntasks <= 0x7fffffffLL) {
@@ -722,7 +724,7 @@ struct TwoAxisBatch {
     if (st != SBP_OK) return st;
     if (pl.p.mode == MODE_SCATTER_P || pl.pitched || g_copy_engine.load() == 2)
       return (st = flush()) != SBP_OK ? st : boxing_one_axis(src, const_cast<sbp_tensor*>(dst), -1, stream, false);
-    const bool alike = n > 0 && n < kBoxGroups && pl.op == first.op && pl.vbytes == first.vbytes && pl.shift == first.shift &&
+    const bool alike = n > 0 && n < kBoxGroups && pl.op == first.op && pl.vbytes == first.vbytes && pl.shift == first.shift && pl.copy_j == first.copy_j &&
                        pl.p.mode == first.p.mode && pl.p.k == first.p.k;
     if (n > 0 && !alike && (st = flush()) != SBP_OK) return st;
     if (n == 0) first = pl;

@@ -48,7 +48,7 @@ struct DisjointParams {
   int cv_log2, rows_per_tile, ntasks;
   unsigned char pair_s[kMaxPairs], pair_d[kMaxPairs];
   long long src_bytes[SBP_MAX_K];   // 16-byte path for unaligned data (boxing_shift.h)
-  int shift_team_log2;
+  int shift_team_log2, shift_copy_j;
   unsigned shift_chunks;
   // quotient and remainder of each axis by each side's shard count: the balanced split without a division
   long long a_base_s, a_rem_s, a_base_d, a_rem_d, b_base_s, b_rem_s, b_base_d, b_rem_d;
@@ -112,7 +112,8 @@ __device__ __forceinline__ void disjoint_sources(const DisjointParams& p, int d,
   }
 }
 
-// The same tasks over data that is not 16-byte aligned (boxing_shift.h).
+// The same tasks over data that is not 16-byte aligned (boxing_shift.h).  KB: sources of a reduction at once, vectors a
+// thread of a copy.
 template <int ESZ, int OP, int KB>
 __global__ void __launch_bounds__(256, shift_ctas(OP, KB)) box_disjoint_shift_kernel(const __grid_constant__ DisjointParams p) {
   SBP_PDL_RELEASE();
@@ -132,7 +133,7 @@ __global__ void __launch_bounds__(256, shift_ctas(OP, KB)) box_disjoint_shift_ke
   if (OP != OP_COPY) disjoint_sources(p, d, &first, &stride, &count);
   const bool all = p.mode == DJ_TO_ALL || p.mode == DJ_REDUCE_ALL;
   const ShiftPlan sp{p.shift_team_log2, p.shift_chunks};
-  if constexpr (OP == OP_COPY) shift_copy_unit<ESZ>(v, sp, tile, p.src[first], p.src_bytes[first], all ? p.dst : p.dst + d, all ? p.n_dst : 1);
+  if constexpr (OP == OP_COPY) shift_copy_unit<ESZ, KB>(v, sp, tile, p.src[first], p.src_bytes[first], all ? p.dst : p.dst + d, all ? p.n_dst : 1);
   else shift_reduce_unit<ESZ, OP, shift_j(KB), KB>(v, sp, tile, p.src, p.src_bytes, first, stride, count, all ? p.dst : p.dst + d, all ? p.n_dst : 1);
 }
 
@@ -274,11 +275,11 @@ static void launch_disjoint(const DisjointParams& p, int vbytes, long long grid,
 template <int ESZ, int OP>
 static void launch_disjoint_shift_k(const DisjointParams& p, long long grid, cudaStream_t st) {
   const dim3 g((unsigned)grid), b(256);
-  switch (OP == OP_COPY ? 1 : shift_kb(p.ks)) {
-    case 1: launch_dependent(box_disjoint_shift_kernel<ESZ, OP, 1>, g, b, 0, st, p); break;
+  switch (OP == OP_COPY ? p.shift_copy_j : shift_kb(p.ks)) {
+    case 1: if constexpr (OP == OP_COPY) launch_dependent(box_disjoint_shift_kernel<ESZ, OP, 1>, g, b, 0, st, p); break;
     case 2: if constexpr (OP != OP_COPY) launch_dependent(box_disjoint_shift_kernel<ESZ, OP, 2>, g, b, 0, st, p); break;
     case 3: if constexpr (OP != OP_COPY) launch_dependent(box_disjoint_shift_kernel<ESZ, OP, 3>, g, b, 0, st, p); break;
-    default: if constexpr (OP != OP_COPY) launch_dependent(box_disjoint_shift_kernel<ESZ, OP, 4>, g, b, 0, st, p); break;
+    default: launch_dependent(box_disjoint_shift_kernel<ESZ, OP, 4>, g, b, 0, st, p); break;
   }
 }
 
@@ -460,14 +461,15 @@ sbp_status boxing_disjoint(const sbp_tensor* src, sbp_tensor* dst, int dst_shard
   p.tiles_per_task = p.col_tiles * row_tiles;
   long long grid = p.tiles_per_task * p.ntasks;
   // unaligned data in 16-byte vectors, by the rule of the same-placement kernels
-  bool shift = vbytes < 16 && seg_bytes_max >= kShiftMinSegment && numel(src) >= kShiftMinElements;
+  bool shift = shift_pays(op == OP_COPY, esz, vbytes, ks, p.n_dst, seg_bytes_max, numel(src));
+  p.shift_copy_j = shift_copy_j(esz, p.n_dst, numel(src));
   if (op != OP_COPY)
     for (int r = 1; r < ks; ++r)
       shift = shift && (reinterpret_cast<uintptr_t>(src->local[r]) - reinterpret_cast<uintptr_t>(src->local[0])) % 16 == 0;
   for (int q = 1; q < p.n_dst; ++q)
     shift = shift && (reinterpret_cast<uintptr_t>(p.dst[q]) - reinterpret_cast<uintptr_t>(p.dst[0])) % 16 == 0;
   if (shift) {
-    const ShiftPlan sp = op == OP_COPY ? shift_plan_copy(seg_bytes_max) : shift_plan_reduce(seg_bytes_max, shift_j(shift_kb(ks)));
+    const ShiftPlan sp = op == OP_COPY ? shift_plan_copy(seg_bytes_max, p.shift_copy_j) : shift_plan_reduce(seg_bytes_max, shift_j(shift_kb(ks)));
     const long long units = nseg_max * sp.chunks, teams = 256 >> sp.team_log2;
     const long long tiles = std::max(1LL, (units + teams - 1) / teams);
     if (units < 0x7fffff00LL && tiles * p.ntasks <= 0x7fffffffLL) {

@@ -28,33 +28,62 @@ struct SegView {
   long long d0, dx, di, dm;
 };
 
-// Segments shorter than this (bytes) are mostly incomplete vectors: they keep the element-wise kernels.
-constexpr long long kShiftMinSegment = 64;
-// Tensors below this many elements too: bf16 [60, 8001] takes 2.0-3.1 us either way, fp32 [100, 777] 1.2 us element
-// by element and 1.6-2.9 in shifted vectors.
-constexpr long long kShiftMinElements = 400000;
-
 // How the segments of a transform are dealt out: teams of 1 << team_log2 threads (16 to 256), `chunks` units per segment.
 struct ShiftPlan {
   int team_log2;
   unsigned chunks;
 };
 
-// Vectors per thread and sources at once: 4 to 8 loads of 16 bytes in flight whatever the transform.
-constexpr int kShiftJCopy = 4;
+// Vectors per thread and sources at once: 4 to 8 loads of 16 bytes in flight whatever the transform.  A copy that fills the
+// device only once or twice, or that writes each value to eight places, takes one vector a thread: more CTAs, whose stores
+// begin earlier (us, four vectors / one: bf16 [60, 8001] S(0) -> B over three 2.6 / 1.8, fp32 [129, 65, 97] over six 6.8 / 4.4,
+// over eight 9.1 / 5.5, bf16 [17, 300001] S(1) -> B over eight 18.7 / 13.3; fp32 [4096, 4096] over three 42 / 82, [3000, 3001]
+// over six 41 / 45).  elements: of the tensor; n_dst: destinations of each value (0 or 1: one).
+inline int shift_copy_j(int esz, int n_dst, long long elements) {
+  const long long bytes = elements * esz;
+  return n_dst >= 8 || (n_dst >= 4 && bytes < 6400000) || (n_dst > 1 && bytes < 2000000) ? 1 : 4;
+}
 constexpr int shift_kb(int k) { return k <= 2 ? 2 : (k == 3 ? 3 : 4); }
 constexpr int shift_j(int kb) { return kb == 2 ? 4 : 2; }
+// When a transform of unaligned data takes this path, from both paths timed on the device over some 700 transforms of 14
+// shapes (us, element-wise tiles / this path):
+//   copies      segments of 32 elements and more, 64 where several destinations take four vectors a thread: i64 [200001, 33]
+//               over three S(1) -> S(0), segments of 11, 38 / 144, [129, 65, 97] over eight S(0) -> S(2), of 12, 8.2 / 20; over
+//               three, of 32, 11.3 / 7.5
+//   reductions  of up to four sources the same; of more, 48 elements: bf16 [50, 200, 301] over eight P(sum) -> S(2), of 38,
+//               33 / 45, over six, of 50, 31 / 27.  More than four sources whose segments are long keep the tiles' loads in
+//               flight (one position, all sources) up to 1.2 M elements: [513, 1025] over eight P(sum) -> B 4.4 / 7.1, [1021,
+//               1537] bf16 11.8 / 9.7; and fp32 sums that go to several destinations at any size: [200001, 33] 65 / 71
+//   where the tiles move several elements an access they are as good: up to 1.2 M bf16 or fp32 elements ([60, 8001] bf16
+//               P(sum) -> B over three 2.6 / 3.8), and 8 bytes an access are enough for i64 gathers to few replicas unless the rows are short and many
+//               ([1021, 1537] over three S(0) -> B 7.4 / 8.1, S(1) -> B 12 / 9.4)
+// Below 400 000 elements (500 000 of more than four sources) a call is all latency: bf16 [60, 8001] takes 2.0-3.1 us either way, fp32 [100, 777] 1.2 us element
+// by element and 1.6-2.9 in shifted vectors.
+// vbytes: what the tiles would move per access.
+inline bool shift_pays(bool copy, int esz, int vbytes, int k, int n_dst, long long seg_bytes, long long elements) {
+  const long long seg = seg_bytes / esz;
+  const bool few = copy || k <= 4, small = elements < 1200000;
+  if (vbytes >= 16 || elements < (few ? 400000 : 500000) || seg < (few ? 32 : 48)) return false;
+  if (esz < 8 && vbytes > esz && small) return false;
+  if (copy) {
+    if (n_dst > 1 && seg < 64 && shift_copy_j(esz, n_dst, elements) > 1) return false;
+    if (esz < 8 || n_dst <= 1 || n_dst >= 8) return true;
+    return n_dst >= 4 ? seg < (1 << 17) || elements < 800000 : seg < 2048 || (seg < (1 << 17) && elements >= 2000000);
+  }
+  if (k <= 4 || seg < 4096) return true;
+  return !small && !(esz == 4 && n_dst > 1);
+}
+
 // CTAs per SM the registers are held to (P(sum) -> S(1), us with 2 / 3 / 4: bf16 [1429, 4727] over two shards, four
 // vectors a thread, 13.2 / 11.9, with two vectors and four CTAs 12.0; bf16 [1249, 6988] over three 19.4 / 19.7 / 17.3; bf16
 // [7894, 4206] over eight 169 / 136 / 128).
 constexpr int shift_ctas(int op, int kb) { return op != OP_COPY && kb == 2 ? 3 : 4; }
 
 // How the segments of a copy are dealt out.
-inline ShiftPlan shift_plan_copy(long long seg_bytes) {
-  constexpr int J = kShiftJCopy;
+inline ShiftPlan shift_plan_copy(long long seg_bytes, int J) {
   const long long nv = seg_bytes / 16 > 0 ? seg_bytes / 16 : 1;
   int t = 4;      // at least as many threads as elements beside the whole vectors
-  while (t < 8 && (J << t) < nv) ++t;
+  while (t < 8 && ((long long)J << t) < nv) ++t;
   return ShiftPlan{t, (unsigned)((nv + ((long long)J << t) - 1) / ((long long)J << t))};
 }
 
@@ -105,10 +134,9 @@ __device__ __forceinline__ uint4 shift_pair(uint4 a, uint4 b, unsigned sh) {
 }
 
 // One unit of a copy (a team of threads and J vectors for each of them) to n_dst destinations whose bases agree modulo 16.
-template <int ESZ>
+template <int ESZ, int J>
 __device__ __forceinline__ void shift_copy_unit(const SegView& g, ShiftPlan sp, unsigned tile, const char* src, long long src_bytes,
                                                 char* const* dst, int n_dst) {
-  constexpr int J = kShiftJCopy;
   using E = typename ShiftElem<ESZ>::type;
   const unsigned T = 1u << sp.team_log2, tl = threadIdx.x & (T - 1);
   const unsigned unit = tile * (256u >> sp.team_log2) + (threadIdx.x >> sp.team_log2);
