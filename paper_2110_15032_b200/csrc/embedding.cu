@@ -11,6 +11,7 @@
 // lookups; all id loads, then all row loads, are issued before the first store.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <atomic>
 
 #include "bounds_check.h"
@@ -530,7 +531,7 @@ __global__ void __launch_bounds__(256, 3) embedding_backward_kernel(const __grid
       if (first + i < p.n_lookups) {
         const long long id = SBP_GUARD(p.ids + first + i, 8) ? __ldg(p.ids + first + i) : -1;
         if (id >= 0 && id < p.rows) k[r] = ((unsigned long long)id << kShift) | (unsigned)i;
-        else if (p.oob && SBP_GUARD(p.oob, 4)) atomicAdd(p.oob, 1);
+        else if (p.oob && blockIdx.y == 0 && SBP_GUARD(p.oob, 4)) atomicAdd(p.oob, 1);
       }
     }
 #pragma unroll
@@ -542,8 +543,8 @@ __global__ void __launch_bounds__(256, 3) embedding_backward_kernel(const __grid
     __syncthreads();
     if (!waited) SBP_PDL_WAIT();          // the gradient has been cleared from here on
     waited = true;
-    // runs of equal ids -> one atomic row add each
-    for (long long cb = 0; cb < p.vpr; cb += lanes) {
+    // runs of equal ids -> one atomic row add each; long rows are dealt out to the CTAs of grid.y, 32 vectors at a time
+    for (long long cb = (long long)blockIdx.y * lanes; cb < p.vpr; cb += (long long)gridDim.y * lanes) {
       const long long col = cb + tl;
       const bool active = col < p.vpr;
       long long cur = -1;
@@ -755,7 +756,12 @@ extern "C" sbp_status sbp_embedding_backward(const sbp_tensor* grad_out, const s
     int chunk = 1024;
     while (chunk > 256 && (chunk * p.vpr > 8192 || p.n_lookups < chunk * 222LL)) chunk /= 2;
     const long long chunks = (p.n_lookups + chunk - 1) / chunk;
-    const dim3 sb((unsigned)(chunks < 148 * 8 ? chunks : 148 * 8)), b(256);
+    // Few chunks of long rows: several CTAs sort a chunk each for itself and take their columns of it, so that the
+    // device is full three CTAs deep (us,
+    // one CTA a chunk / so: [20000, 1000], 3000 lookups 93 / 25; [2000, 8192], 500 lookups 609 / 20; [100, 40000], 64 lookups
+    // 2436 / 15).
+    const long long passes = (p.vpr + p.lanes - 1) / p.lanes, split = std::min(passes, std::max(1LL, 444 / chunks));
+    const dim3 sb((unsigned)(chunks < 148 * 8 ? chunks : 148 * 8), (unsigned)split), b(256);
     if (chunk == 1024) e = launch_dependent(embedding_backward_kernel<1024>, sb, b, 0, stream, p);
     else if (chunk == 512) e = launch_dependent(embedding_backward_kernel<512>, sb, b, 0, stream, p);
     else e = launch_dependent(embedding_backward_kernel<256>, sb, b, 0, stream, p);
