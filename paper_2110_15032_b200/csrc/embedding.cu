@@ -225,6 +225,7 @@ __global__ void __launch_bounds__(256, 4) embedding_rows_kernel(const __grid_con
     V val[J];
 #pragma unroll
     for (int j = 0; j < J; ++j) {
+      if (j * 256u >= pieces) break;                // short rows leave most of a chunk's steps empty
       const unsigned f = j * 256 + threadIdx.x;
       val[j] = zero_vec<V>();
       if (f >= pieces) continue;
@@ -238,6 +239,7 @@ __global__ void __launch_bounds__(256, 4) embedding_rows_kernel(const __grid_con
       V* o = reinterpret_cast<V*>(p.out[q]) + out0;
 #pragma unroll
       for (int j = 0; j < J; ++j) {
+        if (j * 256u >= pieces) break;
         const unsigned f = j * 256 + threadIdx.x;
         if (f < pieces && SBP_GUARD(o + f, sizeof(V))) __stcs(o + f, p.canon_neg_zero ? canon<V, ESZ>(val[j]) : val[j]);
       }
