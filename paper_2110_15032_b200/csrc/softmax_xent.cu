@@ -85,6 +85,27 @@ __device__ __forceinline__ void write_row(const XentCombineParams& p, long long 
     if (SBP_GUARD(p.row_sum[j] + row, 4)) p.row_sum[j][row] = S;
 }
 
+// The (m, s) pairs of a warp's lanes into one, the same in all of them: the maximum first, then every sum rescaled once.
+// (Merging pair by pair rescales a sum at every level, and the unit's exponentials are 5e-8 low on the average: sums of
+// PAIRWISE.)
+__device__ __forceinline__ void merge_warp(float& m, float& s) {
+  float top = m;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, off));
+  s = m == -INFINITY ? 0.f : s * ex2((m - top) * kLog2e);
+  m = top;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+}
+
+// n pairs into one, in their order.
+__device__ __forceinline__ void merge_all(const float* ms, const float* ss, int n, float& m, float& s) {
+  m = ms[0];
+  for (int w = 1; w < n; ++w) m = fmaxf(m, ms[w]);
+  s = 0.f;
+  for (int w = 0; w < n; ++w) s += ms[w] == -INFINITY ? 0.f : ss[w] * ex2((ms[w] - m) * kLog2e);
+}
+
 // ---- chunk policies: how one thread of a team loads, maxes and exp-sums its kLoadsPerThread vectors of 16 bytes.  z
 // points at the first vector (16-byte aligned), nv counts the vectors there are.
 
@@ -179,12 +200,15 @@ __device__ __forceinline__ int to_boundary(const T* z, long long n) {
   return h < n ? h : (int)n;
 }
 
-// A team's pass over the n > 0 logits at z: the running (m, s) of each of its threads.
+// A team's pass over the n > 0 logits at z: the running (m, s) of each of its threads, s a sum of exp(z - m).
 // A row starts wherever the class count and the pitch put it: up to 15 bytes on either end of the span are taken
 // element by element, one element a thread, and what lies between as aligned vectors; the loads of the next chunk
 // are issued before the current one is reduced.  (Unaligned rows element by element throughout: fp32 [256, 100003]
 // over four shards 33 us, backward 76; as here 25 and 35: 0.62 and 0.89 of the copy bandwidth.)
-template <typename Chunk, bool UNITS>
+// An exponential is 2^(z log2e - c), c = m log2e rounded: one FMA an element.  What the rounding of c leaves, r = m log2e - c,
+// is a factor 2^r on all that the thread adds up in a chunk, up to 3e-7 at a maximum of 8; it is taken out of the chunk's
+// sum.  What is carried from chunk to chunk is rescaled by the difference of the maxima: exactly 1 while the maximum stands.
+template <typename Chunk>
 __device__ __forceinline__ void walk_span(const typename Chunk::T* z, long long n, int tid, int team, float& m, float& s) {
   using T = typename Chunk::T;
   constexpr int VEC = Chunk::VEC;
@@ -200,34 +224,19 @@ __device__ __forceinline__ void walk_span(const typename Chunk::T* z, long long 
     const float x = static_cast<float>(*lone);
     if (x != -INFINITY) merge(m, s, x, 1.f);
   }
-  // UNITS: inside the loop s counts in units of 2^e, e the integer above m log2 e.  Without, the rounding of m log2 e
-  // scales what a thread has so far once more with every chunk, which only many threads to a row average out.
-  float e = 0.f;
-  if constexpr (UNITS) {
-    e = ceilf(m * kLog2e);      // -inf as long as there is nothing
-    if (m != -INFINITY) s *= ex2(fmaf(m, kLog2e, -e));
-  }
   for (long long off = 0; off < nv; off += step) {
     const bool more = off + step < nv;
     if (more) nxt.load(zv + (off + step) * VEC, nv - off - step, tid, team);
     const float cm = cur.max();
-    if (cm != -INFINITY) {
-      const float mm = fmaxf(m, cm);
-      if constexpr (UNITS) {
-        const float ee = ceilf(mm * kLog2e);
-        const float carried = e == ee ? s : (e == -INFINITY ? 0.f : s * ex2(e - ee));
-        s = carried + cur.expsum(-ee);
-        e = ee;
-      } else {
-        const float neg = -mm * kLog2e;
-        const float carried = (m == -INFINITY) ? 0.f : s * ex2(fmaf(m, kLog2e, neg));
-        s = carried + cur.expsum(neg);
-      }
+    if (cm != -INFINITY) {                                      // not the threads of a short row that have nothing
+      const float mm = fmaxf(m, cm), c = fmaxf(mm * kLog2e, -3.4e38f);      // finite under masks of the type's lowest value
+      const float carried = s * ex2((m - mm) * kLog2e);         // s is 0 as long as m is -inf
+      const float sum = cur.expsum(-c);
+      s = carried + fmaf(sum, -0.69314718f * fmaf(mm, kLog2e, -c), sum);
       m = mm;
     }
     if (more) cur = nxt;
   }
-  if (UNITS && m != -INFINITY) s *= ex2(fmaf(-m, kLog2e, e));
 }
 
 // Many rows: a team of 1 << team_log2 threads takes a whole row, shard after shard, and finishes it -- no partials,
@@ -236,8 +245,7 @@ __device__ __forceinline__ void walk_span(const typename Chunk::T* z, long long 
 // four 39 / 24.)  The team grows with the row, so that a thread adds up no more elements than in the partial kernel;
 // rows that take more than 128 threads so are left to that kernel, which is as fast for them or faster (fp32 [2000,
 // 134217] over four 254 us with teams of 64, 168 there; [3000, 30000] over two 73 either way; bf16 [2000, 100000] over
-// two 92 with teams of 256, 75 there).  Relative error of the row sums with 64 threads and 9000 fp32 classes 3.3e-7, with no
-// bound on the team's share and without UNITS 3e-6 to 9e-6, in the partial kernel 3e-7 to 4e-7.
+// two 92 with teams of 256, 75 there).  Relative error of the row sums at any team 0.6e-7 to 0.9e-7 rms, 3.5e-7 at most.
 constexpr long long kRowsForTeams = 740;
 
 // log2 of the team for this many rows and classes in vectors of `vec` elements; 0: the partial kernel
@@ -264,16 +272,11 @@ __global__ void __launch_bounds__(kThreads) xent_rows_kernel(const __grid_consta
       long long c_start, c_len;
       split_range(p.classes, p.k, r, (int64_t*)&c_start, (int64_t*)&c_len);
       const T* z = reinterpret_cast<const T*>(p.logits[r]) + row * p.pitch[r];
-      if (c_len > 0) walk_span<Chunk, true>(z, c_len, tl, team, m, s);
+      if (c_len > 0) walk_span<Chunk>(z, c_len, tl, team, m, s);
       if (tl == 0 && y >= c_start && y < c_start + c_len && SBP_GUARD(z + (y - c_start), sizeof(T))) t = static_cast<float>(z[y - c_start]);
     }
   }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const float m2 = __shfl_xor_sync(0xffffffffu, m, off);
-    const float s2 = __shfl_xor_sync(0xffffffffu, s, off);
-    merge(m, s, m2, s2);
-  }
+  merge_warp(m, s);
   if (team > 32) {
     __shared__ float sm[kThreads / 32], ss[kThreads / 32];
     const int w0 = threadIdx.x >> 5;
@@ -282,17 +285,16 @@ __global__ void __launch_bounds__(kThreads) xent_rows_kernel(const __grid_consta
       ss[w0] = s;
     }
     __syncthreads();
-    if (tl == 0)
-      for (int w = 1; w < team / 32; ++w) merge(m, s, sm[w0 + w], ss[w0 + w]);
+    if (tl == 0) merge_all(sm + w0, ss + w0, team / 32, m, s);
   }
   if (tl == 0 && row < p.rows) write_row(c, row, m, s, t);
 }
 
 // One CTA per (row, shard, column span).  Each thread keeps a running (m, s) over the chunks
 // of its span -- the loads of the next chunk are issued before the current one is reduced --
-// and the CTA merges the 256 pairs with a fixed tree.
-template <typename Chunk>
-__global__ void __launch_bounds__(kThreads) xent_partial_kernel(const __grid_constant__ XentParams p) {
+// and the CTA merges its threads' pairs in a fixed order.
+template <typename Chunk, int THREADS>
+__global__ void __launch_bounds__(THREADS) xent_partial_kernel(const __grid_constant__ XentParams p) {
   using T = typename Chunk::T;
   const long long row = blockIdx.x;
   const int split = blockIdx.y;
@@ -311,24 +313,18 @@ __global__ void __launch_bounds__(kThreads) xent_partial_kernel(const __grid_con
   SBP_PDL_WAIT();
 
   float m = -INFINITY, s = 0.f;
-  if (n > 0) walk_span<Chunk, false>(z, n, tid, kThreads, m, s);
+  if (n > 0) walk_span<Chunk>(z, n, tid, THREADS, m, s);
 
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const float m2 = __shfl_xor_sync(0xffffffffu, m, off);
-    const float s2 = __shfl_xor_sync(0xffffffffu, s, off);
-    merge(m, s, m2, s2);
-  }
-  __shared__ float sm[kThreads / 32], ss[kThreads / 32];
+  merge_warp(m, s);
+  __shared__ float sm[THREADS / 32], ss[THREADS / 32];
   if ((tid & 31) == 0) {
     sm[tid >> 5] = m;
     ss[tid >> 5] = s;
   }
   __syncthreads();
   if (tid == 0) {
-    float mm = sm[0], sv = ss[0];
-#pragma unroll
-    for (int w = 1; w < kThreads / 32; ++w) merge(mm, sv, sm[w], ss[w]);
+    float mm, sv;
+    merge_all(sm, ss, THREADS / 32, mm, sv);
     float t = 0.f;
     const long long y = (SBP_GUARD(p.labels + row, 8) ? p.labels[row] : -1) - c_start - c0;
     if (y >= 0 && y < n && SBP_GUARD(z + y, sizeof(T))) t = static_cast<float>(z[y]);
@@ -337,6 +333,16 @@ __global__ void __launch_bounds__(kThreads) xent_partial_kernel(const __grid_con
     if (SBP_GUARD(p.part_s + at, 4)) p.part_s[at] = sv;
     if (SBP_GUARD(p.part_t + at, 4)) p.part_t[at] = t;
   }
+}
+
+// Short rows get no more threads than there are vectors (fp32 [700, 100] over four S256 us with 256 threads, S32 with 32).
+template <typename Chunk>
+static void launch_partial(const XentParams& p, dim3 grid, long long widest, cudaStream_t st) {
+  const long long vectors = (widest + Chunk::VEC - 1) / Chunk::VEC;
+  if (vectors <= 32) launch_dependent(xent_partial_kernel<Chunk, 32>, grid, dim3(32), 0, st, p);
+  else if (vectors <= 64) launch_dependent(xent_partial_kernel<Chunk, 64>, grid, dim3(64), 0, st, p);
+  else if (vectors <= 128) launch_dependent(xent_partial_kernel<Chunk, 128>, grid, dim3(128), 0, st, p);
+  else launch_dependent(xent_partial_kernel<Chunk, kThreads>, grid, dim3(kThreads), 0, st, p);
 }
 
 // One warp per row: lane j takes the parts j, j + 32, ... in ascending order, then the lanes
@@ -358,13 +364,9 @@ __global__ void __launch_bounds__(kCombineThreads) xent_combine_kernel(const __g
     merge(m, S, p.part_m[at], p.part_s[at]);
     zy += p.part_t[at];
   }
+  merge_warp(m, S);
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const float m2 = __shfl_xor_sync(0xffffffffu, m, off);
-    const float s2 = __shfl_xor_sync(0xffffffffu, S, off);
-    zy += __shfl_xor_sync(0xffffffffu, zy, off);
-    merge(m, S, m2, s2);
-  }
+  for (int off = 16; off > 0; off >>= 1) zy += __shfl_xor_sync(0xffffffffu, zy, off);
   if (lane == 0) write_row(p, row, m, S, zy);
 }
 
@@ -739,8 +741,8 @@ sbp_status sbp_softmax_xent(const sbp_tensor* logits, const sbp_tensor* labels, 
     return SBP_OK;
   }
   dim3 grid((unsigned)rows, (unsigned)nsplit, (unsigned)k);
-  if (logits->dtype == SBP_BF16) launch_dependent(xent_partial_kernel<ChunkBF16>, grid, dim3(kThreads), 0, stream, p);
-  else launch_dependent(xent_partial_kernel<ChunkF32>, grid, dim3(kThreads), 0, stream, p);
+  if (logits->dtype == SBP_BF16) launch_partial<ChunkBF16>(p, grid, (classes + k - 1) / k, stream);
+  else launch_partial<ChunkF32>(p, grid, (classes + k - 1) / k, stream);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "softmax partial launch");
 
