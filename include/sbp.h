@@ -308,7 +308,7 @@ void sbp_boxing_set_copy_engine(int32_t engine);
  * dW = X^T dY (x = X with SBP_TRANS_X) and dX = dY W^T (w = W with SBP_TRANS_W).  Data
  * parallelism (Section 3.1: X S(0), W B) then gives dW = (S(1), S(0)) -> P(sum), and asking
  * for y as B folds the gradient all-reduce into the product.  One-axis placements only.
- * ws: scratch for the tensor-core path (see below; may be NULL when the query returns 0).
+ * ws: scratch for the tensor-core path (see below; may be NULL when sbp_matmul_workspace_bytes_for returns 0).
  * A result whose base or leading dimension the copy engine cannot address is written by the
  * kernel's own stores instead; that needs no workspace.
  */
@@ -324,11 +324,16 @@ void sbp_boxing_set_copy_engine(int32_t engine);
  * aligned local tensors or add the operands' sizes yourself); ws must be 256-byte aligned.  Without
  * a large enough workspace such a product runs on the FMA kernel: same results within the stated
  * tolerance, far slower.  sbp_matmul_workspace_bytes is the same query for flags = 0.
- * A 16-byte aligned workspace with more room than that is used as well where it helps: a small result of a
- * long contraction (the feature gradient of a classifier) is cut along K over the whole device when `ws`
- * holds at least two fp32 copies of the result. */
+ * sbp_matmul_workspace_bytes_preferred is at least as large: it adds the room for partial results that a small
+ * result of a long contraction profits from (the feature gradient of a classifier, [512, 2^20] x [2^20, 512], takes
+ * 570 us with it, 770 without); asked of the device that is current.  Such a product is cut along K
+ * over the whole device when `ws` has room for at least two sets of fp32 partial results, and the more the finer, so its
+ * last bits depend on how much room there is; where the two queries answer the same, a product whose local tensors are
+ * aligned as the queries take them to be leaves the rest of a larger workspace alone.  ws is scratch: any of it may be
+ * written by the call, so calls that may run at the same time need one each. */
 size_t sbp_matmul_workspace_bytes_for(const sbp_tensor* x, const sbp_tensor* w, const sbp_tensor* y, uint32_t flags);
 size_t sbp_matmul_workspace_bytes(const sbp_tensor* x, const sbp_tensor* w, const sbp_tensor* y);
+size_t sbp_matmul_workspace_bytes_preferred(const sbp_tensor* x, const sbp_tensor* w, const sbp_tensor* y, uint32_t flags);
 
 /* The tensor-core path describes every operand and result tile layout to the copy engine with a
  * descriptor that the driver encodes on the host.  The library keeps the descriptors it has
@@ -347,7 +352,8 @@ void sbp_tensor_map_stats(uint64_t* reused, uint64_t* encoded);
  * per tile, each pair with its part of the contraction, the parts added in a fixed order (its results
  * may differ from the other forms' in the last bits, and are the same from call to call).  This reports the launches since the
  * library was loaded (process-wide): [0] square
- * or split, [1] tall, [2] the square launch that ends a mixed run.
+ * or split, [1] tall, [2] the square launch that ends a mixed run; sbp_matmul_split_launches tells how many of [0] were
+ * split.
  * sbp_matmul_set_form overrides the choice for tests and measurements (process-wide, not a tuning
  * knob): form 0 = the library chooses, 1 = square, 2 = tall, 3 = mixed, 4 = split (where a product cannot run
  * the forced form -- softmax epilogues, results written element-wise, fewer tiles than one wave
@@ -372,6 +378,7 @@ void sbp_matmul_set_form(int32_t form, int32_t max_pairs);
 int32_t sbp_matmul_route(int64_t m, int64_t n, int64_t k, int32_t pairs, uint32_t flags, int32_t replicas, int32_t out_f32,
                          int64_t* tall_tiles);
 void sbp_matmul_form_stats(uint64_t launches[3]);
+uint64_t sbp_matmul_split_launches(void);
 sbp_status sbp_matmul(const sbp_tensor* x, const sbp_tensor* w, sbp_tensor* y, uint32_t flags,
                       void* ws, size_t ws_bytes, void* cuda_stream);
 

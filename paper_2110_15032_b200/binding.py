@@ -117,12 +117,16 @@ def load_library():
     lib.sbp_matmul_workspace_bytes.argtypes = [T, T, T]
     lib.sbp_matmul_workspace_bytes_for.restype = C.c_size_t
     lib.sbp_matmul_workspace_bytes_for.argtypes = [T, T, T, C.c_uint32]
+    lib.sbp_matmul_workspace_bytes_preferred.restype = C.c_size_t
+    lib.sbp_matmul_workspace_bytes_preferred.argtypes = [T, T, T, C.c_uint32]
     lib.sbp_matmul.argtypes = [T, T, T, C.c_uint32, C.c_void_p, C.c_size_t, C.c_void_p]
     lib.sbp_tensor_map_stats.argtypes = [C.POINTER(C.c_uint64), C.POINTER(C.c_uint64)]
     lib.sbp_tensor_map_stats.restype = None
     lib.sbp_matmul_set_form.argtypes = [C.c_int32, C.c_int32]
     lib.sbp_matmul_set_form.restype = None
     lib.sbp_matmul_form_stats.argtypes = [C.POINTER(C.c_uint64)]
+    lib.sbp_matmul_split_launches.restype = C.c_uint64
+    lib.sbp_matmul_split_launches.argtypes = []
     lib.sbp_matmul_route.argtypes = [C.c_int64, C.c_int64, C.c_int64, C.c_int32, C.c_uint32, C.c_int32, C.c_int32, C.POINTER(C.c_int64)]
     lib.sbp_matmul_route.restype = C.c_int32
     lib.sbp_matmul_form_stats.restype = None
@@ -339,6 +343,11 @@ def sbp_matmul_form_stats():
     return int(v[0]), int(v[1]), int(v[2])
 
 
+def sbp_matmul_split_launches() -> int:
+    """Launches of the tensor-core MatMul's split form since the library was loaded (counted among the square ones too)."""
+    return int(load_library().sbp_matmul_split_launches())
+
+
 def sbp_selftest_debug_bounds(buf: torch.Tensor, stream=None) -> None:
     _check(load_library().sbp_selftest_debug_bounds(C.c_void_p(buf.data_ptr()), buf.numel() * buf.element_size(),
                                                     _stream_ptr(stream)))
@@ -427,6 +436,13 @@ def sbp_boxing_host(src_host: SbpTensor, dst_host: SbpTensor, dev_ws: torch.Tens
 def sbp_matmul_workspace_bytes(x: SbpTensor, w: SbpTensor, y: SbpTensor, flags: int = 0) -> int:
     a, b, c = x._c(), w._c(), y._c()
     return int(load_library().sbp_matmul_workspace_bytes_for(C.byref(a), C.byref(b), C.byref(c), flags))
+
+
+def sbp_matmul_workspace_bytes_preferred(x: SbpTensor, w: SbpTensor, y: SbpTensor, flags: int = 0) -> int:
+    """What the product can make use of: at least sbp_matmul_workspace_bytes, more where partial results of a long
+    contraction pay (see include/sbp.h)."""
+    a, b, c = x._c(), w._c(), y._c()
+    return int(load_library().sbp_matmul_workspace_bytes_preferred(C.byref(a), C.byref(b), C.byref(c), flags))
 
 
 def sbp_matmul(x: SbpTensor, w: SbpTensor, y: SbpTensor, flags: int = 0,

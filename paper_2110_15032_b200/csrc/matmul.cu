@@ -26,9 +26,12 @@ sbp_status launch_xent_finish(float* part_m, float* part_s, float* part_t, int p
 sbp_status check_xent_outputs(const sbp_tensor* labels, const sbp_tensor* loss, const sbp_tensor* row_max,
                               const sbp_tensor* row_sum, long long rows, int k);
 size_t xent_finish_stage_floats(long long rows);
-size_t matmul_tc_workspace_bytes(const MatmulPlan& plan);
+// Defined in matmul_tc.cu.  True when the tensor-core kernels take the plan as it stands; *room: the workspace they would
+// use for partial results if they were given it.  Launches nothing.
+bool matmul_tc_room(const MatmulPlan& plan, size_t* room);
 void tensor_map_cache_stats(unsigned long long* hits, unsigned long long* encodes);
 void tc_form_stats(unsigned long long out[3]);
+unsigned long long tc_split_launches();
 void tc_set_form(int form, int max_pairs);
 int tc_route(long long tiles_sq, long long tiles_tall, long long kb, int pairs, bool gelu, int n_rep, bool out_f32, int forced,
              long long* tall_tiles);
@@ -231,8 +234,8 @@ static PackNeed pack_need(const MatmulPlan& p, bool with_ptrs) {
   return n;
 }
 
-// Copies the operands named by `need` into ws and rewrites the plan to read the copies.
-static sbp_status pack_operands(MatmulPlan* plan, const PackNeed& need, void* ws, cudaStream_t st) {
+// Copies the operands named by `need` into ws (unless dry) and rewrites the plan to read the copies.
+static sbp_status pack_operands(MatmulPlan* plan, const PackNeed& need, void* ws, cudaStream_t st, bool dry = false) {
   MatmulPlan& p = *plan;
   PackList list{};
   int nb = 0;
@@ -254,7 +257,7 @@ static sbp_status pack_operands(MatmulPlan* plan, const PackNeed& need, void* ws
     return SBP_OK;
   };
   auto add = [&](const void* src, void* dst, long long rows, long long cols, long long sld, long long dld) -> sbp_status {
-    if (rows == 0 || cols == 0) return SBP_OK;
+    if (rows == 0 || cols == 0 || dry) return SBP_OK;
     list.b[nb++] = PackBlock{static_cast<const unsigned short*>(src), static_cast<unsigned short*>(dst), rows, cols, sld, dld};
     return nb == kPackBlocks ? flush() : SBP_OK;
   };
@@ -526,7 +529,21 @@ size_t sbp_matmul_workspace_bytes_for(const sbp_tensor* x, const sbp_tensor* w, 
   const sbp_status st = two_axes ? build_plan_2d(x, w, y, flags, false, &plan) : build_plan(x, w, y, flags, false, &plan);
   if (st != SBP_OK) return 0;
   // without pointers to look at, an operand counts as misaligned only by its shape
-  return pack_need(plan, false).bytes + matmul_tc_workspace_bytes(plan);
+  return pack_need(plan, false).bytes;
+}
+
+size_t sbp_matmul_workspace_bytes_preferred(const sbp_tensor* x, const sbp_tensor* w, const sbp_tensor* y, uint32_t flags) {
+  MatmulPlan plan;
+  const bool two_axes = x && w && y && (x->pdims == 2 || w->pdims == 2 || y->pdims == 2);
+  const sbp_status st = two_axes ? build_plan_2d(x, w, y, flags, false, &plan) : build_plan(x, w, y, flags, false, &plan);
+  if (st != SBP_OK) return 0;
+  const PackNeed need = pack_need(plan, false);
+  if (plan.in_dtype != SBP_BF16) return need.bytes;
+  size_t room = 0;
+  if (matmul_tc_room(plan, &room)) return room > need.bytes ? room : need.bytes;
+  if (need.bytes == 0 || pack_operands(&plan, need, nullptr, nullptr, true) != SBP_OK) return need.bytes;
+  matmul_tc_room(plan, &room);
+  return need.bytes + room;
 }
 
 size_t sbp_matmul_workspace_bytes(const sbp_tensor* x, const sbp_tensor* w, const sbp_tensor* y) {
@@ -559,6 +576,8 @@ void sbp_matmul_form_stats(uint64_t launches[3]) {
   if (launches)
     for (int i = 0; i < 3; ++i) launches[i] = v[i];
 }
+
+uint64_t sbp_matmul_split_launches(void) { return tc_split_launches(); }
 
 sbp_status sbp_matmul(const sbp_tensor* x, const sbp_tensor* w, sbp_tensor* y, uint32_t flags, void* ws,
                       size_t ws_bytes, void* cuda_stream) {

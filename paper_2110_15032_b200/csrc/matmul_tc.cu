@@ -1614,8 +1614,8 @@ void tensor_map_cache_stats(unsigned long long* hits, unsigned long long* encode
   *encodes = g_map_encodes;
 }
 
-// launches of the kernel by form: square, tall, square over the halves that a mixed run leaves
-static std::atomic<unsigned long long> g_form_launches[3];
+// launches of the kernel by form: square or split, tall, square over the halves that a mixed run leaves; and the split ones
+static std::atomic<unsigned long long> g_form_launches[3], g_split_launches;
 
 // Overrides of the form choice and of the CTA pairs a launch may use (tests and measurements):
 // set by tc_set_form, else taken once from SBP_TC_FORM (square | tall | mixed | split) and SBP_TC_PAIRS.
@@ -1649,6 +1649,8 @@ void tc_set_form(int form, int max_pairs) {
 void tc_form_stats(unsigned long long out[3]) {
   for (int i = 0; i < 3; ++i) out[i] = g_form_launches[i].load();
 }
+
+unsigned long long tc_split_launches() { return g_split_launches.load(); }
 
 // 2-D row-major tensor [rows, cols] with leading dimension ld (elements), box [box_rows, box_cols].
 static bool make_map(CUtensorMap* map, const void* base, int esz, long long rows, long long cols, long long ld,
@@ -1684,8 +1686,6 @@ static bool make_map(CUtensorMap* map, const void* base, int esz, long long rows
   slot.used = true;
   return true;
 }
-
-size_t matmul_tc_workspace_bytes(const MatmulPlan&) { return 0; }
 
 static bool aligned16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
 
@@ -1868,6 +1868,7 @@ static sbp_status launch_split_form(const TcSplitParams* p, int splits, int tile
   if (e != cudaSuccess) return cuda_fail(e, "tensor-core matmul launch");
   count_launch();
   g_form_launches[0]++;
+  g_split_launches++;
   return SBP_OK;
 }
 
@@ -1942,11 +1943,11 @@ static SplitChoice choose_split(const MatmulPlan& plan, const int* kblocks, doub
     kb_max = kb > kb_max ? kb : kb_max;
     kb_min = kb_min < 0 || kb < kb_min ? kb : kb_min;
   }
-  SplitChoice best{0, 0, 0, 1};
+  SplitChoice best{0, 0, 0, 1}, cut{0, 0, 0, 1};
   const OperandRows rows = operand_rows(plan);
   const long long pf = part_floats(plan);
-  const long long room = pf > 0 ? (long long)(ws_bytes / 4) / pf : 0;      // sets of partial results the workspace holds
-  double best_cost = forced == 4 ? 1e300 : cost_persistent;
+  const long long room = pf > 0 ? (long long)std::min<size_t>(ws_bytes / 4, size_t(1) << 60) / pf : 0;      // sets of partial results the workspace holds
+  double best_cost = forced == 4 ? 1e300 : cost_persistent, cut_cost = 1e300, any_cut_cost = 1e300;
   for (int swap = 0; swap < 2; ++swap) {
     if (swap && plan.a_trans) continue;      // X would be the N-major operand: boxes of 64 rows and more
     if (swap && m_max > 192) continue;       // its tiles read the weight once per 128 rows, the plain ones once per 256
@@ -1972,19 +1973,25 @@ static SplitChoice choose_split(const MatmulPlan& plan, const int* kblocks, doub
           best = SplitChoice{nb, s, swap, 1};
         }
         // as many clusters a tile as run at once; adding their results up is a launch, one write and one read
-        const long long outer = std::min({tiles > 0 ? cap / tiles : 0, room, kb_min / (8 * s), 128LL});
-        if (outer >= 2) {
+        auto cut_over = [&](long long outer) {
           const double kbo = (double)((kb_max + s * outer - 1) / (s * outer));
           const double sum = 4.0 + (double)pf * (8.0 * outer + (plan.out_dtype == SBP_F32 ? 4.0 : 2.0) * (1 + plan.n_rep)) / 5e6;
-          const double co = k_time(kbo) + per_wave + (s > 1 ? 0.8 + 0.08 * s : 0.0) + sum;
-          if (co < best_cost) {
-            best_cost = co;
-            best = SplitChoice{nb, s, swap, (int)outer};
+          return k_time(kbo) + per_wave + (s > 1 ? 0.8 + 0.08 * s : 0.0) + sum;
+        };
+        const long long all = std::min({tiles > 0 ? cap / tiles : 0, kb_min / (8 * s), 128LL}), outer = std::min(all, room);
+        if (all >= 2) any_cut_cost = std::min(any_cut_cost, cut_over(all));
+        if (outer >= 2) {
+          const double co = cut_over(outer);
+          if (co < cut_cost) {
+            cut_cost = co;
+            cut = SplitChoice{nb, s, swap, (int)outer};
           }
         }
       }
     }
   }
+  // The workspace is used only where the size query reports room for it: not where a cut pays with less room alone.
+  if (any_cut_cost < best_cost && cut_cost < best_cost) return cut;
   return best;
 }
 
@@ -2190,7 +2197,8 @@ static sbp_status launch_narrow(const MatmulPlan& plan, const XentFusion& xf, cu
   }
 }
 
-sbp_status launch_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, void* ws, size_t ws_bytes, cudaStream_t st, bool* taken) {
+// room != nullptr: nothing is launched; *room is the workspace that the product would use if it were given all it can use.
+static sbp_status run_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, void* ws, size_t ws_bytes, cudaStream_t st, bool* taken, size_t* room) {
   *taken = false;
   if (plan.in_dtype != SBP_BF16) return SBP_ERR_UNSUPPORTED;
   const int oesz = plan.out_dtype == SBP_F32 ? 4 : 2;
@@ -2269,10 +2277,19 @@ sbp_status launch_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, void* 
     }
     if (forced == 4 || (forced == 0 && pair_cap() == 0)) {
       const SplitChoice sc = choose_split(as_one ? merged : plan, kblocks, 0.92 * (form.cost + 5.5), forced, aligned16(ws) ? ws_bytes : 0);
+      if (room) {
+        *taken = sc.splits > 0 || rows_aligned;
+        *room = sc.outer > 1 ? (size_t)sc.outer * (size_t)part_floats(plan) * 4 : 0;
+        return SBP_OK;
+      }
       if (sc.splits > 0) return launch_split(plan, as_one ? &merged : nullptr, kblocks, sc, !y_direct, static_cast<float*>(ws), st, taken);
     }
   }
   if (!rows_aligned) return SBP_ERR_UNSUPPORTED;
+  if (room) {
+    *taken = true;
+    return SBP_OK;
+  }
 
   p.ngroups = plan.ngroups;
   p.nseg = plan.nseg;
@@ -2369,6 +2386,16 @@ sbp_status launch_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, void* 
   p.half_split = 1;
   p.total_tiles = 2 * (tiles - tall_tiles);
   return launch_tc(kFormSquare, plan.a_trans, plan.b_trans, &p, st, nullptr);
+}
+
+sbp_status launch_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, void* ws, size_t ws_bytes, cudaStream_t st, bool* taken) {
+  return run_matmul_tc(plan, xf, ws, ws_bytes, st, taken, nullptr);
+}
+
+bool matmul_tc_room(const MatmulPlan& plan, size_t* room) {
+  *room = 0;
+  bool taken = false;
+  return run_matmul_tc(plan, nullptr, nullptr, ~size_t(0), nullptr, &taken, room) == SBP_OK && taken;
 }
 
 sbp_status read_and_clear_tc_timeout(bool* timed_out) {
