@@ -1929,7 +1929,9 @@ static int split_capacity(int splits) {
 // with 128 and fewer (the single-issue roles); set-up, drain and stores 9.6 / 6.6 us (256 / 128 columns),
 // 6.5 / 5.3 / 4.4 for the exchanged form (128 / 64 / 32).  Fitted to 1208 timings of 54 products (rms error
 // 12 %; the pick within 8 % of the best cut of each).  The persistent kernel keeps what it does as well:
-// `cost_persistent` includes the 5.5 us it takes besides its waves, and a split has to win by 8 %.
+// `cost_persistent` includes the 5.5 us it takes besides its waves, and a split has to win by 8 %.  An fp32 result is
+// twice the stores, like another replica ([16384 x 512] x [512 x 64] over four devices to fp32 S(0): 12.3 us split, which
+// the rule took without that term, 7.9 persistent; three [333 x 333] x [333 x 111] to fp32 14.0 / 18.4).
 // (us, persistent / split, one product in a row of them: 16 rows [4096 x 16384] 31 / 24 and [16384 x 4096]
 // 79 / 26; 1000 rows [4096 x 1024] written to four replicas 28 / 16; 500 rows [1024 x 4096] + GeLU 15 / 11;
 // 512 x 512 over 2^20 classes 4569 / 621; 64 x 256 over 2^17 578 / 48.)
@@ -1967,7 +1969,7 @@ static SplitChoice choose_split(const MatmulPlan& plan, const int* kblocks, doub
         auto k_time = [&](double kbs) { return kbs * per_kb + (swap ? rows.extra(nb / 2, BMH, kbs, per_kb) : rows.extra(BMH, nb / 2, kbs, per_kb)); };
         const double per_wave = nb == 256 ? 9.6 : (nb == 128 ? 6.6 : (nb == 64 ? 5.3 : 4.4));
         const double cost = waves * (k_time(kb) + per_wave + (s > 1 ? 0.8 + 0.08 * s : 0.0) + (plan.gelu ? 0.4 : 0.0) +
-                                     plan.n_rep * 2.0 * nb / (256.0 * s));
+                                     (plan.n_rep + (plan.out_dtype == SBP_F32 ? 1 : 0)) * 2.0 * nb / (256.0 * s));
         if (cost < best_cost) {
           best_cost = cost;
           best = SplitChoice{nb, s, swap, 1};
@@ -2270,7 +2272,10 @@ static sbp_status run_matmul_tc(const MatmulPlan& plan, const XentFusion* xf, vo
     }
     form = choose_form(tiles_sq, tiles_tall, kb_tile, cap_sq, cap_tall, plan.gelu != 0, plan.n_rep, plan.out_dtype == SBP_F32, rows,
                        forced == 4 ? 0 : forced);
-    if (y_direct) form.walk_tall = false;
+    if (y_direct) {      // its shifted row stores are exposed at the end, where a split deals them out to its pairs
+      form.walk_tall = false;
+      form.cost += 1.0;
+    }
     if (!rows_aligned) {      // the copy: a launch, one read and one write
       form.cost += 4.0;
       for (int s = 0; s < plan.nseg; ++s) form.cost += (double)plan.kseg[s] * merged.m[0] * 4.0 / 4e6;
