@@ -836,7 +836,8 @@ static sbp_status boxing_one_axis(const sbp_tensor* src, sbp_tensor* dst, int ds
   Plan pl;
   st = make_plan(src, dst, dst_shard, &pl);
   if (st != SBP_OK) return st;
-  if (dry || numel(src) == 0) return SBP_OK;
+  // a grid for a shard that holds nothing would finish without having waited for the kernel before it
+  if (dry || numel(src) == 0 || (dst_shard >= 0 && local_numel(dst, dst_shard) == 0)) return SBP_OK;
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   SBP_BOUNDS_RESET();
   SBP_BOUNDS_TENSOR(src);

@@ -483,6 +483,7 @@ sbp_status boxing_disjoint(const sbp_tensor* src, sbp_tensor* dst, int dst_shard
   }
   if (copy_needed && grid > 0x7fffffffLL) return fail(SBP_ERR_UNSUPPORTED, "tensor too large for one launch");
   if (dry) return SBP_OK;   // every refusal lies above this line, every launch below it
+  if (dst_shard >= 0 && local_numel(dst, dst_shard) == 0) return SBP_OK;   // no grid that finishes without having waited
   SBP_BOUNDS_RESET();
   SBP_BOUNDS_TENSOR(src);
   if (dst_shard >= 0) SBP_BOUNDS_SHARD(dst, dst_shard);
