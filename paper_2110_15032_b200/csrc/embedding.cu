@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(256, 4) embedding_rows_kernel(const __grid_con
     V val[J];
 #pragma unroll
     for (int j = 0; j < J; ++j) {
-      if (j * 256u >= pieces) break;                // short rows leave most of a chunk's steps empty
+      if (sizeof(V) < 16 && j * 256u >= pieces) break;      // short rows leave most of the 16 steps empty
       const unsigned f = j * 256 + threadIdx.x;
       val[j] = zero_vec<V>();
       if (f >= pieces) continue;
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(256, 4) embedding_rows_kernel(const __grid_con
       V* o = reinterpret_cast<V*>(p.out[q]) + out0;
 #pragma unroll
       for (int j = 0; j < J; ++j) {
-        if (j * 256u >= pieces) break;
+        if (sizeof(V) < 16 && j * 256u >= pieces) break;
         const unsigned f = j * 256 + threadIdx.x;
         if (f < pieces && SBP_GUARD(o + f, sizeof(V))) __stcs(o + f, p.canon_neg_zero ? canon<V, ESZ>(val[j]) : val[j]);
       }
@@ -253,7 +253,9 @@ __global__ void __launch_bounds__(256, 4) embedding_rows_kernel(const __grid_con
   SBP_PDL_RELEASE();
 }
 
-// Pieces per thread of a chunk: eight 16-byte ones, and more of narrower pieces.
+// Pieces per thread of a chunk: eight 16-byte ones, and more of narrower pieces.  (Leaving out the empty steps of a chunk pays
+// with 16 of them: bf16 [10^6, 12], 300 K lookups to eight replicas 20.5 -> 14.3 us; with eight it costs full chunks more:
+// [2^24, 128] 191.2 -> 192.3.)
 template <typename V>
 constexpr int rows_j() { return sizeof(V) == 16 ? 8 : 16; }
 
