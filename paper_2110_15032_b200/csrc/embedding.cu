@@ -266,19 +266,19 @@ static void launch_emb(const EmbParams& given, bool fused, cudaStream_t st) {
   constexpr int J = rows_j<V>();
   SBP_BOUNDS_UPLOAD(st);
   if (fused && given.vpr <= 256 * J) {
-    // persistent: as many CTAs as fit at once
-    static std::atomic<int> resident{0};
-    int r = resident.load(std::memory_order_relaxed);
+    // persistent: as many CTAs as fit at once, asked once a device
+    static std::atomic<int> resident[64];
+    int dev = 0, r = 0;
+    const bool known = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64;
+    if (known) r = resident[dev].load(std::memory_order_relaxed);
     if (r == 0) {
-      int dev = 0, sms = 148, per_sm = 4;
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+      int per_sm = 4;
       if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, embedding_rows_kernel<V, ESZ, J>, 256, 0) != cudaSuccess || per_sm < 1) {
         cudaGetLastError();
         per_sm = 4;
       }
-      r = sms * per_sm;
-      resident.store(r, std::memory_order_relaxed);
+      r = device_sms() * per_sm;
+      if (known) resident[dev].store(r, std::memory_order_relaxed);
     }
     // Chunks in whole waves of CTAs: a last wave of a few full chunks costs as much as a full one ([4096, 64] with
     // 65 K lookups 7.4 us with full chunks, 6.4 us so; [50 000, 32] with 2400 5.8 and 4.2 us).
@@ -758,14 +758,15 @@ extern "C" sbp_status sbp_embedding_backward(const sbp_tensor* grad_out, const s
     // than 1.5 chunks per SM (us for chunks of 256 / 512 / 1024: [2 x 10^6, 16], 426 K lookups 63 / 52 / 47.5;
     // [10^6, 64], 213 K lookups 68 / 65 / 74; [300 000, 100], 104 K lookups 41 / 48 / 65).
     int chunk = 1024;
-    while (chunk > 256 && (chunk * p.vpr > 8192 || p.n_lookups < chunk * 222LL)) chunk /= 2;
+    const long long sms = device_sms();
+    while (chunk > 256 && (chunk * p.vpr > 8192 || 2 * p.n_lookups < 3 * chunk * sms)) chunk /= 2;
     const long long chunks = (p.n_lookups + chunk - 1) / chunk;
     // Few chunks of long rows: several CTAs sort a chunk each for itself and take their columns of it, so that the
     // device is full three CTAs deep (us,
     // one CTA a chunk / so: [20000, 1000], 3000 lookups 93 / 25; [2000, 8192], 500 lookups 609 / 20; [100, 40000], 64 lookups
     // 2436 / 15).
-    const long long passes = (p.vpr + p.lanes - 1) / p.lanes, split = std::min(passes, std::max(1LL, 444 / chunks));
-    const dim3 sb((unsigned)(chunks < 148 * 8 ? chunks : 148 * 8), (unsigned)split), b(256);
+    const long long passes = (p.vpr + p.lanes - 1) / p.lanes, split = std::min(passes, std::max(1LL, 3 * sms / chunks));
+    const dim3 sb((unsigned)std::min(chunks, sms * 8), (unsigned)split), b(256);
     if (chunk == 1024) e = launch_dependent(embedding_backward_kernel<1024>, sb, b, 0, stream, p);
     else if (chunk == 512) e = launch_dependent(embedding_backward_kernel<512>, sb, b, 0, stream, p);
     else e = launch_dependent(embedding_backward_kernel<256>, sb, b, 0, stream, p);

@@ -365,7 +365,7 @@ sbp_status launch_matmul_f32(const MatmulPlan& plan, cudaStream_t st) {
   // 1075 each from three.  A round of CTAs costs about 4000 clocks of launch and pipeline fill, a split
   // its exchange through distributed shared memory.  (us, this rule / the other choices: 1000 x 1500 x 777
   // on four shards 92 / 98-189, 700 x 2000 x 700 81 / 88-232, 100 x 2000 x 100 16 / 28-226.)
-  const int sms = 148;
+  const int sms = device_sms();
   int best_t = 0, best_s = 1;
   double best = 1e300;
   for (int t = 0; t < 2; ++t) {

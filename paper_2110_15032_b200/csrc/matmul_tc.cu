@@ -2110,7 +2110,7 @@ static sbp_status launch_split(const MatmulPlan& given, const MatmulPlan* merged
   p.y_vec = 1;
   const sbp_status rs = launch_split_any(plan.a_trans, plan.b_trans, c, &p, tiles, st);
   if (rs != SBP_OK) return rs;
-  const long long blocks = std::min(148LL * 8, (quads + 255) / 256);
+  const long long blocks = std::min(8LL * device_sms(), (quads + 255) / 256);
   const cudaError_t e = launch_dependent(matmul_parts_kernel, dim3((unsigned)blocks, (unsigned)given.ngroups), dim3(256), 0, st, q);
   if (e != cudaSuccess) return cuda_fail(e, "matmul partial sums launch");
   count_launch();

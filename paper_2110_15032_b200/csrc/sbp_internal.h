@@ -84,6 +84,9 @@ sbp_status refuse_ld(const sbp_tensor* t, const char* name, const char* entry);
 
 sbp_status cuda_fail(cudaError_t e, const char* what);
 
+// SMs of the current device (asked once a device; a B200's 148 where there is none).
+int device_sms();
+
 // Launch of `kernel` as a programmatic dependent of the kernel before it in the stream: if that
 // kernel releases its dependents early (SBP_PDL_RELEASE), this one's CTAs may be set up while its
 // last CTAs still run.  Such a kernel must execute SBP_PDL_WAIT before its first access to

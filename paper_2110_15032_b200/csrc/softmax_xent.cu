@@ -240,18 +240,17 @@ __device__ __forceinline__ void walk_span(const typename Chunk::T* z, long long 
 }
 
 // Many rows: a team of 1 << team_log2 threads takes a whole row, shard after shard, and finishes it -- no partials,
-// no second kernel.  Taken from 740 rows on (five CTAs an SM), with the team that spreads the rows over the device
+// no second kernel.  Taken from five rows an SM on (740), with the team that spreads the rows over the device
 // once.  (us, partial + combine kernels / this: fp32 [4096, 1003] over two shards 24 / 8.5, bf16 [1000, 30000] over
 // four 39 / 24.)  The team grows with the row, so that a thread adds up no more elements than in the partial kernel;
 // rows that take more than 128 threads so are left to that kernel, which is as fast for them or faster (fp32 [2000,
 // 134217] over four 254 us with teams of 64, 168 there; [3000, 30000] over two 73 either way; bf16 [2000, 100000] over
 // two 92 with teams of 256, 75 there).  Relative error of the row sums at any team 0.6e-7 to 0.9e-7 rms, 3.5e-7 at most.
-constexpr long long kRowsForTeams = 740;
-
 // log2 of the team for this many rows and classes in vectors of `vec` elements; 0: the partial kernel
 static int team_for(long long rows, long long classes, int vec) {
-  if (rows < kRowsForTeams) return 0;
-  int t = rows < 2 * kRowsForTeams ? 7 : (rows < 4 * kRowsForTeams ? 6 : 5);
+  const long long least = 5LL * device_sms();
+  if (rows < least) return 0;
+  int t = rows < 2 * least ? 7 : (rows < 4 * least ? 6 : 5);
   const long long most = (long long)kMaxChunksPerCta * kLoadsPerThread * vec;
   while (t <= 7 && (classes >> t) > most) ++t;
   return t <= 7 ? t : 0;
@@ -401,7 +400,7 @@ static void tiling_in(const sbp_tensor* logits, size_t ws_bytes, long long* span
   // (never more scratch than the size query answers or the built-in array holds, so that both entry points cut alike)
   const size_t most = std::min({ws_bytes, sbp_softmax_xent_workspace_bytes(logits), (size_t)SBP_SOFTMAX_XENT_STATIC_SCRATCH_BYTES});
   const long long room = (long long)(most / (3 * sizeof(float) * (size_t)k * (size_t)rows));
-  while (*nsplit * rows * k < 148 * 4 && *span > chunk) {
+  while (*nsplit * rows * k < 4LL * device_sms() && *span > chunk) {
     const long long sp = (*span / chunk + 1) / 2 * chunk, ns = (c_max + sp - 1) / sp;
     if (ns > room) break;
     *span = sp;
@@ -501,7 +500,7 @@ constexpr int kMaxSlices = 64;
 // parts of 64 rows: 8 CTAs with 32 parts a thread before.)
 static int slices_for(int parts, long long rows) {
   const long long row_ctas = (rows + 31) / 32;
-  long long s = std::min((long long)parts / 16, 592 / row_ctas);
+  long long s = std::min((long long)parts / 16, 4LL * device_sms() / row_ctas);
   s = std::max(s, (long long)parts / 256);
   return (int)std::max(1LL, std::min(s, (long long)kMaxSlices));
 }
