@@ -23,8 +23,9 @@
  *   - Source and destination buffers must not overlap.
  *   - Balanced split of an axis of length n over k shards: shard r holds
  *     ceil(n/k) elements if r < n mod k, else floor(n/k), contiguous, in rank order.
- *   - 16-byte aligned pointers and row segments take the 128-bit vector path; anything
- *     else takes an element-wise path with identical results.
+ *   - 16-byte aligned pointers and row segments move in 128-bit vectors.  Anything else gives the same
+ *     values (in a sum over many terms perhaps in another order): large boxing transforms, softmax rows and
+ *     stored products still move in 16-byte vectors, shifted, the rest in narrower ones or element by element.
  *   - sbp_last_error() returns a thread-local, human readable detail for the last
  *     non-OK status returned on the calling thread.
  */
@@ -374,7 +375,8 @@ void sbp_matmul_set_form(int32_t form, int32_t max_pairs);
  * in the tall form; 0 for square), -1 for arguments out of range.  Host arithmetic only: no
  * device is touched, overrides set with sbp_matmul_set_form are not applied, and products that
  * cannot leave the square form (softmax epilogues, element-wise stores) are not modelled, nor is the split
- * form. */
+ * form: it is what the persistent kernel would do, and a product with few tiles or few rows may run split
+ * instead (sbp_matmul_split_launches before and after a call tells). */
 int32_t sbp_matmul_route(int64_t m, int64_t n, int64_t k, int32_t pairs, uint32_t flags, int32_t replicas, int32_t out_f32,
                          int64_t* tall_tiles);
 void sbp_matmul_form_stats(uint64_t launches[3]);

@@ -3,9 +3,9 @@
 // Three kernels execute a plan:
 //   * the tensor-core kernel (matmul_tc.cu): bf16 operands, fp32 accumulation in tensor
 //     memory, TMA-fed tiles; taken whenever the shapes meet its alignment rules;
-//   * the fp32 kernel (matmul_f32.cu): fp32 operands, fp32 fused multiply-adds, k ascending;
+//   * the fp32 kernel (matmul_f32.cu): fp32 operands, fp32 fused multiply-adds, k ascending (in up to eight parts);
 //   * the FMA kernel in this file: bf16 operands that the tensor-core kernel cannot take and that no
-//     workspace was given for, same arithmetic.
+//     workspace was given for, one such chain.
 #include <cuda_bf16.h>
 
 #include "bounds_check.h"

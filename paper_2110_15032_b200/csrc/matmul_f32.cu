@@ -1,6 +1,7 @@
 // fp32 MatMul: executes a grouped-GEMM plan (matmul_plan.h) on the FMA pipes.
 //
-// Every element of the result is one chain of fused multiply-adds in fp32, k ascending, segments in rank
+// Every element of the result is a chain of fused multiply-adds in fp32, k ascending, segments in rank order; where K is
+// split over the CTAs of a cluster (below) one chain for each, the chains added in their
 // order; there is no reduced-precision product.  Bound: the FMA pipe (128 lanes per SM and clock, 74
 // TFLOP/s at 1.965 GHz) once a product fills the device, the latency of load -> shared memory -> first
 // FMA and the launch for the small ones.

@@ -776,7 +776,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
                   else store_shifted<2>(yb + (row0 + r) * ld * 2, bytes, lane & 7, 8, at);
                 }
               }
-              __syncwarp();      // the buffer is rewritten two slabs from now
+              __syncwarp();      // every lane has read the slab before its buffer is staged again
             } else {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
