@@ -796,6 +796,20 @@ def whole_job_gbs(world: int, ms_step: float) -> float:
     return world * step_bytes() / (ms_step * 1e-3) / 1e9
 
 
+def split_record(line):
+    """The record that goes to standard output, short enough for whoever keeps only the end of it, and the rest, which goes
+    to standard error: every operator line, every transform, the per-config lines of the roofline and of the CPU baseline."""
+    record, detail = dict(line), {}
+    for key in ("ops", "transforms"):
+        if key in record:
+            detail[key] = record.pop(key)
+    for key in ("roofline", "cpu_baseline"):
+        if isinstance(record.get(key), dict) and "configs" in record[key]:
+            record[key] = dict(record[key])
+            detail[key + "_configs"] = record[key].pop("configs")
+    return record, detail
+
+
 # ------------------------------------------------------------------------------ main
 
 def parse():
@@ -1039,7 +1053,9 @@ def main():
             base["configs"] = cfgs
             line["cpu_baseline"] = base
     if rank == 0:
-        print(json.dumps(line))
+        record, detail = split_record(line)
+        sys.stderr.write("detail: " + json.dumps(detail) + "\n")
+        print(json.dumps(record))
     if dist is not None:
         dist.destroy_process_group()
     return 0
