@@ -259,13 +259,20 @@ __global__ void __launch_bounds__(256, 4) embedding_rows_kernel(const __grid_con
 template <typename V>
 constexpr int rows_j() { return sizeof(V) == 16 ? 8 : 16; }
 
-// A fused gather runs the chunked kernel unless one row is longer than a chunk; the unfused one (k outputs, all but one
-// of them zeros) is bound by its stores and runs element by element, four per thread.
+// Results of this many bytes in all, written to four replicas and more, are bound by their stores, which CTAs that come and
+// go in order spread better than persistent ones do (us, chunked / element by element, two pieces a thread: fp32 rows of 128,
+// 1.7 M lookups to eight replicas 1365 / 1231, 400 K 317 / 295, 150 K 117 / 116, to four 172 / 159, 200 K 87 / 84; to three
+// 171 / 165; to two 97 / 111, 1.7 M 407 / 457; bf16 rows of 36 in 8-byte pieces, 1.7 M to four 122 / 156).
+constexpr long long kSpreadBytes = 600000000;
+
+// A fused gather runs the chunked kernel unless one row is longer than a chunk or its result is spread so; the unfused one
+// (k outputs, all but one of them zeros) is bound by its stores and runs element by element, four per thread.
 template <typename V, int ESZ>
 static void launch_emb(const EmbParams& given, bool fused, cudaStream_t st) {
   constexpr int J = rows_j<V>();
   SBP_BOUNDS_UPLOAD(st);
-  if (fused && given.vpr <= 256 * J) {
+  const bool spread = fused && sizeof(V) == 16 && given.n_dst >= 4 && given.n_dst * given.n_lookups * given.vpr * 16 >= kSpreadBytes;
+  if (fused && !spread && given.vpr <= 256 * J) {
     // persistent: as many CTAs as fit at once, asked once a device
     static std::atomic<int> resident[64];
     int dev = 0, r = 0;
@@ -293,7 +300,8 @@ static void launch_emb(const EmbParams& given, bool fused, cudaStream_t st) {
     return;
   }
   const long long blocks = (given.n_lookups * given.vpr + 1023) / 1024;
-  if (fused) embedding_kernel<V, ESZ, 4, true><<<dim3((unsigned)blocks), 256, 0, st>>>(given);
+  if (spread) embedding_kernel<V, ESZ, 2, true><<<dim3((unsigned)((given.n_lookups * given.vpr + 511) / 512)), 256, 0, st>>>(given);
+  else if (fused) embedding_kernel<V, ESZ, 4, true><<<dim3((unsigned)blocks), 256, 0, st>>>(given);
   else embedding_kernel<V, ESZ, 4, false><<<dim3((unsigned)blocks), 256, 0, st>>>(given);
 }
 

@@ -1,6 +1,7 @@
-"""Table gradients of long rows and few lookups, whose columns are dealt out to several CTAs: one pass of 32 vectors and one
-vector more, more CTAs than columns, ids outside the table (counted once, not once a CTA), every chunk's last position.
-Bound of an n-term fp32 sum: n u sum|terms|, u = 2^-24."""
+"""Embedding calls whose shape decides how they are dealt out.  Table gradients of long rows and few lookups, whose columns are
+dealt out to several CTAs: one pass of 32 vectors and one vector more, more CTAs than columns, ids outside the table (counted
+once, not once a CTA), every chunk's last position; bound of an n-term fp32 sum: n u sum|terms|, u = 2^-24.  Lookups of short
+rows, and results just below and above the size at which several replicas are written element by element."""
 import numpy as np
 import pytest
 import torch
@@ -47,3 +48,19 @@ def test_lookup_of_short_rows_to_several_replicas(dtype, dim, lookups):
     sbp.sbp_embedding(table, make_global([ids] * k, (lookups,), I64, sbp.B), out)
     for t in out.locals:
         assert torch.equal(t.cpu(), T[ids])
+
+
+@pytest.mark.parametrize("lookups", [292968, 292969, 300001])
+def test_large_results_to_four_replicas(lookups):
+    rows, dim, k = 3001, 128, 4
+    T = torch.randn(rows, dim, device="cuda")
+    ids = torch.randint(0, rows, (lookups,), device="cuda")
+    ids[5] = rows
+    oob = torch.zeros(1, dtype=torch.int32, device="cuda")
+    table = sbp.SbpTensor((rows, dim), F32, sbp.S(0), [t.contiguous() for t in torch.tensor_split(T, k, 0)])
+    out = sbp.empty_global((lookups, dim), F32, sbp.B, k)
+    sbp.sbp_embedding(table, sbp.SbpTensor((lookups,), I64, sbp.B, [ids] * k), out, oob)
+    want = torch.cat([T, torch.zeros(1, dim, device="cuda")])[ids]
+    assert int(oob.item()) == 1
+    for t in out.locals:
+        assert torch.equal(t, want)
