@@ -617,7 +617,7 @@ static sbp_status make_plan(const sbp_tensor* src, const sbp_tensor* dst, int ds
   pl->shift = false;
   pl->copy_j = shift_copy_j(p.esz, p.n_dst, numel(src));
   if (p.mode != MODE_SCATTER_P && src->dtype == dst->dtype &&
-      shift_pays(pl->op == OP_COPY, p.esz, pl->vbytes, k, p.n_dst, seg_bytes_max, numel(src))) {
+      shift_pays(pl->op == OP_COPY, true, p.esz, pl->vbytes, k, p.n_dst, seg_bytes_max, numel(src))) {
     bool ok = true;
     for (int q = 1; q < p.n_dst; ++q)
       ok = ok && (reinterpret_cast<uintptr_t>(p.dst[q]) - reinterpret_cast<uintptr_t>(p.dst[0])) % 16 == 0;

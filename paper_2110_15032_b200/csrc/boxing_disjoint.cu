@@ -461,7 +461,7 @@ sbp_status boxing_disjoint(const sbp_tensor* src, sbp_tensor* dst, int dst_shard
   p.tiles_per_task = p.col_tiles * row_tiles;
   long long grid = p.tiles_per_task * p.ntasks;
   // unaligned data in 16-byte vectors, by the rule of the same-placement kernels
-  bool shift = shift_pays(op == OP_COPY, esz, vbytes, ks, p.n_dst, seg_bytes_max, numel(src));
+  bool shift = shift_pays(op == OP_COPY, false, esz, vbytes, ks, p.n_dst, seg_bytes_max, numel(src));
   p.shift_copy_j = shift_copy_j(esz, p.n_dst, numel(src));
   if (op != OP_COPY)
     for (int r = 1; r < ks; ++r)

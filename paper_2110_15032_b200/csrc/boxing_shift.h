@@ -49,29 +49,48 @@ constexpr int shift_j(int kb) { return kb == 2 ? 4 : 2; }
 // shapes (us, element-wise tiles / this path):
 //   copies      segments of 32 elements and more, 64 where several destinations take four vectors a thread: i64 [200001, 33]
 //               over three S(1) -> S(0), segments of 11, 38 / 144, [129, 65, 97] over eight S(0) -> S(2), of 12, 8.2 / 20; over
-//               three, of 32, 11.3 / 7.5
-//   reductions  of up to four sources the same; of more, 48 elements: bf16 [50, 200, 301] over eight P(sum) -> S(2), of 38,
-//               33 / 45, over six, of 50, 31 / 27.  More than four sources whose segments are long keep the tiles' loads in
-//               flight (one position, all sources) up to 1.2 M elements: [513, 1025] over eight P(sum) -> B 4.4 / 7.1, [1021,
-//               1537] bf16 11.8 / 9.7; and fp32 sums that go to several destinations at any size: [200001, 33] 65 / 71
+//               three, of 32, 11.3 / 7.5.  Aligned pairs in segments of up to 32 of them fill half a row of a tile and stay
+//               there: [20001, 100] over two S(0) -> S(1), bf16 5.5 / 11.2, fp32 5.5 / 11.6
+//   reductions  of one placement keep the tiles up to 64 units (what a tile moves per access) a segment, which is one pass of a
+//               row: [50, 200, 100] bf16 over two P(sum) -> S(2) 4.7 / 13.6, [60001, 127] 42 / 67, [50, 200, 301] over five 21 / 24,
+//               over eight 33 / 45, of 65 units 62 / 50; the same with 120 to 128 units of pairs (fp32 [50, 100, 500] over two 7.5 /
+//               11.0).  Three sources, and the last three of seven, the tiles read one after the other, and are slower: fp32
+//               [50, 200, 301] over seven 38 / 33, [50, 200, 106] over three 12.3 / 10.6.
+//               The eight sources of one placement they read all at once: long segments pay only from 1.2 M elements on
+//               ([513, 1025] P(sum) -> B 4.4 / 7.1, [1021, 1537] bf16 11.8 / 9.7), and never in fp32 pairs ([50, 100, 2000] 52 / 66)
+//               or 4 bytes and more that go to several destinations ([200001, 33] 65 / 71, bf16 [1429, 4726] 35 / 42)
+//               Between different placements the tiles read a few sources at a time as well and only two keep them: bf16
+//               [50, 200, 306] over two to three 17 / 19, over eight to seven, of 38, 45 / 40; [4095, 8193] over five to two 320 / 144
 //   where the tiles move several elements an access they are as good: up to 1.2 M bf16 or fp32 elements ([60, 8001] bf16
-//               P(sum) -> B over three 2.6 / 3.8), and 8 bytes an access are enough for i64 gathers to few replicas unless the rows are short and many
-//               ([1021, 1537] over three S(0) -> B 7.4 / 8.1, S(1) -> B 12 / 9.4)
-// Below 400 000 elements (500 000 of more than four sources) a call is all latency: bf16 [60, 8001] takes 2.0-3.1 us either way, fp32 [100, 777] 1.2 us element
-// by element and 1.6-2.9 in shifted vectors.
+//               P(sum) -> B over three 2.6 / 3.8), and 8 bytes an access are enough for i64 gathers to few replicas unless
+//               the rows are short and many ([1021, 1537] over three S(0) -> B 7.4 / 8.1, S(1) -> B 12 / 9.4)
+// Below 400 000 elements (500 000 of those eight sources, 800 000 of more than four sources and eight destinations: [513, 1025]
+// over eight to nine P(sum) -> B 6.2 / 8.4) a call is all latency: bf16 [60, 8001] takes 2.0-3.1 us either way, fp32 [100, 777]
+// 1.2 us element by element and 1.6-2.9 in shifted vectors.
+// same: one placement on both sides.
 // vbytes: what the tiles would move per access.
-inline bool shift_pays(bool copy, int esz, int vbytes, int k, int n_dst, long long seg_bytes, long long elements) {
+inline bool shift_pays(bool copy, bool same, int esz, int vbytes, int k, int n_dst, long long seg_bytes, long long elements) {
   const long long seg = seg_bytes / esz;
-  const bool few = copy || k <= 4, small = elements < 1200000;
-  if (vbytes >= 16 || elements < (few ? 400000 : 500000) || seg < (few ? 32 : 48)) return false;
+  const long long units = seg_bytes / vbytes;
+  const bool eight = !copy && same && k == 8, small = elements < 1200000;
+  if (vbytes >= 16 || elements < (eight ? 500000 : 400000) || seg < 32) return false;
+  if (copy) {
+    if (vbytes > esz && units <= 32) return false;
+  } else if (!same) {
+    if (units <= 64 && k == 2) return false;
+  } else {
+    const bool one_by_one = k % 4 == 3 && (vbytes == esz ? k == 3 || esz > 2 : units > 32 && units <= 56);
+    if ((units <= 64 && !one_by_one) || (vbytes > esz && units > 120 && units <= 128)) return false;
+    if (eight && esz == 4 && vbytes == 8) return false;
+  }
   if (esz < 8 && vbytes > esz && small) return false;
   if (copy) {
     if (n_dst > 1 && seg < 64 && shift_copy_j(esz, n_dst, elements) > 1) return false;
     if (esz < 8 || n_dst <= 1 || n_dst >= 8) return true;
     return n_dst >= 4 ? seg < (1 << 17) || elements < 800000 : seg < 2048 || (seg < (1 << 17) && elements >= 2000000);
   }
-  if (k <= 4 || seg < 4096) return true;
-  return !small && !(esz == 4 && n_dst > 1);
+  if (!eight) return k <= 4 || n_dst < 8 || elements >= 800000;
+  return seg < 4096 || (!small && !(vbytes >= 4 && n_dst > 1));
 }
 
 // CTAs per SM the registers are held to (P(sum) -> S(1), us with 2 / 3 / 4: bf16 [1429, 4727] over two shards, four

@@ -1,5 +1,5 @@
 """Boxing of unaligned data on either side of the lines at which it takes the shifted 16-byte path, and with one vector a
-thread (several destinations) or four: segments of 31 to 33 and 47 to 49 elements, tensors just below and above the element
+thread (several destinations) or four: segments of 31 to 33 and 47 to 49 elements and of few aligned pairs, tensors just below and above the element
 counts, destinations that are one buffer or many.  Bit-exact against the oracle."""
 import pytest
 import torch
@@ -24,14 +24,26 @@ def test_short_segments(cols, dtype):
 @pytest.mark.parametrize("dtype", [F32, BF16])
 def test_short_segments_of_many_sources(cols, dtype):
     _run((1901, cols), dtype, P, S1, 5)
+    _run((1201, cols * 8 // 5), dtype, P, S1, 8)
     run_disjoint((1901, cols), dtype, P, S1, 6, 5)
 
 
-@pytest.mark.parametrize("shape", [(631, 633), (635, 637), (1093, 1095), (1097, 1099)])
+@pytest.mark.parametrize("units", [31, 33, 55, 57, 63, 65, 119, 121, 129])
+@pytest.mark.parametrize("dtype", [F32, BF16])
+def test_rows_of_few_pairs(units, dtype):
+    for k in (2, 3, 7, 8):
+        rows = 1300000 // (2 * units * k) + 1
+        _run((rows, 2 * units * k), dtype, P, S1, k)
+        _run((rows, 2 * units * k), dtype, S0, S1, k)
+
+
+@pytest.mark.parametrize("shape", [(631, 633), (635, 637), (893, 895), (895, 899), (1093, 1095), (1097, 1099)])
 @pytest.mark.parametrize("dtype", [F32, BF16])
 def test_element_counts(shape, dtype):
-    _run(shape, dtype, P, B, 5)
-    _run(shape, dtype, P, S0, 5)
+    for k in (5, 8):
+        _run(shape, dtype, P, B, k)
+        _run(shape, dtype, P, S0, k)
+    run_disjoint(shape, dtype, P, B, 5, 9)
     _run(shape, dtype, S0, B, 5)
 
 
