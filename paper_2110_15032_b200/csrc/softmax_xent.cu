@@ -86,8 +86,7 @@ __device__ __forceinline__ void write_row(const XentCombineParams& p, long long 
 }
 
 // The (m, s) pairs of a warp's lanes into one, the same in all of them: the maximum first, then every sum rescaled once.
-// (Merging pair by pair rescales a sum at every level, and the unit's exponentials are 5e-8 low on the average: sums of
-// PAIRWISE.)
+// (Merging pair by pair rescales a sum at every level, and the unit's exponentials are 5e-8 low on the average.)
 __device__ __forceinline__ void merge_warp(float& m, float& s) {
   float top = m;
 #pragma unroll
@@ -154,6 +153,20 @@ struct ChunkBF16 {
     }
     return s0 + s1;
   }
+  // sum of 2^((z - m) log2e): exact in m, finite for every finite z
+  __device__ __forceinline__ float expsum_far(float m) const {
+    float s = 0.f;
+#pragma unroll
+    for (int u = 0; u < kLoadsPerThread; ++u) {
+      const uint32_t* w = reinterpret_cast<const uint32_t*>(&raw[u]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        s += ex2((__uint_as_float(w[i] << 16) - m) * kLog2e);
+        s += ex2((__uint_as_float(w[i] & 0xffff0000u) - m) * kLog2e);
+      }
+    }
+    return s;
+  }
 };
 
 // fp32, 4 elements per load.
@@ -191,6 +204,16 @@ struct ChunkF32 {
     }
     return s0 + s1;
   }
+  __device__ __forceinline__ float expsum_far(float m) const {
+    float s = 0.f;
+#pragma unroll
+    for (int u = 0; u < kLoadsPerThread; ++u) {
+      const float* f = reinterpret_cast<const float*>(&raw[u]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) s += ex2((f[i] - m) * kLog2e);
+    }
+    return s;
+  }
 };
 
 // Elements before the first 16-byte boundary at or after z, at most n.
@@ -207,7 +230,11 @@ __device__ __forceinline__ int to_boundary(const T* z, long long n) {
 // over four shards 33 us, backward 76; as here 25 and 35: 0.62 and 0.89 of the copy bandwidth.)
 // An exponential is 2^(z log2e - c), c = m log2e rounded: one FMA an element.  What the rounding of c leaves, r = m log2e - c,
 // is a factor 2^r on all that the thread adds up in a chunk, up to 3e-7 at a maximum of 8; it is taken out of the chunk's
-// sum.  What is carried from chunk to chunk is rescaled by the difference of the maxima: exactly 1 while the maximum stands.
+// sum, to first order, which is enough (1e-9) up to a maximum of kNear; beyond that, where r grows to many units -- rows
+// masked with -1e9 and the like -- every exponent is formed from z - m.
+// What is carried from chunk to chunk is rescaled by the difference of the maxima: exactly 1 while the maximum stands.
+constexpr float kNear = 1024.f;
+
 template <typename Chunk>
 __device__ __forceinline__ void walk_span(const typename Chunk::T* z, long long n, int tid, int team, float& m, float& s) {
   using T = typename Chunk::T;
@@ -229,10 +256,14 @@ __device__ __forceinline__ void walk_span(const typename Chunk::T* z, long long 
     if (more) nxt.load(zv + (off + step) * VEC, nv - off - step, tid, team);
     const float cm = cur.max();
     if (cm != -INFINITY) {                                      // not the threads of a short row that have nothing
-      const float mm = fmaxf(m, cm), c = fmaxf(mm * kLog2e, -3.4e38f);      // finite under masks of the type's lowest value
+      const float mm = fmaxf(m, cm), c = mm * kLog2e;
       const float carried = s * ex2((m - mm) * kLog2e);         // s is 0 as long as m is -inf
-      const float sum = cur.expsum(-c);
-      s = carried + fmaf(sum, -0.69314718f * fmaf(mm, kLog2e, -c), sum);
+      if (fabsf(mm) <= kNear) {
+        const float sum = cur.expsum(-c);
+        s = carried + fmaf(sum, -0.69314718f * fmaf(mm, kLog2e, -c), sum);
+      } else {
+        s = carried + cur.expsum_far(mm);
+      }
       m = mm;
     }
     if (more) cur = nxt;
@@ -334,7 +365,7 @@ __global__ void __launch_bounds__(THREADS) xent_partial_kernel(const __grid_cons
   }
 }
 
-// Short rows get no more threads than there are vectors (fp32 [700, 100] over four S256 us with 256 threads, S32 with 32).
+// Short rows get no more threads than there are vectors (fp32 [700, 100] over four 11.0 us with 256 threads, 6.1 with 32).
 template <typename Chunk>
 static void launch_partial(const XentParams& p, dim3 grid, long long widest, cudaStream_t st) {
   const long long vectors = (widest + Chunk::VEC - 1) / Chunk::VEC;
@@ -597,9 +628,10 @@ __global__ void __launch_bounds__(kThreads) xent_backward_kernel(const __grid_co
   T* g = reinterpret_cast<T*>(p.grad[shard]) + row * p.gpitch[shard];
   SBP_PDL_RELEASE();
   SBP_PDL_WAIT();
-  // softmax = 2^(z log2e - m log2e - log2 S): the division by the row sum is folded into the exponent
+  // softmax = 2^((z - m) log2e - log2 S): the division by the row sum is folded into the exponent, and z - m keeps it exact
+  // at any maximum
   if (!SBP_GUARD(p.row_max + row, 4) || !SBP_GUARD(p.row_sum + row, 4) || !SBP_GUARD(p.labels + row, 8)) return;
-  const float neg = -p.row_max[row] * kLog2e - log2f(p.row_sum[row]);
+  const float m = p.row_max[row], neg = -log2f(p.row_sum[row]);
   const long long y = p.labels[row] - c_start;      // label's column inside this shard, if any
   const int head = VEC > 1 ? to_boundary(z, c_len) : 0;
   const long long nv = (c_len - head) / VEC;
@@ -608,7 +640,7 @@ __global__ void __launch_bounds__(kThreads) xent_backward_kernel(const __grid_co
   if (VEC > 1 && blockIdx.y == 0) {
     const long long at = tid < head ? tid : (tid >= 16 && tid - 16 < tail ? head + nv * VEC + (tid - 16) : -1);
     if (at >= 0 && SBP_GUARD(z + at, sizeof(T)) && SBP_GUARD(g + at, sizeof(T))) {
-      float v = ex2(fmaf(static_cast<float>(z[at]), kLog2e, neg));
+      float v = ex2(fmaf(static_cast<float>(z[at]) - m, kLog2e, neg));
       if (at == y) v -= 1.0f;
       g[at] = static_cast<T>(v);
     }
@@ -634,7 +666,7 @@ __global__ void __launch_bounds__(kThreads) xent_backward_kernel(const __grid_co
       Pack out;
 #pragma unroll
       for (int i = 0; i < VEC; ++i) {
-        float f = ex2(fmaf(static_cast<float>(in[u].e[i]), kLog2e, neg));
+        float f = ex2(fmaf(static_cast<float>(in[u].e[i]) - m, kLog2e, neg));
         if (i == y_rel) f -= 1.0f;
         out.e[i] = static_cast<T>(f);
       }

@@ -61,3 +61,30 @@ def test_infinities_and_nan_reach_the_loss():
         loss = _forward(part, 2)[0]
         bad = torch.isnan(loss) | torch.isinf(loss)
         assert bool(bad[7]) and bool(bad[8]) and not bool(bad[9]) and int(bad[:100].sum()) == 2
+
+
+@pytest.mark.parametrize("top", [3e4, 1e6, -3e4, -1e8, -1e9, -1e10, -1e20, -1e30, None])
+@pytest.mark.parametrize("rows,classes,k", [(40, 1000, 2), (300, 20001, 4), (4000, 515, 2)])
+@pytest.mark.parametrize("dtype", [F32, BF16])
+def test_maxima_of_any_size(top, rows, classes, k, dtype):
+    """Rows wholly at one value, as a padded row under a mask is: the sum is the class count and the gradient 1 / classes; and
+    the same rows with half of their classes lower by a few units in the last place, or by ln 2 where those are finer."""
+    v = torch.tensor(torch.finfo(dtype).min if top is None else top, dtype=dtype, device="cuda")
+    Z = v.expand(rows, classes).clone()
+    step = max(0.6931471805599453, float(v.abs()) * 2.0 ** (-22 if dtype == F32 else -6))
+    Z[rows // 2:, ::2] = v.float() * 1.0 - step if top is not None else v
+    Zd = Z.double()
+    E = torch.exp(Zd - Zd.max(1, keepdim=True)[0])
+    want = E.sum(1)
+    loss, m, s = _forward(Z, k)
+    assert torch.equal(m.double(), Zd.max(1)[0])
+    assert float(((s.double() - want) / want).abs().max()) <= 2.0 ** -21
+    z = sbp.SbpTensor((rows, classes), dtype, sbp.S(1), [t.contiguous() for t in torch.tensor_split(Z, k, 1)])
+    lab = sbp.SbpTensor((rows,), torch.int64, sbp.B, [torch.zeros(rows, dtype=torch.int64, device="cuda")] * k)
+    rm, rs = (sbp.SbpTensor((rows,), F32, sbp.B, [t] * k) for t in (m, s))
+    g = sbp.empty_global((rows, classes), dtype, sbp.S(1), k)
+    sbp.sbp_softmax_xent_backward(z, lab, rm, rs, g)
+    G = torch.cat(g.locals, 1).double()
+    ref = E / want[:, None]
+    ref[:, 0] -= 1.0
+    assert float((G - ref).abs().max()) <= (2.0 ** -20 if dtype == F32 else 2.0 ** -8)
