@@ -42,6 +42,7 @@
 #include "bounds_check.h"
 #include "matmul_plan.h"
 #include "sbp_internal.h"
+#include "tc_ptx.h"
 
 namespace sbp {
 
@@ -80,9 +81,6 @@ static_assert(kStagesShort * kStageBytes + kEpiWarps * kEpiBufsShort * kSlabByte
 constexpr int kMaxStages = kStages > kStagesTall ? kStages : kStagesTall;
 constexpr int kThreadsTc = 32 * (2 + kEpiWarps);
 constexpr int kTmemCols = 512;
-constexpr unsigned long long kWaitLimitNs = 2000000000ull;
-
-__device__ int g_tc_timeout_flag = 0;
 
 struct TcParams {
   CUtensorMap map_a[SBP_MAX_K];
@@ -113,167 +111,6 @@ struct TcParams {
   long long ldy[SBP_MAX_K];
 };
 
-// ------------------------------------------------------------------ PTX helpers
-
-__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ unsigned long long now_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-__device__ __forceinline__ void mbar_init(unsigned bar, unsigned count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-
-// One try_wait with a suspend-time hint: the thread sleeps in hardware until the phase completes
-// or the hint (in ns) runs out, instead of spinning and taking issue slots and power from the
-// tensor pipe (measured: +8 % MatMul throughput against a bare polling loop).
-__device__ __forceinline__ bool mbar_try(unsigned bar, unsigned parity) {
-  unsigned done;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 0x10000;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(done)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return done != 0;
-}
-
-// Bounded wait.  Returns false (and raises the abort flag) when the limit expires.
-__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, volatile int* abort_flag) {
-  if (mbar_try(bar, parity)) return true;
-  const unsigned long long t0 = now_ns();
-  for (;;) {
-    if (mbar_try(bar, parity)) return true;
-    if (*abort_flag) return false;
-    if (now_ns() - t0 > kWaitLimitNs) {
-      *abort_flag = 1;
-      atomicExch(&g_tc_timeout_flag, 1);
-      return false;
-    }
-  }
-}
-
-// The same wait made by a whole converged warp; the answer is the same in all of its lanes.
-__device__ __forceinline__ bool mbar_wait_warp(unsigned bar, unsigned parity, volatile int* abort_flag) {
-  if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag)) != 0;
-}
-
-// One lane of a converged warp, the same one every time.
-__device__ __forceinline__ bool elect_one() {
-  unsigned p;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
-  return p != 0;
-}
-
-__device__ __forceinline__ void mbar_expect_tx(unsigned bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(unsigned bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
-// Address of the same shared-memory object in CTA `rank` of this cluster.
-__device__ __forceinline__ unsigned map_to_cta(unsigned addr, unsigned rank) {
-  unsigned r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-
-// Arrive on an mbarrier that may live in the partner CTA (cluster-space address).  The arrive
-// carries the default (CTA-scope) release: what it hands over is tensor memory whose reads have
-// completed (tcgen05.wait::ld, then tcgen05.fence::before_thread_sync), not data in memory, and a
-// cluster-scope release here cost every epilogue warp some thousand clocks per tile (fused
-// classifier forward 0.472 -> 0.450 ms, backward 0.577 -> 0.533 ms).
-__device__ __forceinline__ void mbar_arrive_cluster(unsigned cluster_addr) {
-  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-
-__device__ __forceinline__ unsigned cluster_ctarank() {
-  unsigned r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-}
-
-// TMA load into this CTA's shared memory; the byte count is credited to `bar`, which may be the
-// partner CTA's barrier (pair form of the instruction; no multicast).
-__device__ __forceinline__ void tma_load_2d(unsigned dst, const CUtensorMap* map, int x, int y, unsigned bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-      "l"(map), "r"(x), "r"(y), "r"(bar)
-      : "memory");
-}
-
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int x, int y, unsigned src) {
-  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(map), "r"(x),
-               "r"(y), "r"(src)
-               : "memory");
-}
-
-// One MMA across the CTA pair: D[256 x 256] (+)= A[256 x 16] * B[16 x 256].
-__device__ __forceinline__ void umma_bf16(unsigned d_tmem, unsigned long long a_desc, unsigned long long b_desc,
-                                          unsigned idesc, unsigned accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-// Arrives on the barrier at this offset in BOTH CTAs of the pair once every tcgen05 operation
-// issued so far by this thread is done.  (mask: the pair's two CTAs inside the cluster.)
-__device__ __forceinline__ void umma_commit_pair(unsigned bar, unsigned short mask = 3) {
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-               "h"(mask)
-               : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld8(unsigned taddr, float* v) {
-  unsigned* r = reinterpret_cast<unsigned*>(v);
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr)
-               : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld32(unsigned taddr, float* v) {
-  unsigned* r = reinterpret_cast<unsigned*>(v);
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr)
-      : "memory");
-}
-
-// Shared-memory matrix descriptor, 128-byte swizzle (lbo / sbo in bytes): bits 0-13 start address
-// >> 4, bits 16-29 lbo >> 4, bits 32-45 sbo >> 4, bit 46 the descriptor version of this architecture,
-// bits 61-63 = 2 the 128-byte swizzle.  It is handled in two parts: what never changes (the high
-// word, and the leading-dimension field of the low word) and the start-address field, so that the
-// MMA-issuing thread builds a descriptor with one add and one register pair.
-__host__ __device__ constexpr unsigned desc_lo_fixed(unsigned lbo) { return (lbo >> 4) << 16; }
-__host__ __device__ constexpr unsigned desc_hi_fixed(unsigned sbo) { return (sbo >> 4) | (1u << 14) | (2u << 29); }
-__device__ __forceinline__ unsigned long long desc_pack(unsigned lo, unsigned hi) {
-  unsigned long long d;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi));
-  return d;
-}
-
 // Instruction descriptor: D fp32, A and B bf16, M = 256 (pair), N = `n`.  Bit 15 / bit 16 say
 // that A / B lies in shared memory with its M / N index contiguous ("MN-major") instead of its
 // K index.  Operands as given: A [M,K] row-major is K-major, B [K,N] row-major is N-major; a
@@ -283,24 +120,53 @@ __host__ __device__ constexpr unsigned make_idesc(int a_trans, int b_trans, int 
   return kIdescBase | ((unsigned)(n >> 3) << 17) | ((a_trans ? 1u : 0u) << 15) | ((b_trans ? 0u : 1u) << 16);
 }
 
-// erf by the rational approximation 7.1.26 of Abramowitz & Stegun (|error| <= 1.5e-7), which is
-// far below the rounding of the bf16 / fp32 store that follows and costs two special-function
-// operations where erff costs a long polynomial.
-__device__ __forceinline__ float erf_as(float x) {
-  const float ax = fabsf(x);
-  float t;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(0.3275911f, ax, 1.0f)));
-  float poly = fmaf(1.061405429f, t, -1.453152027f);
-  poly = fmaf(poly, t, 1.421413741f);
-  poly = fmaf(poly, t, -0.284496736f);
-  poly = fmaf(poly, t, 0.254829592f);
-  poly *= t;
-  float e;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(-ax * ax * 1.4426950408889634f));
-  return copysignf(fmaf(-poly, e, 1.0f), x);
+// Two numbers in one register pair.
+__device__ __forceinline__ unsigned long long two(float x, float y) {
+  unsigned long long v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
+  return v;
+}
+__device__ __forceinline__ unsigned long long two(float x) { return two(x, x); }
+__device__ __forceinline__ unsigned long long fma_two(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long v;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
+  return v;
+}
+__device__ __forceinline__ unsigned long long mul_two(unsigned long long a, unsigned long long b) {
+  unsigned long long v;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+  return v;
 }
 
-__device__ __forceinline__ float gelu_erf_tc(float v) { return 0.5f * v * (1.0f + erf_as(v * 0.70710678118654752440f)); }
+// GeLU of two numbers, erf by the rational approximation 7.1.26 of Abramowitz & Stegun (|error| <= 1.5e-7), which is far
+// below the rounding of the bf16 / fp32 store that follows and costs two special-function operations where erff costs a
+// long polynomial.  With erf |z| = 1 - q(z), 0.5 v (1 + erf(v / sqrt 2)) = max(v, 0) - 0.5 |v| q: ten instructions a
+// number, the multiply-adds in pairs, where erf by itself and one number at a time took twenty.  The epilogue of a tile
+// that nothing overlaps is these instructions.
+// (|v| stops at 32, where q is 0, so that infinity stays infinity; NaN stays NaN.)
+__device__ __forceinline__ void gelu_two(float& a, float& b) {
+  float ua, ub, pa, pb, ta, tb, ea, eb;
+  asm("min.NaN.f32 %0, %1, 0f42000000;" : "=f"(ua) : "f"(a));
+  asm("min.NaN.f32 %0, %1, 0f42000000;" : "=f"(ub) : "f"(b));
+  asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(pa) : "f"(a));
+  asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(pb) : "f"(b));
+  const unsigned long long u = two(fabsf(ua), fabsf(ub));
+  const unsigned long long d = fma_two(u, two(0.3275911f * 0.70710678118654752440f), two(1.0f));
+  const unsigned long long x = mul_two(mul_two(u, two(-0.72134752044448170368f)), u);      // -(v / sqrt 2)^2 log2 e
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ta) : "f"(__uint_as_float((unsigned)d)));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(tb) : "f"(__uint_as_float((unsigned)(d >> 32))));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ea) : "f"(__uint_as_float((unsigned)x)));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(eb) : "f"(__uint_as_float((unsigned)(x >> 32))));
+  const unsigned long long t = two(ta, tb);
+  unsigned long long q = fma_two(t, two(-0.5f * 1.061405429f), two(0.5f * 1.453152027f));      // -0.5 q
+  q = fma_two(q, t, two(-0.5f * 1.421413741f));
+  q = fma_two(q, t, two(0.5f * 0.284496736f));
+  q = fma_two(q, t, two(-0.5f * 0.254829592f));
+  q = mul_two(mul_two(q, t), two(ea, eb));
+  const unsigned long long v = fma_two(u, q, two(pa, pb));
+  a = __uint_as_float((unsigned)v);
+  b = __uint_as_float((unsigned)(v >> 32));
+}
 
 struct TileCoord {
   int g, m0, n0;
@@ -694,8 +560,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
             float e;
             asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(fmaf(x, 1.4426950408889634f, g_neg)));
             return e;          // the label's column gets its -1 below, outside the per-element path
-          } else if constexpr (MODE == 1) {
-            return gelu_erf_tc(x);
           } else {
             return x;
           }
@@ -718,6 +582,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
 #pragma unroll
               for (int c = 0; c < 8; ++c) {
                 float4 o;
+                if constexpr (MODE == 1) {
+                  gelu_two(v[4 * c], v[4 * c + 1]);
+                  gelu_two(v[4 * c + 2], v[4 * c + 3]);
+                }
                 o.x = xform(v[4 * c + 0], 4 * c + 0); o.y = xform(v[4 * c + 1], 4 * c + 1);
                 o.z = xform(v[4 * c + 2], 4 * c + 2); o.w = xform(v[4 * c + 3], 4 * c + 3);
                 *reinterpret_cast<float4*>(rowp + ((c ^ (lane & 7)) << 4)) = o;
@@ -728,6 +596,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
                 float f[8];
 #pragma unroll
                 for (int e = 0; e < 8; ++e) f[e] = xform(v[8 * c + e], 8 * c + e);
+                if constexpr (MODE == 1) {
+#pragma unroll
+                  for (int e = 0; e < 8; e += 2) gelu_two(f[e], f[e + 1]);
+                }
                 uint4 o;
                 __nv_bfloat162 h;
                 h = __floats2bfloat162_rn(f[0], f[1]); o.x = *reinterpret_cast<unsigned*>(&h);
@@ -1087,7 +959,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) matmul_tc_split_kernel(const __
       }
       if (p.gelu) {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = gelu_erf_tc(v[e]);
+        for (int e = 0; e < 8; e += 2) gelu_two(v[e], v[e + 1]);
       }
       const int cc = (c - lo) * 8;
       if constexpr (SW) {
@@ -1226,7 +1098,7 @@ __global__ void __launch_bounds__(256) matmul_parts_kernel(const __grid_constant
     float f[4] = {v.x, v.y, v.z, v.w};
     if (p.gelu) {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) f[e] = gelu_erf_tc(f[e]);
+      for (int e = 0; e < 4; e += 2) gelu_two(f[e], f[e + 1]);
     }
     const int n_out = (g == 0 ? p.n_rep : 0) + 1;
     for (int o = 0; o < n_out; ++o) {
@@ -2403,12 +2275,6 @@ bool matmul_tc_room(const MatmulPlan& plan, size_t* room) {
   return run_matmul_tc(plan, nullptr, nullptr, ~size_t(0), nullptr, &taken, room) == SBP_OK && taken;
 }
 
-sbp_status read_and_clear_tc_timeout(bool* timed_out) {
-  int flag = 0, zero = 0;
-  SBP_CUDA_TRY(cudaMemcpyFromSymbol(&flag, g_tc_timeout_flag, sizeof(int)));
-  if (flag) SBP_CUDA_TRY(cudaMemcpyToSymbol(g_tc_timeout_flag, &zero, sizeof(int)));
-  *timed_out = flag != 0;
-  return SBP_OK;
-}
+sbp_status read_and_clear_tc_timeout(bool* timed_out) { return read_and_clear_timeout_flag(timed_out); }
 
 }  // namespace sbp
