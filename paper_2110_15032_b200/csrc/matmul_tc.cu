@@ -299,17 +299,24 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  cluster_sync_all();                            // both CTAs' barriers exist before anyone signals them
+  cluster_arrive();
+  const int first = blockIdx.x >> 1, stride = gridDim.x >> 1;   // tiles are dealt to CTA pairs
+  TileCoord tc = tile_coord(p, first);
+  if (warp == 2 && lane == 0) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&p.map_a[p.chain ? 0 : tc.g]) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&p.map_b[p.chain ? 0 : tc.g]) : "memory");
+    if (p.xent != 1 && !p.y_direct) asm volatile("prefetch.tensormap [%0];" ::"l"(&p.map_y[tc.g]) : "memory");
+  }
+  cluster_wait();                                // both CTAs' barriers exist before anyone signals them
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const unsigned tmem_base = tmem_base_slot;
   // A kernel launched behind this one as its programmatic dependent may be set up from here on;
   // it waits on the device for this grid to finish before it reads what this grid writes.  This
   // kernel is launched the same way: barriers and TMEM are set up under the end of the kernel before.
   SBP_PDL_RELEASE();
+  // The first tile's place and descriptors are there before the wait: the first operands land 1.25 us after it, 2.2 to 2.9
+  // where both came after it (500 x 1024 x 1024 over eight devices; 2048 x 1024 x 4096 2.2, 3.3).
   SBP_PDL_WAIT();
-
-  const int first = blockIdx.x >> 1, stride = gridDim.x >> 1;   // tiles are dealt to CTA pairs
 
   if (warp == 0) {
     // ------------------------------------------------ producer (both CTAs)
@@ -328,7 +335,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
     int slot = 0;
     unsigned round = 0;
     for (int tile = first; tile < p.total_tiles; tile += stride) {
-      const TileCoord tc = tile_coord(p, tile);
+      if (tile != first) tc = tile_coord(p, tile);
       const int s_lo = p.chain ? 0 : tc.g, s_hi = p.chain ? p.nseg : tc.g + 1;
       for (int s = s_lo; s < s_hi; ++s) {
         const int nkb = p.kblocks[s];
@@ -384,7 +391,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
       int tile_iter = 0;
       constexpr unsigned idesc = make_idesc(AT, BT);
       for (int tile = first; tile < p.total_tiles; tile += stride, ++tile_iter) {
-        const TileCoord tc = tile_coord(p, tile);
+        if (tile != first) tc = tile_coord(p, tile);
         // Square form: the two accumulators take turns, so a tile's MMAs run while the tile before
         // it is drained.  Tall form: accumulator h belongs to m-half h of every tile; the first
         // m-half may start as soon as ITS accumulator has been drained, the second waits for its own.
@@ -458,7 +465,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
     unsigned slab_iter = 0;
     for (int tile = first; tile < p.total_tiles; tile += stride, ++tile_iter) {
       if (*abort_flag) break;
-      const TileCoord tc = tile_coord(p, tile);
+      if (tile != first) tc = tile_coord(p, tile);
       const int facc = MH == 2 ? 0 : (tile_iter & 1);
       bool ok = true;
       if (lane == 0)
@@ -672,14 +679,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
       if (lane == 0) mbar_arrive_cluster(acc_empty0[acc]);   // tells CTA 0's MMA thread
       }
     }
+    // done with tensor memory and barriers; what is left is the stores
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncwarp();
+    cluster_arrive();
     if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    __syncwarp();
+    cluster_wait();
+    return;
   }
 
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  cluster_sync_all();          // the partner may still signal this CTA's barriers or read its tiles
+  __syncwarp();
+  cluster_arrive();
+  cluster_wait();              // the partner may still signal this CTA's barriers or read its tiles
   if (warp == 1) {
-    __syncwarp();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
   }
@@ -767,7 +781,9 @@ __global__ void __launch_bounds__(kThreadsTc, 1) matmul_tc_split_kernel(const __
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
-  // this cluster's tile and this pair's range of its K-blocks
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncwarp();
+  cluster_arrive();            // and under this barrier: this cluster's tile and this pair's range of its K-blocks
   const int cluster = (int)(blockIdx.x / (unsigned)(2 * S)), part = p.outer > 1 ? cluster / p.tiles : 0;
   const int tile = cluster - part * p.tiles;
   int g = 0;
@@ -783,9 +799,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) matmul_tc_split_kernel(const __
     asm volatile("prefetch.tensormap [%0];" ::"l"(&p.map_a[s_lo]) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&p.map_b[s_lo]) : "memory");
   }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  cluster_sync_all();
+  cluster_wait();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const unsigned tmem_base = tmem_base_slot;
   bool ok = true;
@@ -933,35 +947,19 @@ __global__ void __launch_bounds__(kThreadsTc, 1) matmul_tc_split_kernel(const __
   int lo, hi;
   mine(slice, &lo, &hi);
   const int col0 = n0 + (slice * per + lo) * 8;
-  if (rows_live && ok && lo < hi && col0 < Ng) {
-    const int esz = p.out_f32 ? 4 : 2, cols = (hi - lo) * 8;
+  const bool mine_live = rows_live && ok && lo < hi && col0 < Ng;      // warp-uniform
+  const int esz = p.out_f32 ? 4 : 2, cols = (hi - lo) * 8;
+  const int pitch = SW ? 32 * esz : cols * esz + 16;
+  unsigned char* stage = smem + (S - 1) * per * (BMH * 32) + (warp - 2) * (32 * ((per + 1) / 2 * 8 * esz + 16));
+  if (mine_live) {
     // Staged per warp as rows of the RESULT: 32 rows of `cols` elements, 16 bytes apart so that 32 rows written at
     // once spread over the banks (SW: `cols` rows of 32 elements).
-    const int pitch = SW ? 32 * esz : cols * esz + 16;
-    unsigned char* stage = smem + (S - 1) * per * (BMH * 32) + (warp - 2) * (32 * ((per + 1) / 2 * 8 * esz + 16));
-    for (int c = lo; c < hi; ++c) {
-      float v[8], own[8];
-      tmem_ld8(tq + (slice * per + c) * 8, own);
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      for (int s = 0; s < S; ++s) {
-        float x[8];
-        if (s == slice) {
-#pragma unroll
-          for (int e = 0; e < 8; ++e) x[e] = own[e];
-        } else {
-          const int from = s < slice ? s : s - 1;
-          const unsigned char* at = smem + from * per * (BMH * 32) + (2 * c * BMH + q * 32 + lane) * 16;
-          *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(at);
-          *reinterpret_cast<float4*>(x + 4) = *reinterpret_cast<const float4*>(at + BMH * 16);
-        }
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = s == 0 ? x[e] : v[e] + x[e];
-      }
+    // eight finished sums of this lane's row, columns cc .. cc + 7 of the warp's
+    auto put = [&](int cc, float* v) {
       if (p.gelu) {
 #pragma unroll
         for (int e = 0; e < 8; e += 2) gelu_two(v[e], v[e + 1]);
       }
-      const int cc = (c - lo) * 8;
       if constexpr (SW) {
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
@@ -984,75 +982,122 @@ __global__ void __launch_bounds__(kThreadsTc, 1) matmul_tc_split_kernel(const __
           *reinterpret_cast<uint4*>(at) = o;
         }
       }
-    }
-    __syncwarp();
-    // out: consecutive lanes take consecutive 16-byte pieces of a row of the result
-    const int el = 16 / esz, pieces = (SW ? 32 : cols) / el, nrows = SW ? cols : 32;
-    const long long yr0 = SW ? col0 : row0, yc0 = SW ? row0 : col0, yrows = SW ? Ng : Mg, ycols = SW ? Mg : Ng;
-    const int n_out = (g == 0 ? p.n_rep : 0) + 1;
-    const long long ld = p.ldy[g];
-    const long long left = ycols - yc0;                  // columns of the result from this warp's first on
-    unsigned char* y0 = static_cast<unsigned char*>(p.y_ptr[g]) + part * p.part_bytes + (yr0 * ld + yc0) * esz;
-    const long long row_bytes = ld * esz;
-    // where row r of this warp's lies in destination o
-    auto row_at = [&](int r, int o, auto blocks) -> unsigned char* {
-      if constexpr (decltype(blocks)::value) {
-        int b = 0;
-        while (b + 1 < p.blocks && yr0 + r >= p.block_row[b + 1]) ++b;
-        return static_cast<unsigned char*>(p.block_y[b]) + (yr0 + r - p.block_row[b]) * row_bytes + yc0 * esz;
-      } else {
-        return (o == 0 ? y0 : static_cast<unsigned char*>(p.rep_ptr[o - 1]) + yr0 * row_bytes + yc0 * esz) + r * row_bytes;
-      }
     };
-    auto store = [&](auto blocks, auto one) {
-#pragma unroll 4
-      for (int idx = lane; idx < nrows * pieces; idx += 32) {
-        const int r = idx / pieces, ch = idx - r * pieces;
-        if (yr0 + r >= yrows || ch * el >= left) continue;
-        const uint4 v = *reinterpret_cast<const uint4*>(stage + r * pitch + ch * 16);
-        for (int o = 0; o < (decltype(one)::value ? 1 : n_out); ++o) {
-          unsigned char* at = row_at(r, o, blocks) + ch * 16;
-          if ((ch + 1) * el <= left) {
-            if (SBP_GUARD(at, 16)) *reinterpret_cast<uint4*>(at) = v;
-          } else if (p.out_f32) {
-            const float* f = reinterpret_cast<const float*>(&v);
+    if (S == 1) {            // nothing to add: up to 32 columns a load
+      constexpr int kG = NB / 16 < 4 ? NB / 16 : 4;
+      for (int c = lo; c < hi; c += kG) {
+        float v[8 * kG];
+        if constexpr (kG == 4) {
+          tmem_ld32(tq + c * 8, v);
+        } else {
 #pragma unroll
-            for (int e = 0; e < 3; ++e)
-              if (ch * el + e < left && SBP_GUARD(at + 4 * e, 4)) reinterpret_cast<float*>(at)[e] = f[e];
-          } else {
-            const unsigned short* f = reinterpret_cast<const unsigned short*>(&v);
+          for (int i = 0; i < kG; ++i) tmem_ld8(tq + (c + i) * 8, v + 8 * i);
+        }
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-            for (int e = 0; e < 7; ++e)
-              if (ch * el + e < left && SBP_GUARD(at + 2 * e, 2)) reinterpret_cast<unsigned short*>(at)[e] = f[e];
-          }
-        }
+        for (int i = 0; i < kG; ++i) put((c + i - lo) * 8, v + 8 * i);
       }
-    };
-    auto store_unaligned = [&](auto blocks) {
-      const int bytes = (int)(left < pieces * el ? left : pieces * el) * esz;
-      for (int idx = lane; idx < nrows * pieces; idx += 32) {
-        const int r = idx / pieces, ch = idx - r * pieces;
-        if (yr0 + r >= yrows) continue;
-        auto in = [&](int off) { return stage + r * pitch + off; };
-        for (int o = 0; o < n_out; ++o) {
-          if (p.out_f32) store_shifted<4>(row_at(r, o, blocks), bytes, ch, pieces, in);
-          else store_shifted<2>(row_at(r, o, blocks), bytes, ch, pieces, in);
-        }
-      }
-    };
-    if (p.y_vec) {
-      if (p.blocks) store(std::true_type{}, std::true_type{});
-      else if (n_out == 1) store(std::false_type{}, std::true_type{});
-      else store(std::false_type{}, std::false_type{});
     } else {
-      if (p.blocks) store_unaligned(std::true_type{});
-      else store_unaligned(std::false_type{});
+      for (int c = lo; c < hi; ++c) {
+        float v[8], own[8];
+        tmem_ld8(tq + (slice * per + c) * 8, own);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        for (int s = 0; s < S; ++s) {
+          float x[8];
+          if (s == slice) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) x[e] = own[e];
+          } else {
+            const int from = s < slice ? s : s - 1;
+            const unsigned char* at = smem + from * per * (BMH * 32) + (2 * c * BMH + q * 32 + lane) * 16;
+            *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(at);
+            *reinterpret_cast<float4*>(x + 4) = *reinterpret_cast<const float4*>(at + BMH * 16);
+          }
+#pragma unroll
+          for (int e = 0; e < 8; ++e) v[e] = s == 0 ? x[e] : v[e] + x[e];
+        }
+        put((c - lo) * 8, v);
+      }
     }
   }
-
+  // done with tensor memory and with what the other CTAs may signal or write; what is left is the stores
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  cluster_sync_all();
+  __syncwarp();
+  cluster_arrive();
+  if (mine_live) {
+    // Out: consecutive lanes take consecutive 16-byte pieces of a row of the result.  Where a row lies is worked out once, by
+    // the lane of its number, and handed round; row and piece are stepped, not divided out.  (Both for every piece of every
+    // row: the stores of [2048 x 1024]^T [2048 x 4096] in 256 x 256 tiles to eight row blocks took 9.9 us, 3.7 so; one
+    // result a device, 256 x 128 tiles 3.9, 2.5.)
+    const int el = 16 / esz, pieces = (SW ? 4 : hi - lo) << (p.out_f32 ? 1 : 0), nrows = SW ? cols : 32;
+    const long long yr0 = SW ? col0 : row0, yc0 = SW ? row0 : col0, yrows = SW ? Ng : Mg, ycols = SW ? Mg : Ng;
+    const int n_out = (g == 0 ? p.n_rep : 0) + 1;
+    const long long row_bytes = p.ldy[g] * esz;
+    const int left = (int)min((long long)pieces * el, ycols - yc0);      // columns this warp has
+    // where row r starts, from the start of the result (row blocks: its address)
+    auto row_at = [&](int r) -> unsigned long long {
+      const long long row = yr0 + r;
+      if (!p.blocks) return (unsigned long long)(row * row_bytes + yc0 * esz);
+      int b = 0;
+      while (b + 1 < p.blocks && row >= p.block_row[b + 1]) ++b;
+      return reinterpret_cast<unsigned long long>(p.block_y[b]) + (unsigned long long)((row - p.block_row[b]) * row_bytes + yc0 * esz);
+    };
+    const unsigned long long at0 = row_at(lane), at1 = SW && NB > 64 ? row_at(lane + 32) : 0ull;
+    unsigned char* const y0 = p.blocks ? nullptr : static_cast<unsigned char*>(p.y_ptr[g]) + part * p.part_bytes;
+    const int log2p = 31 - __clz(pieces);
+    const bool pow2 = (1 << log2p) == pieces;
+    int r = pow2 ? lane >> log2p : lane / pieces, ch = lane - r * pieces;
+    const int dr = pow2 ? 32 >> log2p : 32 / pieces, dc = 32 - dr * pieces;
+    const int total = (int)min((long long)nrows, yrows - yr0) * pieces;
+    auto step = [&](auto vec, auto one) {
+#pragma unroll 4
+      for (int i = 0; i < total; i += 32) {
+        unsigned long long off = __shfl_sync(0xffffffffu, at0, r & 31);
+        if (SW && NB > 64) {
+          const unsigned long long far = __shfl_sync(0xffffffffu, at1, r & 31);
+          if (r >= 32) off = far;
+        }
+        if (i + lane < total) {
+          uint4 v;
+          if constexpr (decltype(vec)::value) v = *reinterpret_cast<const uint4*>(stage + r * pitch + ch * 16);
+          for (int o = 0; o < (decltype(one)::value ? 1 : n_out); ++o) {
+            unsigned char* at = (o == 0 ? y0 : static_cast<unsigned char*>(p.rep_ptr[o - 1])) + off;
+            if constexpr (!decltype(vec)::value) {
+              auto in = [&](int b) { return stage + r * pitch + b; };
+              if (p.out_f32) store_shifted<4>(at, left * 4, ch, pieces, in);
+              else store_shifted<2>(at, left * 2, ch, pieces, in);
+            } else {
+              at += ch * 16;
+              if ((ch + 1) * el <= left) {
+                if (SBP_GUARD(at, 16)) *reinterpret_cast<uint4*>(at) = v;
+              } else if (p.out_f32) {
+                const float* f = reinterpret_cast<const float*>(&v);
+#pragma unroll
+                for (int e = 0; e < 3; ++e)
+                  if (ch * el + e < left && SBP_GUARD(at + 4 * e, 4)) reinterpret_cast<float*>(at)[e] = f[e];
+              } else {
+                const unsigned short* f = reinterpret_cast<const unsigned short*>(&v);
+#pragma unroll
+                for (int e = 0; e < 7; ++e)
+                  if (ch * el + e < left && SBP_GUARD(at + 2 * e, 2)) reinterpret_cast<unsigned short*>(at)[e] = f[e];
+              }
+            }
+          }
+        }
+        r += dr;
+        ch += dc;
+        if (ch >= pieces) {
+          ch -= pieces;
+          ++r;
+        }
+      }
+    };
+    if (!p.y_vec) step(std::false_type{}, std::false_type{});
+    else if (n_out == 1) step(std::true_type{}, std::true_type{});
+    else step(std::true_type{}, std::false_type{});
+  }
+  __syncwarp();
+  cluster_wait();
   if (warp == 1) {
     __syncwarp();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
