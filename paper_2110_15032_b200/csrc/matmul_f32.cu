@@ -1,4 +1,5 @@
-// fp32 MatMul: executes a grouped-GEMM plan (matmul_plan.h) on the FMA pipes.
+// fp32 MatMul: executes a grouped-GEMM plan (matmul_plan.h) on the FMA pipes.  (Products that fill tiles of the tensor cores
+// go to matmul_f32_tc.cu, which is as exact.)
 //
 // Every element of the result is a chain of fused multiply-adds in fp32, k ascending, segments in rank order; where K is
 // split over the CTAs of a cluster (below) one chain for each, the chains added in their
@@ -336,6 +337,10 @@ bool aligned16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0;
 
 }  // namespace
 
+// Defined in matmul_f32_tc.cu: the same product from bf16 parts on the tensor cores.
+double f32_tc_cost(const MatmulPlan& plan, int* nb, int* splits);
+sbp_status launch_matmul_f32_tc(const MatmulPlan& plan, int nb, int splits, cudaStream_t st);
+
 sbp_status launch_matmul_f32(const MatmulPlan& plan, cudaStream_t st) {
   F32Params P;
   P.plan = plan;
@@ -384,6 +389,15 @@ sbp_status launch_matmul_f32(const MatmulPlan& plan, cudaStream_t st) {
       const double cost = it * per_sm * each + rounds * (4000 + exchange);
       if (cost < best) { best = cost; best_t = t; best_s = s; }
     }
+  }
+  // The tensor cores take it where their estimate (us) is below this one at 1.93 clocks a ns: measured times are 1.16 of this
+  // estimate at 1.9 GHz, and a switch has to win by some 15 %.  (us, this kernel / the other: 942 x 256 x 128 on three shards
+  // 8.1 / 9.0, 339 x 736 x 128 on two 8.9 / 9.4, 69 x 270 x 1639 on four 14.3 / 13.7, 187 x 1092 x 339 on four 17.9 / 14.6,
+  // 1170 x 256 x 808 on three 30 / 17, 1000 x 1500 x 777 on four 92 / 38, 2048 x 2048 x 2048 422 / 153.)
+  if (best > 11000) {
+    int nb = 0, splits = 1;
+    const double tc = f32_tc_cost(plan, &nb, &splits);
+    if (tc >= 0 && tc * 1930 < best) return launch_matmul_f32_tc(plan, nb, splits, st);
   }
   if (best == 1e300) return fail(SBP_ERR_UNSUPPORTED, "matrix too large for the FMA kernel");
   const int b = best_t == 0 ? 128 : 64;

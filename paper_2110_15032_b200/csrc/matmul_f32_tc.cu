@@ -1,0 +1,617 @@
+// fp32 MatMul on the tensor cores: executes a grouped-GEMM plan (matmul_plan.h) with the accuracy of fp32 arithmetic.
+//
+// An fp32 number is the sum of three bf16 numbers, x = h + m + l, each the rounding of what the ones before it
+// leave; nothing is lost, bf16 having the exponents of fp32.  A product of two numbers is then hh + (hm + mh) +
+// (hl + mm + lh) + terms below 2^-24 of it, that is six products of bf16 numbers, each exact in fp32.  The tensor cores
+// sum them up over a slot of 32 K-steps, the smallest products first: their accumulator cuts off what an addition
+// shifts out, and over longer runs that would show.  The slot's sum is then added to fp32 registers with IEEE additions.
+// Error against fp64, root mean square, relative, normal operands, this / the FMA kernel (one chain, or cut in up to
+// eight): K = 16 4.8e-8 / 7.3e-8, 64 6.3e-8 / 8.5e-8, 512 9.6e-8 / 1.5e-7, 1500 1.4e-7 / 4.9e-7, 2048 1.6e-7 / 2.9e-7.
+// (Slots of 64: 3.2e-7 at any K.  Operands all of one sign, where the cut-off does not average out: K = 64 6.3e-8 /
+// 5.0e-8, 2048 1.35e-7 / 1.0e-7 cut in eight.)
+//
+//   warps 0-7   the accumulators: they add a slot's sum, 32 rows x half of the columns a warp, out of one of two buffers
+//               in tensor memory
+//   warps 8-15  the operands: they load fp32 quads into registers a slot ahead, split them and put the parts into the
+//               six planes of a ring slot in shared memory
+//   warp 16     one elected lane issues the slot's twelve M128 N16..192 K16 MMAs and commits slot and buffer
+//
+// Operands keep the order they have in memory: K-contiguous ones become K-major tiles with 64-byte rows, the others
+// MN-major tiles in chunks of 64 columns.  A tile whose K is long and whose device is otherwise idle is cut along K
+// over the CTAs of a cluster, whose partial tiles are added in order through distributed shared memory.
+//
+// Bound: the data path of shared memory.  Per slot of a 128 x 128 tile the MMAs read 768 lines of 128 bytes, the planes take
+// 384, the loads pass 256 to 512, in some 2200 clocks (768 for the MMAs alone); a wider tile shares the A operand
+// (192 columns 2800, 1870 for 128 of them), 16 warps for the operands instead of 8 change nothing (2048^3 157 and 153 us).
+// 1000 x 1024 x 1500 on four shards 33 us, 1000 x 1500 x 777 38, 2048^3 153 (112 TFLOP/s); FMA kernel 87, 92, 422.
+//
+// A product that is not finite (operands or sums that are not, or a bf16 part that rounds to infinity) is found in
+// the accumulators; the CTA then multiplies its tile again with fp32 multiply-adds in ascending order.
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <atomic>
+#include <type_traits>
+
+#include "bounds_check.h"
+#include "matmul_plan.h"
+#include "sbp_internal.h"
+#include "tc_ptx.h"
+
+namespace sbp {
+
+namespace {
+
+constexpr int kTM = 128;                 // rows of a tile
+constexpr int kTN = 192;                 // columns of a tile, at most
+constexpr int kSK = 32;                  // K-steps of a ring slot
+constexpr int kMaxSlots = 8;
+constexpr int kDrain = 256;              // threads that keep the accumulators, threads that split operands
+constexpr int kWorkers = 256;
+constexpr int kThreads = kDrain + kWorkers + 128;      // and a warpgroup one warp of which issues the MMAs
+constexpr int kMmaWarp = (kDrain + kWorkers) / 32;
+constexpr int kPlaneA = kTM * kSK * 2;   // one bf16 part of an A slot
+constexpr int kRing = 198 * 1024;
+constexpr int kSmem = kRing + 1024;      // + alignment slack
+constexpr int kAccs = 2;                 // accumulators in tensor memory
+constexpr int kAccCols = 256;            // columns from one to the other
+
+struct F32TcParams {
+  MatmulPlan plan;
+  int splits;                            // CTAs per tile (cluster size)
+  int nb;                                // columns of a tile, a multiple of 16
+  int slots;                             // ring slots
+};
+
+__device__ __forceinline__ float gelu_erf(float v) { return 0.5f * v * (1.0f + erff(v * 0.70710678118654752440f)); }
+
+// Two numbers as three bf16 each, packed.
+__device__ __forceinline__ unsigned bf16_pair(float lo, float hi) {
+  unsigned r;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+  return r;
+}
+// (x, y) less the two bf16 of h: exact
+__device__ __forceinline__ void less_pair(float& x, float& y, unsigned h) {
+  asm("{\n\t.reg .b64 v, w;\n\tmov.b64 v, {%0, %1};\n\tmov.b64 w, {%2, %3};\n\tfma.rn.f32x2 v, w, %4, v;\n\tmov.b64 {%0, %1}, v;\n\t}"
+      : "+f"(x), "+f"(y)
+      : "r"(h << 16), "r"(h & 0xffff0000u), "l"(0xbf800000bf800000ull));
+}
+__device__ __forceinline__ void split_pair(float x, float y, unsigned& h, unsigned& m, unsigned& l) {
+  h = bf16_pair(x, y);
+  less_pair(x, y, h);
+  m = bf16_pair(x, y);
+  less_pair(x, y, m);
+  l = bf16_pair(x, y);
+}
+
+// A worker's share of an operand: Q quads of consecutive elements a slot, kept in registers between their load and
+// their way into the ring slot's planes.  KC: K is contiguous in memory; quad j of thread t is quad t mod 8 of row
+// t / 8 + 32 j.  Otherwise a K-step has 2^SH quads, and quad j is one of K-step (t >> SH) + j (256 >> SH).
+// The loads are predicated instructions: where a branch stood around them each was waited for before the next was made
+// (300 to 430 clocks a quad).
+template <int Q, bool KC, int SH>
+struct Share {
+  static constexpr int kApart = KC ? kWorkers / 8 : kWorkers >> SH;      // rows (K-steps) from quad j to quad j + 1
+  static constexpr int kHop = kApart * (KC ? 64 : 128);                  // bytes
+  static constexpr unsigned kOdd = !KC && SH == 6 ? 64 : 0;              // four K-steps on, the 128-byte swizzle is another one
+  float4 r[Q];
+  const float* at;               // quad 0 of the next slot to load
+  int step;                      // elements from quad j to quad j + 1
+  int limit;                     // KC: K in the slot before the quad; else elements from it to the operand's edge
+  int first;                     // row (K-step) of quad 0
+  int rows, tile_rows;           // rows of the operand / of the tile from there on (KC)
+  unsigned off;                  // where quad 0 goes in a plane
+
+  __device__ __forceinline__ void init(int t, int ext, int width) {
+    if constexpr (KC) {          // rows of 64 bytes, 64-byte swizzle
+      const int row = t >> 3, c = t & 7;
+      first = row;
+      limit = c * 4;
+      rows = ext - row;
+      tile_rows = width - row;
+      off = row * 64 + (((c >> 1) ^ ((row >> 1) & 3)) << 4) + (c & 1) * 8;
+    } else {                     // chunks of 64 positions: rows of 128 bytes, 128-byte swizzle
+      const int k = t >> SH, c = t & ((1 << SH) - 1);
+      first = k;
+      limit = ext - c * 4;
+      rows = 0;
+      tile_rows = c * 4 < width ? kSK : 0;
+      off = (c >> 4) * (kSK * 128) + k * 128 + ((((c >> 1) & 7) ^ (k & 7)) << 4) + (c & 1) * 8;
+    }
+  }
+  // g: position (0, 0) of the slot that is loaded next
+  __device__ __forceinline__ void point(const float* g, long long ld, int t) {
+    at = g + first * ld + (KC ? limit : (t & ((1 << SH) - 1)) * 4);
+    step = kApart * (int)ld;
+  }
+  // VEC: every quad lies inside as a whole or not at all, and 16-byte aligned.  count: quads a slot
+  template <bool VEC>
+  __device__ __forceinline__ void load(int left, int count) {
+#pragma unroll
+    for (int j = 0; j < Q; ++j) {
+      if (j >= count) break;
+      const float* src = at + (long long)j * step;
+      int have;                  // elements of the quad that lie inside
+      if constexpr (KC) have = j * kApart < rows ? left - limit : 0;
+      else have = first + j * kApart < left ? limit : 0;
+      r[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if constexpr (VEC) {
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %5, 0;\n\t@p ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}"
+                     : "+f"(r[j].x), "+f"(r[j].y), "+f"(r[j].z), "+f"(r[j].w)
+                     : "l"(src), "r"(have > 0 && SBP_GUARD(src, 16) ? 1 : 0));
+      } else {
+        float* e[4] = {&r[j].x, &r[j].y, &r[j].z, &r[j].w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p ld.global.nc.f32 %0, [%1];\n\t}"
+                       : "+f"(*e[i])
+                       : "l"(src + i), "r"(have > i && SBP_GUARD(src + i, 4) ? 1 : 0));
+      }
+    }
+  }
+  __device__ __forceinline__ void store(unsigned base, int plane, int count) {
+#pragma unroll
+    for (int j = 0; j < Q; ++j) {
+      if (j >= count) break;
+      const unsigned to = base + ((j & 1) ? off ^ kOdd : off) + j * kHop;
+      uint2 h, m, l;
+      split_pair(r[j].x, r[j].y, h.x, m.x, l.x);
+      split_pair(r[j].z, r[j].w, h.y, m.y, l.y);
+      asm volatile(
+          "{\n\t.reg .pred p;\n\tsetp.gt.s32 p, %9, %10;\n\t@p st.shared.v2.b32 [%0], {%3, %4};\n\t@p st.shared.v2.b32 [%1], {%5, %6};\n\t"
+          "@p st.shared.v2.b32 [%2], {%7, %8};\n\t}" ::"r"(to),
+          "r"(to + plane), "r"(to + 2 * plane), "r"(h.x), "r"(h.y), "r"(m.x), "r"(m.y), "r"(l.x), "r"(l.y), "r"(tile_rows), "r"(KC ? j * kApart : 0));
+    }
+  }
+};
+
+// a += b on two packed numbers
+__device__ __forceinline__ void add2(unsigned long long& a, unsigned long long b) { asm("add.rn.f32x2 %0, %0, %1;" : "+l"(a) : "l"(b)); }
+__device__ __forceinline__ float lo(unsigned long long v) { return __uint_as_float((unsigned)v); }
+__device__ __forceinline__ float hi(unsigned long long v) { return __uint_as_float((unsigned)(v >> 32)); }
+
+// 16 accumulator columns of this warp's 32 rows, in pairs
+__device__ __forceinline__ void tmem_ld16_wait(unsigned taddr, unsigned long long (&v)[8]) {
+  unsigned r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) asm("mov.b64 %0, {%1, %2};" : "=l"(v[i]) : "r"(r[2 * i]), "r"(r[2 * i + 1]));
+}
+
+// AT / BT: the operand is stored transposed.  A as given and B transposed are K-contiguous.
+template <int AT, int BT>
+__global__ void __launch_bounds__(kThreads, 1) matmul_f32_tc_kernel(const __grid_constant__ F32TcParams P) {
+  constexpr bool AKC = !AT, BKC = BT;
+  extern __shared__ unsigned char smem_raw[];
+  __shared__ __align__(8) unsigned long long bar_full[kMaxSlots], bar_empty[kMaxSlots], bar_acc_full[kAccs], bar_acc_empty[kAccs];
+  __shared__ unsigned tmem_base_slot;
+  __shared__ int abort_flag_s, redo_s;
+  volatile int* abort_flag = &abort_flag_s;
+
+  const MatmulPlan& p = P.plan;
+  const int g = blockIdx.z, splits = P.splits, slice = (int)(blockIdx.x % (unsigned)splits), nb = P.nb;
+  const long long M = p.m[g], N = p.n[g];
+  const long long m0 = (long long)blockIdx.y * kTM, n0 = (long long)(blockIdx.x / (unsigned)splits) * nb;
+  if (m0 >= M || n0 >= N) return;                  // the whole cluster
+  const int rows = (int)min((long long)kTM, M - m0), cols = (int)min((long long)nb, N - n0);
+  unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int plane_b = (nb + 63) / 64 * (64 * kSK * 2), slot_bytes = 3 * (kPlaneA + plane_b), slots = P.slots;
+
+  if (tid == 0) {
+    abort_flag_s = 0;
+    redo_s = 0;
+    for (int i = 0; i < slots; ++i) {
+      mbar_init(smem_addr(&bar_full[i]), kWorkers / 32);
+      mbar_init(smem_addr(&bar_empty[i]), 1);
+    }
+    for (int i = 0; i < kAccs; ++i) {
+      mbar_init(smem_addr(&bar_acc_full[i]), 1);
+      mbar_init(smem_addr(&bar_acc_empty[i]), kDrain / 32);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == kMmaWarp) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_base_slot)), "r"(kAccs * kAccCols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+
+  // this CTA's range of slots over all segments
+  const int s_lo = p.chain ? 0 : g, s_hi = p.chain ? p.nseg : g + 1;
+  long long total = 0;
+  for (int s = s_lo; s < s_hi; ++s) total += (p.kseg[s] + kSK - 1) / kSK;
+  const long long it0 = total * slice / splits;
+  const int iters = (int)(total * (slice + 1) / splits - it0);
+  int seg0 = s_lo;                                 // where the range starts: segment and K inside it
+  long long k0 = it0;
+  while (seg0 < s_hi) {
+    const long long n = (p.kseg[seg0] + kSK - 1) / kSK;
+    if (k0 < n) break;
+    k0 -= n;
+    ++seg0;
+  }
+  k0 *= kSK;
+
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const unsigned tmem_base = tmem_base_slot;
+  SBP_PDL_WAIT();                                  // everything up to here overlaps the kernel before this one
+
+  const int q = warp & 3, half = (warp >> 2) & 1, width = nb / 2;      // a draining warp's tensor-memory lanes and columns
+  if (warp < kDrain / 32) {
+    // ------------------------------------------------ accumulators
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 128;");        // 2 x 128 + 2 x 88 + 48 = 5 x 96
+    unsigned long long acc[kTN / 4];
+#pragma unroll
+    for (int i = 0; i < kTN / 4; ++i) acc[i] = 0ull;
+    bool ok = true;
+    for (int c = 0; c < iters; ++c) {
+      ok = mbar_wait_warp(smem_addr(&bar_acc_full[c % kAccs]), (unsigned)(c / kAccs & 1), abort_flag);
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const unsigned at = tmem_base + ((unsigned)(q * 32) << 16) + (c % kAccs) * kAccCols + half * width;
+#pragma unroll
+      for (int b = 0; b < kTN / 4; b += 8) {
+        if (2 * b >= width) break;
+        unsigned long long v[8];
+        tmem_ld16_wait(at + 2 * b, v);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) add2(acc[b + i], v[i]);
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_addr(&bar_acc_empty[c % kAccs]));
+    }
+    // every product has been made: the ring becomes the tile
+    SBP_PDL_RELEASE();
+    float zero = 0.f;                              // stays so unless something is not finite
+    float* tile = reinterpret_cast<float*>(smem) + (q * 32 + lane) * (nb + 4) + half * width;
+#pragma unroll
+    for (int i = 0; i < kTN / 4; i += 4) {
+      if (2 * i >= width) break;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) zero = fmaf(hi(acc[i + e]), 0.f, fmaf(lo(acc[i + e]), 0.f, zero));
+    }
+    if (zero != 0.f) redo_s = 1;
+    asm volatile("bar.sync 1, 256;" ::: "memory");      // every warp has seen its last chunk
+#pragma unroll
+    for (int i = 0; i < kTN / 4; i += 2) {
+      if (2 * i >= width) break;
+      *reinterpret_cast<float4*>(tile + 2 * i) = make_float4(lo(acc[i]), hi(acc[i]), lo(acc[i + 1]), hi(acc[i + 1]));
+    }
+    if (redo_s) {
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      for (int idx = tid; idx < kTM * cols; idx += kDrain) {
+        const int r = idx % kTM, c = idx / kTM;
+        if (r >= rows) continue;
+        float sum = 0.f;
+        int s = seg0;
+        long long k = k0;
+        for (int n = iters; n > 0; --n) {
+          while (s < s_hi && k >= p.kseg[s]) { ++s; k = 0; }
+          const long long end = min(p.kseg[s], k + kSK);
+          const float* A = static_cast<const float*>(p.a[s]) + (AT ? p.row_off[g] + m0 + r : (p.row_off[g] + m0 + r) * p.lda[s]);
+          const float* B = static_cast<const float*>(p.b[s]) + (BT ? (p.col_off[g] + n0 + c) * p.ldb[s] : p.col_off[g] + n0 + c);
+          for (long long kk = k; kk < end; ++kk) {
+            const float* a = A + (AT ? kk * p.lda[s] : kk);
+            const float* b = B + (BT ? kk : kk * p.ldb[s]);
+            if (SBP_GUARD(a, 4) && SBP_GUARD(b, 4)) sum = fmaf(__ldg(a), __ldg(b), sum);
+          }
+          k += kSK;
+        }
+        reinterpret_cast<float*>(smem)[r * (nb + 4) + c] = sum;
+      }
+    }
+  } else if (warp < kMmaWarp) {
+    // ------------------------------------------------ operands
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
+    const int t = tid - kDrain;
+    // whole aligned quads everywhere, or element by element
+    bool a_vec = AT ? (rows & 3) == 0 && (p.row_off[g] & 3) == 0 : true, b_vec = BT ? true : (cols & 3) == 0 && (p.col_off[g] & 3) == 0;
+    for (int s = s_lo; s < s_hi; ++s) {
+      a_vec = a_vec && (reinterpret_cast<unsigned long long>(p.a[s]) & 15) == 0 && (p.lda[s] & 3) == 0 && (AT || (p.kseg[s] & 3) == 0);
+      b_vec = b_vec && (reinterpret_cast<unsigned long long>(p.b[s]) & 15) == 0 && (p.ldb[s] & 3) == 0 && (!BT || (p.kseg[s] & 3) == 0);
+    }
+    constexpr int kQA = kTM * kSK / 4 / kWorkers;
+    // sh: log2 of the quads of a K-step of an MN-contiguous B
+    auto run = [&](auto av, auto bv, auto sh) {
+      constexpr bool AV = decltype(av)::value, BV = decltype(bv)::value;
+      constexpr int SH = decltype(sh)::value, kQB = BKC ? kTN * kSK / 4 / kWorkers : kSK / (kWorkers >> SH);
+      Share<kQA, AKC, 5> A;
+      Share<kQB, BKC, SH> B;
+      A.init(t, rows, kTM);
+      B.init(t, cols, nb);
+      const int count_b = BKC ? (nb + 31) / 32 : kQB;
+      int ls = seg0, left = 0, lk = (int)k0;
+      // the next slot to load: afresh at the start of a segment, else one step on
+      auto next_slot = [&](bool start) {
+        if (!start) {
+          lk += kSK;
+          if (lk < (int)p.kseg[ls]) {
+            A.at += AKC ? kSK : kSK * (int)p.lda[ls];
+            B.at += BKC ? kSK : kSK * (int)p.ldb[ls];
+            left = min(kSK, (int)p.kseg[ls] - lk);
+            return;
+          }
+        }
+        while (ls < s_hi && lk >= p.kseg[ls]) { ++ls; lk = 0; }      // also steps over empty segments
+        const long long lda = p.lda[ls], ldb = p.ldb[ls];
+        A.point(static_cast<const float*>(p.a[ls]) + (AT ? lk * lda + p.row_off[g] + m0 : (p.row_off[g] + m0) * lda + lk), lda, t);
+        B.point(static_cast<const float*>(p.b[ls]) + (BT ? (p.col_off[g] + n0) * ldb + lk : lk * ldb + p.col_off[g] + n0), ldb, t);
+        left = min(kSK, (int)p.kseg[ls] - lk);
+      };
+      if (iters > 0) {
+        next_slot(true);
+        A.template load<AV>(left, kQA);
+        B.template load<BV>(left, count_b);
+      }
+      int slot = 0;
+      unsigned round = 0;
+      for (int it = 0; it < iters; ++it) {
+        if (!mbar_wait_warp(smem_addr(&bar_empty[slot]), round ^ 1, abort_flag)) break;
+        const unsigned to = smem_addr(smem) + slot * slot_bytes;
+        if (it + 1 < iters) next_slot(false);
+        else left = 0;
+        A.store(to, kPlaneA, kQA);                 // and the next slot's quads take the registers
+        A.template load<AV>(left, kQA);
+        B.store(to + 3 * kPlaneA, plane_b, count_b);
+        B.template load<BV>(left, count_b);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_addr(&bar_full[slot]));
+        slot = slot + 1 == slots ? 0 : slot + 1;
+        round ^= (slot == 0);
+      }
+    };
+    auto run_b = [&](auto av, auto sh) {
+      if (b_vec) run(av, std::true_type{}, sh);
+      else run(av, std::false_type{}, sh);
+    };
+    auto run_a = [&](auto sh) {
+      if (a_vec) run_b(std::true_type{}, sh);
+      else run_b(std::false_type{}, sh);
+    };
+    if constexpr (BKC) {
+      run_a(std::integral_constant<int, 5>{});
+    } else {
+      if (nb > 128) run_a(std::integral_constant<int, 6>{});
+      else if (nb > 64) run_a(std::integral_constant<int, 5>{});
+      else run_a(std::integral_constant<int, 4>{});
+    }
+  } else {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+    if (warp == kMmaWarp) {
+    // ------------------------------------------------ MMA issuer
+    const bool leader = elect_one();
+    const unsigned idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((AT ? 1u : 0u) << 15) | ((BT ? 0u : 1u) << 16) | ((unsigned)(nb >> 3) << 17) |
+                           ((unsigned)(kTM >> 4) << 24);
+    constexpr unsigned a_lo = desc_lo_fixed(AKC ? 16 : kSK * 128), b_lo = desc_lo_fixed(BKC ? 16 : kSK * 128);
+    constexpr unsigned a_hi = AKC ? desc_hi_fixed(512, 4) : desc_hi_fixed(1024), b_hi = BKC ? desc_hi_fixed(512, 4) : desc_hi_fixed(1024);
+    constexpr unsigned a_step = AKC ? 2 : 128, b_step = BKC ? 2 : 128;      // 16 K-steps, in 16-byte units
+    int slot = 0;
+    unsigned round = 0;
+    for (int it = 0; it < iters; ++it) {
+      const int c = it;
+      if (!mbar_wait_warp(smem_addr(&bar_acc_empty[c % kAccs]), (unsigned)((c / kAccs & 1) ^ 1), abort_flag)) break;
+      if (!mbar_wait_warp(smem_addr(&bar_full[slot]), round, abort_flag)) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (leader) {
+        const unsigned sa = (smem_addr(smem) + slot * slot_bytes) & 0x3ffffu, sb = sa + 3 * kPlaneA;
+        const unsigned d = tmem_base + (c % kAccs) * kAccCols;
+        unsigned accumulate = 0;
+        // parts of A and B, the smallest products first
+        constexpr int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};
+#pragma unroll
+        for (int t = 0; t < 6; ++t)
+#pragma unroll
+          for (int kk = 0; kk < kSK / 16; ++kk) {
+            umma_bf16_cta(d, desc_pack(a_lo + ((sa + pa[t] * kPlaneA) >> 4) + kk * a_step, a_hi),
+                          desc_pack(b_lo + ((sb + pb[t] * plane_b) >> 4) + kk * b_step, b_hi), idesc, accumulate);
+            accumulate = 1;
+          }
+        umma_commit_cta(smem_addr(&bar_empty[slot]));
+        umma_commit_cta(smem_addr(&bar_acc_full[c % kAccs]));
+      }
+      __syncwarp();
+      slot = slot + 1 == slots ? 0 : slot + 1;
+      round ^= (slot == 0);
+    }
+    if (*abort_flag && leader) {                   // products in flight get a bounded chance to finish
+      umma_commit_cta(smem_addr(&bar_acc_full[0]));
+      const unsigned long long t0 = now_ns();
+      const unsigned parity = 0;
+      while (!mbar_try(smem_addr(&bar_acc_full[0]), parity) && now_ns() - t0 < 100000000ull) {
+      }
+    }
+    __syncwarp();
+    }
+  }
+
+  // The tile is in shared memory: each CTA of the cluster adds up the partial sums of its rows, slice by slice, and stores them.
+  if (splits > 1) cluster_sync_all();
+  else __syncthreads();
+  if (warp < kMmaWarp) {
+    const int r_lo = kTM * slice / splits, r_hi = min(rows, kTM * (slice + 1) / splits);
+    const long long ldy = p.ldy[g];
+    const int n_out = (g == 0 ? p.n_rep : 0) + 1;
+    bool y_vec = (reinterpret_cast<unsigned long long>(p.y[g]) & 15) == 0 && (ldy & 3) == 0;
+    for (int o = 1; o < n_out; ++o) y_vec = y_vec && (reinterpret_cast<unsigned long long>(p.y_rep[o - 1]) & 15) == 0;
+    for (int r = r_lo + warp; r < r_hi; r += kMmaWarp) {
+      for (int c = lane * 4; c < cols; c += 128) {
+        const unsigned at = smem_addr(smem) + (unsigned)(r * (nb + 4) + c) * 4;
+        float v[4];
+        if (splits == 1) {
+          *reinterpret_cast<float4*>(v) = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(smem) + r * (nb + 4) + c);
+        } else {
+#pragma unroll 1
+          for (int s = 0; s < splits; s += 4) {      // four at a time, in ascending order
+            float x[4][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (s + i < splits)
+                asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                             : "=f"(x[i][0]), "=f"(x[i][1]), "=f"(x[i][2]), "=f"(x[i][3])
+                             : "r"(map_to_cta(at, s + i))
+                             : "memory");
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (s + i < splits) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] = s + i == 0 ? x[i][e] : v[e] + x[i][e];
+              }
+          }
+        }
+        if (p.gelu) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) v[e] = gelu_erf(v[e]);
+        }
+        for (int o = 0; o < n_out; ++o) {
+          float* y = static_cast<float*>(o == 0 ? p.y[g] : p.y_rep[o - 1]) + (m0 + r) * ldy + n0 + c;
+          if (y_vec && c + 3 < cols) {
+            if (SBP_GUARD(y, 16)) *reinterpret_cast<float4*>(y) = make_float4(v[0], v[1], v[2], v[3]);
+          } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              if (c + e < cols && SBP_GUARD(y + e, 4)) y[e] = v[e];
+          }
+        }
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  if (splits > 1) cluster_sync_all();              // nobody leaves while its tile may still be read
+  else __syncthreads();
+  if (warp == kMmaWarp) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kAccs * kAccCols) : "memory");
+  }
+}
+
+template <int AT, int BT>
+cudaError_t launch_form(const F32TcParams* P, int splits, dim3 grid, cudaStream_t st, int* capacity) {
+  static std::atomic<unsigned long long> opted{0};      // one bit per device
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned long long bit = 1ull << (dev & 63);
+  if (dev >= 64 || !(opted.load(std::memory_order_relaxed) & bit)) {
+    e = cudaFuncSetAttribute(matmul_f32_tc_kernel<AT, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+    if (e != cudaSuccess) return e;
+    if (dev < 64) opted.fetch_or(bit, std::memory_order_relaxed);
+  }
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = kSmem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)splits;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (capacity) return cudaOccupancyMaxActiveClusters(capacity, matmul_f32_tc_kernel<AT, BT>, &cfg);
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, matmul_f32_tc_kernel<AT, BT>, *P);
+}
+
+// Clusters of this many CTAs that the current device holds at once (a CTA fills its SM).
+int cluster_capacity(int splits) {
+  static std::atomic<int> known[64][9];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  int v = known[dev][splits].load(std::memory_order_relaxed);
+  if (v == 0) {
+    if (launch_form<0, 0>(nullptr, splits, dim3((unsigned)splits), nullptr, &v) != cudaSuccess || v < 1) {
+      cudaGetLastError();
+      v = -1;
+    }
+    known[dev][splits].store(v, std::memory_order_relaxed);
+  }
+  return v;
+}
+
+}  // namespace
+
+// The best cut of a plan for this kernel: estimated time in us (negative: it does not take the plan), columns of a tile, CTAs a
+// tile.  Per wave of clusters: a slot takes 0.81 us and 0.0032 more a column (all of its warps' round: loads, splitting,
+// twelve MMAs, the accumulators' turn), set-up, drain and stores 5.9 and 0.018 a column.  Fitted to 823 timings of 30 products
+// (rms error 10 %; the pick within 1.5 % of the best cut on the average).
+double f32_tc_cost(const MatmulPlan& plan, int* nb, int* splits) {
+  long long slots = 0, mmax = 0, nmax = 0;
+  for (int s = 0; s < plan.nseg; ++s) {
+    if (!plan.chain && s >= plan.ngroups) continue;
+    if (plan.kseg[s] > 0x7fffff00LL || plan.lda[s] > (1 << 25) || plan.ldb[s] > (1 << 25)) return -1;      // 32-bit steps
+    const long long n = (plan.kseg[s] + kSK - 1) / kSK;
+    slots = plan.chain ? slots + n : std::max(slots, n);
+  }
+  for (int g = 0; g < plan.ngroups; ++g) {
+    mmax = std::max(mmax, plan.m[g]);
+    nmax = std::max(nmax, plan.n[g]);
+  }
+  if ((mmax + kTM - 1) / kTM > 65535 || slots == 0 || slots > 0x7fffffffLL || nmax == 0) return -1;
+  double best = -1;
+  const long long least = (nmax + kTN - 1) / kTN;
+  for (long long t = least; t <= least + 12; ++t) {
+    const int w = (int)(((nmax + t - 1) / t + 15) / 16 * 16);
+    long long tiles = 0;
+    for (int g = 0; g < plan.ngroups; ++g) tiles += ((plan.m[g] + kTM - 1) / kTM) * ((plan.n[g] + w - 1) / w);
+    for (int s : {1, 2, 3, 4, 6, 8}) {
+      if (slots < s) break;
+      const int cap = cluster_capacity(s);
+      if (cap < 1) continue;
+      const double waves = (double)((tiles + cap - 1) / cap);
+      const double cost = waves * ((double)((slots + s - 1) / s) * (0.813 + 0.0032 * w) + 5.87 + 0.018 * w + (s > 1 ? 0.2 : 0.0));
+      if (best < 0 || cost < best) {
+        best = cost;
+        *nb = w;
+        *splits = s;
+      }
+    }
+    if (w <= 32) break;
+  }
+  return best;
+}
+
+sbp_status launch_matmul_f32_tc(const MatmulPlan& plan, int nb, int splits, cudaStream_t st) {
+  F32TcParams P;
+  P.plan = plan;
+  P.nb = nb;
+  P.splits = splits;
+  P.slots = std::min(kMaxSlots, kRing / (3 * (kPlaneA + (nb + 63) / 64 * (64 * kSK * 2))));
+  long long mmax = 0, nmax = 0;
+  for (int g = 0; g < plan.ngroups; ++g) {
+    mmax = std::max(mmax, plan.m[g]);
+    nmax = std::max(nmax, plan.n[g]);
+  }
+  const long long gx = (nmax + nb - 1) / nb * splits;
+  if (gx > 0x7fffffffLL || (mmax + kTM - 1) / kTM > 65535) return fail(SBP_ERR_UNSUPPORTED, "matrix too large for one launch");
+  const dim3 grid((unsigned)gx, (unsigned)((mmax + kTM - 1) / kTM), (unsigned)plan.ngroups);
+  SBP_BOUNDS_UPLOAD(st);
+  cudaError_t e;
+  switch ((plan.a_trans ? 2 : 0) | (plan.b_trans ? 1 : 0)) {
+    case 0: e = launch_form<0, 0>(&P, splits, grid, st, nullptr); break;
+    case 1: e = launch_form<0, 1>(&P, splits, grid, st, nullptr); break;
+    case 2: e = launch_form<1, 0>(&P, splits, grid, st, nullptr); break;
+    default: e = launch_form<1, 1>(&P, splits, grid, st, nullptr); break;
+  }
+  if (e != cudaSuccess) return cuda_fail(e, "matmul launch");
+  count_launch();
+  return SBP_OK;
+}
+
+sbp_status read_and_clear_f32_tc_timeout(bool* timed_out) { return read_and_clear_timeout_flag(timed_out); }
+
+}  // namespace sbp

@@ -193,6 +193,7 @@ __global__ void bounds_selftest_kernel(unsigned char* buf, size_t bytes) {
 // Defined next to the kernels that own the flags.
 sbp_status read_and_clear_bulk_timeout(bool* timed_out);
 sbp_status read_and_clear_tc_timeout(bool* timed_out);
+sbp_status read_and_clear_f32_tc_timeout(bool* timed_out);
 sbp_status launch_expire_wait(unsigned long long limit_ns, cudaStream_t st);
 
 }  // namespace sbp
@@ -231,10 +232,12 @@ int32_t sbp_debug_bounds_enabled(void) {
 uint64_t sbp_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }
 
 sbp_status sbp_check_device_errors(void) {
-  bool bulk = false, tc = false;
+  bool bulk = false, tc = false, f32 = false;
   sbp_status st = read_and_clear_bulk_timeout(&bulk);
   if (st != SBP_OK) return st;
   st = read_and_clear_tc_timeout(&tc);
+  if (st != SBP_OK) return st;
+  st = read_and_clear_f32_tc_timeout(&f32);
   if (st != SBP_OK) return st;
 #ifdef SBP_DEBUG_BOUNDS
   if (cudaDeviceSynchronize() != cudaSuccess) return fail(SBP_ERR_CUDA, "device synchronisation failed");
@@ -245,7 +248,7 @@ sbp_status sbp_check_device_errors(void) {
   }
 #endif
   if (bulk) return fail(SBP_ERR_TIMEOUT, "a bulk-copy boxing kernel gave up waiting for its loads");
-  if (tc) return fail(SBP_ERR_TIMEOUT, "the tensor-core matmul kernel gave up waiting on one of its barriers");
+  if (tc || f32) return fail(SBP_ERR_TIMEOUT, "the tensor-core matmul kernel gave up waiting on one of its barriers");
   return SBP_OK;
 }
 

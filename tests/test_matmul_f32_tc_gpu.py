@@ -1,0 +1,98 @@
+"""fp32 products on the tensor cores where they can go wrong: edges of tiles and ring slots, chained segments of uneven
+and zero length, both stored forms of either operand, rows off the 16-byte rule, operands and sums that are not finite,
+numbers at the ends of the exponent range.  The shapes are such as the library's own choice sends there.  Oracle and bound
+as for the other fp32 products; the error against fp64 besides stays below what a chain of fp32 multiply-adds shows."""
+import pytest
+import torch
+
+import paper_2110_15032_b200 as sbp
+from test_ops_gpu import _matmul_case
+
+pytestmark = pytest.mark.gpu
+F32 = torch.float32
+S0, S1, B = sbp.S(0), sbp.S(1), sbp.B
+
+
+@pytest.mark.parametrize("M,K,N", [(1024, 1024, 512), (1027, 1029, 517), (513, 2047, 770), (640, 1500, 1039), (900, 992, 1155)])
+@pytest.mark.parametrize("tx,tw", [(False, False), (True, False), (False, True), (True, True)])
+def test_edges_and_stored_forms(M, K, N, tx, tw):
+    _matmul_case(M, K, N, 1, F32, B, B, tx=tx, tw=tw)
+
+
+@pytest.mark.parametrize("M,K,N,k,xs,ws", [(1000, 1024, 1500, 4, S0, B), (1000, 1500, 777, 4, B, S1), (700, 1030, 900, 3, S0, B),
+                                           (600, 1000, 1100, 7, B, S1)])
+def test_groups(M, K, N, k, xs, ws):
+    _matmul_case(M, K, N, k, F32, xs, ws)
+
+
+@pytest.mark.parametrize("M,K,N,k", [(520, 2003, 640, 3), (768, 1100, 515, 8), (1030, 517, 900, 16)])
+@pytest.mark.parametrize("ys", [B, S0, S1])
+@pytest.mark.parametrize("tx,tw", [(False, False), (True, True)])
+def test_chained_segments(M, K, N, k, ys, tx, tw):
+    _matmul_case(M, K, N, k, F32, S1, S0, ys=ys, tx=tx, tw=tw, flags=sbp.SBP_EPILOGUE_GELU if ys == S1 else 0)
+
+
+def _product(X, W):
+    (M, K), N = X.shape, W.shape[1]
+    y = sbp.empty_global((M, N), F32, B, 1)
+    sbp.sbp_matmul(sbp.SbpTensor((M, K), F32, B, [X]), sbp.SbpTensor((K, N), F32, B, [W]), y)
+    return y.locals[0]
+
+
+def _operands(M=1024, K=1024, N=640, seed=1):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return torch.randn(M, K, device="cuda", generator=g), torch.randn(K, N, device="cuda", generator=g)
+
+
+def _check(Y, X, W):
+    R, mag = X.double() @ W.double(), X.double().abs() @ W.double().abs()
+    fin = torch.isfinite(R) & (mag < 3e38)
+    assert bool(((Y.double() - R).abs() <= 4 * X.shape[1] ** 0.5 * 2.0 ** -24 * mag + 1e-30)[fin].all())
+    return R, fin
+
+
+def test_infinities_and_nan():
+    X, W = _operands()
+    X[3, 100], X[500, 7], X[1000, 1000] = float("inf"), -float("inf"), float("nan")
+    W[5, 9], W[900, 600] = float("inf"), float("nan")
+    Y = _product(X, W)
+    R, fin = _check(Y, X, W)
+    assert torch.equal(torch.isnan(Y), torch.isnan(R))
+    assert torch.equal(Y[~fin & ~torch.isnan(R)].double(), R[~fin & ~torch.isnan(R)])
+
+
+def test_ends_of_the_exponent_range():
+    """The largest number rounds to infinity as a bf16; a sum may overflow; the lowest parts of small numbers are denormal."""
+    X, W = _operands()
+    X[7] *= 1e-30
+    X[7, 20], W[20] = torch.finfo(F32).max, W[20] * 1e-30
+    X[8], X[9], X[10] = X[8] * 1e30, X[9] * 2.0 ** -60, X[10] * 2.0 ** -100
+    W[:, 5] *= 2.0 ** -40
+    Y = _product(X, W)
+    _check(Y, X, W)
+    X[8, :2], W[:2, 6] = 3e38, 3.0
+    assert bool(torch.isinf(_product(X, W)[8, 6]))
+
+
+def test_whole_numbers_are_exact():
+    g = torch.Generator(device="cuda").manual_seed(2)
+    X = torch.randint(-90, 91, (1000, 1111), device="cuda", generator=g).float()
+    W = torch.randint(-90, 91, (1111, 700), device="cuda", generator=g).float()
+    assert torch.equal(_product(X, W).double(), X.double() @ W.double())
+
+
+@pytest.mark.parametrize("M,K,N", [(1024, 512, 1024), (1000, 1500, 777), (2048, 2048, 512)])
+def test_error_against_fp64(M, K, N):
+    """A chain of K fp32 multiply-adds of independent normal numbers is off by about 0.21 sqrt(K / 2) 2^-23 of the result
+    (2.8e-7 at 512, 5.6e-7 at 2048), a cut one by less in proportion to the root of the cut, at most eight."""
+    X, W = _operands(M, K, N)
+    R = X.double() @ W.double()
+    err = float((_product(X, W).double() - R).norm() / R.norm())
+    assert err <= 0.21 * (K / 16) ** 0.5 * 2.0 ** -23 + 6e-8
+
+
+def test_the_same_bits_every_time():
+    X, W = _operands(1000, 1500, 300)
+    ref = _product(X, W).clone()
+    for _ in range(20):
+        assert torch.equal(ref, _product(X, W))
