@@ -65,19 +65,25 @@ sbp_status fail(sbp_status s, const char* fmt, ...) {
 
 void count_launch(uint64_t n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
-int device_sms() {
+// An attribute of the current device, asked once a device; `none` where there is no device.
+template <cudaDeviceAttr ATTR>
+static int device_attribute(int none) {
   static std::atomic<int> known[64];
-  int dev = 0, n = 148;
+  int dev = 0, n = none;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
     cudaGetLastError();
     return n;
   }
   const int k = known[dev].load(std::memory_order_relaxed);
   if (k > 0) return k;
-  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) cudaGetLastError();
+  if (cudaDeviceGetAttribute(&n, ATTR, dev) != cudaSuccess) cudaGetLastError();
   known[dev].store(n, std::memory_order_relaxed);
   return n;
 }
+
+int device_sms() { return device_attribute<cudaDevAttrMultiProcessorCount>(148); }
+
+int device_l2_bytes() { return device_attribute<cudaDevAttrL2CacheSize>(126 << 20); }
 
 sbp_status cuda_fail(cudaError_t e, const char* what) {
   return fail(SBP_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));

@@ -87,6 +87,9 @@ sbp_status cuda_fail(cudaError_t e, const char* what);
 // SMs of the current device (asked once a device; a B200's 148 where there is none).
 int device_sms();
 
+// Bytes of its L2 cache.
+int device_l2_bytes();
+
 // Launch of `kernel` as a programmatic dependent of the kernel before it in the stream: if that
 // kernel releases its dependents early (SBP_PDL_RELEASE), this one's CTAs may be set up while its
 // last CTAs still run.  Such a kernel must execute SBP_PDL_WAIT before its first access to

@@ -42,6 +42,7 @@ struct XentParams {
   long long pitch[SBP_MAX_K];   // elements between consecutive rows of shard r's logits
   int k, nsplit;
   long long span;    // elements per CTA
+  long long keep_from;          // row, or CTA of the partial kernel, from which on what is read stays in L2
 };
 
 struct XentCombineParams {
@@ -108,10 +109,45 @@ __device__ __forceinline__ void merge_all(const float* ms, const float* ss, int 
 // ---- chunk policies: how one thread of a team loads, maxes and exp-sums its kLoadsPerThread vectors of 16 bytes.  z
 // points at the first vector (16-byte aligned), nv counts the vectors there are.
 
-__device__ __forceinline__ uint4 ld_logits(const void* p) {
+// The logits are read twice, by the forward pass and from their end by the backward.  What the forward pass reads last, as
+// much as stays in L2 beside the gradient, it reads with the usual priority, the rest as first to go; the backward's reads
+// and its results are the first to go as well.  (us, forward and backward, all with the usual priority / so: fp32
+// [256, 100003] over four 57.7 / 54.7, [128, 100003] 30.5 / 29.0, [256, 200000] 106.5 / 102.9, [4000, 8000] 72.7 / 71.1;
+// bf16 [512, 100000] 65.8 / 63.1.  The part to keep, MB, [256, 100003]: 40 55.4, 50 54.8, 60 54.7, 70 55.1, 100 55.4; the
+// priority to keep longest instead of the usual one 0.1 to 1 us slower.)
+constexpr long long kKeepNum = 7, kKeepDen = 16;      // of the device's L2 (126 MB: 55)
+__device__ __forceinline__ unsigned long long l2_usual() {
+  unsigned long long p;
+  asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
+// (made where it is used: kept in a register across the backward's loop it cost a CTA an SM, and more than it gave)
+__device__ __forceinline__ unsigned long long l2_first() {
+  unsigned long long p;
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
+
+__device__ __forceinline__ uint4 ld_logits(const void* p, unsigned long long priority) {
   uint4 r;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
+  asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %5;"
+               : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
+               : "l"(p), "l"(priority));
   return r;
+}
+
+// Two numbers in a register pair; two exponentials of (z - m) log2e, added to two sums.  The difference is exact in m, and in
+// pairs it and the product cost no more than one multiply-add an element did.
+__device__ __forceinline__ unsigned long long pair(float x, float y) {
+  unsigned long long v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
+  return v;
+}
+__device__ __forceinline__ void expsum_pair(unsigned long long z, unsigned long long neg_m, float& s0, float& s1) {
+  asm("add.rn.f32x2 %0, %0, %1;" : "+l"(z) : "l"(neg_m));
+  asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(z) : "l"(pair(kLog2e, kLog2e)));
+  s0 += ex2(__uint_as_float((unsigned)z));
+  s1 += ex2(__uint_as_float((unsigned)(z >> 32)));
 }
 
 // bf16, 8 elements per load; max on packed pairs, exp in fp32.
@@ -119,11 +155,11 @@ struct ChunkBF16 {
   using T = __nv_bfloat16;
   static constexpr int VEC = 8;
   uint4 raw[kLoadsPerThread];
-  __device__ __forceinline__ void load(const T* z, long long nv, int tid, int team) {
+  __device__ __forceinline__ void load(const T* z, long long nv, int tid, int team, unsigned long long priority) {
 #pragma unroll
     for (int u = 0; u < kLoadsPerThread; ++u) {
       const long long v = (long long)u * team + tid;
-      if (v < nv && SBP_GUARD(z + v * VEC, 16)) raw[u] = ld_logits(z + v * VEC);
+      if (v < nv && SBP_GUARD(z + v * VEC, 16)) raw[u] = ld_logits(z + v * VEC, priority);
       else raw[u] = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);   // -inf, -inf
     }
   }
@@ -137,35 +173,17 @@ struct ChunkBF16 {
     }
     return fmaxf(__low2float(mx), __high2float(mx));
   }
-  // sum of 2^(z*log2e + neg_m_l2e) over the thread's elements
-  __device__ __forceinline__ float expsum(float neg_m_l2e) const {
+  // sum of 2^((z - m) log2e) over the thread's elements
+  __device__ __forceinline__ float expsum(float m) const {
+    const unsigned long long neg = pair(-m, -m);
     float s0 = 0.f, s1 = 0.f;
 #pragma unroll
     for (int u = 0; u < kLoadsPerThread; ++u) {
       const uint32_t* w = reinterpret_cast<const uint32_t*>(&raw[u]);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float lo = __uint_as_float(w[i] << 16);
-        const float hi = __uint_as_float(w[i] & 0xffff0000u);
-        s0 += ex2(fmaf(lo, kLog2e, neg_m_l2e));
-        s1 += ex2(fmaf(hi, kLog2e, neg_m_l2e));
-      }
+      for (int i = 0; i < 4; ++i) expsum_pair(pair(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xffff0000u)), neg, s0, s1);
     }
     return s0 + s1;
-  }
-  // sum of 2^((z - m) log2e): exact in m, finite for every finite z
-  __device__ __forceinline__ float expsum_far(float m) const {
-    float s = 0.f;
-#pragma unroll
-    for (int u = 0; u < kLoadsPerThread; ++u) {
-      const uint32_t* w = reinterpret_cast<const uint32_t*>(&raw[u]);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        s += ex2((__uint_as_float(w[i] << 16) - m) * kLog2e);
-        s += ex2((__uint_as_float(w[i] & 0xffff0000u) - m) * kLog2e);
-      }
-    }
-    return s;
   }
 };
 
@@ -174,11 +192,11 @@ struct ChunkF32 {
   using T = float;
   static constexpr int VEC = 4;
   uint4 raw[kLoadsPerThread];
-  __device__ __forceinline__ void load(const T* z, long long nv, int tid, int team) {
+  __device__ __forceinline__ void load(const T* z, long long nv, int tid, int team, unsigned long long priority) {
 #pragma unroll
     for (int u = 0; u < kLoadsPerThread; ++u) {
       const long long v = (long long)u * team + tid;
-      if (v < nv && SBP_GUARD(z + v * VEC, 16)) raw[u] = ld_logits(z + v * VEC);
+      if (v < nv && SBP_GUARD(z + v * VEC, 16)) raw[u] = ld_logits(z + v * VEC, priority);
       else raw[u] = make_uint4(0xFF800000u, 0xFF800000u, 0xFF800000u, 0xFF800000u);   // -inf
     }
   }
@@ -192,27 +210,16 @@ struct ChunkF32 {
     }
     return m;
   }
-  __device__ __forceinline__ float expsum(float neg_m_l2e) const {
+  __device__ __forceinline__ float expsum(float m) const {
+    const unsigned long long neg = pair(-m, -m);
     float s0 = 0.f, s1 = 0.f;
 #pragma unroll
     for (int u = 0; u < kLoadsPerThread; ++u) {
       const float* f = reinterpret_cast<const float*>(&raw[u]);
-      s0 += ex2(fmaf(f[0], kLog2e, neg_m_l2e));
-      s1 += ex2(fmaf(f[1], kLog2e, neg_m_l2e));
-      s0 += ex2(fmaf(f[2], kLog2e, neg_m_l2e));
-      s1 += ex2(fmaf(f[3], kLog2e, neg_m_l2e));
+      expsum_pair(pair(f[0], f[1]), neg, s0, s1);
+      expsum_pair(pair(f[2], f[3]), neg, s0, s1);
     }
     return s0 + s1;
-  }
-  __device__ __forceinline__ float expsum_far(float m) const {
-    float s = 0.f;
-#pragma unroll
-    for (int u = 0; u < kLoadsPerThread; ++u) {
-      const float* f = reinterpret_cast<const float*>(&raw[u]);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) s += ex2((f[i] - m) * kLog2e);
-    }
-    return s;
   }
 };
 
@@ -228,15 +235,11 @@ __device__ __forceinline__ int to_boundary(const T* z, long long n) {
 // element by element, one element a thread, and what lies between as aligned vectors; the loads of the next chunk
 // are issued before the current one is reduced.  (Unaligned rows element by element throughout: fp32 [256, 100003]
 // over four shards 33 us, backward 76; as here 25 and 35: 0.62 and 0.89 of the copy bandwidth.)
-// An exponential is 2^(z log2e - c), c = m log2e rounded: one FMA an element.  What the rounding of c leaves, r = m log2e - c,
-// is a factor 2^r on all that the thread adds up in a chunk, up to 3e-7 at a maximum of 8; it is taken out of the chunk's
-// sum, to first order, which is enough (1e-9) up to a maximum of kNear; beyond that, where r grows to many units -- rows
-// masked with -1e9 and the like -- every exponent is formed from z - m.
+// An exponential is 2^((z - m) log2e): exact in the maximum, finite for every finite z.  (As 2^(z log2e - c), c = m log2e rounded,
+// with what the rounding leaves taken out of the sum to first order, rows wholly at -1e8 had a negative sum.)
 // What is carried from chunk to chunk is rescaled by the difference of the maxima: exactly 1 while the maximum stands.
-constexpr float kNear = 1024.f;
-
 template <typename Chunk>
-__device__ __forceinline__ void walk_span(const typename Chunk::T* z, long long n, int tid, int team, float& m, float& s) {
+__device__ __forceinline__ void walk_span(const typename Chunk::T* z, long long n, int tid, int team, unsigned long long priority, float& m, float& s) {
   using T = typename Chunk::T;
   constexpr int VEC = Chunk::VEC;
   const int head = to_boundary(z, n);
@@ -245,7 +248,7 @@ __device__ __forceinline__ void walk_span(const typename Chunk::T* z, long long 
   const T* zv = z + head;
   const long long step = (long long)team * kLoadsPerThread;     // vectors per chunk
   Chunk cur, nxt;
-  if (nv > 0) cur.load(zv, nv, tid, team);
+  if (nv > 0) cur.load(zv, nv, tid, team, priority);
   const T* lone = tid < head ? z + tid : (tid >= 16 && tid - 16 < tail ? zv + nv * VEC + (tid - 16) : nullptr);
   if (lone && SBP_GUARD(lone, sizeof(T))) {
     const float x = static_cast<float>(*lone);
@@ -253,17 +256,11 @@ __device__ __forceinline__ void walk_span(const typename Chunk::T* z, long long 
   }
   for (long long off = 0; off < nv; off += step) {
     const bool more = off + step < nv;
-    if (more) nxt.load(zv + (off + step) * VEC, nv - off - step, tid, team);
+    if (more) nxt.load(zv + (off + step) * VEC, nv - off - step, tid, team, priority);
     const float cm = cur.max();
     if (cm != -INFINITY) {                                      // not the threads of a short row that have nothing
-      const float mm = fmaxf(m, cm), c = mm * kLog2e;
-      const float carried = s * ex2((m - mm) * kLog2e);         // s is 0 as long as m is -inf
-      if (fabsf(mm) <= kNear) {
-        const float sum = cur.expsum(-c);
-        s = carried + fmaf(sum, -0.69314718f * fmaf(mm, kLog2e, -c), sum);
-      } else {
-        s = carried + cur.expsum_far(mm);
-      }
+      const float mm = fmaxf(m, cm);
+      s = s * ex2((m - mm) * kLog2e) + cur.expsum(mm);          // s is 0 as long as m is -inf
       m = mm;
     }
     if (more) cur = nxt;
@@ -302,7 +299,7 @@ __global__ void __launch_bounds__(kThreads) xent_rows_kernel(const __grid_consta
       long long c_start, c_len;
       split_range(p.classes, p.k, r, (int64_t*)&c_start, (int64_t*)&c_len);
       const T* z = reinterpret_cast<const T*>(p.logits[r]) + row * p.pitch[r];
-      if (c_len > 0) walk_span<Chunk>(z, c_len, tl, team, m, s);
+      if (c_len > 0) walk_span<Chunk>(z, c_len, tl, team, row >= p.keep_from ? l2_usual() : l2_first(), m, s);
       if (tl == 0 && y >= c_start && y < c_start + c_len && SBP_GUARD(z + (y - c_start), sizeof(T))) t = static_cast<float>(z[y - c_start]);
     }
   }
@@ -343,7 +340,8 @@ __global__ void __launch_bounds__(THREADS) xent_partial_kernel(const __grid_cons
   SBP_PDL_WAIT();
 
   float m = -INFINITY, s = 0.f;
-  if (n > 0) walk_span<Chunk>(z, n, tid, THREADS, m, s);
+  const long long cta = blockIdx.x + (long long)gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
+  if (n > 0) walk_span<Chunk>(z, n, tid, THREADS, cta >= p.keep_from ? l2_usual() : l2_first(), m, s);
 
   merge_warp(m, s);
   __shared__ float sm[THREADS / 32], ss[THREADS / 32];
@@ -654,7 +652,7 @@ __global__ void __launch_bounds__(kThreads) xent_backward_kernel(const __grid_co
     for (int u = 0; u < kBwdVecs; ++u) {
       const long long v = v0 + u * step;
       if (v >= nv || !SBP_GUARD(zv + v * VEC, sizeof(Pack))) continue;
-      if constexpr (VEC > 1) *reinterpret_cast<uint4*>(&in[u]) = ld_logits(zv + v * VEC);
+      if constexpr (VEC > 1) *reinterpret_cast<uint4*>(&in[u]) = ld_logits(zv + v * VEC, l2_first());
       else in[u] = *reinterpret_cast<const Pack*>(zv + v * VEC);
     }
 #pragma unroll
@@ -761,6 +759,10 @@ sbp_status sbp_softmax_xent(const sbp_tensor* logits, const sbp_tensor* labels, 
   SBP_BOUNDS_ADD(ws, 3 * (size_t)parts * rows * sizeof(float));
   SBP_BOUNDS_UPLOAD(stream);
   const int team_log2 = team_for(rows, classes, logits->dtype == SBP_BF16 ? 8 : 4);
+  // the last units of the walk, rows or CTAs, whose logits make up the part to keep
+  const double keep = std::min(1.0, (double)device_l2_bytes() * kKeepNum / kKeepDen / ((double)rows * classes * elem_size(logits->dtype)));
+  const long long units = team_log2 > 0 ? rows : rows * parts;
+  p.keep_from = units - (long long)(keep * units);
   if (team_log2 > 0) {
     const int per_cta = kThreads >> team_log2;
     const dim3 g((unsigned)((rows + per_cta - 1) / per_cta));
