@@ -22,6 +22,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <type_traits>
 
 #include "bounds_check.h"
 #include "matmul_plan.h"
@@ -41,6 +42,8 @@ struct F32Params {
   MatmulPlan plan;
   int splits;                    // CTAs per tile (cluster size)
   int a_vec, b_vec, y_vec;       // 16-byte copies / stores are possible everywhere
+  int early;                     // the small kernel lets the next one in at once
+  int a_quad, b_quad;            // and every quad of an operand lies inside it as a whole or not at all
 };
 
 __device__ __forceinline__ void cp_async16(unsigned dst, const void* src, unsigned bytes) {
@@ -333,6 +336,212 @@ cudaError_t launch_stored(const F32Params& P, dim3 grid, cudaStream_t st) {
   }
 }
 
+// ------------------------------------------------------------------ small products
+//
+// A product of a few small tiles is latency: launch, first loads, a chain of K-slices, an exchange.  Here the eight warps of a
+// CTA share a 32 x 32 tile and cut its contraction between them: a warp loads its slices into registers a slice ahead, passes
+// them through shared memory of its own and multiplies 4 x 8 elements a lane; the eight partial tiles are added in
+// their order.  No cluster to be placed, no barrier but the one before the sums.
+constexpr int kST = 32;                  // tile
+constexpr int kSWarps = 8;
+template <bool KC>
+constexpr int small_floats() { return KC ? kST * kKPitch : kBK * kST; }
+
+// One K-slice of an operand, 16 elements a lane.  KC: quad j of a lane is K quad (lane mod 4) of row lane / 4 + 8 j, else position
+// quad (lane mod 8) of K-step lane / 8 + 4 j.  The loads are predicated instructions, so that none waits for the one before.
+template <bool KC>
+struct SmallSlice {
+  float4 r[4];
+  template <bool VEC>
+  __device__ __forceinline__ void load(const float* g, long long ld, long long ext, long long kk, int lane) {
+    const int row = KC ? lane >> 2 : lane >> 3, col = (KC ? lane & 3 : lane & 7) * 4;
+    const long long rows = KC ? ext : kk, cols = KC ? kk : ext;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int at = row + j * (KC ? 8 : 4);
+      const float* src = g + at * ld + col;
+      const long long have = at < rows ? cols - col : 0;
+      r[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if constexpr (VEC) {       // whole quads inside or none
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %5, 0;\n\t@p ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}"
+                     : "+f"(r[j].x), "+f"(r[j].y), "+f"(r[j].z), "+f"(r[j].w)
+                     : "l"(src), "r"(have > 0 && SBP_GUARD(src, 16) ? 1 : 0));
+      } else {
+        float* e[4] = {&r[j].x, &r[j].y, &r[j].z, &r[j].w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p ld.global.nc.f32 %0, [%1];\n\t}"
+                       : "+f"(*e[i])
+                       : "l"(src + i), "r"(have > i && SBP_GUARD(src + i, 4) ? 1 : 0));
+      }
+    }
+  }
+  __device__ __forceinline__ void store(float* s, int lane) const {
+    const int row = KC ? lane >> 2 : lane >> 3, col = (KC ? lane & 3 : lane & 7) * 4;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) *reinterpret_cast<float4*>(s + (row + j * (KC ? 8 : 4)) * (KC ? kKPitch : kST) + col) = r[j];
+  }
+};
+
+template <int AT, int BT>
+__global__ void __launch_bounds__(32 * kSWarps) matmul_f32_small_kernel(const __grid_constant__ F32Params P) {
+  constexpr bool AKC = !AT, BKC = BT;
+  constexpr int kA = small_floats<AKC>(), kB = small_floats<BKC>(), kPitch = kST + 4;
+  constexpr int kFloats = kSWarps * (kA + kB) > kSWarps * kST * kPitch ? kSWarps * (kA + kB) : kSWarps * kST * kPitch;
+  __shared__ __align__(16) float smem[kFloats];
+  const MatmulPlan& p = P.plan;
+  const int g = blockIdx.z;
+  const long long M = p.m[g], N = p.n[g];
+  const long long m0 = (long long)blockIdx.y * kST, n0 = (long long)blockIdx.x * kST;
+  if (m0 >= M || n0 >= N) return;
+  // A product of a few CTAs lets the next kernel's in at once, they find SMs of their own; one of more, only when its sums are
+  // parked: earlier they delay it.  (Programs, us, at once / then: 64 x 128 x 96 x 80 on two shards, 6 and 8 CTAs, 9.2 / 10.4;
+  // 1734 x 72 x 90 x 16, 110 CTAs, 17.4 / 12.1; 336 x 334 x 435 x 172 on eight 31.4 / 28.4 where it was the slices' end.)
+  if (P.early) SBP_PDL_RELEASE();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ty = lane >> 2, tx = lane & 3;
+  auto row_of = [&](int i) { return AKC ? i * 8 + ty : ty * 4 + i; };
+  auto col_of = [&](int j) { return BKC ? j * 4 + tx : (j / 4) * 16 + tx * 4 + (j & 3); };
+
+  // this warp's range of K-slices over all segments
+  const int s_lo = p.chain ? 0 : g, s_hi = p.chain ? p.nseg : g + 1;
+  long long total = 0;
+  for (int s = s_lo; s < s_hi; ++s) total += (p.kseg[s] + kBK - 1) / kBK;
+  const long long it0 = total * warp / kSWarps;
+  const int iters = (int)(total * (warp + 1) / kSWarps - it0);
+  int ls = s_lo;
+  long long lk = it0;
+  while (ls < s_hi) {
+    const long long n = (p.kseg[ls] + kBK - 1) / kBK;
+    if (lk < n) break;
+    lk -= n;
+    ++ls;
+  }
+  lk *= kBK;
+  unsigned long long acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+  float* sa = smem + warp * (kA + kB);
+  float* sb = sa + kA;
+  SBP_PDL_WAIT();
+
+  auto run = [&](auto av, auto bv) {
+    constexpr bool AV = decltype(av)::value, BV = decltype(bv)::value;
+    SmallSlice<AKC> a;
+    SmallSlice<BKC> b;
+    auto load_next = [&]() {
+      while (ls < s_hi && lk >= p.kseg[ls]) { ++ls; lk = 0; }      // also steps over empty segments
+      const long long lda = p.lda[ls], ldb = p.ldb[ls], left = p.kseg[ls] - lk;
+      a.template load<AV>(static_cast<const float*>(p.a[ls]) + (AT ? lk * lda + p.row_off[g] + m0 : (p.row_off[g] + m0) * lda + lk), lda, M - m0, left, lane);
+      b.template load<BV>(static_cast<const float*>(p.b[ls]) + (BT ? (p.col_off[g] + n0) * ldb + lk : lk * ldb + p.col_off[g] + n0), ldb, N - n0, left, lane);
+      lk += kBK;
+    };
+    if (iters > 0) load_next();
+    for (int it = 0; it < iters; ++it) {
+      a.store(sa, lane);
+      b.store(sb, lane);
+      __syncwarp();
+      if (it + 1 < iters) load_next();
+#pragma unroll
+      for (int k0 = 0; k0 < kBK; k0 += 4) {
+        float x[4][4], w[8][4];
+        if constexpr (AKC) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) *reinterpret_cast<float4*>(x[i]) = *reinterpret_cast<const float4*>(sa + row_of(i) * kKPitch + k0);
+        }
+        if constexpr (BKC) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) *reinterpret_cast<float4*>(w[j]) = *reinterpret_cast<const float4*>(sb + col_of(j) * kKPitch + k0);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          float ak[4], bk[8];
+          if constexpr (AKC) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) ak[i] = x[i][k];
+          } else {
+            *reinterpret_cast<float4*>(ak) = *reinterpret_cast<const float4*>(sa + (k0 + k) * kST + row_of(0));
+          }
+#pragma unroll
+          for (int j = 0; j < 8; j += 4) {
+            if constexpr (BKC) { bk[j] = w[j][k]; bk[j + 1] = w[j + 1][k]; bk[j + 2] = w[j + 2][k]; bk[j + 3] = w[j + 3][k]; }
+            else *reinterpret_cast<float4*>(bk + j) = *reinterpret_cast<const float4*>(sb + (k0 + k) * kST + col_of(j));
+          }
+          unsigned long long bp[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) bp[j] = pack2(bk[2 * j], bk[2 * j + 1]);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const unsigned long long ap = pack2(ak[i], ak[i]);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) fma2(acc[i][j], ap, bp[j]);
+          }
+        }
+      }
+      __syncwarp();              // the slice has been read
+    }
+  };
+  if (P.a_quad && P.b_quad) run(std::true_type{}, std::true_type{});
+  else if (P.a_quad) run(std::true_type{}, std::false_type{});
+  else if (P.b_quad) run(std::false_type{}, std::true_type{});
+  else run(std::false_type{}, std::false_type{});
+
+  __syncthreads();               // every warp is done with its slices
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; j += 4) {
+      float v[4];
+      unpack2(acc[i][j / 2], v[0], v[1]);
+      unpack2(acc[i][j / 2 + 1], v[2], v[3]);
+      float* at = smem + (warp * kST + row_of(i)) * kPitch + col_of(j);
+      if constexpr (BKC) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) at[e * 4] = v[e];
+      } else {
+        *reinterpret_cast<float4*>(at) = make_float4(v[0], v[1], v[2], v[3]);
+      }
+    }
+  __syncthreads();
+  if (!P.early) SBP_PDL_RELEASE();
+  const int r = tid >> 3, c = (tid & 7) * 4;
+  if (m0 + r >= M || n0 + c >= N) return;
+  float v[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int w = 0; w < kSWarps; ++w) {
+    const float4 x = *reinterpret_cast<const float4*>(smem + (w * kST + r) * kPitch + c);
+    v[0] = w == 0 ? x.x : v[0] + x.x;
+    v[1] = w == 0 ? x.y : v[1] + x.y;
+    v[2] = w == 0 ? x.z : v[2] + x.z;
+    v[3] = w == 0 ? x.w : v[3] + x.w;
+  }
+  if (p.gelu) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v[e] = gelu_erf(v[e]);
+  }
+  const int n_out = (g == 0 ? p.n_rep : 0) + 1;
+  for (int q = 0; q < n_out; ++q) {
+    float* at = static_cast<float*>(q == 0 ? p.y[g] : p.y_rep[q - 1]) + (m0 + r) * p.ldy[g] + n0 + c;
+    if (P.y_vec && n0 + c + 3 < N) {
+      if (SBP_GUARD(at, 16)) *reinterpret_cast<float4*>(at) = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (n0 + c + e < N && SBP_GUARD(at + e, 4)) at[e] = v[e];
+    }
+  }
+}
+
+cudaError_t launch_small(const F32Params& P, dim3 grid, cudaStream_t st) {
+  switch ((P.plan.a_trans ? 2 : 0) | (P.plan.b_trans ? 1 : 0)) {
+    case 0: return launch_dependent(matmul_f32_small_kernel<0, 0>, grid, dim3(32 * kSWarps), 0, st, P);
+    case 1: return launch_dependent(matmul_f32_small_kernel<0, 1>, grid, dim3(32 * kSWarps), 0, st, P);
+    case 2: return launch_dependent(matmul_f32_small_kernel<1, 0>, grid, dim3(32 * kSWarps), 0, st, P);
+    default: return launch_dependent(matmul_f32_small_kernel<1, 1>, grid, dim3(32 * kSWarps), 0, st, P);
+  }
+}
+
 bool aligned16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
 
 }  // namespace
@@ -345,23 +554,29 @@ sbp_status launch_matmul_f32(const MatmulPlan& plan, cudaStream_t st) {
   F32Params P;
   P.plan = plan;
   P.a_vec = P.b_vec = P.y_vec = 1;
+  bool whole_k = true, whole_m = true, whole_n = true;
   long long iters = 0, mmax = 0, nmax = 0;
   for (int s = 0; s < plan.nseg; ++s) {
     if (!plan.chain && s >= plan.ngroups) continue;
     if (!aligned16(plan.a[s]) || plan.lda[s] % 4 != 0) P.a_vec = 0;
     if (!aligned16(plan.b[s]) || plan.ldb[s] % 4 != 0) P.b_vec = 0;
+    if (plan.kseg[s] % 4 != 0) whole_k = false;
     const long long n = (plan.kseg[s] + kBK - 1) / kBK;
     iters = plan.chain ? iters + n : (n > iters ? n : iters);
   }
   for (int g = 0; g < plan.ngroups; ++g) {
     mmax = plan.m[g] > mmax ? plan.m[g] : mmax;
     nmax = plan.n[g] > nmax ? plan.n[g] : nmax;
+    if (plan.m[g] % 4 != 0) whole_m = false;
+    if (plan.n[g] % 4 != 0) whole_n = false;
     if (plan.a_trans && plan.row_off[g] % 4 != 0) P.a_vec = 0;
     if (!plan.b_trans && plan.col_off[g] % 4 != 0) P.b_vec = 0;
     if (!aligned16(plan.y[g]) || plan.ldy[g] % 4 != 0) P.y_vec = 0;
   }
   for (int q = 0; q < plan.n_rep; ++q)
     if (!aligned16(plan.y_rep[q])) P.y_vec = 0;
+  P.a_quad = P.a_vec && (plan.a_trans ? whole_m : whole_k);
+  P.b_quad = P.b_vec && (plan.b_trans ? whole_k : whole_n);
   if (mmax == 0 || nmax == 0) return SBP_OK;
   if (iters > 0x7fffffffLL) return fail(SBP_ERR_UNSUPPORTED, "contraction too long for one launch");
 
@@ -373,7 +588,7 @@ sbp_status launch_matmul_f32(const MatmulPlan& plan, cudaStream_t st) {
   // on four shards 92 / 98-189, 700 x 2000 x 700 81 / 88-232, 100 x 2000 x 100 16 / 28-226.)
   const int sms = device_sms();
   int best_t = 0, best_s = 1;
-  double best = 1e300;
+  double best = 1e300, best_per_sm = 0;
   for (int t = 0; t < 2; ++t) {
     const int b = t == 0 ? 128 : 64;
     long long tiles = 0;
@@ -387,17 +602,45 @@ sbp_status launch_matmul_f32(const MatmulPlan& plan, cudaStream_t st) {
       const double exchange = s == 1 ? 0 : (t == 0 ? 4000 : 1000 + 450 * s);
       const double rounds = (double)(long long)((per_sm + resident - 1) / resident);
       const double cost = it * per_sm * each + rounds * (4000 + exchange);
-      if (cost < best) { best = cost; best_t = t; best_s = s; }
+      if (cost < best) { best = cost; best_per_sm = per_sm; best_t = t; best_s = s; }
     }
   }
-  // The tensor cores take it where their estimate (us) is below this one at 1.93 clocks a ns: measured times are 1.16 of this
-  // estimate at 1.9 GHz, and a switch has to win by some 15 %.  (us, this kernel / the other: 942 x 256 x 128 on three shards
+  // The small kernel: 2.2 us and 1.25 a slice of a warp's, 0.45 more for an operand that comes element by element, CTAs that
+  // share an SM 0.6 each.  Against it this kernel's estimate as measured, 1.16 of it at 1.9 GHz, less where every CTA has an SM of
+  // its own.  (us, this kernel / the small one: 64 x 96 x 80 on two shards 4.9 / 3.4, 40 x 98 x 640 5.0 / 3.4, 215 x 89 x 113 on
+  // eight 5.2 / 3.8, 1031 x 325 x 228 on three 17.4 / 10.4, 722 x 258 x 99 on two 8.1 / 9.1, 32 x 512 x 32 6.3 / 7.2, 90 x 789 x 85
+  // 10.0 / 12.4: a long contraction wants the cluster, and from four slices a warp on the switch has to win by a fifth: in a
+  // program of 133 x 620 x 622 x 187 on three the small kernel alone took 9.4, this one 13.0, the program 26.4 and 24.9.)
+  double fma_us = best_per_sm > 1 ? best / 1640 : 1.6 + 0.00032 * best;
+  const long long small_x = (nmax + kST - 1) / kST, small_y = (mmax + kST - 1) / kST;
+  bool small = false;
+  if (small_x <= 0x7fffffffLL && small_y <= 65535) {
+    long long tiles = 0;
+    for (int g = 0; g < plan.ngroups; ++g) tiles += ((plan.m[g] + kST - 1) / kST) * ((plan.n[g] + kST - 1) / kST);
+    const double per_sm = (double)((tiles + sms - 1) / sms);
+    const double slices = (double)((iters + kSWarps - 1) / kSWarps);
+    const double cost = 2.2 + slices * (1.25 + (P.a_quad ? 0 : 0.45) + (P.b_quad ? 0 : 0.45)) * (0.4 + 0.6 * per_sm);
+    if (cost < (slices > 3 ? 0.8 : 0.95) * fma_us) {
+      small = true;
+      P.early = 8 * tiles <= sms;
+      fma_us = cost;
+    }
+  }
+  // The tensor cores take it where their estimate (us) is below this kernel's at 1.93 clocks a ns -- a switch has to win by some
+  // 15 % -- and below the small one's.  (us, this kernel / the other: 942 x 256 x 128 on three shards
   // 8.1 / 9.0, 339 x 736 x 128 on two 8.9 / 9.4, 69 x 270 x 1639 on four 14.3 / 13.7, 187 x 1092 x 339 on four 17.9 / 14.6,
   // 1170 x 256 x 808 on three 30 / 17, 1000 x 1500 x 777 on four 92 / 38, 2048 x 2048 x 2048 422 / 153.)
   if (best > 11000) {
     int nb = 0, splits = 1;
     const double tc = f32_tc_cost(plan, &nb, &splits);
-    if (tc >= 0 && tc * 1930 < best) return launch_matmul_f32_tc(plan, nb, splits, st);
+    if (tc >= 0 && tc * 1930 < best && (!small || tc < fma_us)) return launch_matmul_f32_tc(plan, nb, splits, st);
+  }
+  if (small) {
+    SBP_BOUNDS_UPLOAD(st);
+    const cudaError_t e = launch_small(P, dim3((unsigned)small_x, (unsigned)small_y, (unsigned)plan.ngroups), st);
+    if (e != cudaSuccess) return cuda_fail(e, "matmul launch");
+    count_launch();
+    return SBP_OK;
   }
   if (best == 1e300) return fail(SBP_ERR_UNSUPPORTED, "matrix too large for the FMA kernel");
   const int b = best_t == 0 ? 128 : 64;

@@ -546,13 +546,17 @@ int cluster_capacity(int splits) {
 }  // namespace
 
 // The best cut of a plan for this kernel: estimated time in us (negative: it does not take the plan), columns of a tile, CTAs a
-// tile.  Per wave of clusters: a slot takes 0.81 us and 0.0032 more a column (all of its warps' round: loads, splitting,
-// twelve MMAs, the accumulators' turn), set-up, drain and stores 5.9 and 0.018 a column.  Fitted to 823 timings of 30 products
-// (rms error 10 %; the pick within 1.5 % of the best cut on the average).
+// tile.  Per wave of clusters: a slot takes 0.705 us and 0.0034 more a column (all of its warps' round: loads, splitting,
+// twelve MMAs, the accumulators' turn), 0.15 and 0.001 a column more where A / B come element by element, set-up, drain and
+// stores 6 and 0.016 a column.  Fitted to 823 timings of 30 products (rms error 8 %; the pick within 1.5 % of the best cut on
+// the average); the exchange is set dearer than in a row of equal calls, between others large clusters wait for their SMs.
 double f32_tc_cost(const MatmulPlan& plan, int* nb, int* splits) {
   long long slots = 0, mmax = 0, nmax = 0;
+  bool a_vec = true, b_vec = true;
   for (int s = 0; s < plan.nseg; ++s) {
     if (!plan.chain && s >= plan.ngroups) continue;
+    if (plan.lda[s] % 4 != 0) a_vec = false;
+    if (plan.ldb[s] % 4 != 0) b_vec = false;
     if (plan.kseg[s] > 0x7fffff00LL || plan.lda[s] > (1 << 25) || plan.ldb[s] > (1 << 25)) return -1;      // 32-bit steps
     const long long n = (plan.kseg[s] + kSK - 1) / kSK;
     slots = plan.chain ? slots + n : std::max(slots, n);
@@ -568,12 +572,13 @@ double f32_tc_cost(const MatmulPlan& plan, int* nb, int* splits) {
     const int w = (int)(((nmax + t - 1) / t + 15) / 16 * 16);
     long long tiles = 0;
     for (int g = 0; g < plan.ngroups; ++g) tiles += ((plan.m[g] + kTM - 1) / kTM) * ((plan.n[g] + w - 1) / w);
+    const double per_slot = 0.705 + 0.0034 * w + (a_vec ? 0 : 0.15) + (b_vec ? 0 : 0.001 * w);
     for (int s : {1, 2, 3, 4, 6, 8}) {
       if (slots < s) break;
       const int cap = cluster_capacity(s);
       if (cap < 1) continue;
       const double waves = (double)((tiles + cap - 1) / cap);
-      const double cost = waves * ((double)((slots + s - 1) / s) * (0.813 + 0.0032 * w) + 5.87 + 0.018 * w + (s > 1 ? 0.2 : 0.0));
+      const double cost = waves * ((double)((slots + s - 1) / s) * per_slot + 6.0 + 0.016 * w + (s > 1 ? 0.25 * s : 0.0));
       if (best < 0 || cost < best) {
         best = cost;
         *nb = w;
