@@ -293,7 +293,8 @@ void sbp_boxing_set_copy_engine(int32_t engine);
  * exactly the deduced pair, and every device multiplies its local tensors (no fused boxing).
  *
  * x: [M,K], w: [K,N], y: [M,N] logical, all 2-D, same dtype for x and w:
- *   SBP_F32  : fp32 FMA accumulation, y SBP_F32.
+ *   SBP_F32  : fp32 accuracy, y SBP_F32: fp32 multiply-adds, or for larger products six tensor-core products of bf16 parts
+ *              whose sums are added in fp32, no further from the exact result.
  *   SBP_BF16 : bf16 operands, fp32 accumulation on the tensor cores, y SBP_BF16 or SBP_F32.
  * flags: SBP_EPILOGUE_GELU applies GeLU(v) = v/2 (1 + erf(v/sqrt 2)) to the fp32
  * accumulator before the store; only where Y is S or B (GeLU is not linear, so it cannot
