@@ -20,9 +20,11 @@
 // MN-major tiles in chunks of 64 columns.  A tile whose K is long and whose device is otherwise idle is cut along K
 // over the CTAs of a cluster, whose partial tiles are added in order through distributed shared memory.
 //
-// Bound: the data path of shared memory.  Per slot of a 128 x 128 tile the MMAs read 768 lines of 128 bytes, the planes take
-// 384, the loads pass 256 to 512, in some 2200 clocks (768 for the MMAs alone); a wider tile shares the A operand
-// (192 columns 2800, 1870 for 128 of them), 16 warps for the operands instead of 8 change nothing (2048^3 157 and 153 us).
+// Bound: no one unit.  At 2048^3 the data path of shared memory is busy 65 % of the clocks (per slot of a 128 x 128 tile the MMAs
+// read 768 lines of 128 bytes, the planes take 384, the loads pass 256 to 512, in some 2200 clocks), the schedulers issue in 51 %,
+// the tensor pipe works in 30 %; a slot's round through loads, splitting, barriers and accumulators sets the pace.
+// A wider tile shares the A operand (192 columns 2800 clocks, 1870 for 128 of them); 16 warps for the operands instead of 8 change
+// nothing (2048^3 157 and 153 us).
 // 1000 x 1024 x 1500 on four shards 33 us, 1000 x 1500 x 777 38, 2048^3 153 (112 TFLOP/s); FMA kernel 87, 92, 422.
 //
 // A product that is not finite (operands or sums that are not, or a bf16 part that rounds to infinity) is found in
