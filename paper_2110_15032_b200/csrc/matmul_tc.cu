@@ -138,34 +138,37 @@ __device__ __forceinline__ unsigned long long mul_two(unsigned long long a, unsi
   return v;
 }
 
-// GeLU of two numbers, erf by the rational approximation 7.1.26 of Abramowitz & Stegun (|error| <= 1.5e-7), which is far
-// below the rounding of the bf16 / fp32 store that follows and costs two special-function operations where erff costs a
-// long polynomial.  With erf |z| = 1 - q(z), 0.5 v (1 + erf(v / sqrt 2)) = max(v, 0) - 0.5 |v| q: ten instructions a
-// number, the multiply-adds in pairs, where erf by itself and one number at a time took twenty.  The epilogue of a tile
-// that nothing overlaps is these instructions.
-// (|v| stops at 32, where q is 0, so that infinity stays infinity; NaN stays NaN.)
+__device__ __forceinline__ unsigned long long add_two(unsigned long long a, unsigned long long b) {
+  unsigned long long v;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+  return v;
+}
+
+// GeLU(v) = 0.5 v (1 + erf(v / sqrt 2)) of two numbers, erf by the rational approximation 7.1.26 of Abramowitz & Stegun
+// (|error| <= 1.5e-7), which is far below the rounding of the bf16 / fp32 store that follows and costs two special-function
+// operations where erff costs a long polynomial.  Each number goes through the operations of the formula in its order, so the
+// bits are those of the scalar form; in pairs they are ten and a half instructions a number where that takes twenty.  The
+// epilogue of a tile that nothing overlaps is these instructions.
 __device__ __forceinline__ void gelu_two(float& a, float& b) {
-  float ua, ub, pa, pb, ta, tb, ea, eb;
-  asm("min.NaN.f32 %0, %1, 0f42000000;" : "=f"(ua) : "f"(a));
-  asm("min.NaN.f32 %0, %1, 0f42000000;" : "=f"(ub) : "f"(b));
-  asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(pa) : "f"(a));
-  asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(pb) : "f"(b));
-  const unsigned long long u = two(fabsf(ua), fabsf(ub));
-  const unsigned long long d = fma_two(u, two(0.3275911f * 0.70710678118654752440f), two(1.0f));
-  const unsigned long long x = mul_two(mul_two(u, two(-0.72134752044448170368f)), u);      // -(v / sqrt 2)^2 log2 e
+  const unsigned long long v = two(a, b), x = mul_two(v, two(0.70710678118654752440f));
+  const unsigned x0 = (unsigned)x, x1 = (unsigned)(x >> 32);
+  const unsigned long long ax = two(fabsf(__uint_as_float(x0)), fabsf(__uint_as_float(x1)));
+  const unsigned long long d = fma_two(two(0.3275911f), ax, two(1.0f)), y = mul_two(mul_two(ax, ax), two(-1.4426950408889634f));
+  float ta, tb, ea, eb;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ta) : "f"(__uint_as_float((unsigned)d)));
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(tb) : "f"(__uint_as_float((unsigned)(d >> 32))));
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ea) : "f"(__uint_as_float((unsigned)x)));
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(eb) : "f"(__uint_as_float((unsigned)(x >> 32))));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ea) : "f"(__uint_as_float((unsigned)y)));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(eb) : "f"(__uint_as_float((unsigned)(y >> 32))));
   const unsigned long long t = two(ta, tb);
-  unsigned long long q = fma_two(t, two(-0.5f * 1.061405429f), two(0.5f * 1.453152027f));      // -0.5 q
-  q = fma_two(q, t, two(-0.5f * 1.421413741f));
-  q = fma_two(q, t, two(0.5f * 0.284496736f));
-  q = fma_two(q, t, two(-0.5f * 0.254829592f));
-  q = mul_two(mul_two(q, t), two(ea, eb));
-  const unsigned long long v = fma_two(u, q, two(pa, pb));
-  a = __uint_as_float((unsigned)v);
-  b = __uint_as_float((unsigned)(v >> 32));
+  unsigned long long q = fma_two(t, two(-1.061405429f), two(1.453152027f));      // the polynomial, negated
+  q = fma_two(q, t, two(-1.421413741f));
+  q = fma_two(q, t, two(0.284496736f));
+  q = fma_two(q, t, two(-0.254829592f));
+  q = fma_two(mul_two(q, t), two(ea, eb), two(1.0f));
+  const unsigned r0 = ((unsigned)q & 0x7fffffffu) | (x0 & 0x80000000u), r1 = ((unsigned)(q >> 32) & 0x7fffffffu) | (x1 & 0x80000000u);
+  const unsigned long long g = mul_two(mul_two(v, two(0.5f)), add_two(two(1.0f), two(__uint_as_float(r0), __uint_as_float(r1))));
+  a = __uint_as_float((unsigned)g);
+  b = __uint_as_float((unsigned)(g >> 32));
 }
 
 struct TileCoord {

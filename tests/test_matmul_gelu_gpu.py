@@ -1,4 +1,7 @@
 """GeLU in the epilogue of the tensor-core products, number by number: a contraction of one with ones leaves W itself."""
+import hashlib
+import os
+
 import pytest
 import torch
 
@@ -31,3 +34,26 @@ def test_gelu_of_every_kind_of_number(form, out):
     want = 0.5 * vd * torch.special.erfc(-vd / 2 ** 0.5)
     tol = vd.abs() * (0.75e-7 + 2.0 ** -22) + (want.abs() * 2.0 ** -8 if out == BF16 else 0.0) + 1e-37
     assert bool(((got - want).abs() <= tol)[:, :-2].all())
+
+
+@pytest.mark.parametrize("form", [sbp.SBP_TC_FORM_SQUARE, sbp.SBP_TC_FORM_TALL, sbp.SBP_TC_FORM_SPLIT])
+@pytest.mark.parametrize("out", [F32, BF16])
+def test_gelu_keeps_its_bits(form, out):
+    """The formula's operations in the formula's order, whichever way they are issued: a program's results do not move."""
+    v = torch.arange(1 << 16, dtype=torch.int32, device="cuda").to(torch.int16).view(BF16)
+    X = torch.ones(300, 1, dtype=BF16, device="cuda")
+    x, w = sbp.SbpTensor((300, 1), BF16, sbp.B, [X]), sbp.SbpTensor((1, 1 << 16), BF16, sbp.B, [v[None, :].contiguous()])
+    y = sbp.empty_global((300, 1 << 16), out, sbp.B, 1)
+    ws = torch.empty(max(256, sbp.sbp_matmul_workspace_bytes(x, w, y, sbp.SBP_EPILOGUE_GELU)), dtype=torch.uint8, device="cuda")
+    sbp.sbp_matmul_set_form(form, 0)
+    try:
+        sbp.sbp_matmul(x, w, y, sbp.SBP_EPILOGUE_GELU, ws)
+    finally:
+        sbp.sbp_matmul_set_form(sbp.SBP_TC_FORM_AUTO, 0)
+    Y = y.locals[0].cpu()
+    Y[torch.isnan(Y)] = float("nan")
+    bits = Y.view(torch.int32 if out == F32 else torch.int16)
+    assert bool((bits == bits[0]).all())
+    with open(os.path.join(os.path.dirname(__file__), "golden", "gelu_of_every_bf16.txt")) as f:
+        golden = dict(line.split() for line in f if not line.startswith("#"))
+    assert hashlib.sha256(bits[0].numpy().tobytes()).hexdigest() == golden["f32" if out == F32 else "bf16"]
