@@ -382,6 +382,17 @@ int32_t sbp_matmul_route(int64_t m, int64_t n, int64_t k, int32_t pairs, uint32_
                          int64_t* tall_tiles);
 void sbp_matmul_form_stats(uint64_t launches[3]);
 uint64_t sbp_matmul_split_launches(void);
+/* An fp32 product runs on one of three kernels: "tiled" (multiply-adds, 128 x 128 or 64 x 64 tiles), "small" (multiply-adds, 32 x 32
+ * tiles whose contraction the warps of a block share) or "tensor" (six tensor-core products of bf16 parts).  The library picks
+ * per product by estimated time.  sbp_matmul_set_f32_form overrides the choice for tests and measurements (process-wide, not a
+ * tuning knob; a product that the forced kernel does not take runs tiled); sbp_matmul_f32_form_stats reports the launches
+ * since the library was loaded: [0] tiled, [1] small, [2] tensor. */
+#define SBP_F32_FORM_AUTO 0
+#define SBP_F32_FORM_TILED 1
+#define SBP_F32_FORM_SMALL 2
+#define SBP_F32_FORM_TENSOR 3
+void sbp_matmul_set_f32_form(int32_t form);
+void sbp_matmul_f32_form_stats(uint64_t launches[3]);
 sbp_status sbp_matmul(const sbp_tensor* x, const sbp_tensor* w, sbp_tensor* y, uint32_t flags,
                       void* ws, size_t ws_bytes, void* cuda_stream);
 

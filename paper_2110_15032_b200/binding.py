@@ -130,6 +130,10 @@ def load_library():
     lib.sbp_matmul_route.argtypes = [C.c_int64, C.c_int64, C.c_int64, C.c_int32, C.c_uint32, C.c_int32, C.c_int32, C.POINTER(C.c_int64)]
     lib.sbp_matmul_route.restype = C.c_int32
     lib.sbp_matmul_form_stats.restype = None
+    lib.sbp_matmul_set_f32_form.argtypes = [C.c_int32]
+    lib.sbp_matmul_set_f32_form.restype = None
+    lib.sbp_matmul_f32_form_stats.argtypes = [C.POINTER(C.c_uint64)]
+    lib.sbp_matmul_f32_form_stats.restype = None
     lib.sbp_softmax_xent_workspace_bytes.restype = C.c_size_t
     lib.sbp_softmax_xent_workspace_bytes.argtypes = [T]
     lib.sbp_softmax_xent.argtypes = [T, T, T, T, T, C.c_void_p, C.c_size_t, C.c_void_p]
@@ -346,6 +350,21 @@ def sbp_matmul_form_stats():
 def sbp_matmul_split_launches() -> int:
     """Launches of the tensor-core MatMul's split form since the library was loaded (counted among the square ones too)."""
     return int(load_library().sbp_matmul_split_launches())
+
+
+SBP_F32_FORM_AUTO, SBP_F32_FORM_TILED, SBP_F32_FORM_SMALL, SBP_F32_FORM_TENSOR = 0, 1, 2, 3
+
+
+def sbp_matmul_set_f32_form(form: int = 0) -> None:
+    """Test and measurement override of the kernel that fp32 products run on."""
+    load_library().sbp_matmul_set_f32_form(int(form))
+
+
+def sbp_matmul_f32_form_stats():
+    """Launches of the fp32 kernels: (tiled, small, tensor cores)."""
+    v = (C.c_uint64 * 3)()
+    load_library().sbp_matmul_f32_form_stats(v)
+    return int(v[0]), int(v[1]), int(v[2])
 
 
 def sbp_selftest_debug_bounds(buf: torch.Tensor, stream=None) -> None:

@@ -34,6 +34,8 @@ void tensor_map_cache_stats(unsigned long long* hits, unsigned long long* encode
 void tc_form_stats(unsigned long long out[3]);
 unsigned long long tc_split_launches();
 void tc_set_form(int form, int max_pairs);
+void f32_set_form(int form);                        // matmul_f32.cu
+void f32_form_stats(unsigned long long out[3]);
 int tc_route(long long tiles_sq, long long tiles_tall, long long kb, int pairs, bool gelu, int n_rep, bool out_f32, int forced,
              long long* tall_tiles);
 
@@ -574,6 +576,15 @@ int32_t sbp_matmul_route(int64_t m, int64_t n, int64_t k, int32_t pairs, uint32_
 void sbp_matmul_form_stats(uint64_t launches[3]) {
   unsigned long long v[3] = {0, 0, 0};
   tc_form_stats(v);
+  if (launches)
+    for (int i = 0; i < 3; ++i) launches[i] = v[i];
+}
+
+void sbp_matmul_set_f32_form(int32_t form) { f32_set_form(form); }
+
+void sbp_matmul_f32_form_stats(uint64_t launches[3]) {
+  unsigned long long v[3] = {0, 0, 0};
+  f32_form_stats(v);
   if (launches)
     for (int i = 0; i < 3; ++i) launches[i] = v[i];
 }

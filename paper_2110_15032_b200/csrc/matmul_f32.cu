@@ -546,6 +546,19 @@ bool aligned16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0;
 
 }  // namespace
 
+// Test and measurement override of the choice below, and the launches of each kernel: [0] tiled, [1] small, [2] tensor cores.
+static std::atomic<int> g_f32_form{SBP_F32_FORM_AUTO};
+static std::atomic<unsigned long long> g_f32_launches[3];
+
+void f32_set_form(int form) { g_f32_form.store(form, std::memory_order_relaxed); }
+void f32_form_stats(unsigned long long out[3]) {
+  for (int i = 0; i < 3; ++i) out[i] = g_f32_launches[i].load(std::memory_order_relaxed);
+}
+static void count_f32_launch(int form) {
+  g_f32_launches[form - 1].fetch_add(1, std::memory_order_relaxed);
+  count_launch();
+}
+
 // Defined in matmul_f32_tc.cu: the same product from bf16 parts on the tensor cores.
 double f32_tc_cost(const MatmulPlan& plan, int* nb, int* splits);
 sbp_status launch_matmul_f32_tc(const MatmulPlan& plan, int nb, int splits, cudaStream_t st);
@@ -586,7 +599,7 @@ sbp_status launch_matmul_f32(const MatmulPlan& plan, cudaStream_t st) {
   // 1075 each from three.  A round of CTAs costs about 4000 clocks of launch and pipeline fill, a split
   // its exchange through distributed shared memory.  (us, this rule / the other choices: 1000 x 1500 x 777
   // on four shards 92 / 98-189, 700 x 2000 x 700 81 / 88-232, 100 x 2000 x 100 16 / 28-226.)
-  const int sms = device_sms();
+  const int sms = device_sms(), form = g_f32_form.load(std::memory_order_relaxed);
   int best_t = 0, best_s = 1;
   double best = 1e300, best_per_sm = 0;
   for (int t = 0; t < 2; ++t) {
@@ -622,7 +635,8 @@ sbp_status launch_matmul_f32(const MatmulPlan& plan, cudaStream_t st) {
     const double per_sm = (double)((tiles + sms - 1) / sms);
     const double slices = (double)((iters + kSWarps - 1) / kSWarps);
     const double cost = 2.2 + slices * (1.25 + (P.a_quad ? 0 : 0.45) + (P.b_quad ? 0 : 0.45)) * (0.4 + 0.6 * per_sm);
-    if (slices == 1 && per_sm > 1 ? cost + 2.5 < fma_us : cost < (slices > 3 ? 0.8 : 0.95) * fma_us) {
+    const bool wins = slices == 1 && per_sm > 1 ? cost + 2.5 < fma_us : cost < (slices > 3 ? 0.8 : 0.95) * fma_us;
+    if (form == SBP_F32_FORM_AUTO ? wins : form == SBP_F32_FORM_SMALL) {
       small = true;
       P.early = 8 * tiles <= sms;
       fma_us = cost;
@@ -633,16 +647,20 @@ sbp_status launch_matmul_f32(const MatmulPlan& plan, cudaStream_t st) {
   // other, alone: 69 x 270 x 1639 on four shards 14.3 / 13.7, 187 x 1092 x 339 on four 17.9 / 14.6, 1170 x 256 x 808 on three 30 / 17,
   // 1000 x 1500 x 777 on four 92 / 38, 2048 x 2048 x 2048 422 / 153; programs of 116 x 1047 x 387 x 16 on three 24.8 / 27.3, 58 x 79 x
   // 1132 x 1272 on eight 28.4 / 30.7, 1809 x 26 x 1014 x 51 on three 59 / 53.)
-  if (best > 11000) {
+  if (form == SBP_F32_FORM_AUTO ? best > 11000 : form == SBP_F32_FORM_TENSOR) {
     int nb = 0, splits = 1;
     const double tc = f32_tc_cost(plan, &nb, &splits);
-    if (tc >= 0 && tc + 4 < best / 1750 && (!small || tc + 4 < fma_us)) return launch_matmul_f32_tc(plan, nb, splits, st);
+    if (tc >= 0 && (form != SBP_F32_FORM_AUTO || (tc + 4 < best / 1750 && (!small || tc + 4 < fma_us)))) {
+      const sbp_status status = launch_matmul_f32_tc(plan, nb, splits, st);
+      if (status == SBP_OK) count_f32_launch(SBP_F32_FORM_TENSOR);
+      return status;
+    }
   }
   if (small) {
     SBP_BOUNDS_UPLOAD(st);
     const cudaError_t e = launch_small(P, dim3((unsigned)small_x, (unsigned)small_y, (unsigned)plan.ngroups), st);
     if (e != cudaSuccess) return cuda_fail(e, "matmul launch");
-    count_launch();
+    count_f32_launch(SBP_F32_FORM_SMALL);
     return SBP_OK;
   }
   if (best == 1e300) return fail(SBP_ERR_UNSUPPORTED, "matrix too large for the FMA kernel");
@@ -654,7 +672,7 @@ sbp_status launch_matmul_f32(const MatmulPlan& plan, cudaStream_t st) {
   SBP_BOUNDS_UPLOAD(st);
   const cudaError_t e = best_t == 0 ? launch_stored<8, 8>(P, grid, st) : launch_stored<4, 4>(P, grid, st);
   if (e != cudaSuccess) return cuda_fail(e, "matmul launch");
-  count_launch();
+  count_f32_launch(SBP_F32_FORM_TILED);
   return SBP_OK;
 }
 

@@ -615,7 +615,6 @@ sbp_status launch_matmul_f32_tc(const MatmulPlan& plan, int nb, int splits, cuda
     default: e = launch_form<1, 1>(&P, splits, grid, st, nullptr); break;
   }
   if (e != cudaSuccess) return cuda_fail(e, "matmul launch");
-  count_launch();
   return SBP_OK;
 }
 

@@ -1,0 +1,68 @@
+"""The three kernels of fp32 products, each forced and each counted: edges of its tiles and K-slices, contractions of one slice and
+of many a warp, chained segments of uneven and zero length, both stored forms, more tiles than the early release of the small
+kernel allows.  And what the library picks by itself, where the other tests of these kernels rely on it."""
+import pytest
+import torch
+
+import paper_2110_15032_b200 as sbp
+from test_ops_gpu import _matmul_case
+
+pytestmark = pytest.mark.gpu
+F32 = torch.float32
+S0, S1, B = sbp.S(0), sbp.S(1), sbp.B
+TILED, SMALL, TENSOR = sbp.SBP_F32_FORM_TILED, sbp.SBP_F32_FORM_SMALL, sbp.SBP_F32_FORM_TENSOR
+
+
+@pytest.fixture(autouse=True)
+def _the_librarys_choice_afterwards():
+    yield
+    sbp.sbp_matmul_set_f32_form(sbp.SBP_F32_FORM_AUTO)
+
+
+def _case(form, *args, **kw):
+    """One product on the kernel `form`, forced or (0) as chosen; returns the kernel that ran."""
+    sbp.sbp_matmul_set_f32_form(form)
+    before = sbp.sbp_matmul_f32_form_stats()
+    _matmul_case(*args, **kw)
+    ran = [b - a for a, b in zip(before, sbp.sbp_matmul_f32_form_stats())]
+    assert sum(ran) == 1 and (not form or ran[form - 1] == 1), (form, ran)
+    return ran.index(1) + 1
+
+
+@pytest.mark.parametrize("M,K,N", [(2048, 64, 2048), (1153, 37, 2050), (512, 256, 512), (500, 250, 509),      # 128 x 128, the latter cut in eight
+                                   (64, 16, 64), (65, 17, 63), (40, 2500, 24), (257, 130, 1030)])               # 64 x 64
+@pytest.mark.parametrize("tx,tw", [(False, False), (True, True)])
+def test_tiled(M, K, N, tx, tw):
+    _case(TILED, M, K, N, 1, F32, B, B, tx=tx, tw=tw)
+
+
+@pytest.mark.parametrize("K", [1, 16, 17, 127, 129, 260, 1000])
+@pytest.mark.parametrize("M,N", [(1, 1), (33, 65), (100, 36), (31, 200), (225, 131)])
+@pytest.mark.parametrize("tx,tw", [(False, False), (True, False), (False, True), (True, True)])
+def test_small(M, K, N, tx, tw):
+    _case(SMALL, M, K, N, 1, F32, B, B, tx=tx, tw=tw)
+
+
+@pytest.mark.parametrize("K", [1, 31, 33, 64, 257])
+@pytest.mark.parametrize("M,N", [(1, 1), (128, 16), (129, 17), (127, 193), (130, 400)])
+@pytest.mark.parametrize("tx,tw", [(False, False), (True, False), (False, True), (True, True)])
+def test_tensor(M, K, N, tx, tw):
+    _case(TENSOR, M, K, N, 1, F32, B, B, tx=tx, tw=tw)
+
+
+@pytest.mark.parametrize("form", [TILED, SMALL, TENSOR])
+@pytest.mark.parametrize("M,K,N,k", [(70, 45, 83, 3), (33, 5, 130, 8), (200, 700, 90, 5)])
+@pytest.mark.parametrize("ys", [B, S0, S1])
+@pytest.mark.parametrize("tx,tw", [(False, False), (True, True)])
+def test_groups_and_segments(form, M, K, N, k, ys, tx, tw):
+    _case(form, M, K, N, k, F32, S0, B, tx=tx, tw=tw)
+    _case(form, M, K, N, k, F32, B, S1, tx=tx, tw=tw)
+    _case(form, M, K, N, k, F32, S1, S0, ys=ys, tx=tx, tw=tw, flags=sbp.SBP_EPILOGUE_GELU if ys == S0 else 0)
+
+
+def test_the_librarys_choice():
+    """Far from the lines between them: tests of the tensor cores' accuracy and of its ranges count on this one."""
+    assert _case(0, 64, 128, 96, 2, F32, S0, B) == SMALL
+    assert _case(0, 32, 512, 32, 1, F32, B, B) == TILED
+    for M, K, N in ((1024, 1024, 640), (1000, 1500, 777), (1000, 1111, 700), (1024, 512, 1024), (2048, 2048, 512), (1000, 1500, 300)):
+        assert _case(0, M, K, N, 1, F32, B, B) == TENSOR
