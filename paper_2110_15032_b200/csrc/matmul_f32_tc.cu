@@ -28,7 +28,7 @@
 // 1000 x 1024 x 1500 on four shards 33 us, 1000 x 1500 x 777 38, 2048^3 153 (112 TFLOP/s); FMA kernel 87, 92, 422.
 //
 // A product that is not finite (operands or sums that are not, or a bf16 part that rounds to infinity) is found in
-// the accumulators; the CTA then multiplies its tile again with fp32 multiply-adds in ascending order.
+// the accumulators; the CTA then multiplies its tile again with fp32 multiply-adds (multiply_again).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -174,6 +174,12 @@ __device__ __forceinline__ void add2(unsigned long long& a, unsigned long long b
 __device__ __forceinline__ float lo(unsigned long long v) { return __uint_as_float((unsigned)v); }
 __device__ __forceinline__ float hi(unsigned long long v) { return __uint_as_float((unsigned)(v >> 32)); }
 
+__device__ __forceinline__ unsigned long long pack(float x, float y) {
+  unsigned long long v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
+  return v;
+}
+
 // 16 accumulator columns of this warp's 32 rows, in pairs
 __device__ __forceinline__ void tmem_ld16_wait(unsigned taddr, unsigned long long (&v)[8]) {
   unsigned r[16];
@@ -188,6 +194,147 @@ __device__ __forceinline__ void tmem_ld16_wait(unsigned taddr, unsigned long lon
   for (int i = 0; i < 8; ++i) asm("mov.b64 %0, {%1, %2};" : "=l"(v[i]) : "r"(r[2 * i]), "r"(r[2 * i + 1]));
 }
 
+// 4 * QUARTERS bytes, or as many zeros
+template <int QUARTERS>
+__device__ __forceinline__ void copy_async(const float* to, const float* from, const float* somewhere, bool in) {
+  if constexpr (QUARTERS == 4)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(to)), "l"(in ? from : somewhere), "r"(in ? 16u : 0u) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_addr(to)), "l"(in ? from : somewhere), "r"(in ? 4u : 0u) : "memory");
+}
+
+// Whole aligned quads everywhere, or element by element?
+template <int AT, int BT>
+__device__ __forceinline__ void whole_quads(const MatmulPlan& p, int g, int s_lo, int s_hi, int rows, int cols, bool& a, bool& b) {
+  a = AT ? (rows & 3) == 0 && (p.row_off[g] & 3) == 0 : true;
+  b = BT ? true : (cols & 3) == 0 && (p.col_off[g] & 3) == 0;
+  for (int s = s_lo; s < s_hi; ++s) {
+    a = a && (reinterpret_cast<unsigned long long>(p.a[s]) & 15) == 0 && (p.lda[s] & 3) == 0 && (AT || (p.kseg[s] & 3) == 0);
+    b = b && (reinterpret_cast<unsigned long long>(p.b[s]) & 15) == 0 && (p.ldb[s] & 3) == 0 && (!BT || (p.kseg[s] & 3) == 0);
+  }
+}
+
+// A slot of an operand on its way into shared memory, in the order it has: K-contiguous as rows of kSK + 4, else `width` positions a
+// K-step, `pitch` apart.  Q elements at once.
+constexpr int kAll = kDrain + kWorkers, kPitchK = kSK + 4;
+template <int Q, bool KC>
+__device__ __forceinline__ void fill_slot(float* to, const float* from, long long ld, int ext, int left, int width, int pitch, int tid) {
+  if constexpr (KC) {
+    constexpr int kPer = kSK / Q;
+    for (int r = tid / kPer; r < width; r += kAll / kPer) {
+      const int k = tid % kPer * Q;
+      const float* src = from + r * ld + k;
+      copy_async<Q>(to + r * kPitchK + k, src, from, r < ext && k < left && SBP_GUARD(src, Q * 4));
+    }
+  } else {
+    for (int k = tid >> 5; k < kSK; k += kAll / 32)
+      for (int c = (tid & 31) * Q; c < width; c += 32 * Q) {
+        const float* src = from + k * ld + c;
+        copy_async<Q>(to + k * pitch + c, src, from, k < left && c < ext && SBP_GUARD(src, Q * 4));
+      }
+  }
+}
+
+// A tile that bf16 parts do not serve, once more with fp32 multiply-adds, by the warps of the accumulators and of the operands:
+// 4 x 12 elements a thread, slots of fp32 operands in two buffers at the ring's end.  A chain is four slots, its sum goes to the
+// tile.  Bound: the FMA pipe, 64 clocks a K-step and 64 columns.
+// (us, a product on the tensor cores / with every tile once more / on the FMA kernel, whose tiles fill the device more evenly:
+// 1024^3 27 / 123 / 61, 2048^3 165 / 908 / 422, 1000 x 1500 x 777 36 / 168 / 95; one chain of loads an element: 4740, 35200, 3200.)
+template <int AT, int BT>
+__device__ __forceinline__ void multiply_again(const MatmulPlan& p, int g, int s, int s_hi, long long k, int iters, long long m0, long long n0,
+                                               int rows, int cols, int nb, bool a_vec, bool b_vec, unsigned char* smem, int tid) {
+  constexpr bool AKC = !AT, BKC = BT;
+  constexpr int kPitchA = kTM + 4, kPitchB = kTN + 4, kChain = 4;
+  constexpr int kA = AKC ? kTM * kPitchK : kSK * kPitchA, kB = BKC ? kTN * kPitchK : kSK * kPitchB;
+  static_assert(kTM * (kTN + 4) * 4 + 2 * (kA + kB) * 4 <= kRing, "tile and two buffers");
+  float* const buffers = reinterpret_cast<float*>(smem + kRing) - 2 * (kA + kB);
+  const int ty = tid >> 4, tx = tid & 15;
+  float* const out = reinterpret_cast<float*>(smem) + ty * 4 * (nb + 4) + (BKC ? tx : tx * 4);
+  auto fill = [&](int b) {
+    while (s < s_hi && k >= p.kseg[s]) { ++s; k = 0; }      // also steps over empty segments
+    const int left = (int)min((long long)kSK, p.kseg[s] - k);
+    const long long lda = p.lda[s], ldb = p.ldb[s];
+    const float* A = static_cast<const float*>(p.a[s]) + (AT ? k * lda + p.row_off[g] + m0 : (p.row_off[g] + m0) * lda + k);
+    const float* B = static_cast<const float*>(p.b[s]) + (BT ? (p.col_off[g] + n0) * ldb + k : k * ldb + p.col_off[g] + n0);
+    float* to = buffers + b * (kA + kB);
+    if (a_vec) fill_slot<4, AKC>(to, A, lda, rows, left, kTM, kPitchA, tid);
+    else fill_slot<1, AKC>(to, A, lda, rows, left, kTM, kPitchA, tid);
+    if (b_vec) fill_slot<4, BKC>(to + kA, B, ldb, cols, left, nb, kPitchB, tid);
+    else fill_slot<1, BKC>(to + kA, B, ldb, cols, left, nb, kPitchB, tid);
+    k += kSK;
+  };
+  unsigned long long acc[4][6];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 6; ++j) acc[i][j] = 0ull;
+  if (iters > 0) fill(0);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+#pragma unroll 1
+  for (int it = 0; it < iters; ++it) {
+    if (it + 1 < iters) fill((it + 1) & 1);
+    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 1;" ::: "memory");
+    asm volatile("bar.sync 2, 512;" ::: "memory");
+    const float* sa = buffers + (it & 1) * (kA + kB) + ty * 4 * (AKC ? kPitchK : 1);
+    const float* sb = buffers + (it & 1) * (kA + kB) + kA + tx * (BKC ? kPitchK : 4);
+#pragma unroll 2
+    for (int k0 = 0; k0 < kSK; k0 += 2) {
+      float2 x[4];                                     // of row i, two K-steps
+      if constexpr (AKC) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = *reinterpret_cast<const float2*>(sa + i * kPitchK + k0);
+      } else {
+        const float4 u = *reinterpret_cast<const float4*>(sa + k0 * kPitchA), v = *reinterpret_cast<const float4*>(sa + (k0 + 1) * kPitchA);
+        x[0] = make_float2(u.x, v.x); x[1] = make_float2(u.y, v.y); x[2] = make_float2(u.z, v.z); x[3] = make_float2(u.w, v.w);
+      }
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {                    // columns past nb: whatever lies there, never stored
+        if (j * 64 >= nb) break;
+        unsigned long long w[2][2];                    // K-step, pair of columns
+        if constexpr (BKC) {
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const float2 u = *reinterpret_cast<const float2*>(sb + (j * 64 + e * 32) * kPitchK + k0);
+            const float2 v = *reinterpret_cast<const float2*>(sb + (j * 64 + e * 32 + 16) * kPitchK + k0);
+            w[0][e] = pack(u.x, v.x);
+            w[1][e] = pack(u.y, v.y);
+          }
+        } else {
+#pragma unroll
+          for (int kk = 0; kk < 2; ++kk) {
+            const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(sb + (k0 + kk) * kPitchB + j * 64);
+            w[kk][0] = u.x;
+            w[kk][1] = u.y;
+          }
+        }
+#pragma unroll
+        for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const unsigned long long a = kk ? pack(x[i].y, x[i].y) : pack(x[i].x, x[i].x);
+            asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[i][2 * j]) : "l"(a), "l"(w[kk][0]));
+            asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[i][2 * j + 1]) : "l"(a), "l"(w[kk][1]));
+          }
+      }
+    }
+    if ((it + 1) % kChain == 0 || it + 1 == iters) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          const float v[4] = {lo(acc[i][2 * j]), hi(acc[i][2 * j]), lo(acc[i][2 * j + 1]), hi(acc[i][2 * j + 1])};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            float* at = out + i * (nb + 4) + j * 64 + (BKC ? e * 16 : e);
+            if (j * 64 + (BKC ? e * 16 + tx : tx * 4 + e) < nb) *at = it >= kChain ? *at + v[e] : v[e];
+          }
+          acc[i][2 * j] = acc[i][2 * j + 1] = 0ull;
+        }
+    }
+    asm volatile("bar.sync 2, 512;" ::: "memory");      // the buffer has been read
+  }
+}
+
 // AT / BT: the operand is stored transposed.  A as given and B transposed are K-contiguous.
 template <int AT, int BT>
 __global__ void __launch_bounds__(kThreads, 1) matmul_f32_tc_kernel(const __grid_constant__ F32TcParams P) {
@@ -195,7 +342,7 @@ __global__ void __launch_bounds__(kThreads, 1) matmul_f32_tc_kernel(const __grid
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long bar_full[kMaxSlots], bar_empty[kMaxSlots], bar_acc_full[kAccs], bar_acc_empty[kAccs];
   __shared__ unsigned tmem_base_slot;
-  __shared__ int abort_flag_s, redo_s;
+  __shared__ int abort_flag_s, again_s;
   volatile int* abort_flag = &abort_flag_s;
 
   const MatmulPlan& p = P.plan;
@@ -210,7 +357,7 @@ __global__ void __launch_bounds__(kThreads, 1) matmul_f32_tc_kernel(const __grid
 
   if (tid == 0) {
     abort_flag_s = 0;
-    redo_s = 0;
+    again_s = 0;
     for (int i = 0; i < slots; ++i) {
       mbar_init(smem_addr(&bar_full[i]), kWorkers / 32);
       mbar_init(smem_addr(&bar_empty[i]), 1);
@@ -241,6 +388,8 @@ __global__ void __launch_bounds__(kThreads, 1) matmul_f32_tc_kernel(const __grid
     ++seg0;
   }
   k0 *= kSK;
+  bool a_vec, b_vec;
+  whole_quads<AT, BT>(p, g, s_lo, s_hi, rows, cols, a_vec, b_vec);
 
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -249,6 +398,7 @@ __global__ void __launch_bounds__(kThreads, 1) matmul_f32_tc_kernel(const __grid
   SBP_PDL_WAIT();                                  // everything up to here overlaps the kernel before this one
 
   const int q = warp & 3, half = (warp >> 2) & 1, width = nb / 2;      // a draining warp's tensor-memory lanes and columns
+  if (warp < kMmaWarp) {                           // two roles that end with the same registers
   if (warp < kDrain / 32) {
     // ------------------------------------------------ accumulators
     asm volatile("setmaxnreg.inc.sync.aligned.u32 128;");        // 2 x 128 + 2 x 88 + 48 = 5 x 96
@@ -283,46 +433,18 @@ __global__ void __launch_bounds__(kThreads, 1) matmul_f32_tc_kernel(const __grid
 #pragma unroll
       for (int e = 0; e < 4; ++e) zero = fmaf(hi(acc[i + e]), 0.f, fmaf(lo(acc[i + e]), 0.f, zero));
     }
-    if (zero != 0.f) redo_s = 1;
+    if (zero != 0.f) again_s = 1;
     asm volatile("bar.sync 1, 256;" ::: "memory");      // every warp has seen its last chunk
 #pragma unroll
     for (int i = 0; i < kTN / 4; i += 2) {
       if (2 * i >= width) break;
       *reinterpret_cast<float4*>(tile + 2 * i) = make_float4(lo(acc[i]), hi(acc[i]), lo(acc[i + 1]), hi(acc[i + 1]));
     }
-    if (redo_s) {
-      asm volatile("bar.sync 1, 256;" ::: "memory");
-      for (int idx = tid; idx < kTM * cols; idx += kDrain) {
-        const int r = idx % kTM, c = idx / kTM;
-        if (r >= rows) continue;
-        float sum = 0.f;
-        int s = seg0;
-        long long k = k0;
-        for (int n = iters; n > 0; --n) {
-          while (s < s_hi && k >= p.kseg[s]) { ++s; k = 0; }
-          const long long end = min(p.kseg[s], k + kSK);
-          const float* A = static_cast<const float*>(p.a[s]) + (AT ? p.row_off[g] + m0 + r : (p.row_off[g] + m0 + r) * p.lda[s]);
-          const float* B = static_cast<const float*>(p.b[s]) + (BT ? (p.col_off[g] + n0 + c) * p.ldb[s] : p.col_off[g] + n0 + c);
-          for (long long kk = k; kk < end; ++kk) {
-            const float* a = A + (AT ? kk * p.lda[s] : kk);
-            const float* b = B + (BT ? kk : kk * p.ldb[s]);
-            if (SBP_GUARD(a, 4) && SBP_GUARD(b, 4)) sum = fmaf(__ldg(a), __ldg(b), sum);
-          }
-          k += kSK;
-        }
-        reinterpret_cast<float*>(smem)[r * (nb + 4) + c] = sum;
-      }
-    }
-  } else if (warp < kMmaWarp) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");         // as the others that go on
+  } else {
     // ------------------------------------------------ operands
     asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
     const int t = tid - kDrain;
-    // whole aligned quads everywhere, or element by element
-    bool a_vec = AT ? (rows & 3) == 0 && (p.row_off[g] & 3) == 0 : true, b_vec = BT ? true : (cols & 3) == 0 && (p.col_off[g] & 3) == 0;
-    for (int s = s_lo; s < s_hi; ++s) {
-      a_vec = a_vec && (reinterpret_cast<unsigned long long>(p.a[s]) & 15) == 0 && (p.lda[s] & 3) == 0 && (AT || (p.kseg[s] & 3) == 0);
-      b_vec = b_vec && (reinterpret_cast<unsigned long long>(p.b[s]) & 15) == 0 && (p.ldb[s] & 3) == 0 && (!BT || (p.kseg[s] & 3) == 0);
-    }
     constexpr int kQA = kTM * kSK / 4 / kWorkers;
     // sh: log2 of the quads of a K-step of an MN-contiguous B
     auto run = [&](auto av, auto bv, auto sh) {
@@ -389,6 +511,9 @@ __global__ void __launch_bounds__(kThreads, 1) matmul_f32_tc_kernel(const __grid
       else if (nb > 64) run_a(std::integral_constant<int, 5>{});
       else run_a(std::integral_constant<int, 4>{});
     }
+  }
+  asm volatile("bar.sync 2, 512;" ::: "memory");
+  if (again_s) multiply_again<AT, BT>(p, g, seg0, s_hi, k0, iters, m0, n0, rows, cols, nb, a_vec, b_vec, smem, tid);
   } else {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
     if (warp == kMmaWarp) {
