@@ -1,7 +1,10 @@
 // fp32 MatMul on the tensor cores: executes a grouped-GEMM plan (matmul_plan.h) with the accuracy of fp32 arithmetic.
 //
-// An fp32 number is the sum of three bf16 numbers, x = h + m + l, each the rounding of what the ones before it
-// leave; nothing is lost, bf16 having the exponents of fp32.  A product of two numbers is then hh + (hm + mh) +
+// An fp32 number from 2^-110 on is the sum of three bf16 numbers, x = h + m + l, each the rounding of what the ones before it
+// leave; below, bits would fall under bf16's smallest step of 2^-133.  So every operand is taken 2^39 times, which brings fp32's
+// smallest step to 2^-110 and the results, 2^78 times as large, clear of where low products would be lost, and the sums are put
+// back at the end.  What that carries past fp32's range, operands from 2^88 and sums from 2^49 on, is found like infinities.
+// A product of two numbers is then hh + (hm + mh) +
 // (hl + mm + lh) + terms below 2^-24 of it, that is six products of bf16 numbers, each exact in fp32.  The tensor cores
 // sum them up over a slot of 32 K-steps, the smallest products first: their accumulator cuts off what an addition
 // shifts out, and over longer runs that would show.  The slot's sum is then added to fp32 registers with IEEE additions.
@@ -27,8 +30,8 @@
 // nothing (2048^3 157 and 153 us).
 // 1000 x 1024 x 1500 on four shards 33 us, 1000 x 1500 x 777 38, 2048^3 153 (112 TFLOP/s); FMA kernel 87, 92, 422.
 //
-// A product that is not finite (operands or sums that are not, or a bf16 part that rounds to infinity) is found in
-// the accumulators; the CTA then multiplies its tile again with fp32 multiply-adds (multiply_again).
+// A result that is not finite (operands or sums that are not, or not once scaled, or a bf16 part that rounds to infinity) is found
+// in the accumulators; the CTA then multiplies its tile again with fp32 multiply-adds (multiply_again).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -68,7 +71,14 @@ struct F32TcParams {
 
 __device__ __forceinline__ float gelu_erf(float v) { return 0.5f * v * (1.0f + erff(v * 0.70710678118654752440f)); }
 
-// Two numbers as three bf16 each, packed.
+__device__ __forceinline__ unsigned long long pack(float x, float y) {
+  unsigned long long v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
+  return v;
+}
+
+// Two numbers, scaled, as three bf16 each, packed.
+constexpr float kScale = 0x1p39f;
 __device__ __forceinline__ unsigned bf16_pair(float lo, float hi) {
   unsigned r;
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
@@ -81,6 +91,9 @@ __device__ __forceinline__ void less_pair(float& x, float& y, unsigned h) {
       : "r"(h << 16), "r"(h & 0xffff0000u), "l"(0xbf800000bf800000ull));
 }
 __device__ __forceinline__ void split_pair(float x, float y, unsigned& h, unsigned& m, unsigned& l) {
+  asm("{\n\t.reg .b64 v;\n\tmov.b64 v, {%0, %1};\n\tmul.rn.f32x2 v, v, %2;\n\tmov.b64 {%0, %1}, v;\n\t}"
+      : "+f"(x), "+f"(y)
+      : "l"(pack(kScale, kScale)));
   h = bf16_pair(x, y);
   less_pair(x, y, h);
   m = bf16_pair(x, y);
@@ -173,12 +186,6 @@ struct Share {
 __device__ __forceinline__ void add2(unsigned long long& a, unsigned long long b) { asm("add.rn.f32x2 %0, %0, %1;" : "+l"(a) : "l"(b)); }
 __device__ __forceinline__ float lo(unsigned long long v) { return __uint_as_float((unsigned)v); }
 __device__ __forceinline__ float hi(unsigned long long v) { return __uint_as_float((unsigned)(v >> 32)); }
-
-__device__ __forceinline__ unsigned long long pack(float x, float y) {
-  unsigned long long v;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
-  return v;
-}
 
 // 16 accumulator columns of this warp's 32 rows, in pairs
 __device__ __forceinline__ void tmem_ld16_wait(unsigned taddr, unsigned long long (&v)[8]) {
@@ -438,7 +445,8 @@ __global__ void __launch_bounds__(kThreads, 1) matmul_f32_tc_kernel(const __grid
 #pragma unroll
     for (int i = 0; i < kTN / 4; i += 2) {
       if (2 * i >= width) break;
-      *reinterpret_cast<float4*>(tile + 2 * i) = make_float4(lo(acc[i]), hi(acc[i]), lo(acc[i + 1]), hi(acc[i + 1]));
+      constexpr float kBack = 1.0f / (kScale * kScale);
+      *reinterpret_cast<float4*>(tile + 2 * i) = make_float4(lo(acc[i]) * kBack, hi(acc[i]) * kBack, lo(acc[i + 1]) * kBack, hi(acc[i + 1]) * kBack);
     }
     asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");         // as the others that go on
   } else {

@@ -47,7 +47,7 @@ def _operands(M=1024, K=1024, N=640, seed=1):
 def _check(Y, X, W):
     R, mag = X.double() @ W.double(), X.double().abs() @ W.double().abs()
     fin = torch.isfinite(R) & (mag < 3e38)
-    assert bool(((Y.double() - R).abs() <= 4 * X.shape[1] ** 0.5 * 2.0 ** -24 * mag + 1e-30)[fin].all())
+    assert bool(((Y.double() - R).abs() <= 4 * X.shape[1] ** 0.5 * (2.0 ** -24 * mag + 2.0 ** -149))[fin].all())      # 2^-149: subnormal results
     return R, fin
 
 
@@ -62,7 +62,7 @@ def test_infinities_and_nan():
 
 
 def test_ends_of_the_exponent_range():
-    """The largest number rounds to infinity as a bf16; a sum may overflow; the lowest parts of small numbers are denormal."""
+    """The largest number is infinite once it is scaled; a sum may overflow; rows of small numbers and of large ones side by side."""
     X, W = _operands()
     X[7] *= 1e-30
     X[7, 20], W[20] = torch.finfo(F32).max, W[20] * 1e-30
@@ -140,3 +140,63 @@ def test_what_is_not_finite_costs_no_more_than_multiply_adds():
         t1.synchronize()
         times.append(t0.elapsed_time(t1))
     assert times[1] < 12 * times[0], times
+
+
+def _close(Y, X, W):
+    """The bound of a chain of fp32 multiply-adds with nothing added but what subnormal numbers are rounded to; and as a whole the
+    error of chains of K / 8 and their sum (0.21 sqrt(K / 16) 2^-23), the K roundings to 2^-149 being 0.29 of that each."""
+    K = X.shape[1]
+    R, mag = X.double() @ W.double(), X.double().abs() @ W.double().abs()
+    assert bool(((Y.double() - R).abs() <= 4 * K ** 0.5 * 2.0 ** -24 * mag + 4 * K ** 0.5 * 2.0 ** -149).all())
+    assert float((Y.double() - R).norm()) <= (0.21 * (K / 16) ** 0.5 * 2.0 ** -23 + 6e-8) * float(R.norm()) + K ** 0.5 / 3 * 2.0 ** -149 * R.numel() ** 0.5
+
+
+def _scaled(T, e):
+    """T 2^e by steps that lose nothing before the last."""
+    while e < -120:
+        T, e = T * 2.0 ** -120, e + 120
+    return T * 2.0 ** e
+
+
+@pytest.mark.parametrize("e", [-100, -108, -110, -112, -116, -120, -126, -130, -140])
+@pytest.mark.parametrize("which", ["x", "w"])
+def test_small_operands(e, which):
+    """Numbers down to the subnormal ones, against others that make ordinary results of them."""
+    X, W = _operands()
+    X, W = (_scaled(X, e), W * 2.0 ** min(120, -e)) if which == "x" else (X * 2.0 ** min(120, -e), _scaled(W, e))
+    _close(_product(X, W), X, W)
+
+
+@pytest.mark.parametrize("e", [-105, -115, -126])
+def test_some_small_operands(e):
+    """Rows, columns and lone elements of them among ordinary ones, and results that lie wholly in the subnormal range."""
+    X, W = _operands()
+    X[::50], W[:, ::30] = _scaled(X[::50], e), W[:, ::30] * 2.0 ** 40
+    X[5, ::3], W[::7, 4] = _scaled(X[5, ::3], e), _scaled(W[::7, 4], e)
+    X[6] = 0.0
+    X[6, 9], W[9] = 1.25 * 2.0 ** e * (1 + 2.0 ** -23), W[9] * 2.0 ** 60
+    _close(_product(X, W), X, W)
+
+
+@pytest.mark.parametrize("a,b", [(85, -85), (40, 9), (100, -100), (45, 45), (60, 2), (-60, -60), (-70, -60), (-40, -90), (-74, -74), (-20, -110)])
+def test_results_of_any_size(a, b):
+    """Small ones down to the subnormal, large operands and large sums."""
+    X, W = _operands()
+    X, W = X * 2.0 ** a, W * 2.0 ** b
+    _close(_product(X, W), X, W)
+
+
+@pytest.mark.parametrize("e", [-100, -112, -120, -126, -135, -145])
+def test_a_permutation_moves_bits(e):
+    X, _ = _operands(1024, 1024, 16)
+    X = _scaled(X, e)
+    order = torch.randperm(1024, generator=torch.Generator().manual_seed(3)).cuda()
+    assert torch.equal(_product(X, torch.eye(1024, device="cuda")[order]), X[:, torch.argsort(order)])
+
+
+def test_small_operands_that_do_not_matter():
+    """Probabilities whose smallest are far below what the results can see."""
+    _, W = _operands(1024, 1024, 1024)
+    X = torch.softmax(torch.randn(1024, 1024, device="cuda", generator=torch.Generator(device="cuda").manual_seed(5)) * 25, 1)
+    assert int(((X > 0) & (X < 2.0 ** -110)).sum()) > 1000
+    _close(_product(X, W), X, W)
