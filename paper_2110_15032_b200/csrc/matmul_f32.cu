@@ -363,14 +363,14 @@ struct SmallSlice {
       const long long have = at < rows ? cols - col : 0;
       r[j] = make_float4(0.f, 0.f, 0.f, 0.f);
       if constexpr (VEC) {       // whole quads inside or none
-        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %5, 0;\n\t@p ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}"
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %5, 0;\n\t@p ld.global.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}"
                      : "+f"(r[j].x), "+f"(r[j].y), "+f"(r[j].z), "+f"(r[j].w)
                      : "l"(src), "r"(have > 0 && SBP_GUARD(src, 16) ? 1 : 0));
       } else {
         float* e[4] = {&r[j].x, &r[j].y, &r[j].z, &r[j].w};
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-          asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p ld.global.nc.f32 %0, [%1];\n\t}"
+          asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p ld.global.f32 %0, [%1];\n\t}"
                        : "+f"(*e[i])
                        : "l"(src + i), "r"(have > i && SBP_GUARD(src + i, 4) ? 1 : 0));
       }

@@ -102,6 +102,8 @@ int device_l2_bytes();
 // reads and then writes one buffer must use plain loads.  tests/test_boxing_gpu.py
 // (test_ping_pong_between_two_buffers_without_a_host_sync) rewrites a source between two reads of
 // it with no synchronisation in between.
+// The fp32 products read their operands by plain loads: the small one lets the next kernel in before its own wait, so a
+// reader, the writer after it and the next reader may be resident on one SM.
 // The wait is for the ONE grid before, so the order of the stream rests on a chain: a grid that has finished must itself
 // have waited.  A kernel some of whose grids would wait in no thread (all of its CTAs leave early) is not launched at
 // all, and a kernel whose dependent reads anything ahead of its own wait (the scatter of the embedding gradient reads the

@@ -1,5 +1,5 @@
-"""Ids and labels that one library call writes and the next one reads, with no synchronisation in between: sbp_boxing moves
-them into one buffer again and again while lookups, table gradients and losses follow on the same stream.  Every kernel
+"""Ids, labels and fp32 operands that one library call writes and the next one reads, with no synchronisation in between: sbp_boxing moves
+them into one buffer again and again while lookups, table gradients, losses and products follow on the same stream.  Every kernel
 may be set up while the one before it still runs, so each has to wait before it reads."""
 import numpy as np
 import pytest
@@ -71,3 +71,39 @@ def test_labels_written_just_before(rows, classes):
         grad = O.from_locals([to_np(t) for t in grads[i].locals], O.S1)
         hit = grad[np.arange(rows), values[-1 - i].numpy()]
         assert np.all(hit < 0.0) and int((grad < 0.0).sum()) == rows, f"round {i}: gradient of other labels"
+
+
+@pytest.mark.parametrize("form", [sbp.SBP_F32_FORM_TILED, sbp.SBP_F32_FORM_SMALL, sbp.SBP_F32_FORM_TENSOR])
+@pytest.mark.parametrize("M,K,N", [(64, 128, 96), (64, 129, 95), (33, 17, 40), (200, 520, 300)])
+def test_operands_written_just_before(form, M, K, N):
+    """Both operands rewritten between two products that read them; each as the same product of tensors that nothing writes."""
+    k = 2
+    xs = [make_global(split_cpu(dg.normal(63, i, (M, K), 0.0, 1.0, F32), sbp.S(0), k), (M, K), F32, sbp.S(0)) for i in range(ROUNDS)]
+    ws = [make_global(split_cpu(dg.normal(64, i, (K, N), 0.0, 1.0, F32), sbp.S(1), k), (K, N), F32, sbp.S(1)) for i in range(ROUNDS)]
+    x, w = sbp.empty_global((M, K), F32, sbp.B, k, alias_replicas=True), sbp.empty_global((K, N), F32, sbp.B, k, alias_replicas=True)
+    fixed = []
+    for i in range(ROUNDS):
+        xi, wi = sbp.empty_global((M, K), F32, sbp.B, k, alias_replicas=True), sbp.empty_global((K, N), F32, sbp.B, k, alias_replicas=True)
+        sbp.sbp_boxing(xs[i], xi)
+        sbp.sbp_boxing(ws[i], wi)
+        fixed.append((xi, wi))
+    out, want = ([[sbp.empty_global((M, N), F32, sbp.B, k) for _ in range(2 * ROUNDS)] for _ in range(2)])
+    torch.cuda.synchronize()
+    sbp.sbp_matmul_set_f32_form(form)
+    try:
+        for i in range(ROUNDS):
+            j = (i + 1) % ROUNDS
+            sbp.sbp_matmul(*fixed[i], want[2 * i])
+            sbp.sbp_matmul(fixed[j][0], fixed[i][1], want[2 * i + 1])
+        torch.cuda.synchronize()
+        for i in range(ROUNDS):
+            sbp.sbp_boxing(ws[i], w)
+            sbp.sbp_boxing(xs[i], x)
+            sbp.sbp_matmul(x, w, out[2 * i])
+            sbp.sbp_boxing(xs[(i + 1) % ROUNDS], x)
+            sbp.sbp_matmul(x, w, out[2 * i + 1])
+        torch.cuda.synchronize()
+    finally:
+        sbp.sbp_matmul_set_f32_form(sbp.SBP_F32_FORM_AUTO)
+    for i, (a, b) in enumerate(zip(out, want)):
+        assert torch.equal(a.locals[0], b.locals[0]), f"product {i}: of other operands"
