@@ -221,6 +221,24 @@ __device__ __forceinline__ void whole_quads(const MatmulPlan& p, int g, int s_lo
   }
 }
 
+// The slots of CTA `slice` of the `splits` that share a tile of group g: segment and K inside it where they start, and how many.
+__device__ __forceinline__ void slots_of(const MatmulPlan& p, int g, int slice, int splits, int& seg, long long& k, int& n) {
+  const int s_lo = p.chain ? 0 : g, s_hi = p.chain ? p.nseg : g + 1;
+  long long total = 0;
+  for (int s = s_lo; s < s_hi; ++s) total += (p.kseg[s] + kSK - 1) / kSK;
+  const long long first = total * slice / splits;
+  n = (int)(total * (slice + 1) / splits - first);
+  seg = s_lo;
+  k = first;
+  while (seg < s_hi) {
+    const long long slots = (p.kseg[seg] + kSK - 1) / kSK;
+    if (k < slots) break;
+    k -= slots;
+    ++seg;
+  }
+  k *= kSK;
+}
+
 // A slot of an operand on its way into shared memory, in the order it has: K-contiguous as rows of kSK + 4, else `width` positions a
 // K-step, `pitch` apart.  Q elements at once.
 constexpr int kAll = kDrain + kWorkers, kPitchK = kSK + 4;
@@ -248,8 +266,20 @@ __device__ __forceinline__ void fill_slot(float* to, const float* from, long lon
 // (us, a product on the tensor cores / with every tile once more / on the FMA kernel, whose tiles fill the device more evenly:
 // 1024^3 27 / 123 / 61, 2048^3 165 / 908 / 422, 1000 x 1500 x 777 36 / 168 / 95; one chain of loads an element: 4740, 35200, 3200.)
 template <int AT, int BT>
-__device__ __forceinline__ void multiply_again(const MatmulPlan& p, int g, int s, int s_hi, long long k, int iters, long long m0, long long n0,
-                                               int rows, int cols, int nb, bool a_vec, bool b_vec, unsigned char* smem, int tid) {
+__device__ __forceinline__ void multiply_again(const F32TcParams& P, unsigned char* smem, int tid) {
+  // Where the tile lies, once more: kept from the start it would take registers from the operands' loop.
+  unsigned bx, by, bz;
+  asm volatile("mov.u32 %0, %%ctaid.x;\n\tmov.u32 %1, %%ctaid.y;\n\tmov.u32 %2, %%ctaid.z;" : "=r"(bx), "=r"(by), "=r"(bz));
+  const MatmulPlan& p = P.plan;
+  const int g = (int)bz, nb = P.nb;
+  const long long m0 = (long long)by * kTM, n0 = (long long)(bx / (unsigned)P.splits) * nb;
+  const int rows = (int)min((long long)kTM, p.m[g] - m0), cols = (int)min((long long)nb, p.n[g] - n0);
+  const int s_hi = p.chain ? p.nseg : g + 1;
+  int s, iters;
+  long long k;
+  slots_of(p, g, (int)(bx % (unsigned)P.splits), P.splits, s, k, iters);
+  bool a_vec, b_vec;
+  whole_quads<AT, BT>(p, g, p.chain ? 0 : g, s_hi, rows, cols, a_vec, b_vec);
   constexpr bool AKC = !AT, BKC = BT;
   constexpr int kPitchA = kTM + 4, kPitchB = kTN + 4, kChain = 4;
   constexpr int kA = AKC ? kTM * kPitchK : kSK * kPitchA, kB = BKC ? kTN * kPitchK : kSK * kPitchB;
@@ -382,21 +412,9 @@ __global__ void __launch_bounds__(kThreads, 1) matmul_f32_tc_kernel(const __grid
 
   // this CTA's range of slots over all segments
   const int s_lo = p.chain ? 0 : g, s_hi = p.chain ? p.nseg : g + 1;
-  long long total = 0;
-  for (int s = s_lo; s < s_hi; ++s) total += (p.kseg[s] + kSK - 1) / kSK;
-  const long long it0 = total * slice / splits;
-  const int iters = (int)(total * (slice + 1) / splits - it0);
-  int seg0 = s_lo;                                 // where the range starts: segment and K inside it
-  long long k0 = it0;
-  while (seg0 < s_hi) {
-    const long long n = (p.kseg[seg0] + kSK - 1) / kSK;
-    if (k0 < n) break;
-    k0 -= n;
-    ++seg0;
-  }
-  k0 *= kSK;
-  bool a_vec, b_vec;
-  whole_quads<AT, BT>(p, g, s_lo, s_hi, rows, cols, a_vec, b_vec);
+  int seg0, iters;
+  long long k0;
+  slots_of(p, g, slice, splits, seg0, k0, iters);
 
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -453,6 +471,8 @@ __global__ void __launch_bounds__(kThreads, 1) matmul_f32_tc_kernel(const __grid
     // ------------------------------------------------ operands
     asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
     const int t = tid - kDrain;
+    bool a_vec, b_vec;
+    whole_quads<AT, BT>(p, g, s_lo, s_hi, rows, cols, a_vec, b_vec);
     constexpr int kQA = kTM * kSK / 4 / kWorkers;
     // sh: log2 of the quads of a K-step of an MN-contiguous B
     auto run = [&](auto av, auto bv, auto sh) {
@@ -521,7 +541,7 @@ __global__ void __launch_bounds__(kThreads, 1) matmul_f32_tc_kernel(const __grid
     }
   }
   asm volatile("bar.sync 2, 512;" ::: "memory");
-  if (again_s) multiply_again<AT, BT>(p, g, seg0, s_hi, k0, iters, m0, n0, rows, cols, nb, a_vec, b_vec, smem, tid);
+  if (again_s) multiply_again<AT, BT>(P, smem, tid);
   } else {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
     if (warp == kMmaWarp) {
