@@ -144,6 +144,19 @@ __device__ __forceinline__ unsigned long long add_two(unsigned long long a, unsi
   return v;
 }
 
+// 2^((a - m) log2e + c) and the same of b: the difference is exact in m, and in pairs it costs no more than one multiply-add an
+// element.  (m log2e folded into c: its rounding is a factor on the whole row, 3e-4 at a maximum of 1e4, 4 % at 1e6.)
+__device__ __forceinline__ void exp_two(float& a, float& b, unsigned long long neg_m, unsigned long long c) {
+  const unsigned long long v = fma_two(add_two(two(a, b), neg_m), two(1.4426950408889634f), c);
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(a) : "f"(__uint_as_float((unsigned)v)));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(b) : "f"(__uint_as_float((unsigned)(v >> 32))));
+}
+__device__ __forceinline__ float exp_one(float a, float m, float c) {
+  float e;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(fmaf(a - m, 1.4426950408889634f, c)));
+  return e;
+}
+
 // GeLU(v) = 0.5 v (1 + erf(v / sqrt 2)) of two numbers, erf by the rational approximation 7.1.26 of Abramowitz & Stegun
 // (|error| <= 1.5e-7), which is far below the rounding of the bf16 / fp32 store that follows and costs two special-function
 // operations where erff costs a long polynomial.  Each number goes through the operations of the formula in its order, so the
@@ -487,7 +500,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
         // Softmax partials of this warp's 32 rows x 128 columns; one thread owns one row, so
         // nothing crosses lanes.  Columns are taken 32 at a time: batch max, then the running
         // (m, s) is rescaled and the batch's exponentials are added.
-        constexpr float kL2e = 1.4426950408889634f;
         const int colbase = tc.n0 + half * (BN / 2);
         const long long row = row0 + lane;
         if (row0 < Mg && colbase < Ng) {            // warp-uniform
@@ -510,21 +522,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
 #pragma unroll
             for (int i = 1; i < 32; ++i) bm = fmaxf(bm, v[i]);
             const float mm = fmaxf(m, bm);
-            const float neg = -mm * kL2e;
-            float carried = 0.f;
-            if (m != -INFINITY) {
-              float e;
-              asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(fmaf(m, kL2e, neg)));
-              carried = s * e;
-            }
+            const float carried = m != -INFINITY ? s * exp_one(m, mm, 0.f) : 0.f;
+            const unsigned long long neg = two(-mm);
             float s0 = 0.f, s1 = 0.f;
 #pragma unroll
             for (int i = 0; i < 32; i += 2) {
-              float e0, e1;
-              asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(fmaf(v[i], kL2e, neg)));
-              asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(fmaf(v[i + 1], kL2e, neg)));
-              s0 += e0;
-              s1 += e1;
+              exp_two(v[i], v[i + 1], neg, 0ull);
+              s0 += v[i];
+              s1 += v[i + 1];
             }
             s = carried + (s0 + s1);
             m = mm;
@@ -553,26 +558,26 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
       // The element-wise modes are compiled apart (MODE 0 plain, 1 GeLU, 2 softmax - onehot of the
       // recomputed logits) so that the plain store, which the short-K classifier product leans
       // on, carries none of the others' instructions.
-      // softmax = 2^(z log2e - m log2e - log2 S): the division by the row sum is folded into the exponent
-      float g_neg = 0.f;
-      long long g_lab = -1;
-      if (p.xent == 2 && row0 + lane < Mg && SBP_GUARD(p.xf.row_max + row0 + lane, 4) &&
-          SBP_GUARD(p.xf.row_sum + row0 + lane, 4) && SBP_GUARD(p.xf.labels + row0 + lane, 8)) {      // this thread's row constants
-        const long long row = row0 + lane;
-        g_neg = -p.xf.row_max[row] * 1.4426950408889634f - log2f(p.xf.row_sum[row]);
-        g_lab = p.xf.labels[row] - p.xf.class_start[tc.g];
-      }
       auto slabs = [&](auto mode_tag) {
         constexpr int MODE = decltype(mode_tag)::value;
-        int lab_rel = -1;   // the label's column inside the current slab, if it lies there
-        auto xform = [&](float x, int idx) -> float {
-          if constexpr (MODE == 2) {
-            float e;
-            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(fmaf(x, 1.4426950408889634f, g_neg)));
-            return e;          // the label's column gets its -1 below, outside the per-element path
-          } else {
-            return x;
+        // softmax = 2^((z - m) log2e - log2 S): the division by the row sum is folded into the exponent
+        float g_max = 0.f, g_neg = 0.f;       // this thread's row
+        long long g_lab = -1;
+        if constexpr (MODE == 2) {
+          const long long row = row0 + lane;
+          if (row < Mg && SBP_GUARD(p.xf.row_max + row, 4) && SBP_GUARD(p.xf.row_sum + row, 4) && SBP_GUARD(p.xf.labels + row, 8)) {
+            g_max = p.xf.row_max[row];
+            g_neg = -log2f(p.xf.row_sum[row]);
+            g_lab = p.xf.labels[row] - p.xf.class_start[tc.g];
           }
+        }
+        int lab_rel = -1;   // the label's column inside the current slab, if it lies there
+        auto xform = [&](float& a, float& b) {
+          if constexpr (MODE == 1) gelu_two(a, b);
+          if constexpr (MODE == 2) {      // (as a pair its constants took two registers more: the kernel spilled, GeLU was 2 % slower)
+            a = exp_one(a, g_max, g_neg);
+            b = exp_one(b, g_max, g_neg);
+          }                               // the label's column gets its -1 below
         };
         for (int sl = 0; sl < nslabs; ++sl) {
           const int col0 = tc.n0 + half * (BN / 2) + sl * cols_per_slab;
@@ -592,12 +597,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
 #pragma unroll
               for (int c = 0; c < 8; ++c) {
                 float4 o;
-                if constexpr (MODE == 1) {
-                  gelu_two(v[4 * c], v[4 * c + 1]);
-                  gelu_two(v[4 * c + 2], v[4 * c + 3]);
-                }
-                o.x = xform(v[4 * c + 0], 4 * c + 0); o.y = xform(v[4 * c + 1], 4 * c + 1);
-                o.z = xform(v[4 * c + 2], 4 * c + 2); o.w = xform(v[4 * c + 3], 4 * c + 3);
+                xform(v[4 * c], v[4 * c + 1]);
+                xform(v[4 * c + 2], v[4 * c + 3]);
+                o.x = v[4 * c]; o.y = v[4 * c + 1]; o.z = v[4 * c + 2]; o.w = v[4 * c + 3];
                 *reinterpret_cast<float4*>(rowp + ((c ^ (lane & 7)) << 4)) = o;
               }
             } else {
@@ -605,11 +607,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
               for (int c = 0; c < 8; ++c) {
                 float f[8];
 #pragma unroll
-                for (int e = 0; e < 8; ++e) f[e] = xform(v[8 * c + e], 8 * c + e);
-                if constexpr (MODE == 1) {
+                for (int e = 0; e < 8; ++e) f[e] = v[8 * c + e];
 #pragma unroll
-                  for (int e = 0; e < 8; e += 2) gelu_two(f[e], f[e + 1]);
-                }
+                for (int e = 0; e < 8; e += 2) xform(f[e], f[e + 1]);
                 uint4 o;
                 __nv_bfloat162 h;
                 h = __floats2bfloat162_rn(f[0], f[1]); o.x = *reinterpret_cast<unsigned*>(&h);
@@ -633,9 +633,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
                 asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(bitsv) : "r"(taddr + sl * cols_per_slab + col) : "memory");
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                 if (lane == src_lane) {
-                  float e;
-                  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(fmaf(__uint_as_float(bitsv), 1.4426950408889634f, g_neg)));
-                  e -= 1.0f;
+                  const float e = exp_one(__uint_as_float(bitsv), g_max, g_neg) - 1.0f;
                   if (p.out_f32) *reinterpret_cast<float*>(rowp + (((col >> 2) ^ (lane & 7)) << 4) + ((col & 3) << 2)) = e;
                   else *reinterpret_cast<__nv_bfloat16*>(rowp + (((col >> 3) ^ (lane & 7)) << 4) + ((col & 7) << 1)) = __float2bfloat16_rn(e);
                 }
@@ -1221,7 +1219,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1) xent_
       bar_acc_empty[kNarrowAccs];
   __shared__ unsigned tmem_base_slot;
   __shared__ int abort_flag_s;
-  __shared__ __align__(16) float neg_s[MODE == 2 ? NB : 4];
+  __shared__ __align__(16) float less_s[MODE == 2 ? NB : 4], neg_s[MODE == 2 ? NB : 4];
   __shared__ long long lab_s[NB];
   volatile int* abort_flag = &abort_flag_s;
 
@@ -1257,9 +1255,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1) xent_
   if (threadIdx.x < NB) {
     const int row = threadIdx.x;
     lab_s[row] = row < p.rows && SBP_GUARD(p.xf.labels + row, 8) ? p.xf.labels[row] : -1;
-    // softmax = 2^(z log2e - m log2e - log2 S): the division by the row sum is folded into the exponent
-    if (MODE == 2 && row < p.rows && SBP_GUARD(p.xf.row_max + row, 4) && SBP_GUARD(p.xf.row_sum + row, 4))
-      neg_s[row] = -p.xf.row_max[row] * 1.4426950408889634f - log2f(p.xf.row_sum[row]);
+    // softmax = 2^((z - m) log2e - log2 S): the division by the row sum is folded into the exponent
+    if (MODE == 2 && row < p.rows && SBP_GUARD(p.xf.row_max + row, 4) && SBP_GUARD(p.xf.row_sum + row, 4)) {
+      less_s[row] = -p.xf.row_max[row];
+      neg_s[row] = -log2f(p.xf.row_sum[row]);
+    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -1368,7 +1368,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1) xent_
         }
         if (r0 >= p.rows || chunk0 >= Ng) continue;    // the same for the four warps of a half
         if constexpr (MODE == 1) {
-          constexpr float kL2e = 1.4426950408889634f;
 #pragma unroll
           for (int c = 0; c < 8; ++c) {
             float4 f = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
@@ -1383,13 +1382,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1) xent_
 #pragma unroll
           for (int i = 4; i < 32; ++i) top[i & 3] = fmaxf(top[i & 3], x[i]);
           const float m = fmaxf(fmaxf(top[0], top[1]), fmaxf(top[2], top[3]));
-          const float neg = m == -INFINITY ? 0.f : -m * kL2e;      // no class of the shard here: sum 0
+          const unsigned long long neg = two(m == -INFINITY ? 0.f : -m);      // no class of the shard here: sum 0
           float sum[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            float e;
-            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(fmaf(x[i], kL2e, neg)));
-            sum[i & 3] += e;
+          for (int i = 0; i < 32; i += 2) {
+            exp_two(x[i], x[i + 1], neg, 0ull);
+            sum[i & 3] += x[i];
+            sum[(i & 3) + 1] += x[i + 1];
           }
           const long long want = lab_s[r0 + lane] - p.class_start[g] - chunk0 - q * 32;
           const float t = want >= 0 && want < 32 && want < Ng - chunk0 - q * 32 ? mine[(int)want * kNarrowPitch + lane] : 0.f;
@@ -1402,9 +1401,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1) xent_
             float M = fmaxf(fmaxf(out[0], out[96]), fmaxf(out[192], out[288])), S = 0.f, T = 0.f;
 #pragma unroll
             for (int w = 0; w < 4; ++w) {
-              float e;
-              asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"((out[w * 96] - M) * kL2e));
-              S = fmaf(out[w * 96 + 32], e, S);
+              S = fmaf(out[w * 96 + 32], exp_one(out[w * 96], M, 0.f), S);
               T += out[w * 96 + 64];
             }
             const long long at = (long long)(p.xf.part_base[g] + chunk0 / BMH) * p.rows + r0 + lane;
@@ -1417,11 +1414,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1) xent_
           const long long first_class = p.class_start[g] + chunk0 + q * 32, step = p.ldy[g];
 #pragma unroll
           for (int c = 0; c < 32; c += 4) {
-            const float4 neg = *reinterpret_cast<const float4*>(neg_s + r0 + c);
-            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(v[c]) : "f"(fmaf(v[c], 1.4426950408889634f, neg.x)));
-            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(v[c + 1]) : "f"(fmaf(v[c + 1], 1.4426950408889634f, neg.y)));
-            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(v[c + 2]) : "f"(fmaf(v[c + 2], 1.4426950408889634f, neg.z)));
-            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(v[c + 3]) : "f"(fmaf(v[c + 3], 1.4426950408889634f, neg.w)));
+            const ulonglong2 less = *reinterpret_cast<const ulonglong2*>(less_s + r0 + c), neg = *reinterpret_cast<const ulonglong2*>(neg_s + r0 + c);
+            exp_two(v[c], v[c + 1], less.x, neg.x);
+            exp_two(v[c + 2], v[c + 3], less.y, neg.y);
           }
           // rows whose label is one of this warp's 32 classes are rare
           const long long want = lab_s[r0 + lane] - first_class;
