@@ -77,7 +77,7 @@ __device__ __forceinline__ void merge(float& m, float& s, float m2, float s2) {
 
 // Loss, max and sum of a finished row, to every replica.
 __device__ __forceinline__ void write_row(const XentCombineParams& p, long long row, float m, float S, float zy) {
-  const float loss = logf(S) + m - zy;
+  const float loss = logf(S) + (m - zy);       // in this order: the sum of a large m and the logarithm would be rounded to m's last place
   for (int j = 0; j < p.n_loss; ++j)
     if (SBP_GUARD(p.loss[j] + row, 4)) p.loss[j][row] = loss;
   for (int j = 0; j < p.n_max; ++j)

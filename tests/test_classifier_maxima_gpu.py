@@ -33,6 +33,8 @@ def test_maxima_of_any_size(top, rows, classes, k):
     S = E.sum(1)
     assert torch.equal(m.locals[0].double(), Z.max(1)[0])
     assert float(((s.locals[0].double() - S) / S).abs().max()) <= 2.0 ** -21
+    want = S.log() + (Z.max(1)[0] - Z[torch.arange(rows), labels.cuda()])
+    assert float((loss.locals[0].double() - want).abs().max()) <= 2.0 ** -20 + 2.0 ** -23 * float(want.max())
     hit = torch.zeros(rows, classes, dtype=torch.bool, device="cuda")
     hit[torch.arange(rows), labels.cuda()] = True
     P = E / S[:, None]

@@ -79,6 +79,8 @@ def test_maxima_of_any_size(top, rows, classes, k, dtype):
     loss, m, s = _forward(Z, k)
     assert torch.equal(m.double(), Zd.max(1)[0])
     assert float(((s.double() - want) / want).abs().max()) <= 2.0 ** -21
+    gone = Zd.max(1)[0] - Zd[:, 0]
+    assert bool(((loss.double() - want.log() - gone).abs() <= 2.0 ** -20 + 2.0 ** -23 * gone).all())
     z = sbp.SbpTensor((rows, classes), dtype, sbp.S(1), [t.contiguous() for t in torch.tensor_split(Z, k, 1)])
     lab = sbp.SbpTensor((rows,), torch.int64, sbp.B, [torch.zeros(rows, dtype=torch.int64, device="cuda")] * k)
     rm, rs = (sbp.SbpTensor((rows,), F32, sbp.B, [t] * k) for t in (m, s))
