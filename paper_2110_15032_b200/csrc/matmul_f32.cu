@@ -560,7 +560,7 @@ static void count_f32_launch(int form) {
 }
 
 // Defined in matmul_f32_tc.cu: the same product from bf16 parts on the tensor cores.
-double f32_tc_cost(const MatmulPlan& plan, int* nb, int* splits);
+double f32_tc_cost(const MatmulPlan& plan, double limit, int* nb, int* splits);
 sbp_status launch_matmul_f32_tc(const MatmulPlan& plan, int nb, int splits, cudaStream_t st);
 
 sbp_status launch_matmul_f32(const MatmulPlan& plan, cudaStream_t st) {
@@ -649,8 +649,9 @@ sbp_status launch_matmul_f32(const MatmulPlan& plan, cudaStream_t st) {
   // 1132 x 1272 on eight 28.4 / 30.7, 1809 x 26 x 1014 x 51 on three 59 / 53.)
   if (form == SBP_F32_FORM_AUTO ? best > 11000 : form == SBP_F32_FORM_TENSOR) {
     int nb = 0, splits = 1;
-    const double tc = f32_tc_cost(plan, &nb, &splits);
-    if (tc >= 0 && (form != SBP_F32_FORM_AUTO || (tc + 4 < best / 1750 && (!small || tc + 4 < fma_us)))) {
+    const double limit = form != SBP_F32_FORM_AUTO ? 1e300 : (small && fma_us < best / 1750 ? fma_us : best / 1750) - 4;
+    const double tc = f32_tc_cost(plan, limit, &nb, &splits);
+    if (tc >= 0 && tc < limit) {
       const sbp_status status = launch_matmul_f32_tc(plan, nb, splits, st);
       if (status == SBP_OK) count_f32_launch(SBP_F32_FORM_TENSOR);
       return status;

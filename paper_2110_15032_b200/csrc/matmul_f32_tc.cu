@@ -682,20 +682,24 @@ cudaError_t launch_form(const F32TcParams* P, int splits, dim3 grid, cudaStream_
   return cudaLaunchKernelEx(&cfg, matmul_f32_tc_kernel<AT, BT>, *P);
 }
 
-// Clusters of this many CTAs that the current device holds at once (a CTA fills its SM).
-int cluster_capacity(int splits) {
-  static std::atomic<int> known[64][9];
+constexpr int kCuts[6] = {1, 2, 3, 4, 6, 8};      // CTAs that may share a tile
+
+// Clusters of kCuts[i] CTAs that the current device holds at once (a CTA fills its SM), asked once a device.
+bool cluster_capacities(int (&cap)[6]) {
+  static std::atomic<int> known[64][6];
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  int v = known[dev][splits].load(std::memory_order_relaxed);
-  if (v == 0) {
-    if (launch_form<0, 0>(nullptr, splits, dim3((unsigned)splits), nullptr, &v) != cudaSuccess || v < 1) {
-      cudaGetLastError();
-      v = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+  for (int i = 0; i < 6; ++i) {
+    cap[i] = known[dev][i].load(std::memory_order_relaxed);
+    if (cap[i] == 0) {
+      if (launch_form<0, 0>(nullptr, kCuts[i], dim3((unsigned)kCuts[i]), nullptr, &cap[i]) != cudaSuccess || cap[i] < 1) {
+        cudaGetLastError();
+        cap[i] = -1;
+      }
+      known[dev][i].store(cap[i], std::memory_order_relaxed);
     }
-    known[dev][splits].store(v, std::memory_order_relaxed);
   }
-  return v;
+  return true;
 }
 
 }  // namespace
@@ -705,7 +709,8 @@ int cluster_capacity(int splits) {
 // twelve MMAs, the accumulators' turn), 0.15 and 0.001 a column more where A / B come element by element, set-up, drain and
 // stores 6 and 0.016 a column.  Fitted to 823 timings of 30 products (rms error 8 %; the pick within 1.5 % of the best cut on
 // the average); the exchange is set dearer than in a row of equal calls, between others large clusters wait for their SMs.
-double f32_tc_cost(const MatmulPlan& plan, int* nb, int* splits) {
+// Nothing is looked for (negative) where the least that any cut takes is not below `limit`.
+double f32_tc_cost(const MatmulPlan& plan, double limit, int* nb, int* splits) {
   long long slots = 0, mmax = 0, nmax = 0;
   bool a_vec = true, b_vec = true;
   for (int s = 0; s < plan.nseg; ++s) {
@@ -721,18 +726,24 @@ double f32_tc_cost(const MatmulPlan& plan, int* nb, int* splits) {
     nmax = std::max(nmax, plan.n[g]);
   }
   if ((mmax + kTM - 1) / kTM > 65535 || slots == 0 || slots > 0x7fffffffLL || nmax == 0) return -1;
+  if ((double)((slots + 7) / 8) * 0.76 + 6.2 >= limit) return -1;
+  int cap[6];
+  if (!cluster_capacities(cap)) return -1;
   double best = -1;
   const long long least = (nmax + kTN - 1) / kTN;
   for (long long t = least; t <= least + 12; ++t) {
     const int w = (int)(((nmax + t - 1) / t + 15) / 16 * 16);
-    long long tiles = 0;
-    for (int g = 0; g < plan.ngroups; ++g) tiles += ((plan.m[g] + kTM - 1) / kTM) * ((plan.n[g] + w - 1) / w);
+    long long tiles = 0, of_one = 0;
+    for (int g = 0; g < plan.ngroups; ++g) {
+      if (g == 0 || plan.m[g] != plan.m[g - 1] || plan.n[g] != plan.n[g - 1]) of_one = ((plan.m[g] + kTM - 1) / kTM) * ((plan.n[g] + w - 1) / w);
+      tiles += of_one;
+    }
     const double per_slot = 0.705 + 0.0034 * w + (a_vec ? 0 : 0.15) + (b_vec ? 0 : 0.001 * w);
-    for (int s : {1, 2, 3, 4, 6, 8}) {
+    for (int i = 0; i < 6; ++i) {
+      const int s = kCuts[i];
       if (slots < s) break;
-      const int cap = cluster_capacity(s);
-      if (cap < 1) continue;
-      const double waves = (double)((tiles + cap - 1) / cap);
+      if (cap[i] < 1) continue;
+      const double waves = (double)((tiles + cap[i] - 1) / cap[i]);
       const double cost = waves * ((double)((slots + s - 1) / s) * per_slot + 6.0 + 0.016 * w + (s > 1 ? 0.25 * s : 0.0));
       if (best < 0 || cost < best) {
         best = cost;
