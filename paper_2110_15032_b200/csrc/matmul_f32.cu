@@ -617,15 +617,22 @@ sbp_status launch_matmul_f32(const MatmulPlan& plan, cudaStream_t st) {
       if (cost < best) { best = cost; best_per_sm = per_sm; best_t = t; best_s = s; }
     }
   }
+  // Alone and in a row this kernel takes 0.5 us and a us for 1950 of those clocks (1680 where CTAs share an SM), 5 more with the
+  // large tile, 6 % more off the 16-byte rule (rms 13 %).  Another kernel is taken only where it beats less than that, since
+  // between kernels of another kind it loses part of what it gains alone: the small one against best / 1640, or 1.6 + best / 3125
+  // where every CTA has an SM of its own, the tensor cores against best / 1750.  (1600 drawn products, alone and after a boxing op
+  // of their operand: one of what these lines pick is over 4 % slower than this kernel, by 10 %; on the geometric mean it is 9 %
+  // off the best of the three.  By the prices as they are it would be 4 % off, and 27 to 60 of the picks slower than this kernel, by up to 46 %.)
+  //
   // The small kernel: 2.2 us and 1.25 a slice of a warp's, 0.45 more for an operand that comes element by element, CTAs that
-  // share an SM 0.6 each.  Against it this kernel's estimate as measured, 1.16 of it at 1.9 GHz, less where every CTA has an SM of
-  // its own.  (us, this kernel / the small one: 64 x 96 x 80 on two shards 4.9 / 3.4, 40 x 98 x 640 5.0 / 3.4, 215 x 89 x 113 on
+  // share an SM 0.6 each, from seven on 1.6 us each (they no longer run at once: 1155 x 124 x 416 on three, ten an SM, 20.7 us, 17.2
+  // here).  (us, this kernel / the small one: 64 x 96 x 80 on two shards 4.9 / 3.4, 40 x 98 x 640 5.0 / 3.4, 215 x 89 x 113 on
   // eight 5.2 / 3.8, 1031 x 325 x 228 on three 17.4 / 10.4, 722 x 258 x 99 on two 8.1 / 9.1, 32 x 512 x 32 6.3 / 7.2, 90 x 789 x 85
   // 10.0 / 12.4: a long contraction wants the cluster.  From four slices a warp on the switch has to win by a fifth, and with one
   // slice and CTAs that share an SM by 2.5 us: in a program of 133 x 620 x 622 x 187 on three the small kernel alone took
   // 9.4, this one 13.0, the program 26.4 and 24.9; one of 185 x 112 x 1082 x 100 on four took 29.9 with the small kernel's 272 CTAs
   // first, 27.2 without.)
-  double fma_us = best_per_sm > 1 ? best / 1640 : 1.6 + 0.00032 * best;
+  double beat_us = best_per_sm > 1 ? best / 1640 : 1.6 + best / 3125;
   const long long small_x = (nmax + kST - 1) / kST, small_y = (mmax + kST - 1) / kST;
   bool small = false;
   if (small_x <= 0x7fffffffLL && small_y <= 65535) {
@@ -633,22 +640,23 @@ sbp_status launch_matmul_f32(const MatmulPlan& plan, cudaStream_t st) {
     for (int g = 0; g < plan.ngroups; ++g) tiles += ((plan.m[g] + kST - 1) / kST) * ((plan.n[g] + kST - 1) / kST);
     const double per_sm = (double)((tiles + sms - 1) / sms);
     const double slices = (double)((iters + kSWarps - 1) / kSWarps);
-    const double cost = 2.2 + slices * (1.25 + (P.a_quad ? 0 : 0.45) + (P.b_quad ? 0 : 0.45)) * (0.4 + 0.6 * per_sm);
-    const bool wins = slices == 1 && per_sm > 1 ? cost + 2.5 < fma_us : cost < (slices > 3 ? 0.8 : 0.95) * fma_us;
+    double cost = 2.2 + slices * (1.25 + (P.a_quad ? 0 : 0.45) + (P.b_quad ? 0 : 0.45)) * (0.4 + 0.6 * per_sm);
+    if (per_sm >= 7 && cost < 2.2 + 1.6 * slices * per_sm) cost = 2.2 + 1.6 * slices * per_sm;
+    const bool wins = slices == 1 && per_sm > 1 ? cost + 2.5 < beat_us : cost < (slices > 3 ? 0.8 : 0.95) * beat_us;
     if (form == SBP_F32_FORM_AUTO ? wins : form == SBP_F32_FORM_SMALL) {
       small = true;
       P.early = 8 * tiles <= sms;
-      fma_us = cost;
+      beat_us = cost;
     }
   }
-  // The tensor cores take it where their estimate (us) and 4 are below this kernel's, and the small one's: alone the other kernel
+  // The tensor cores take it where their estimate (us) and 4 are below best / 1750, and the small kernel's estimate: alone the other kernel
   // wins earlier, but between kernels of another kind each of its launches waits some 5 us for whole SMs.  (us, this kernel / the
   // other, alone: 69 x 270 x 1639 on four shards 14.3 / 13.7, 187 x 1092 x 339 on four 17.9 / 14.6, 1170 x 256 x 808 on three 30 / 17,
   // 1000 x 1500 x 777 on four 92 / 38, 2048 x 2048 x 2048 422 / 153; programs of 116 x 1047 x 387 x 16 on three 24.8 / 27.3, 58 x 79 x
   // 1132 x 1272 on eight 28.4 / 30.7, 1809 x 26 x 1014 x 51 on three 59 / 53.)
   if (form == SBP_F32_FORM_AUTO ? best > 11000 : form == SBP_F32_FORM_TENSOR) {
     int nb = 0, splits = 1;
-    const double limit = form != SBP_F32_FORM_AUTO ? 1e300 : (small && fma_us < best / 1750 ? fma_us : best / 1750) - 4;
+    const double limit = form != SBP_F32_FORM_AUTO ? 1e300 : (small && beat_us < best / 1750 ? beat_us : best / 1750) - 4;
     const double tc = f32_tc_cost(plan, limit, &nb, &splits);
     if (tc >= 0 && tc < limit) {
       const sbp_status status = launch_matmul_f32_tc(plan, nb, splits, st);

@@ -66,6 +66,7 @@ def test_the_librarys_choice():
     """Far from the lines between them: tests of the tensor cores' accuracy and of its ranges count on this one."""
     assert _case(0, 64, 128, 96, 2, F32, S0, B) == SMALL
     assert _case(0, 32, 512, 32, 1, F32, B, B) == TILED
+    assert _case(0, 1155, 124, 1248, 3, F32, B, S1) != SMALL      # ten CTAs an SM: 20.7 us, tiled 17.2, tensor cores 12.6
     for M, K, N in ((1024, 1024, 640), (1000, 1500, 777), (1000, 1111, 700), (1024, 512, 1024), (2048, 2048, 512), (1000, 1500, 300)):
         assert _case(0, M, K, N, 1, F32, B, B) == TENSOR
 
