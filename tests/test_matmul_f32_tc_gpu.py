@@ -100,7 +100,7 @@ def test_the_same_bits_every_time():
 
 @pytest.mark.parametrize("M,K,N,k", [(1024, 1024, 640, 1), (300, 1029, 517, 3)])
 @pytest.mark.parametrize("tx,tw", [(False, False), (True, False), (False, True), (True, True)])
-def test_the_second_time_with_multiply_adds(M, K, N, k, tx, tw):
+def test_second_multiplication_edges(M, K, N, k, tx, tw):
     """One infinity in every row of X makes every tile be multiplied again: what is finite (columns where W is 0 there would be
     NaN, so W is not) is infinite, and with it out of the way of all but the first rows the others are ordinary results."""
     X, W = _operands(M, K, N)
