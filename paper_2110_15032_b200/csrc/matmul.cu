@@ -4,7 +4,7 @@
 //   * the tensor-core kernel (matmul_tc.cu): bf16 operands, fp32 accumulation in tensor
 //     memory, TMA-fed tiles; taken whenever the shapes meet its alignment rules;
 //   * the fp32 kernels (matmul_f32.cu, matmul_f32_tc.cu): fp32 operands, fp32 fused multiply-adds, k ascending (in up to eight
-//     parts), or tensor-core products of three bf16 parts a number, as exact;
+//     parts), or tensor-core products of three bf16 parts a number;
 //   * the FMA kernel in this file: bf16 operands that the tensor-core kernel cannot take and that no
 //     workspace was given for, one such chain.
 #include <cuda_bf16.h>

@@ -1,5 +1,5 @@
 // fp32 MatMul: executes a grouped-GEMM plan (matmul_plan.h) on the FMA pipes.  (Products that fill tiles of the tensor cores
-// go to matmul_f32_tc.cu, which is as exact.)
+// go to matmul_f32_tc.cu.)
 //
 // Every element of the result is a chain of fused multiply-adds in fp32, k ascending, segments in rank order; where K is
 // split over the CTAs of a cluster (below) one chain for each, the chains added in their

@@ -4,14 +4,21 @@
 // leave; below, bits would fall under bf16's smallest step of 2^-133.  So every operand is taken 2^39 times, which brings fp32's
 // smallest step to 2^-110 and the results, 2^78 times as large, clear of where low products would be lost, and the sums are put
 // back at the end.  What that carries past fp32's range, operands from 2^88 and sums from 2^49 on, is found like infinities.
-// A product of two numbers is then hh + (hm + mh) +
-// (hl + mm + lh) + terms below 2^-24 of it, that is six products of bf16 numbers, each exact in fp32.  The tensor cores
-// sum them up over a slot of 32 K-steps, the smallest products first: their accumulator cuts off what an addition
-// shifts out, and over longer runs that would show.  The slot's sum is then added to fp32 registers with IEEE additions.
-// Error against fp64, root mean square, relative, normal operands, this / the FMA kernel (one chain, or cut in up to
-// eight): K = 16 4.8e-8 / 7.3e-8, 64 6.3e-8 / 8.5e-8, 512 9.6e-8 / 1.5e-7, 1500 1.4e-7 / 4.9e-7, 2048 1.6e-7 / 2.9e-7.
-// (Slots of 64: 3.2e-7 at any K.  Operands all of one sign, where the cut-off does not average out: K = 64 6.3e-8 /
-// 5.0e-8, 2048 1.35e-7 / 1.0e-7 cut in eight.)
+// A product of two numbers is then hh + (hm + mh) + (hl + mm + lh) + terms below 2^-24 of it, that is six products of bf16
+// numbers, each exact in fp32.  The tensor cores sum them up over a slot of 32 K-steps, the smallest products first: their
+// accumulator cuts off what an addition shifts out, and over longer runs that would show.  The slot's sum is then added to
+// fp32 registers with IEEE additions.  (The split and the six products: Henry, Tang and Heinecke, Leveraging the bfloat16
+// artificial intelligence datatype for higher-precision computations, 2019; sums outside the tensor cores: Ootomo and Yokota,
+// Recovering single precision accuracy from tensor cores, 2022.)
+// Error against fp64, root mean square, relative, this / the tiled FMA kernel as it would be cut:
+//   1024 x K x 1024, K =      64               128              1024             2048 (2048^3)
+//   normal operands           6.3e-8 / 14e-8   7.0e-8 / 11e-8   10e-8 / 29e-8    12e-8 / 41e-8
+//   their magnitudes          6.4e-8 / 12e-8   6.6e-8 / 5.8e-8  7.7e-8 / 13e-8   8.8e-8 / 18e-8
+//   log-normal, sigma 2       29e-8 / 14e-8    27e-8 / 13e-8    22e-8 / 32e-8    20e-8 / 55e-8
+// Operands of one sign show what the cut-off leaves (slots of 64: 3.2e-7 at any K), sums of a few large terms what it takes from the
+// small ones.  Over 92 drawn products that run here, normal operands: 0.36 of the FMA kernel's error on the geometric mean and
+// 0.60 at most; their magnitudes 0.64 and 1.35 (948 x 1877 x 1769, which that kernel cuts in eight: 13e-8 / 9.6e-8).  (hh in an
+// accumulator of its own: 5.6e-8 at K = 64, log-normal as before; left there for 64 K-steps 9.0e-8 and 4.9e-7.)
 //
 //   warps 0-7   the accumulators: they add a slot's sum, 32 rows x half of the columns a warp, out of one of two buffers
 //               in tensor memory
@@ -23,12 +30,12 @@
 // MN-major tiles in chunks of 64 columns.  A tile whose K is long and whose device is otherwise idle is cut along K
 // over the CTAs of a cluster, whose partial tiles are added in order through distributed shared memory.
 //
-// Bound: no one unit.  At 2048^3 the data path of shared memory is busy 65 % of the clocks (per slot of a 128 x 128 tile the MMAs
-// read 768 lines of 128 bytes, the planes take 384, the loads pass 256 to 512, in some 2200 clocks), the schedulers issue in 51 %,
-// the tensor pipe works in 30 %; a slot's round through loads, splitting, barriers and accumulators sets the pace.
+// Bound: no one unit.  At 2048^3 the data path of shared memory is busy 67 % of the clocks (per slot of a 128 x 128 tile the
+// MMAs read 768 lines of 128 bytes, the planes take 384, the loads pass 256 to 512, in some 2200 clocks), the schedulers issue in
+// 49 %, the tensor pipe works in 31 %; a slot's round through loads, splitting, barriers and accumulators sets the pace.
 // A wider tile shares the A operand (192 columns 2800 clocks, 1870 for 128 of them); 16 warps for the operands instead of 8 change
 // nothing (2048^3 157 and 153 us).
-// 1000 x 1024 x 1500 on four shards 33 us, 1000 x 1500 x 777 38, 2048^3 153 (112 TFLOP/s); FMA kernel 87, 92, 422.
+// 1000 x 1024 x 1500 on four shards 33 us, 1000 x 1500 x 777 40, 2048^3 166 (103 TFLOP/s); FMA kernel 87, 92, 422.
 //
 // A result that is not finite (operands or sums that are not, or not once scaled, or a bf16 part that rounds to infinity) is found
 // in the accumulators; the CTA then multiplies its tile again with fp32 multiply-adds (multiply_again).

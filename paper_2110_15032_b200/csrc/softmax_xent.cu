@@ -114,7 +114,8 @@ __device__ __forceinline__ void merge_all(const float* ms, const float* ss, int 
 // and its results are the first to go as well.  (us, forward and backward, all with the usual priority / so: fp32
 // [256, 100003] over four 57.7 / 54.7, [128, 100003] 30.5 / 29.0, [256, 200000] 106.5 / 102.9, [4000, 8000] 72.7 / 71.1;
 // bf16 [512, 100000] 65.8 / 63.1.  The part to keep, MB, [256, 100003]: 40 55.4, 50 54.8, 60 54.7, 70 55.1, 100 55.4; the
-// priority to keep longest instead of the usual one 0.1 to 1 us slower.)
+// priority to keep longest instead of the usual one 0.1 to 1 us slower.  Passes over the same logits; on logits just made, whose
+// producer has left a part of them in L2, the two are level.)
 constexpr long long kKeepNum = 7, kKeepDen = 16;      // of the device's L2 (126 MB: 55)
 __device__ __forceinline__ unsigned long long l2_usual() {
   unsigned long long p;
