@@ -298,8 +298,8 @@ void sbp_boxing_set_copy_engine(int32_t engine);
  *              against exact ones, contractions of 64 to 2048, tensor cores / multiply-adds: operands of both signs 0.6 to 1.2e-7 /
  *              1.1 to 4.1e-7; of one sign 0.6 to 1.3e-7 / 0.6 to 2.6e-7 (at most 1.35 times as far, where multiply-adds are cut
  *              in eight chains); sums of which a few terms are most (log-normal factors, sigma 2) 2.0 to 2.9e-7 / 1.3 to 7e-7
- *              (twice as far up to a contraction of 128).  Products that touch what is not finite, operands from 2^88 or sums
- *              from 2^49 on take up to twice the time of multiply-adds alone.
+ *              (twice as far up to a contraction of 128).  Where operands or sums are not finite, or operands from 2^88 or sums from
+ *              2^49 on, tiles are multiplied twice: a product whose tiles all are takes 1.2 to 2.7 times as long as by multiply-adds.
  *   SBP_BF16 : bf16 operands, fp32 accumulation on the tensor cores, y SBP_BF16 or SBP_F32.
  * flags: SBP_EPILOGUE_GELU applies GeLU(v) = v/2 (1 + erf(v/sqrt 2)) to the fp32
  * accumulator before the store; only where Y is S or B (GeLU is not linear, so it cannot
