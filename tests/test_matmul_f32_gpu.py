@@ -1,7 +1,7 @@
-"""The fp32 MatMul kernel where it can go wrong: the edges of its two tile sizes, K-slices with a
+"""fp32 products on the kernel that the library picks, where they can go wrong: edges of tiles, K-slices with a
 remainder, contractions split over a cluster, chained segments of uneven and zero length, operands that
 miss the 16-byte rule, both stored forms of either operand.  Same oracle and the same bound
-(probabilistic bound on recursive summation) as the other fp32 products."""
+(probabilistic bound on recursive summation) as the other fp32 products.  test_matmul_f32_forms_gpu.py forces each kernel."""
 import pytest
 import torch
 

@@ -1,6 +1,6 @@
-"""The small fp32 products, whose eight warps share a 32 x 32 tile and cut its contraction between them: edges of the tile,
-contractions around one slice a warp, chained segments of uneven and zero length, both stored forms, rows off the 16-byte
-rule, replicas.  Oracle and bound as for the other fp32 products."""
+"""Small fp32 products on the kernel that the library picks for them, the small one or the tiled one: edges of the small kernel's
+32 x 32 tile, contractions around one slice a warp, chained segments of uneven length, both stored forms, rows off the 16-byte
+rule, replicas.  Oracle and bound as for the other fp32 products.  test_matmul_f32_forms_gpu.py forces each kernel."""
 import pytest
 import torch
 

@@ -1,6 +1,7 @@
 """fp32 products on the tensor cores where they can go wrong: edges of tiles and ring slots, chained segments of uneven
-and zero length, both stored forms of either operand, rows off the 16-byte rule, operands and sums that are not finite,
-numbers at the ends of the exponent range.  The shapes are such as the library's own choice sends there.  Oracle and bound
+length, both stored forms of either operand, rows off the 16-byte rule, operands and sums that are not finite,
+numbers at the ends of the exponent range.  The shapes are such as the library's own choice sends there (which
+test_matmul_f32_forms_gpu.py checks, beside shapes that are forced).  Oracle and bound
 as for the other fp32 products; the error against fp64 besides stays below what a chain of fp32 multiply-adds shows."""
 import pytest
 import torch
